@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -108,6 +109,23 @@ int tune_lookup(const std::string& key);
 void tune_store(const std::string& key, int choice);
 std::string tune_device_tag();
 
+// Twiddle tables of the line transforms (line.cuh) of one grid's axis lengths,
+// for both plans. kind 0: cx<T> entries; kind 1: paired entries (c, c, s, s)
+// in single precision, fixed-point words in double precision.
+template <typename T>
+class LineTables {
+ public:
+  explicit LineTables(const Grid& g);
+  ~LineTables();
+  LineTables(const LineTables&) = delete;
+  LineTables& operator=(const LineTables&) = delete;
+  const void* get(int L, bool narrow, int kind) const;
+
+ private:
+  unsigned char* dev_ = nullptr;
+  long off_[44];
+};
+
 // Batched power-of-two FFTs and Fourier multipliers on one grid, in precision T.
 template <typename T>
 class Spectral {
@@ -133,46 +151,23 @@ class Spectral {
   void fwd(const T* u, C* U);
   // packed spectrum -> real field (normalised by 1/N); U is overwritten
   void inv(C* U, T* u);
-  // G[i] = d/dx_i u, i < d  (first derivatives with the Nyquist mode dropped)
-  void grad(const T* u, T* G, C* U, C* W);
-  // out = sum_i d/dx_i q_i
-  void div(const T* q, T* out, C* U, C* S);
-  // W = i k~_axis U (W may equal U)
-  void mult_deriv(const C* U, C* W, int axis);
-  // S (+)= i k~_axis U
-  void mult_deriv_acc(const C* U, C* S, int axis, bool first);
-  // in place Leray projection of d spectra (stride Nc)
-  void mult_leray(C* W);
-
   const C* twiddles(int L) const;   // Stockham stage tables for length L
   const C* rc_twiddles() const;     // exp(-2 pi i k / L_last), k < M
-  // single precision, two-stage plans (L = 32..256): the stage-1 twiddle
-  // block of length L with each entry (c, s) stored as (c, c, s, s), for the
-  // paired column passes; null otherwise
-  const float4* pair_twiddles(int L) const;
-
-  // A second stream with a fork and a join event, for independent passes of
-  // one stage (created on first use).
-  cudaStream_t aux_stream();
-  cudaEvent_t fork_event() const { return ev_fork_; }
-  cudaEvent_t join_event() const { return ev_join_; }
+  const void* line_table(int L, bool narrow, int kind) const { return lines_->get(L, narrow, kind); }
 
  private:
   void cols(C* U, int axis, bool inverse);
   Grid g_;
   cudaStream_t s_;
-  cudaStream_t aux_ = nullptr;
-  cudaEvent_t ev_fork_ = nullptr, ev_join_ = nullptr;
   C* tw_ = nullptr;  // device: tables per length + real/complex table
-  float4* tw2_ = nullptr;  // device: paired twiddle blocks (single precision only)
-  long tw2_off_[11] = {0};
+  std::unique_ptr<LineTables<T>> lines_;
   bool owns_ = true;
   long tw_off_[11] = {0};  // offset of the table of length 2^e
   long rc_off_ = 0;
 };
 
 // ---------------------------------------------------------------------------
-// Fused Heun stages (fused.cuh): advection k = -v.grad u [- grad m . v~] and
+// Transport stages (stage.cuh): advection k = -v.grad u [- grad m . v~] and
 // divergence k = div(v lam), each with its Runge-Kutta update in the last pass.
 // ---------------------------------------------------------------------------
 // bounded waits of the TMA column pass that gave up since the last call
@@ -186,20 +181,16 @@ struct AdvEpi;
 template <typename T>
 struct DivEpi;
 }  // namespace fused
-// three packed-spectrum scratch buffers per call (Zx unused in 2D). u_ready:
-// U already holds the packed spectrum of u (no real-to-complex pass); emit:
-// the last pass leaves the packed spectrum of the stage's out1 in U.
+// gx, gy: scratch fields (gy unused in 2D)
 template <typename T>
-void adv_stage(Spectral<T>& sp, const T* u, const fused::AdvEpi<T>& e, cx<T>* U, cx<T>* Zx, cx<T>* Zy,
-               bool u_ready = false, bool emit = false);
-// two 3D advection stages (fields uA, uB) sharing their passes; Z: six
-// spectral work arrays of Nc values
+void adv_stage(Spectral<T>& sp, const T* u, const fused::AdvEpi<T>& e, T* gx, T* gy);
+// two 3D advection stages (fields uA, uB) sharing their launches; Z: four scratch fields
 template <typename T>
 void adv2_stage(Spectral<T>& sp, const T* uA, const fused::AdvEpi<T>& eA, const T* uB, const fused::AdvEpi<T>& eB,
-                cx<T>* const* Z);
+                T* const* Z);
 // a: d velocity fields at stride N
 template <typename T>
-void div_stage(Spectral<T>& sp, const T* lam, const T* a, const fused::DivEpi<T>& e, cx<T>* Q0, cx<T>* Q1, cx<T>* Q2);
+void div_stage(Spectral<T>& sp, const T* lam, const T* a, const fused::DivEpi<T>& e, T* kx, T* ky);
 
 // ---------------------------------------------------------------------------
 // Fourier-diagonal operators on whole coefficient vectors (FP64), with the

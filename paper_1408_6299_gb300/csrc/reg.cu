@@ -25,7 +25,7 @@
 
 #include "../../include/reg.h"
 #include "internal.h"
-#include "fused.cuh"
+#include "stage.cuh"
 #include "pointwise.h"
 
 using namespace reg;
@@ -101,9 +101,8 @@ bool invert_small(int n, const std::vector<double>& A, std::vector<double>& Ai) 
 // per-precision scratch of the sweeps
 template <typename T>
 struct Work {
-  using C = cx<T>;
-  DBuf<C> U, W, X;         // spectra
-  DBuf<C> U2, W2, X2;      // spectra of the second field of a two-field stage
+  DBuf<T> gx, gy;          // column derivatives of a stage
+  DBuf<T> gx2, gy2;        // and of the second field of a two-field stage
   DBuf<T> yhS, accS, srcS; // state stage values and one source of the fused forward sweep
   DBuf<T> G, q, va, vb, wa, wb;  // d fields
   DBuf<T> m, yh, acc, k, lam;    // fields
@@ -255,12 +254,6 @@ Spectral<float>& spectral<float>(reg_ctx* c) {
   return *c->sp32;
 }
 
-template <typename T>
-void grad_into(reg_ctx* c, const T* u, T* G) {
-  Work<T>& w = work<T>(c);
-  spectral<T>(c).grad(u, G, w.U.get(c->g.Nc), w.W.get(c->g.Nc));
-}
-
 // velocity (coefficients in precision T) at node j: a pointer to d fields
 template <typename T>
 const T* vel_node(reg_ctx* c, const T* coef, int j, T* buf) {
@@ -269,16 +262,12 @@ const T* vel_node(reg_ctx* c, const T* coef, int j, T* buf) {
   return buf;
 }
 
-// fused advection stage on u: k = -a.grad u [- gm.w], Heun stage update.
-// u_ready: w.U already holds the spectrum of u (left there by the previous
-// stage); emit: leave the spectrum of out1 in w.U for the next stage;
-// spec_only: out1 is needed only as that spectrum (no real store).
+// advection stage on u: k = -a.grad u [- gm.w], Heun stage update
 template <typename T>
 void adv(reg_ctx* c, const T* u, const T* a, const T* gm, const T* wv, const T* y, T* out1, T* out2, T* Gkeep,
-         int stage, const T* src = nullptr, const T* sw = nullptr, T* Sout = nullptr, bool u_ready = false,
-         bool emit = false, bool spec_only = false) {
+         int stage, const T* src = nullptr, const T* sw = nullptr, T* Sout = nullptr) {
   Work<T>& w = work<T>(c);
-  const long N = c->N(), Nc = c->g.Nc;
+  const long N = c->N();
   fused::AdvEpi<T> e{};
   for (int i = 0; i < c->d; ++i) {
     e.a[i] = a ? a + i * N : nullptr;
@@ -294,8 +283,7 @@ void adv(reg_ctx* c, const T* u, const T* a, const T* gm, const T* wv, const T* 
   e.out2 = out2;
   e.h = (T)c->h();
   e.stage = stage;
-  e.out1_spectral_only = spec_only ? 1 : 0;
-  adv_stage<T>(spectral<T>(c), u, e, w.U.get(Nc), w.W.get(Nc), w.X.get(Nc), u_ready, emit);
+  adv_stage<T>(spectral<T>(c), u, e, w.gx.get(N), c->d == 3 ? w.gy.get(N) : nullptr);
 }
 
 // epilogue of an advection stage without stored-gradient source terms
@@ -322,15 +310,15 @@ fused::AdvEpi<T> adv_epi(reg_ctx* c, const T* a, const T* y, T* out1, T* out2, i
 template <typename T>
 void adv2(reg_ctx* c, const T* uA, const fused::AdvEpi<T>& eA, const T* uB, const fused::AdvEpi<T>& eB) {
   Work<T>& w = work<T>(c);
-  const long Nc = c->g.Nc;
-  cx<T>* Z[6] = {w.U.get(Nc), w.W.get(Nc), w.X.get(Nc), w.U2.get(Nc), w.W2.get(Nc), w.X2.get(Nc)};
+  const long N = c->N();
+  T* Z[4] = {w.gx.get(N), w.gy.get(N), w.gx2.get(N), w.gy2.get(N)};
   adv2_stage<T>(spectral<T>(c), uA, eA, uB, eB, Z);
 }
 
-// grad u into G (d fields) through the fused stage passes
+// grad u into G (d fields) through the stage passes
 template <typename T>
-void grad_fused(reg_ctx* c, const T* u, T* G, bool u_ready = false) {
-  adv<T>(c, u, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, G, 1, nullptr, nullptr, nullptr, u_ready);
+void grad_fused(reg_ctx* c, const T* u, T* G) {
+  adv<T>(c, u, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, G, 1);
 }
 
 // fused divergence stage on lam: k = div(a lam), Heun stage update; e carries
@@ -339,13 +327,13 @@ template <typename T>
 void divh(reg_ctx* c, const T* lam, const T* a, const T* y, T* out1, T* out2, int stage,
           fused::DivEpi<T> e = fused::DivEpi<T>{}) {
   Work<T>& w = work<T>(c);
-  const long Nc = c->g.Nc;
+  const long N = c->N();
   e.y = y;
   e.out1 = out1;
   e.out2 = out2;
   e.h = (T)c->h();
   e.stage = stage;
-  div_stage<T>(spectral<T>(c), lam, a, e, w.U.get(Nc), w.W.get(Nc), w.X.get(Nc));
+  div_stage<T>(spectral<T>(c), lam, a, e, w.gx.get(N), c->d == 3 ? w.gy.get(N) : nullptr);
 }
 
 // ---------------------------------------------------------------------------
@@ -359,29 +347,22 @@ template <typename T>
 void state_steps(reg_ctx* c, const T* vcoef, int j0, int j1, T* gm, T* gmh, int base, T* ck) {
   Work<T>& w = work<T>(c);
   const long N = c->N(), dN = c->dN();
-  const T h = (T)c->h();
   T* m = w.m.get(N);
   T* yh = w.yh.get(N);
   T* acc = w.acc.get(N);
-  T* G = w.G.get(dN);
   T* va = w.va.get(dN);
   T* vb = w.vb.get(dN);
-  // each stage leaves the spectrum of its out1 in w.U for the next one; the
-  // predictor yh is needed only as that spectrum
-  bool ready = false;
   for (int j = j0; j < j1; ++j) {
     if (ck && c->ckpt > 0 && j % c->ckpt == 0)
       REG_CUDA(cudaMemcpyAsync(ck + (long)(j / c->ckpt) * N, m, N * sizeof(T), cudaMemcpyDeviceToDevice, c->s));
     adv<T>(c, m, vel_node<T>(c, vcoef, j, va), nullptr, nullptr, m, yh, acc, gm ? gm + (long)(j - base) * dN : nullptr,
-           1, nullptr, nullptr, nullptr, ready, true, true);
-    const bool more = j + 1 < j1 || gm;  // the spectrum of m is read next
+           1);
     adv<T>(c, yh, vel_node<T>(c, vcoef, j + 1, vb), nullptr, nullptr, acc, m, nullptr,
-           gmh ? gmh + (long)(j + 1 - base) * dN : nullptr, 2, nullptr, nullptr, nullptr, true, more);
-    ready = more;
+           gmh ? gmh + (long)(j + 1 - base) * dN : nullptr, 2);
   }
   if (ck && c->ckpt > 0 && j1 % c->ckpt == 0)
     REG_CUDA(cudaMemcpyAsync(ck + (long)(j1 / c->ckpt) * N, m, N * sizeof(T), cudaMemcpyDeviceToDevice, c->s));
-  if (gm) grad_fused<T>(c, m, gm + (long)(j1 - base) * dN, ready);
+  if (gm) grad_fused<T>(c, m, gm + (long)(j1 - base) * dN);
 }
 
 // Recompute state gradients of segment [j0, j1] from the checkpoint at j0.
@@ -410,16 +391,13 @@ void recompute_segment_src(reg_ctx* c, const T* vcoef, const T* wcoef, int j0, i
   T* wa = w.wa.get(dN);
   T* src = w.src.get((size_t)(c->ckpt + 1) * N);
   REG_CUDA(cudaMemcpyAsync(m, w.ck.p + (long)(j0 / c->ckpt) * N, N * sizeof(T), cudaMemcpyDeviceToDevice, c->s));
-  bool ready = false;  // w.U holds the spectrum of m
   for (int j = j0; j < j1; ++j) {
     adv<T>(c, m, vel_node<T>(c, vcoef, j, va), nullptr, nullptr, m, yh, acc, nullptr, 1, nullptr,
-           vel_node<T>(c, wcoef, j, wa), src + (long)(j - j0) * N, ready, true, true);
-    adv<T>(c, yh, vel_node<T>(c, vcoef, j + 1, vb), nullptr, nullptr, acc, m, nullptr, nullptr, 2, nullptr, nullptr,
-           nullptr, true, true);
-    ready = true;
+           vel_node<T>(c, wcoef, j, wa), src + (long)(j - j0) * N);
+    adv<T>(c, yh, vel_node<T>(c, vcoef, j + 1, vb), nullptr, nullptr, acc, m, nullptr, nullptr, 2);
   }
   adv<T>(c, m, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 1, nullptr,
-         vel_node<T>(c, wcoef, j1, wa), src + (long)(j1 - j0) * N, ready);
+         vel_node<T>(c, wcoef, j1, wa), src + (long)(j1 - j0) * N);
 }
 
 // Gradient slots available for node j (after ensure_segment)
@@ -637,8 +615,7 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
         const T* wA = vel_node<T>(c, wcoef, j, wa);
         fused::AdvEpi<T> sA = adv_epi<T>(c, vA, m, yhS, accS, 1, nullptr, wA, sj);
         if (j == 0) {
-          // the state's stage 1 leaves the spectrum of yhS for its stage 2
-          adv<T>(c, m, vA, nullptr, nullptr, m, yhS, accS, nullptr, 1, nullptr, wA, sj, false, true, true);
+          adv<T>(c, m, vA, nullptr, nullptr, m, yhS, accS, nullptr, 1, nullptr, wA, sj);
         } else {
           fused::AdvEpi<T> iB = adv_epi<T>(c, vA, acc, y, nullptr, 2);
           iB.src_from_a = 1;
@@ -648,7 +625,7 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
         }
         const T* vB = vel_node<T>(c, vcoef, j + 1, vb);
         if (j == 0) {
-          adv<T>(c, yhS, vB, nullptr, nullptr, accS, m, nullptr, nullptr, 2, nullptr, nullptr, nullptr, true);
+          adv<T>(c, yhS, vB, nullptr, nullptr, accS, m, nullptr, nullptr, 2);
           lincomb_t<T>(-h, sj, (T)0, nullptr, yh, N, c->s);
           lincomb_t<T>((T)(-0.5) * h, sj, (T)0, nullptr, acc, N, c->s);
         } else {
@@ -668,10 +645,6 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
     if (mtil)
       REG_CUDA(cudaMemcpyAsync(mtil + (long)c->n_t * N, y, N * sizeof(T), cudaMemcpyDeviceToDevice, c->s));
   }
-  // each stage leaves the spectrum of its out1 in w.U for the next one (the
-  // state re-advance of a segment overwrites it); the predictor yh is needed
-  // only as that spectrum
-  bool ready = false;
   for (int seg = 0; seg * K < c->n_t && !(use_src && c->ckpt > 0 && c->d == 3); ++seg) {
     int j0 = seg * K, j1 = j0 + K;
     int base = 0;
@@ -679,12 +652,9 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
       if (use_src) recompute_segment_src<T>(c, vcoef, wcoef, j0, j1);
       else recompute_segment<T>(c, vcoef, j0, j1);
       base = j0;
-      ready = false;
     }
     for (int j = j0; j < j1; ++j) {
       const T* vA = vel_node<T>(c, vcoef, j, va);
-      const bool more = j + 1 < j1;  // the next stage of this segment reads the spectrum of y
-      const bool yh_ready = j > 0;
       if (use_src) {
         const T* s1 = w.src.p + (long)(j - base) * N;
         const T* s2 = w.src.p + (long)(j + 1 - base) * N;
@@ -692,10 +662,9 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
           lincomb_t<T>(-h, s1, (T)0, nullptr, yh, N, c->s);
           lincomb_t<T>((T)(-0.5) * h, s1, (T)0, nullptr, acc, N, c->s);
         } else {
-          adv<T>(c, y, vA, nullptr, nullptr, y, yh, acc, nullptr, 1, s1, nullptr, nullptr, ready, true, true);
+          adv<T>(c, y, vA, nullptr, nullptr, y, yh, acc, nullptr, 1, s1);
         }
-        adv<T>(c, yh, vel_node<T>(c, vcoef, j + 1, vb), nullptr, nullptr, acc, y, nullptr, nullptr, 2, s2, nullptr,
-               nullptr, yh_ready, more);
+        adv<T>(c, yh, vel_node<T>(c, vcoef, j + 1, vb), nullptr, nullptr, acc, y, nullptr, nullptr, 2, s2);
         if (mtil)
           REG_CUDA(cudaMemcpyAsync(mtil + (long)(j + 1) * N, y, N * sizeof(T), cudaMemcpyDeviceToDevice, c->s));
       } else {
@@ -705,12 +674,11 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
         if (j == 0) {
           transport_stage1<T>(nullptr, vA, g1, wA, nullptr, h, yh, acc, c->d, N, c->s);
         } else {
-          adv<T>(c, y, vA, g1, wA, y, yh, acc, nullptr, 1, nullptr, nullptr, nullptr, ready, true, true);
+          adv<T>(c, y, vA, g1, wA, y, yh, acc, nullptr, 1);
         }
         adv<T>(c, yh, vel_node<T>(c, vcoef, j + 1, vb), g2, vel_node<T>(c, wcoef, j + 1, wb), acc, y, nullptr,
-               nullptr, 2, nullptr, nullptr, nullptr, yh_ready, more);
+               nullptr, 2);
       }
-      ready = more;
     }
   }
   // lam~_1 = -m~_1
@@ -847,16 +815,16 @@ void hessvec_body(reg_ctx* c, const double* vt, double* out) {
 // graph would read or write stale memory and must be captured again
 size_t graph_signature(reg_ctx* c) {
   const void* ptrs[] = {c->f.p,        c->SV.p,       c->SF.p,       c->vlin.p,     c->gdir.p,     c->gout.p,
-                        c->w64.U.p,    c->w64.W.p,    c->w64.X.p,    c->w64.m.p,    c->w64.yh.p,   c->w64.acc.p,
+                        c->w64.gx.p,   c->w64.gy.p,    c->w64.m.p,    c->w64.yh.p,   c->w64.acc.p,
                         c->w64.lam.p,  c->w64.va.p,   c->w64.vb.p,   c->w64.wa.p,   c->w64.wb.p,   c->w64.gm.p,
-                        c->w64.gmh.p,  c->w64.ck.p,   c->w32.U.p,    c->w32.W.p,    c->w32.X.p,    c->w32.m.p,
+                        c->w64.gmh.p,  c->w64.ck.p,   c->w32.gx.p,   c->w32.gy.p,    c->w32.m.p,
                         c->w32.yh.p,   c->w32.acc.p,  c->w32.lam.p,  c->w32.va.p,   c->w32.vb.p,   c->w32.wa.p,
                         c->w32.wb.p,   c->w32.gm.p,   c->w32.gmh.p,  c->w32.ck.p,   c->w32.vcoef.p, c->w32.wcoef.p,
                         c->w32.fhi.p,  c->w32.flo.p,  c->w64.G.p,    c->w32.G.p,    c->w64.src.p,  c->w32.src.p,
                         c->w64.mtil.p, c->w32.mtil.p, c->w64.lamN.p, c->w32.lamN.p, c->w64.yh2.p, c->w32.yh2.p,
                         c->w64.acc2.p, c->w32.acc2.p, c->w64.st0.p,  c->w32.st0.p,  c->w64.st1.p,  c->w32.st1.p,
-                        c->w64.Gt.p,   c->w32.Gt.p,   c->w64.U2.p,   c->w32.U2.p,   c->w64.W2.p,   c->w32.W2.p,
-                        c->w64.X2.p,   c->w32.X2.p,   c->w64.yhS.p,  c->w32.yhS.p,  c->w64.accS.p, c->w32.accS.p,
+                        c->w64.Gt.p,   c->w32.Gt.p,   c->w64.gx2.p,  c->w32.gx2.p,  c->w64.gy2.p,  c->w32.gy2.p,
+                        c->w64.yhS.p,  c->w32.yhS.p,  c->w64.accS.p, c->w32.accS.p,
                         c->w64.srcS.p, c->w32.srcS.p};
   size_t h = 1469598103934665603ull;
   for (const void* p : ptrs) h = (h ^ (size_t)p) * 1099511628211ull;
@@ -941,7 +909,7 @@ double* defgrad(reg_ctx* c, const double* v, int substeps) {
   const long ddN = (long)dd * N;
   double* gvl = c->gvl.get((size_t)nc * ddN);
   for (int l = 0; l < nc; ++l)
-    for (int i = 0; i < d; ++i) grad_into<double>(c, v + ((long)l * d + i) * N, gvl + ((long)l * dd + i * d) * N);
+    for (int i = 0; i < d; ++i) grad_fused<double>(c, v + ((long)l * d + i) * N, gvl + ((long)l * dd + i * d) * N);
   double* F = c->F.get(ddN);
   double* Fh = c->Fh.get(ddN);
   double* K1 = c->K1.get(ddN);
@@ -967,7 +935,7 @@ double* defgrad(reg_ctx* c, const double* v, int substeps) {
       const double* Fin = stage ? Fh : F;
       double* Kout = stage ? K2 : K1;
       for (int q = 0; q < dd; ++q) {
-        grad_into<double>(c, Fin + q * N, G);
+        grad_fused<double>(c, Fin + q * N, G);
         detF_rhs(G, vv, gg, Fin, q, Kout, d, N, c->s);
       }
       if (stage == 0) {

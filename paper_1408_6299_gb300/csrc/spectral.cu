@@ -15,7 +15,7 @@
 #include <atomic>
 #include <stdexcept>
 
-#include "internal.h"
+#include "tune.h"
 
 namespace reg {
 
@@ -174,42 +174,6 @@ __device__ inline long encode_neg(long q0, const ModeIdx& m, const GridArgs& g) 
 __device__ inline double masked_k(const ModeIdx& m, const GridArgs& g, int a) {
   if (a == g.d - 1) return (double)m.j[a];  // slot 0 -> 0 for both DC and Nyquist halves
   return (double)kmask(m.j[a], g.n[a]);
-}
-
-template <typename T>
-__global__ void k_mult_deriv(const cx<T>* __restrict__ U, cx<T>* __restrict__ W, GridArgs g, int axis, int acc) {
-  long q = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= g.Nc) return;
-  ModeIdx m = decode(q, g.d, g.n, g.M);
-  T k = (T)masked_k(m, g, axis);
-  cx<T> u = U[q];
-  cx<T> r = mk<cx<T>>(-k * u.y, k * u.x);
-  if (acc) r = cadd(W[q], r);
-  W[q] = r;
-}
-
-template <typename T>
-__global__ void k_mult_leray(cx<T>* __restrict__ W, GridArgs g) {
-  long q = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= g.Nc) return;
-  ModeIdx m = decode(q, g.d, g.n, g.M);
-  T k[3];
-  T kk = 0;
-  for (int a = 0; a < g.d; ++a) {
-    k[a] = (T)masked_k(m, g, a);
-    kk += k[a] * k[a];
-  }
-  if (kk == (T)0) return;
-  T dr = 0, di = 0;
-  for (int a = 0; a < g.d; ++a) {
-    cx<T> w = W[a * g.Nc + q];
-    dr += k[a] * w.x;
-    di += k[a] * w.y;
-  }
-  for (int a = 0; a < g.d; ++a) {
-    cx<T> w = W[a * g.Nc + q];
-    W[a * g.Nc + q] = mk<cx<T>>(w.x - k[a] * dr / kk, w.y - k[a] * di / kk);
-  }
 }
 
 // |k|^2 over the leading axes (full wavenumbers, Nyquist kept)
@@ -404,19 +368,30 @@ void launch_rows(bool inverse, const void* in, void* out, long nrows, const cx<T
   REG_LAUNCH();
 }
 
+// tune: the autotuner may halve the rows per block of the real-to-complex pass
+template <typename T, int L, int RB>
+void tuned_rows(bool inverse, const void* in, void* out, long nrows, const cx<T>* tw, const cx<T>* twrc,
+                cudaStream_t s, bool tune) {
+  auto run = [&](int v) {
+    if (v == 0) launch_rows<T, L, RB>(inverse, in, out, nrows, tw, twrc, s);
+    else launch_rows<T, L, RB / 2>(inverse, in, out, nrows, tw, twrc, s);
+  };
+  run(!inverse && tune ? tuned_choice("rows_r2c", sizeof(T), L, tune_size(nrows), 2, s, run) : 0);
+}
+
 template <typename T>
 void dispatch_rows(int L, bool inverse, const void* in, void* out, long nrows, const cx<T>* tw,
-                   const cx<T>* twrc, cudaStream_t s) {
+                   const cx<T>* twrc, cudaStream_t s, bool tune) {
   // about 2048 (fp32) / 1024 (fp64) complex values per block
   constexpr int E = sizeof(T) == 4 ? 2048 : 1024;
   switch (L) {
-    case 8: return launch_rows<T, 8, E / 4>(inverse, in, out, nrows, tw, twrc, s);
-    case 16: return launch_rows<T, 16, E / 8>(inverse, in, out, nrows, tw, twrc, s);
-    case 32: return launch_rows<T, 32, E / 16>(inverse, in, out, nrows, tw, twrc, s);
-    case 64: return launch_rows<T, 64, E / 32>(inverse, in, out, nrows, tw, twrc, s);
-    case 128: return launch_rows<T, 128, E / 64>(inverse, in, out, nrows, tw, twrc, s);
-    case 256: return launch_rows<T, 256, E / 128>(inverse, in, out, nrows, tw, twrc, s);
-    case 512: return launch_rows<T, 512, E / 256>(inverse, in, out, nrows, tw, twrc, s);
+    case 8: return tuned_rows<T, 8, E / 4>(inverse, in, out, nrows, tw, twrc, s, tune);
+    case 16: return tuned_rows<T, 16, E / 8>(inverse, in, out, nrows, tw, twrc, s, tune);
+    case 32: return tuned_rows<T, 32, E / 16>(inverse, in, out, nrows, tw, twrc, s, tune);
+    case 64: return tuned_rows<T, 64, E / 32>(inverse, in, out, nrows, tw, twrc, s, tune);
+    case 128: return tuned_rows<T, 128, E / 64>(inverse, in, out, nrows, tw, twrc, s, tune);
+    case 256: return tuned_rows<T, 256, E / 128>(inverse, in, out, nrows, tw, twrc, s, tune);
+    case 512: return tuned_rows<T, 512, E / 256>(inverse, in, out, nrows, tw, twrc, s, tune);
   }
   throw StatusError{1, "unsupported last-axis length " + std::to_string(L)};
 }
@@ -499,18 +474,7 @@ Spectral<T>::Spectral(const Grid& g, cudaStream_t s) : g_(g), s_(s) {
   for (size_t i = 0; i < all.size(); ++i) h[i] = (T)all[i];
   REG_CUDA(cudaMalloc(&tw_, h.size() * sizeof(T)));
   REG_CUDA(cudaMemcpy(tw_, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice));
-  if (sizeof(T) == 4) {
-    // the two-stage plans' stage-1 blocks (L = 32..256) with duplicated entries
-    std::vector<float4> p2;
-    for (int e = 5; e <= 8; ++e) {
-      tw2_off_[e] = (long)p2.size();
-      std::vector<double> t = stage_table(1 << e);
-      for (size_t i = 0; i + 1 < t.size(); i += 2)
-        p2.push_back(make_float4((float)t[i], (float)t[i], (float)t[i + 1], (float)t[i + 1]));
-    }
-    REG_CUDA(cudaMalloc(&tw2_, p2.size() * sizeof(float4)));
-    REG_CUDA(cudaMemcpy(tw2_, p2.data(), p2.size() * sizeof(float4), cudaMemcpyHostToDevice));
-  }
+  lines_.reset(new LineTables<T>(g));
 }
 
 template <typename T>
@@ -565,20 +529,6 @@ long Spectral<T>::write_tables(double* out, long* tw_off, long* rc_off) {
 template <typename T>
 Spectral<T>::~Spectral() {
   if (tw_ && owns_) cudaFree(tw_);
-  if (tw2_ && owns_) cudaFree(tw2_);
-  if (ev_fork_) cudaEventDestroy(ev_fork_);
-  if (ev_join_) cudaEventDestroy(ev_join_);
-  if (aux_) cudaStreamDestroy(aux_);
-}
-
-template <typename T>
-cudaStream_t Spectral<T>::aux_stream() {
-  if (!aux_) {
-    REG_CUDA(cudaEventCreateWithFlags(&ev_fork_, cudaEventDisableTiming));
-    REG_CUDA(cudaEventCreateWithFlags(&ev_join_, cudaEventDisableTiming));
-    REG_CUDA(cudaStreamCreateWithFlags(&aux_, cudaStreamNonBlocking));
-  }
-  return aux_;
 }
 
 template <typename T>
@@ -590,12 +540,6 @@ const cx<T>* Spectral<T>::rc_twiddles() const {
   return tw_ + rc_off_;
 }
 template <typename T>
-const float4* Spectral<T>::pair_twiddles(int L) const {
-  if (!tw2_ || L < 32 || L > 256) return nullptr;
-  return tw2_ + tw2_off_[ilog2(L)];
-}
-
-template <typename T>
 void Spectral<T>::cols(C* U, int axis, bool inverse) {
   long s = g_.M;
   for (int a = axis + 1; a < g_.d - 1; ++a) s *= g_.n[a];
@@ -605,52 +549,14 @@ void Spectral<T>::cols(C* U, int axis, bool inverse) {
 
 template <typename T>
 void Spectral<T>::fwd(const T* u, C* U) {
-  dispatch_rows<T>(g_.L, false, u, U, g_.rows, twiddles(g_.M), rc_twiddles(), s_);
+  dispatch_rows<T>(g_.L, false, u, U, g_.rows, twiddles(g_.M), rc_twiddles(), s_, owns_);
   for (int a = g_.d - 2; a >= 0; --a) cols(U, a, false);
 }
 
 template <typename T>
 void Spectral<T>::inv(C* U, T* u) {
   for (int a = 0; a <= g_.d - 2; ++a) cols(U, a, true);
-  dispatch_rows<T>(g_.L, true, U, u, g_.rows, twiddles(g_.M), rc_twiddles(), s_);
-}
-
-template <typename T>
-void Spectral<T>::mult_deriv(const C* U, C* W, int axis) {
-  ProfScope ps(KK_MULT, s_, 2.0 * g_.Nc * sizeof(C));
-  k_mult_deriv<T><<<blocks_for(g_.Nc), 256, 0, s_>>>(U, W, args(g_), axis, 0);
-  REG_LAUNCH();
-}
-
-template <typename T>
-void Spectral<T>::mult_deriv_acc(const C* U, C* S, int axis, bool first) {
-  ProfScope ps(KK_MULT, s_, (first ? 2.0 : 3.0) * g_.Nc * sizeof(C));
-  k_mult_deriv<T><<<blocks_for(g_.Nc), 256, 0, s_>>>(U, S, args(g_), axis, first ? 0 : 1);
-  REG_LAUNCH();
-}
-
-template <typename T>
-void Spectral<T>::mult_leray(C* W) {
-  k_mult_leray<T><<<blocks_for(g_.Nc), 256, 0, s_>>>(W, args(g_));
-  REG_LAUNCH();
-}
-
-template <typename T>
-void Spectral<T>::grad(const T* u, T* G, C* U, C* W) {
-  fwd(u, U);
-  for (int i = 0; i < g_.d; ++i) {
-    mult_deriv(U, W, i);
-    inv(W, G + (long)i * g_.N);
-  }
-}
-
-template <typename T>
-void Spectral<T>::div(const T* q, T* out, C* U, C* S) {
-  for (int i = 0; i < g_.d; ++i) {
-    fwd(q + (long)i * g_.N, U);
-    mult_deriv_acc(U, S, i, i == 0);
-  }
-  inv(S, out);
+  dispatch_rows<T>(g_.L, true, U, u, g_.rows, twiddles(g_.M), rc_twiddles(), s_, owns_);
 }
 
 template class Spectral<float>;

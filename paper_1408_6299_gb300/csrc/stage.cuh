@@ -1,0 +1,526 @@
+// stage.cuh -- transport stages of the Heun sweeps (Mang & Biros, Eq.
+// first-order-forward / first-order-adjoint / gauss-newton, Sec. 3.3.1).
+//
+// A stage is one launch of column passes and one row pass:
+//   columns  the derivatives along the strided axes, each field (or product of
+//            two fields) read once and its derivative written once;
+//   rows     the derivative along the contiguous last axis, and with it the
+//            stage's pointwise epilogue, which reads the column derivatives:
+//     advection  k = -v . grad u [- grad m . v~], Heun update, optional store of grad u
+//     divergence k = div(v lam),                  Heun update, body-force accumulation
+// Both work on real fields: two neighbouring real lines form one complex line
+// (line.cuh). Spectra are never stored.
+#pragma once
+#include <cuda.h>
+
+#include "internal.h"
+#include "fixed.cuh"
+#include "line.cuh"
+
+namespace reg {
+namespace fused {
+
+// Epilogue parameters of the advection stage (state / incremental state).
+template <typename T>
+struct AdvEpi {
+  const T* a[3];   // velocity components at the stage time
+  const T* gm[3];  // source: grad m at the stage time (null: no source)
+  const T* w[3];   // source: incremental velocity at the stage time
+  const T* y;      // stage 1: y_j (null = 0); stage 2: acc
+  T* out1;         // stage 1: y_j + h k; stage 2: acc + h/2 k (null: only keep grad u)
+  T* out2;         // stage 1: y_j + h/2 k
+  T* G[3];         // optional: keep grad u (null: not stored)
+  const T* src;    // optional precomputed source sum_i gm_i w_i (used instead of gm/w)
+  const T* sw[3];  // optional: with Sout, store Sout = sum_i (grad u)_i sw_i
+  T* Sout;
+  T h;
+  int stage;
+  int src_from_a;  // two-field stage, second field: the source is the first field's Sout value
+  int a_from_a;    // two-field stage, second field: same velocity as the first (reuse its loaded values)
+};
+
+// Epilogue parameters of the divergence stage (adjoint / incremental adjoint).
+// Stage 1 can also accumulate the body force f_l,i += cA_l y gmA_i (+ cB_l out1
+// gmB_i): the trapezoid term of node j+1, or the two stage terms of the
+// discrete adjoint. The accumulator is f_hi (+ f_lo) with layout [n_c][d][N];
+// with f_lo set, (f_hi, f_lo) is a compensated pair (exact two-sum per add).
+// Stage 0 only evaluates: out1 = div(v lam) (+ src). src (optional) is added
+// to the divergence (the div(v~ lam) source of the full Newton incremental
+// adjoint). gmC/yC (optional) add the Newton force term cA_l yC gmC_i.
+template <typename T>
+struct DivEpi {
+  const T* y;  // stage 1: lam_{j+1}; stage 2: acc
+  T* out1;
+  T* out2;
+  T h;
+  int stage;
+  T* f_hi;          // null: no force accumulation
+  T* f_lo;          // null: plain accumulation into f_hi
+  const T* gmA;     // d fields at stride N
+  const T* gmB;     // d fields or null
+  T cA[16], cB[16]; // per-coefficient weights
+  int nc, d;
+  long N;
+  const T* src;     // added to the divergence
+  const T* gmC;     // d fields or null
+  const T* yC;
+};
+
+// Advection epilogue on the point pair q with the gradient components g[0..D)
+// (-a.g [- source], Heun update, optional keep of g or of g.sw). srcv, when
+// given, is the source value instead of e.src. Returns the Sout value.
+// av_in: the velocity values at q (null: load them); av_out: receives the
+// loaded velocity values when the Heun update ran.
+template <typename T, int D>
+__device__ __forceinline__ cx<T> adv_point(const AdvEpi<T>& e, const cx<T>* g, long q, const cx<T>* srcv,
+                                           const cx<T>* av_in = nullptr, cx<T>* av_out = nullptr) {
+  using C = cx<T>;
+  C so = mk<C>(0, 0);
+  if (e.G[0]) {
+#pragma unroll
+    for (int f = 0; f < D; ++f) reinterpret_cast<C*>(e.G[f])[q] = g[f];
+  }
+  if (e.Sout) {
+    T s0 = 0, s1 = 0;
+#pragma unroll
+    for (int f = 0; f < D; ++f) {
+      C w = reinterpret_cast<const C*>(e.sw[f])[q];
+      s0 += g[f].x * w.x;
+      s1 += g[f].y * w.y;
+    }
+    so = mk<C>(s0, s1);
+    reinterpret_cast<C*>(e.Sout)[q] = so;
+  }
+  if (!e.out1) return so;
+  T k0 = 0, k1 = 0;
+#pragma unroll
+  for (int f = 0; f < D; ++f) {
+    C a = av_in ? av_in[f] : reinterpret_cast<const C*>(e.a[f])[q];
+    if (av_out) av_out[f] = a;
+    k0 -= a.x * g[f].x;
+    k1 -= a.y * g[f].y;
+  }
+  if (srcv) {
+    k0 -= srcv->x;
+    k1 -= srcv->y;
+  } else if (e.src) {
+    C sv = reinterpret_cast<const C*>(e.src)[q];
+    k0 -= sv.x;
+    k1 -= sv.y;
+  } else if (e.gm[0]) {
+#pragma unroll
+    for (int f = 0; f < D; ++f) {
+      C gm = reinterpret_cast<const C*>(e.gm[f])[q];
+      C w = reinterpret_cast<const C*>(e.w[f])[q];
+      k0 -= gm.x * w.x;
+      k1 -= gm.y * w.y;
+    }
+  }
+  C r1;
+  if (e.stage == 1) {
+    C yv = e.y ? reinterpret_cast<const C*>(e.y)[q] : mk<C>(0, 0);
+    r1 = mk<C>(yv.x + e.h * k0, yv.y + e.h * k1);
+    reinterpret_cast<C*>(e.out2)[q] = mk<C>(yv.x + (T)0.5 * e.h * k0, yv.y + (T)0.5 * e.h * k1);
+  } else {
+    C yv = reinterpret_cast<const C*>(e.y)[q];
+    r1 = mk<C>(yv.x + (T)0.5 * e.h * k0, yv.y + (T)0.5 * e.h * k1);
+  }
+  reinterpret_cast<C*>(e.out1)[q] = r1;
+  return so;
+}
+
+// Divergence epilogue on the point pair q with the divergence value k (scaled,
+// real space): Heun stage update and, in stage 1, the optional body-force
+// accumulation (see DivEpi).
+template <typename T>
+__device__ __forceinline__ void div_point(const DivEpi<T>& dv, cx<T> k, long q) {
+  using C = cx<T>;
+  if (dv.src) {
+    C sv = reinterpret_cast<const C*>(dv.src)[q];
+    k = mk<C>(k.x + sv.x, k.y + sv.y);
+  }
+  if (dv.stage == 0) {
+    reinterpret_cast<C*>(dv.out1)[q] = k;
+    return;
+  }
+  C yv = reinterpret_cast<const C*>(dv.y)[q];
+  if (dv.stage != 1) {
+    reinterpret_cast<C*>(dv.out1)[q] = mk<C>(yv.x + (T)0.5 * dv.h * k.x, yv.y + (T)0.5 * dv.h * k.y);
+    return;
+  }
+  C o1 = mk<C>(yv.x + dv.h * k.x, yv.y + dv.h * k.y);
+  reinterpret_cast<C*>(dv.out1)[q] = o1;
+  reinterpret_cast<C*>(dv.out2)[q] = mk<C>(yv.x + (T)0.5 * dv.h * k.x, yv.y + (T)0.5 * dv.h * k.y);
+  if (!dv.f_hi) return;
+  // products of the point pair with every component, then per coefficient
+  // all loads before any store
+  C ta[3], tb[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    ta[i] = tb[i] = mk<C>(0, 0);
+    if (i < dv.d) {
+      C ga = reinterpret_cast<const C*>(dv.gmA + i * dv.N)[q];
+      ta[i] = mk<C>(yv.x * ga.x, yv.y * ga.y);
+      if (dv.gmC) {
+        C gc = reinterpret_cast<const C*>(dv.gmC + i * dv.N)[q];
+        C yc = reinterpret_cast<const C*>(dv.yC)[q];
+        ta[i] = mk<C>(ta[i].x + yc.x * gc.x, ta[i].y + yc.y * gc.y);
+      }
+      if (dv.gmB) {
+        C gb = reinterpret_cast<const C*>(dv.gmB + i * dv.N)[q];
+        tb[i] = mk<C>(o1.x * gb.x, o1.y * gb.y);
+      }
+    }
+  }
+  for (int l = 0; l < dv.nc; ++l) {
+    C hi[3], lo[3];
+    C* Hf = reinterpret_cast<C*>(dv.f_hi + (long)l * dv.d * dv.N);
+    C* Lo = dv.f_lo ? reinterpret_cast<C*>(dv.f_lo + (long)l * dv.d * dv.N) : nullptr;
+    const long hN = dv.N / 2;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      if (i < dv.d) {
+        hi[i] = Hf[i * hN + q];
+        lo[i] = Lo ? Lo[i * hN + q] : mk<C>(0, 0);
+      }
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      if (i < dv.d) {
+        T t0 = dv.cA[l] * ta[i].x + dv.cB[l] * tb[i].x;
+        T t1 = dv.cA[l] * ta[i].y + dv.cB[l] * tb[i].y;
+        if (Lo) {
+          C h = hi[i];
+          T s0 = h.x + t0, b0 = s0 - h.x, s1 = h.y + t1, b1 = s1 - h.y;
+          lo[i].x += (h.x - (s0 - b0)) + (t0 - b0);
+          lo[i].y += (h.y - (s1 - b1)) + (t1 - b1);
+          Hf[i * hN + q] = mk<C>(s0, s1);
+          Lo[i * hN + q] = lo[i];
+        } else {
+          Hf[i * hN + q] = mk<C>(hi[i].x + t0, hi[i].y + t1);
+        }
+      }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Column passes
+// ---------------------------------------------------------------------------
+constexpr int kColJobs = 4;
+// Up to four derivative passes along axes of the same length L: out = D in, or
+// D (in mul). s: distance of two line elements (complex values, a power of
+// two); n: complex lines of the field (the pairs of neighbouring real lines).
+template <typename T>
+struct ColJobs {
+  const T* in[kColJobs];
+  const T* mul[kColJobs];
+  T* out[kColJobs];
+  int log2s[kColJobs];
+  int start[kColJobs + 1];  // first block of each job; start[nj] = all blocks
+  int nj;
+  int n;
+};
+
+// Threads of a block: TS along a line times TC neighbouring lines (128-byte
+// row segments where the block allows it). VAR: 0, or 1 for the other block
+// size the autotuner may choose; both give the same bits.
+template <class A, int L, bool NARROW, int VAR>
+struct ColTile {
+  static constexpr int TS = LinePlan<L, NARROW>::TS;
+  static constexpr int LINE = L * (int)sizeof(typename A::V);  // shared bytes of a line
+  static constexpr int NT0 = (NARROW ? 64 : (sizeof(typename A::V) == 8 ? 256 : 128)) * (VAR ? (NARROW ? 2 : 1) : 1) /
+                             (VAR && !NARROW ? 2 : 1);
+  static constexpr int MINTC = NARROW ? 4 : (VAR ? 4 : 8);
+  static constexpr int TC1 = NT0 / TS < MINTC ? MINTC : NT0 / TS;
+  static constexpr int fit(int tc) { return tc * LINE <= 49152 ? tc : fit(tc / 2); }  // 48 KB of shared memory
+  static constexpr int TC = fit(TC1);
+  static constexpr int NT = TC * TS;
+};
+
+// the largest mag of the TS threads (c, j), j < TS, of a column; thread c + j TC
+// of the block holds (c, j). red: scratch, free again after the next barrier.
+template <int TC, int TS>
+__device__ __forceinline__ unsigned line_max(unsigned mag, unsigned* red, int c, int j) {
+  if constexpr (TS == 1) {
+    return mag;
+  } else {
+#pragma unroll
+    for (int o = TC; o < 32; o *= 2) mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, o));
+    constexpr int NW = TC >= 32 ? TS : TC * TS / 32;  // partial results per column
+    if constexpr (NW > 1) {
+      red[(TC >= 32 ? j : (int)threadIdx.x / 32) * TC + c] = mag;  // equal values where lanes share a slot
+      __syncthreads();
+#pragma unroll
+      for (int w = 0; w < NW; ++w) mag = max(mag, red[w * TC + c]);
+      __syncthreads();
+    }
+    return mag;
+  }
+}
+
+__device__ __forceinline__ float2 gmul(float2 a, float2 b) { return make_float2(a.x * b.x, a.y * b.y); }
+__device__ __forceinline__ double2 gmul(double2 a, double2 b) { return make_double2(a.x * b.x, a.y * b.y); }
+__device__ __forceinline__ float4 gmul(float4 a, float4 b) {
+  return make_float4(a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w);
+}
+
+template <class A, typename T, int L, bool NARROW, bool PROD, int VAR>
+__global__ void __launch_bounds__(ColTile<A, L, NARROW, VAR>::NT) k_cols_line(ColJobs<T> J,
+                                                                          const typename A::W* __restrict__ tw) {
+  using Tile = ColTile<A, L, NARROW, VAR>;
+  using Ln = Line<A, L, NARROW>;
+  using V = typename A::V;
+  using G = typename A::G;
+  constexpr int E = Ln::E, TC = Tile::TC;
+  __shared__ V buf[L * TC];
+  int q = 0;
+#pragma unroll
+  for (int k = 1; k < kColJobs; ++k)
+    if (k < J.nj && (int)blockIdx.x >= J.start[k]) q = k;
+  const int c = threadIdx.x % TC, j = threadIdx.x / TC;
+  const int line = ((int)blockIdx.x - J.start[q]) * TC + c;
+  const int ls = J.log2s[q];
+  const long s = 1L << ls;
+  const long off = ((long)(line >> ls) * L << ls) + (line & (int)(s - 1));
+  const bool ok = line < J.n;
+  G x[E];
+  {
+    const G* in = reinterpret_cast<const G*>(J.in[q]) + off;
+#pragma unroll
+    for (int e = 0; e < E; ++e) x[e] = ok ? in[Ln::position(j, e) * s] : G{};
+    if constexpr (PROD) {
+      const G* mul = reinterpret_cast<const G*>(J.mul[q]) + off;
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        if (ok) x[e] = gmul(x[e], mul[Ln::position(j, e) * s]);
+    }
+  }
+  V v[E];
+  auto at = [&](int p) { return buf + p * TC + c; };
+  auto sync = [] { __syncthreads(); };
+  G* out = reinterpret_cast<G*>(J.out[q]) + off;
+  if constexpr (A::SCALED) {
+    unsigned mag = 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) mag = max(mag, fx_mag(x[e]));
+    const FxScale<L, Ln::R0> sc(line_max<TC, Tile::TS>(mag, reinterpret_cast<unsigned*>(buf), c, j));
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = sc.in(x[e]);
+    Ln::derivative(v, j, at, sync, tw);
+    if (!ok) return;
+#pragma unroll
+    for (int e = 0; e < E; ++e) out[Ln::position(j, e) * s] = sc.out(v[e]);
+  } else {
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = A::in(x[e]);
+    Ln::derivative(v, j, at, sync, tw);
+    if (!ok) return;
+#pragma unroll
+    for (int e = 0; e < E; ++e) out[Ln::position(j, e) * s] = A::out(v[e]);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Row pass with the stage epilogue
+// ---------------------------------------------------------------------------
+// ADV2, ADV3: advection in 2D / 3D; ADV33: two 3D advection stages (fields u[0]
+// and u[1]); DIV: divergence (2D and 3D)
+enum { EPI_ADV2 = 0, EPI_ADV3 = 1, EPI_ADV33 = 2, EPI_DIV = 3 };
+
+template <typename T>
+struct RowArgs {
+  const T* u[2];   // differentiated fields (DIV: u[0] times mul)
+  const T* mul;
+  const T* gx[2];  // derivatives along the first axis (DIV: of the first product)
+  const T* gy[2];  // along the second axis (3D)
+  AdvEpi<T> adv, advB;
+  DivEpi<T> dv;
+  long nrows;
+};
+
+// Rows r and r + 1 (r even) form one complex line. A block holds NSEQ lines;
+// a wide line lives in one warp, which also runs the epilogue of its rows, so
+// the warps never wait for one another. A narrow block transforms one or a few
+// lines with part of its threads and spreads their epilogue over all of them.
+template <int L, bool NARROW, int EPI>
+struct RowTile {
+  using P = LinePlan<L, NARROW>;
+  static constexpr int TS = P::TS;
+  static constexpr int NF = EPI == EPI_ADV33 ? 2 : 1;
+  static constexpr int MINSEQ = 32 / TS > NF ? 32 / TS : NF;
+  static constexpr int NSEQ = NARROW ? MINSEQ : 128 / TS;
+  static constexpr int NFFT = NSEQ * TS;  // transforming threads
+  static constexpr int NT = NFFT > 128 ? NFFT : 128;
+  static constexpr bool WARP = !NARROW && 32 / TS >= NF;  // each warp alone
+  static constexpr int PADSH = P::R(0) == 16 ? 4 : (P::R(0) == 8 ? 3 : 2);
+  static constexpr int RS = (L + (L >> PADSH) + 1) / 2 * 2;
+  static constexpr int ROWS = NSEQ / NF * 2;  // rows of one field per block
+};
+
+template <class A, typename T, int L, bool NARROW, int EPI>
+__global__ void __launch_bounds__(RowTile<L, NARROW, EPI>::NT) k_rows_line(RowArgs<T> a,
+                                                                            const typename A::W* __restrict__ tw) {
+  using Tile = RowTile<L, NARROW, EPI>;
+  using Ln = Line<A, L, NARROW>;
+  using V = typename A::V;
+  using C = cx<T>;
+  constexpr int E = Ln::E, TS = Tile::TS, RS = Tile::RS, NF = Tile::NF, M = L / 2;
+  __shared__ __align__(16) V buf[Tile::NSEQ * RS];
+  const long row0 = (long)blockIdx.x * Tile::ROWS;
+  if (Tile::NFFT == Tile::NT || threadIdx.x < Tile::NFFT) {
+    const int seq = threadIdx.x / TS, j = threadIdx.x % TS;
+    const long row = row0 + seq / NF * 2;
+    const bool ok = row < a.nrows;
+    V* b = buf + seq * RS;
+    C x[E];
+    {
+      const T* u = a.u[0];
+      if (NF == 2 && seq % NF) u = a.u[1];
+      u += row * L;
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int p = Ln::position(j, e);
+        x[e] = ok ? mk<C>(u[p], u[L + p]) : mk<C>(0, 0);
+      }
+      if constexpr (EPI == EPI_DIV) {
+        const T* m = a.mul + row * L;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const int p = Ln::position(j, e);
+          if (ok) x[e] = mk<C>(x[e].x * m[p], x[e].y * m[L + p]);
+        }
+      }
+    }
+    V v[E];
+    auto sync = [] {
+      if constexpr (TS <= 32) __syncwarp();
+      else asm volatile("bar.sync 1, %0;" ::"n"(Tile::NFFT) : "memory");
+    };
+    auto at = [&](int p) { return b + p + (p >> Tile::PADSH); };
+    if constexpr (A::SCALED) {
+      unsigned mag = 0;
+#pragma unroll
+      for (int e = 0; e < E; ++e) mag = max(mag, fx_mag(x[e]));
+#pragma unroll
+      for (int o = 1; o < (TS < 32 ? TS : 32); o *= 2) mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, o));
+      if constexpr (TS > 32) {  // the line's warps exchange their maxima
+        unsigned* red = reinterpret_cast<unsigned*>(b);
+        red[j / 32] = mag;
+        sync();
+#pragma unroll
+        for (int w = 0; w < TS / 32; ++w) mag = max(mag, red[w]);
+        sync();
+      }
+      const FxScale<L, Ln::R0> sc(mag);
+#pragma unroll
+      for (int e = 0; e < E; ++e) v[e] = sc.in(x[e]);
+      Ln::derivative(v, j, at, sync, tw);
+#pragma unroll
+      for (int e = 0; e < E; ++e) x[e] = sc.out(v[e]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < E; ++e) v[e] = A::in(x[e]);
+      Ln::derivative(v, j, at, sync, tw);
+#pragma unroll
+      for (int e = 0; e < E; ++e) x[e] = A::out(v[e]);
+    }
+    // the two real rows of the derivative, in place of the exchanged values
+    if constexpr (Ln::S > 1) sync();
+    T* ra = reinterpret_cast<T*>(b);
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int p = Ln::position(j, e);
+      ra[p] = x[e].x;
+      ra[RS + p] = x[e].y;
+    }
+  }
+  if constexpr (Tile::WARP) __syncwarp();
+  else __syncthreads();
+  constexpr int GT = Tile::WARP ? 32 : Tile::NT;                      // threads that share rows
+  constexpr int GROWS = Tile::WARP ? 32 / TS / NF * 2 : Tile::ROWS;  // and those rows
+  const int g0 = Tile::WARP ? (int)(threadIdx.x / 32) * GROWS : 0;
+  const int gt = Tile::WARP ? threadIdx.x % 32 : threadIdx.x;
+#pragma unroll 2
+  for (int i = gt; i < GROWS * M; i += GT) {
+    const int r = g0 + i / M, jj = i % M;
+    const long row = row0 + r;
+    if (row >= a.nrows) break;
+    const long q = row * M + jj;  // the point pair (2 jj, 2 jj + 1) of the row
+    auto dlast = [&](int f) {
+      const T* ra = reinterpret_cast<const T*>(buf + (r / 2 * NF + f) * RS) + (r & 1) * RS;
+      return reinterpret_cast<const C*>(ra)[jj];
+    };
+    auto ld = [&](const T* p) { return reinterpret_cast<const C*>(p)[q]; };
+    if constexpr (EPI == EPI_ADV2) {
+      const C g[2] = {ld(a.gx[0]), dlast(0)};
+      adv_point<T, 2>(a.adv, g, q, nullptr);
+    } else if constexpr (EPI == EPI_ADV3) {
+      const C g[3] = {ld(a.gx[0]), ld(a.gy[0]), dlast(0)};
+      adv_point<T, 3>(a.adv, g, q, nullptr);
+    } else if constexpr (EPI == EPI_ADV33) {
+      const C g[3] = {ld(a.gx[0]), ld(a.gy[0]), dlast(0)};
+      const C h[3] = {ld(a.gx[1]), ld(a.gy[1]), dlast(1)};
+      C av[3];
+      const C sa = adv_point<T, 3>(a.adv, g, q, nullptr, nullptr, av);
+      adv_point<T, 3>(a.advB, h, q, a.advB.src_from_a ? &sa : nullptr, a.advB.a_from_a ? av : nullptr);
+    } else {
+      C k = dlast(0);
+      const C x = ld(a.gx[0]);
+      k = mk<C>(k.x + x.x, k.y + x.y);
+      if (a.gy[0]) {
+        const C y = ld(a.gy[0]);
+        k = mk<C>(k.x + y.x, k.y + y.y);
+      }
+      div_point<T>(a.dv, k, q);
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Bounded waits on tensor copies
+// ---------------------------------------------------------------------------
+static __device__ int g_tma_timeouts;
+
+__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void mbar_init(uint64_t* bar, unsigned count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_addr(bar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_addr(bar)), "r"(bytes)
+               : "memory");
+}
+// wait for the phase with parity `parity`; false when the bound runs out
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, int tries = 1 << 20) {
+  for (int i = 0; i < tries; ++i) {
+    unsigned done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(smem_addr(bar)), "r"(parity)
+        : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n" ::
+          "r"(smem_addr(dst)),
+      "l"(map), "r"(x), "r"(y), "r"(smem_addr(bar))
+      : "memory");
+}
+
+// Failure-path check: one block waits on an mbarrier that nothing completes,
+// gives up after `tries` polls and counts the timeout as the column pass does.
+static __global__ void k_wait_timeout_probe(int tries) {
+  __shared__ __align__(8) uint64_t bar;
+  if (threadIdx.x == 0) {
+    mbar_init(&bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  __syncthreads();
+  if (!__syncthreads_and(mbar_wait(&bar, 0, tries)) && threadIdx.x == 0) atomicAdd(&g_tma_timeouts, 1);
+}
+
+}  // namespace fused
+}  // namespace reg

@@ -1,22 +1,20 @@
-// fused_f32.cu -- single precision instantiation of the fused transport stages.
+// stage_f32.cu -- single precision instantiation of the transport stages.
 #include "../../include/reg.h"
-#include "fused_launch.cuh"
+#include "stage_launch.cuh"
 
 namespace reg {
 template <>
-void adv_stage<float>(Spectral<float>& sp, const float* u, const fused::AdvEpi<float>& e, float2* U, float2* Zx,
-                      float2* Zy, bool u_ready, bool emit) {
-  fused::adv_stage_impl<float>(sp, u, e, U, Zx, Zy, u_ready, emit);
+void adv_stage<float>(Spectral<float>& sp, const float* u, const fused::AdvEpi<float>& e, float* gx, float* gy) {
+  fused::adv_stage_impl<float>(sp, u, e, gx, gy);
 }
 template <>
 void adv2_stage<float>(Spectral<float>& sp, const float* uA, const fused::AdvEpi<float>& eA, const float* uB,
-                      const fused::AdvEpi<float>& eB, float2* const* Z) {
+                     const fused::AdvEpi<float>& eB, float* const* Z) {
   fused::adv2_stage_impl<float>(sp, uA, eA, uB, eB, Z);
 }
 template <>
-void div_stage<float>(Spectral<float>& sp, const float* lam, const float* a, const fused::DivEpi<float>& e,
-                      float2* Q0, float2* Q1, float2* Q2) {
-  fused::div_stage_impl<float>(sp, lam, a, e, Q0, Q1, Q2);
+void div_stage<float>(Spectral<float>& sp, const float* lam, const float* a, const fused::DivEpi<float>& e, float* kx, float* ky) {
+  fused::div_stage_impl<float>(sp, lam, a, e, kx, ky);
 }
 
 // timeouts of the TMA column pass of this precision since the last call (reset on read)

@@ -1,0 +1,230 @@
+// stage_launch.cuh -- host launchers of the transport stages (stage.cuh),
+// instantiated per precision by the stage_*.cu files.
+#pragma once
+#include <stdlib.h>
+
+#include <type_traits>
+
+#include "stage.cuh"
+#include "tune.h"
+
+namespace reg {
+namespace fused {
+
+// line arithmetic per precision
+template <typename T>
+struct Arith;
+template <>
+struct Arith<float> {
+  using Main = LineFloat<float>;
+};
+template <>
+struct Arith<double> {
+  using Main = LineFloat<double>;
+};
+
+// One derivative pass along a strided axis: out = D_axis in, or D_axis (in mul)
+template <typename T>
+struct ColJob {
+  int axis;
+  const T* in;
+  const T* mul;
+  T* out;
+};
+
+// distance of two elements of a line along `axis` (complex values: pairs of reals)
+inline long line_stride(const Grid& g, int axis) {
+  long s = g.M;
+  for (int a = axis + 1; a < g.d - 1; ++a) s *= g.n[a];
+  return s;
+}
+
+inline bool narrow_lines(long threads_wide) {
+  static const long lim = getenv("REG_NARROW") ? atol(getenv("REG_NARROW")) : 152 * 256;
+  return threads_wide < lim;
+}
+
+template <class A, typename T, int L, bool NARROW, bool PROD, int VAR>
+void cols_launch(const Spectral<T>& sp, const ColJob<T>* jobs, int nj, cudaStream_t st) {
+  using Tile = ColTile<A, L, NARROW, VAR>;
+  const Grid& g = sp.grid();
+  ColJobs<T> J{};
+  J.nj = nj;
+  J.n = (int)(g.Nc / L / A::CW);
+  const int per = (J.n + Tile::TC - 1) / Tile::TC;
+  for (int q = 0; q < nj; ++q) {
+    J.in[q] = jobs[q].in;
+    J.mul[q] = jobs[q].mul;
+    J.out[q] = jobs[q].out;
+    J.log2s[q] = ilog2_c((int)(line_stride(g, jobs[q].axis) / A::CW));
+    J.start[q] = q * per;
+  }
+  J.start[nj] = nj * per;
+  ProfScope ps(KK_COLS, st, (double)nj * g.N * sizeof(T) * (PROD ? 3.0 : 2.0),
+               (double)nj * g.Nc / L * (2.0 * fft_flops<L>() + 2.0 * L));
+  k_cols_line<A, T, L, NARROW, PROD, VAR><<<(unsigned)(nj * per), Tile::NT, 0, st>>>(
+      J, static_cast<const typename A::W*>(sp.line_table(L, NARROW, A::TABLE)));
+  REG_LAUNCH();
+}
+
+// Fields up to 16 MB live in L2 between the passes, as in the trials; larger
+// ones stream, which a trial on the same buffers does not show: variant 0.
+template <class A, typename T, int L, bool NARROW, bool PROD>
+void cols_tuned(const Spectral<T>& sp, const ColJob<T>* jobs, int nj, cudaStream_t st) {
+  auto run = [&](int v) {
+    if (v == 0) cols_launch<A, T, L, NARROW, PROD, 0>(sp, jobs, nj, st);
+    else cols_launch<A, T, L, NARROW, PROD, 1>(sp, jobs, nj, st);
+  };
+  const long n = sp.grid().N;
+  if (n * (long)sizeof(T) > (16 << 20)) return run(0);
+  run(tuned_choice(PROD ? "cols|prod" : "cols|plain", sizeof(T), L, tune_size(n * nj), 2, st, run));
+}
+
+template <typename T, int L, bool PROD>
+void cols_L(const Spectral<T>& sp, const ColJob<T>* jobs, int nj, cudaStream_t st) {
+  using A = typename Arith<T>::Main;
+  const Grid& g = sp.grid();
+  const long threads = (long)nj * g.Nc / L * LinePlan<L, false>::TS;
+  if (narrow_lines(threads)) return cols_tuned<A, T, L, true, PROD>(sp, jobs, nj, st);
+  if constexpr (sizeof(T) == 4)
+    if (threads >= 2 * 152 * 512) return cols_tuned<LinePair, T, L, false, PROD>(sp, jobs, nj, st);
+  cols_tuned<A, T, L, false, PROD>(sp, jobs, nj, st);
+}
+
+// The column passes of one stage: one launch per distinct axis length.
+template <typename T, bool PROD>
+void run_cols(const Spectral<T>& sp, const ColJob<T>* jobs, int nj, cudaStream_t st) {
+  const Grid& g = sp.grid();
+  bool done[kColJobs] = {false};
+  for (int a = 0; a < nj; ++a) {
+    if (done[a]) continue;
+    const int L = g.n[jobs[a].axis];
+    ColJob<T> grp[kColJobs];
+    int m = 0;
+    for (int b = a; b < nj; ++b)
+      if (!done[b] && g.n[jobs[b].axis] == L) {
+        grp[m++] = jobs[b];
+        done[b] = true;
+      }
+    switch (L) {
+      case 8: cols_L<T, 8, PROD>(sp, grp, m, st); break;
+      case 16: cols_L<T, 16, PROD>(sp, grp, m, st); break;
+      case 32: cols_L<T, 32, PROD>(sp, grp, m, st); break;
+      case 64: cols_L<T, 64, PROD>(sp, grp, m, st); break;
+      case 128: cols_L<T, 128, PROD>(sp, grp, m, st); break;
+      case 256: cols_L<T, 256, PROD>(sp, grp, m, st); break;
+      case 512: cols_L<T, 512, PROD>(sp, grp, m, st); break;
+      default: throw StatusError{1, "unsupported axis length"};
+    }
+  }
+}
+
+template <typename T, int L, int EPI>
+void rows_L(const Spectral<T>& sp, const RowArgs<T>& a, double bytes, cudaStream_t st) {
+  using A = typename Arith<T>::Main;
+  constexpr int NF = RowTile<L, false, EPI>::NF;
+  ProfScope ps(KK_ROWS_C2R, st, bytes, (double)a.nrows / 2 * NF * (2.0 * fft_flops<L>() + 2.0 * L));
+  auto go = [&](auto narrow) {
+    constexpr bool NARROW = decltype(narrow)::value;
+    using Tile = RowTile<L, NARROW, EPI>;
+    const unsigned grid = (unsigned)((a.nrows + Tile::ROWS - 1) / Tile::ROWS);
+    k_rows_line<A, T, L, NARROW, EPI><<<grid, Tile::NT, 0, st>>>(
+        a, static_cast<const typename A::W*>(sp.line_table(L, NARROW, A::TABLE)));
+    REG_LAUNCH();
+  };
+  if (narrow_lines(a.nrows / 2 * NF * LinePlan<L, false>::TS)) go(std::true_type{});
+  else go(std::false_type{});
+}
+
+template <typename T, int EPI>
+void run_rows(const Spectral<T>& sp, const RowArgs<T>& a, double bytes, cudaStream_t st) {
+  switch (sp.grid().L) {
+    case 8: return rows_L<T, 8, EPI>(sp, a, bytes, st);
+    case 16: return rows_L<T, 16, EPI>(sp, a, bytes, st);
+    case 32: return rows_L<T, 32, EPI>(sp, a, bytes, st);
+    case 64: return rows_L<T, 64, EPI>(sp, a, bytes, st);
+    case 128: return rows_L<T, 128, EPI>(sp, a, bytes, st);
+    case 256: return rows_L<T, 256, EPI>(sp, a, bytes, st);
+    case 512: return rows_L<T, 512, EPI>(sp, a, bytes, st);
+  }
+  throw StatusError{1, "unsupported last-axis length"};
+}
+
+// fields an advection epilogue reads and writes beyond u and its derivatives
+// (stage 1 reads y = u itself)
+template <typename T>
+int adv_fields(const AdvEpi<T>& e, int d, const T* u) {
+  int n = (e.G[0] ? d : 0) + (e.Sout ? d + 1 : 0);
+  if (e.out1)
+    n += d + (e.src ? 1 : (e.gm[0] && !e.src_from_a ? 2 * d : 0)) + (e.y && e.y != u ? 1 : 0) + (e.stage == 1 ? 2 : 1);
+  return n;
+}
+
+// One advection stage on u; gx, gy: scratch fields (gy in 3D).
+template <typename T>
+void adv_stage_impl(Spectral<T>& sp, const T* u, const AdvEpi<T>& e, T* gx, T* gy) {
+  const Grid& g = sp.grid();
+  cudaStream_t s = sp.stream();
+  const ColJob<T> jobs[2] = {{0, u, nullptr, gx}, {1, u, nullptr, gy}};
+  run_cols<T, false>(sp, jobs, g.d - 1, s);
+  RowArgs<T> a{};
+  a.u[0] = u;
+  a.gx[0] = gx;
+  a.gy[0] = g.d == 3 ? gy : nullptr;
+  a.adv = e;
+  a.nrows = g.rows;
+  const double bytes = (double)g.N * sizeof(T) * (g.d + adv_fields(e, g.d, u));
+  if (g.d == 3) run_rows<T, EPI_ADV3>(sp, a, bytes, s);
+  else run_rows<T, EPI_ADV2>(sp, a, bytes, s);
+}
+
+// Two advection stages of 3D fields uA and uB sharing their launches; Z: four
+// scratch fields.
+template <typename T>
+void adv2_stage_impl(Spectral<T>& sp, const T* uA, const AdvEpi<T>& eA, const T* uB, const AdvEpi<T>& eB,
+                     T* const* Z) {
+  const Grid& g = sp.grid();
+  cudaStream_t s = sp.stream();
+  const ColJob<T> jobs[4] = {
+      {0, uA, nullptr, Z[0]}, {1, uA, nullptr, Z[1]}, {0, uB, nullptr, Z[2]}, {1, uB, nullptr, Z[3]}};
+  run_cols<T, false>(sp, jobs, 4, s);
+  RowArgs<T> a{};
+  a.u[0] = uA;
+  a.u[1] = uB;
+  for (int f = 0; f < 2; ++f) {
+    a.gx[f] = Z[2 * f];
+    a.gy[f] = Z[2 * f + 1];
+  }
+  a.adv = eA;
+  a.advB = eB;
+  // a velocity read by both epilogues (the same node, or n_c = 1) is read once
+  const bool shared_a = eA.out1 && eB.out1 && eA.a[0] == eB.a[0] && eA.a[1] == eB.a[1] && eA.a[2] == eB.a[2];
+  a.advB.a_from_a = shared_a ? 1 : 0;
+  a.nrows = g.rows;
+  const double bytes =
+      (double)g.N * sizeof(T) * (6 + adv_fields(eA, 3, uA) + adv_fields(eB, 3, uB) - (shared_a ? 3 : 0));
+  run_rows<T, EPI_ADV33>(sp, a, bytes, s);
+}
+
+// One divergence stage: div(a lam); kx, ky: scratch fields (ky in 3D).
+template <typename T>
+void div_stage_impl(Spectral<T>& sp, const T* lam, const T* a, const DivEpi<T>& e, T* kx, T* ky) {
+  const Grid& g = sp.grid();
+  cudaStream_t s = sp.stream();
+  const long N = g.N;
+  const ColJob<T> jobs[2] = {{0, a, lam, kx}, {1, a + N, lam, ky}};
+  run_cols<T, true>(sp, jobs, g.d - 1, s);
+  RowArgs<T> r{};
+  r.u[0] = a + (g.d - 1) * N;
+  r.mul = lam;
+  r.gx[0] = kx;
+  r.gy[0] = g.d == 3 ? ky : nullptr;
+  r.dv = e;
+  r.nrows = g.rows;
+  double f = 2 + g.d - 1 + (e.stage && e.y != lam ? 1 : 0) + (e.stage == 1 ? 2 : 1) + (e.src ? 1 : 0);
+  if (e.f_hi) f += g.d * (e.gmB ? 2 : 1) + (e.gmC ? g.d + 1 : 0) + 2.0 * e.nc * g.d * (e.f_lo ? 2 : 1);
+  run_rows<T, EPI_DIV>(sp, r, f * N * sizeof(T), s);
+}
+
+}  // namespace fused
+}  // namespace reg

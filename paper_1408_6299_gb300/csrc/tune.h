@@ -1,0 +1,82 @@
+// tune.h -- choice of the autotuner among variants of a pure pass (one that
+// writes only what it does not read, so running it again gives the same
+// result). The variants of a pass give the same bits; they differ in the work
+// per block.
+#pragma once
+#include <stdlib.h>
+
+#include <map>
+#include <mutex>
+#include <string>
+#include <tuple>
+
+#include "internal.h"
+
+namespace reg {
+
+// Variant 0..nv-1 for pass `kind` on elements of `size` bytes, lines of length
+// L and `work` lines: the choice of this process for the shape, or the
+// persistent one (tune.cu), else, outside a stream capture, each variant runs
+// three times on the call's own buffers after one untimed run, timed with
+// CUDA events on the stream, and the fastest is recorded. During a capture, and
+// with REG_AUTOTUNE=0, variant 0 runs and nothing is recorded.
+template <typename Run>
+int tuned_choice(const char* kind, int size, int L, long work, int nv, cudaStream_t st, Run run) {
+  using Key = std::tuple<int, std::string, int, int, long>;
+  static std::mutex mu;
+  static std::map<Key, int> mem;
+  int dev = 0;
+  REG_CUDA(cudaGetDevice(&dev));
+  const Key key(dev, kind, size, L, work);
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = mem.find(key);
+    if (it != mem.end()) return it->second;
+  }
+  const std::string name = tune_device_tag() + "|" + kind + "|" + (size == 4 ? "f32" : "f64") + "|L" +
+                           std::to_string(L) + "|n" + std::to_string(work);
+  int pick = tune_lookup(name);
+  if (pick < 0 || pick >= nv) {
+    const char* env = getenv("REG_AUTOTUNE");
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    REG_CUDA(cudaStreamIsCapturing(st, &cs));
+    if ((env && env[0] == '0') || cs != cudaStreamCaptureStatusNone) return 0;
+    cudaEvent_t e0, e1;
+    REG_CUDA(cudaEventCreate(&e0));
+    REG_CUDA(cudaEventCreate(&e1));
+    float best = 1e30f;
+    pick = 0;
+    for (int v = 0; v < nv; ++v) run(v);
+    for (int v = 0; v < nv; ++v) {
+      float total = 0;
+      for (int r = 0; r < 3; ++r) {
+        REG_CUDA(cudaEventRecord(e0, st));
+        run(v);
+        REG_CUDA(cudaEventRecord(e1, st));
+        REG_CUDA(cudaEventSynchronize(e1));
+        float ms = 0;
+        REG_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+        total += ms;
+      }
+      if (total < best) {
+        best = total;
+        pick = v;
+      }
+    }
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
+    tune_store(name, pick);
+  }
+  std::lock_guard<std::mutex> lk(mu);
+  mem[key] = pick;
+  return pick;
+}
+
+// work sizes rounded up to a power of two: stacks of similar size share a choice
+inline long tune_size(long n) {
+  long r = 1;
+  while (r < n) r *= 2;
+  return r;
+}
+
+}  // namespace reg
