@@ -22,13 +22,34 @@ inline unsigned nblk(long n, int bs = 256) {
   return (unsigned)(b < 1 ? 1 : b);
 }
 
-template <typename T, typename S>
-__global__ void k_vel_at(const S* __restrict__ coef, int nc, Coefs b, T* __restrict__ out, long dN) {
+__global__ void k_vel_at(const double* __restrict__ coef, int nc, Coefs b, double* __restrict__ out, long dN) {
   long x = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= dN) return;
   double s = 0.0;
-  for (int l = 0; l < nc; ++l) s += b.c[l] * (double)coef[l * dN + x];
-  out[x] = (T)s;
+  for (int l = 0; l < nc; ++l) s += b.c[l] * coef[l * dN + x];
+  out[x] = s;
+}
+
+// The single-precision combination, accurate to the last bit without the
+// double-precision unit (two operations per clock and SM; 16 us for 64^3 with
+// three coefficients that way): every weight is a pair of floats, products
+// and sums keep their rounding errors, and the sum is rounded once.
+struct FloatWeights {
+  float hi[16], lo[16];
+};
+__global__ void k_vel_at(const float* __restrict__ coef, int nc, FloatWeights b, float* __restrict__ out, long dN) {
+  long x = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (x >= dN) return;
+  float s = 0.f, err = 0.f;
+  for (int l = 0; l < nc; ++l) {
+    const float c = coef[l * dN + x];
+    const float p = __fmul_rn(b.hi[l], c);
+    err += fmaf(b.hi[l], c, -p) + b.lo[l] * c;
+    const float t = __fadd_rn(s, p), z = __fsub_rn(t, s);
+    err += __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z));
+    s = t;
+  }
+  out[x] = s + err;
 }
 
 template <typename S, typename T>
@@ -67,27 +88,61 @@ __global__ void k_dot_fields(const T* __restrict__ a, const T* __restrict__ b, T
   out[x] = s;
 }
 
-// (f_hi, f_lo)[l][i][x] += c_l lam[x] gm[i][x]; with f_lo null a plain sum
-// into f_hi, else a compensated pair (the rounding error of each add kept in f_lo)
+// Body force of a group of time nodes. Adding each node's term inside the
+// adjoint stage reads and writes the accumulator (n_c d fields, twice that for
+// a compensated pair) at every step; here the nodes of a group share one read
+// and one write of it, and the terms are added in the same order. Bound by
+// the reads of the state gradients. A thread takes one component of a point
+// pair; the blocks of the d components of the same points are neighbours, so
+// they find y in L2.
 template <typename T>
-__global__ void k_force(T* __restrict__ fhi, T* __restrict__ flo, const T* __restrict__ lam,
-                        const T* __restrict__ gm, Coefs c, int nc, int d, long N) {
-  long x = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= N) return;
-  T l = lam[x];
-  for (int i = 0; i < d; ++i) {
-    T p = l * gm[i * N + x];
-    for (int a = 0; a < nc; ++a) {
-      long q = ((long)a * d + i) * N + x;
-      T t = (T)c.c[a] * p;
-      if (!flo) {
-        fhi[q] += t;
-      } else {
-        T h = fhi[q], sm = h + t, bp = sm - h;
-        flo[q] += (h - (sm - bp)) + (t - bp);
-        fhi[q] = sm;
+__global__ void __launch_bounds__(256) k_force(T* __restrict__ fhi, T* __restrict__ flo, ForceNodes<T> F, int nc, int d,
+                                               long N) {
+  using C = cx<T>;
+  const int i = blockIdx.x % d;
+  const long q = (long)(blockIdx.x / d) * blockDim.x + threadIdx.x;
+  if (q >= N / 2) return;
+  auto ld = [&](const T* p) { return reinterpret_cast<const C*>(p)[q]; };
+  C ta[kForceNodes], tb[kForceNodes];
+#pragma unroll
+  for (int k = 0; k < kForceNodes; ++k) {
+    ta[k] = tb[k] = mk<C>(0, 0);
+    if (k < F.count) {
+      const C y = ld(F.yA[k]), g = ld(F.gA[k] + i * N);
+      ta[k] = mk<C>(y.x * g.x, y.y * g.y);
+      if (F.yC[k]) {
+        const C yc = ld(F.yC[k]), gc = ld(F.gC[k] + i * N);
+        ta[k] = mk<C>(ta[k].x + yc.x * gc.x, ta[k].y + yc.y * gc.y);
+      }
+      if (F.yB[k]) {
+        const C yb = ld(F.yB[k]), gb = ld(F.gB[k] + i * N);
+        tb[k] = mk<C>(yb.x * gb.x, yb.y * gb.y);
       }
     }
+  }
+  for (int l = 0; l < nc; ++l) {
+    const long o = ((long)l * d + i) * (N / 2) + q;
+    C h = reinterpret_cast<C*>(fhi)[o];
+    C e = flo ? reinterpret_cast<C*>(flo)[o] : mk<C>(0, 0);
+#pragma unroll
+    for (int k = 0; k < kForceNodes; ++k) {
+      if (k >= F.count) break;
+      T t0 = F.cA[k][l] * ta[k].x, t1 = F.cA[k][l] * ta[k].y;
+      if (F.yB[k]) {
+        t0 += F.cB[k][l] * tb[k].x;
+        t1 += F.cB[k][l] * tb[k].y;
+      }
+      if (flo) {
+        const T s0 = h.x + t0, b0 = s0 - h.x, s1 = h.y + t1, b1 = s1 - h.y;
+        e.x += (h.x - (s0 - b0)) + (t0 - b0);
+        e.y += (h.y - (s1 - b1)) + (t1 - b1);
+        h = mk<C>(s0, s1);
+      } else {
+        h = mk<C>(h.x + t0, h.y + t1);
+      }
+    }
+    reinterpret_cast<C*>(fhi)[o] = h;
+    if (flo) reinterpret_cast<C*>(flo)[o] = e;
   }
 }
 
@@ -241,14 +296,21 @@ __global__ void k_reduce_final(const double* __restrict__ part, double* __restri
 
 }  // namespace
 
-template <typename T, typename S>
-void vel_at(const S* coef, int nc, const Coefs& b, T* out, long dN, cudaStream_t s) {
-  k_vel_at<T, S><<<nblk(dN), 256, 0, s>>>(coef, nc, b, out, dN);
+template <>
+void vel_at<double>(const double* coef, int nc, const Coefs& b, double* out, long dN, cudaStream_t s) {
+  k_vel_at<<<nblk(dN), 256, 0, s>>>(coef, nc, b, out, dN);
   REG_LAUNCH();
 }
-template void vel_at<float, double>(const double*, int, const Coefs&, float*, long, cudaStream_t);
-template void vel_at<double, double>(const double*, int, const Coefs&, double*, long, cudaStream_t);
-template void vel_at<float, float>(const float*, int, const Coefs&, float*, long, cudaStream_t);
+template <>
+void vel_at<float>(const float* coef, int nc, const Coefs& b, float* out, long dN, cudaStream_t s) {
+  FloatWeights w;
+  for (int l = 0; l < 16; ++l) {
+    w.hi[l] = l < nc ? (float)b.c[l] : 0.f;
+    w.lo[l] = l < nc ? (float)(b.c[l] - (double)w.hi[l]) : 0.f;
+  }
+  k_vel_at<<<nblk(dN), 256, 0, s>>>(coef, nc, w, out, dN);
+  REG_LAUNCH();
+}
 
 template <typename S, typename T>
 void convert(const S* in, T* out, long n, cudaStream_t s) {
@@ -275,9 +337,12 @@ void dot_fields(const T* a, const T* b, T* out, int d, long N, cudaStream_t s) {
 }
 
 template <typename T>
-void force_acc(T* fhi, T* flo, const T* lam, const T* gm, const Coefs& c, int nc, int d, long N, cudaStream_t s) {
-  ProfScope ps(KK_FORCE, s, (double)N * sizeof(T) * ((d + 1) + 2.0 * nc * d * (flo ? 2 : 1)));
-  k_force<T><<<nblk(N), 256, 0, s>>>(fhi, flo, lam, gm, c, nc, d, N);
+void force_acc(T* fhi, T* flo, const ForceNodes<T>& F, int nc, int d, long N, cudaStream_t s) {
+  if (!F.count) return;
+  double fields = 2.0 * nc * d * (flo ? 2 : 1);
+  for (int k = 0; k < F.count; ++k) fields += (d + 1) * (1 + (F.yB[k] ? 1 : 0) + (F.yC[k] ? 1 : 0));
+  ProfScope ps(KK_FORCE, s, (double)N * sizeof(T) * fields);
+  k_force<T><<<nblk(N / 2) * d, 256, 0, s>>>(fhi, flo, F, nc, d, N);
   REG_LAUNCH();
 }
 
@@ -290,7 +355,7 @@ void pair_to_double(const float* hi, const float* lo, double* out, long n, cudaS
   template void transport_stage1<T>(const T*, const T*, const T*, const T*, const T*, T, T*, T*, int, long, \
                                     cudaStream_t);                                                       \
   template void dot_fields<T>(const T*, const T*, T*, int, long, cudaStream_t);                             \
-  template void force_acc<T>(T*, T*, const T*, const T*, const Coefs&, int, int, long, cudaStream_t);
+  template void force_acc<T>(T*, T*, const ForceNodes<T>&, int, int, long, cudaStream_t);
 INST(float)
 INST(double)
 #undef INST

@@ -10,9 +10,9 @@ struct Coefs {
   double c[16];
 };
 
-// out[x] = sum_l b_l coef[l*dN + x], x < dN
-template <typename T, typename S>
-void vel_at(const S* coef, int nc, const Coefs& b, T* out, long dN, cudaStream_t s);
+// out[x] = sum_l b_l coef[l*dN + x], x < dN, rounded once to T
+template <typename T>
+void vel_at(const T* coef, int nc, const Coefs& b, T* out, long dN, cudaStream_t s);
 template <typename S, typename T>
 void convert(const S* in, T* out, long n, cudaStream_t s);
 
@@ -25,10 +25,23 @@ void transport_stage1(const T* G, const T* vt, const T* gm, const T* wt, const T
 // out = sum_i a_i b_i (d fields at stride N)
 template <typename T>
 void dot_fields(const T* a, const T* b, T* out, int d, long N, cudaStream_t s);
-// f[l][i] += c_l lam gm_i: plain sum into fhi (flo null) or a compensated
-// (fhi, flo) pair of precision T
+// Body force of up to kForceNodes time nodes (see ForceNodes):
+//   f[l][i] += cA_l (yA gA_i + yC gC_i) + cB_l yB gB_i   for every node in order,
+// a plain sum into fhi (flo null) or a compensated (fhi, flo) pair of precision T
+constexpr int kForceNodes = 8;
 template <typename T>
-void force_acc(T* fhi, T* flo, const T* lam, const T* gm, const Coefs& c, int nc, int d, long N, cudaStream_t s);
+struct ForceNodes {
+  int count = 0;
+  const T* yA[kForceNodes] = {};
+  const T* gA[kForceNodes] = {};  // d fields at stride N
+  const T* yB[kForceNodes] = {};  // second term (discrete adjoint) or null
+  const T* gB[kForceNodes] = {};
+  const T* yC[kForceNodes] = {};  // Newton term or null
+  const T* gC[kForceNodes] = {};
+  T cA[kForceNodes][16], cB[kForceNodes][16];
+};
+template <typename T>
+void force_acc(T* fhi, T* flo, const ForceNodes<T>& nodes, int nc, int d, long N, cudaStream_t s);
 // out = (double)hi + (double)lo
 void pair_to_double(const float* hi, const float* lo, double* out, long n, cudaStream_t s);
 

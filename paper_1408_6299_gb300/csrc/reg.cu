@@ -110,6 +110,7 @@ struct Work {
   DBuf<T> gm, gmh, ck;           // state gradients (all nodes or one segment), stage gradients, checkpoints
   DBuf<T> fhi, flo;              // single precision body force as a compensated pair
   DBuf<T> src;                   // source grad m_j . v~(t_j) per node (all nodes or one segment)
+  DBuf<T> lamR, yhR;             // adjoint (and its predictors) of the nodes whose force is pending
   DBuf<T> mtil, lamN, yh2, acc2, st0, st1, Gt, mR, m1;  // full Newton matvec
 };
 
@@ -254,13 +255,28 @@ Spectral<float>& spectral<float>(reg_ctx* c) {
   return *c->sp32;
 }
 
-// velocity (coefficients in precision T) at node j: a pointer to d fields
+// Velocity (coefficients in precision T) at the time nodes: a pointer to d
+// fields. Consecutive steps share a node, so the last two are kept: get(j)
+// stays valid until two other nodes have been asked for.
 template <typename T>
-const T* vel_node(reg_ctx* c, const T* coef, int j, T* buf) {
-  if (c->n_c == 1) return coef;
-  vel_at<T, T>(coef, c->n_c, c->basis_at_node(j), buf, c->dN(), c->s);
-  return buf;
-}
+struct NodeVel {
+  reg_ctx* c;
+  const T* coef;
+  T* buf[2];
+  int node[2] = {-1, -1}, last = 1;
+  NodeVel(reg_ctx* c_, const T* coef_, DBuf<T>& a, DBuf<T>& b)
+      : c(c_), coef(coef_), buf{c_->n_c > 1 ? a.get(c_->dN()) : nullptr, c_->n_c > 1 ? b.get(c_->dN()) : nullptr} {}
+  const T* get(int j) {
+    if (c->n_c == 1) return coef;
+    if (node[last] == j) return buf[last];
+    last ^= 1;
+    if (node[last] != j) {
+      vel_at<T>(coef, c->n_c, c->basis_at_node(j), buf[last], c->dN(), c->s);
+      node[last] = j;
+    }
+    return buf[last];
+  }
+};
 
 // advection stage on u: k = -a.grad u [- gm.w], Heun stage update
 template <typename T>
@@ -350,14 +366,12 @@ void state_steps(reg_ctx* c, const T* vcoef, int j0, int j1, T* gm, T* gmh, int 
   T* m = w.m.get(N);
   T* yh = w.yh.get(N);
   T* acc = w.acc.get(N);
-  T* va = w.va.get(dN);
-  T* vb = w.vb.get(dN);
+  NodeVel<T> v(c, vcoef, w.va, w.vb);
   for (int j = j0; j < j1; ++j) {
     if (ck && c->ckpt > 0 && j % c->ckpt == 0)
       REG_CUDA(cudaMemcpyAsync(ck + (long)(j / c->ckpt) * N, m, N * sizeof(T), cudaMemcpyDeviceToDevice, c->s));
-    adv<T>(c, m, vel_node<T>(c, vcoef, j, va), nullptr, nullptr, m, yh, acc, gm ? gm + (long)(j - base) * dN : nullptr,
-           1);
-    adv<T>(c, yh, vel_node<T>(c, vcoef, j + 1, vb), nullptr, nullptr, acc, m, nullptr,
+    adv<T>(c, m, v.get(j), nullptr, nullptr, m, yh, acc, gm ? gm + (long)(j - base) * dN : nullptr, 1);
+    adv<T>(c, yh, v.get(j + 1), nullptr, nullptr, acc, m, nullptr,
            gmh ? gmh + (long)(j + 1 - base) * dN : nullptr, 2);
   }
   if (ck && c->ckpt > 0 && j1 % c->ckpt == 0)
@@ -382,22 +396,18 @@ void recompute_segment(reg_ctx* c, const T* vcoef, int j0, int j1) {
 template <typename T>
 void recompute_segment_src(reg_ctx* c, const T* vcoef, const T* wcoef, int j0, int j1) {
   Work<T>& w = work<T>(c);
-  const long N = c->N(), dN = c->dN();
+  const long N = c->N();
   T* m = w.m.get(N);
   T* yh = w.yh.get(N);
   T* acc = w.acc.get(N);
-  T* va = w.va.get(dN);
-  T* vb = w.vb.get(dN);
-  T* wa = w.wa.get(dN);
+  NodeVel<T> v(c, vcoef, w.va, w.vb), vt(c, wcoef, w.wa, w.wb);
   T* src = w.src.get((size_t)(c->ckpt + 1) * N);
   REG_CUDA(cudaMemcpyAsync(m, w.ck.p + (long)(j0 / c->ckpt) * N, N * sizeof(T), cudaMemcpyDeviceToDevice, c->s));
   for (int j = j0; j < j1; ++j) {
-    adv<T>(c, m, vel_node<T>(c, vcoef, j, va), nullptr, nullptr, m, yh, acc, nullptr, 1, nullptr,
-           vel_node<T>(c, wcoef, j, wa), src + (long)(j - j0) * N);
-    adv<T>(c, yh, vel_node<T>(c, vcoef, j + 1, vb), nullptr, nullptr, acc, m, nullptr, nullptr, 2);
+    adv<T>(c, m, v.get(j), nullptr, nullptr, m, yh, acc, nullptr, 1, nullptr, vt.get(j), src + (long)(j - j0) * N);
+    adv<T>(c, yh, v.get(j + 1), nullptr, nullptr, acc, m, nullptr, nullptr, 2);
   }
-  adv<T>(c, m, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 1, nullptr,
-         vel_node<T>(c, wcoef, j1, wa), src + (long)(j1 - j0) * N);
+  adv<T>(c, m, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 1, nullptr, vt.get(j1), src + (long)(j1 - j0) * N);
 }
 
 // Gradient slots available for node j (after ensure_segment)
@@ -424,67 +434,112 @@ void state_solve_store(reg_ctx* c, const T* vcoef, const T* m0) {
   }
 }
 
-// Adjoint solve (Eq. first-order-adjoint) backward from lam (in w.lam at n_t),
-// accumulating the body force f_l = int b_l lam grad m dt into f (double).
-// The force terms of each step are added in the first stage of the step: the
-// trapezoid term of node j+1, or the two stage terms of the discrete adjoint.
-// Single precision sweeps accumulate into a compensated pair of floats that is
-// converted to double at the end. Leaves lam_0 in w.lam.
+// The body-force sum of a backward sweep: the terms of up to kForceNodes nodes
+// are collected and added by one kernel (flush), in the order they were given.
+// Single precision sweeps accumulate into a compensated pair of floats that
+// is converted to double at the end.
 template <typename T>
-void adjoint_solve(reg_ctx* c, const T* vcoef, double* f) {
-  Work<T>& w = work<T>(c);
-  const long N = c->N(), dN = c->dN();
-  const double hd = c->h();
-  T* lam = w.lam.p;
-  T* yh = w.yh.get(N);
-  T* acc = w.acc.get(N);
-  T* va = w.va.get(dN);
-  T* vb = w.vb.get(dN);
-  T* fhi;
-  T* flo = nullptr;
-  if (sizeof(T) == sizeof(double)) {
-    fhi = reinterpret_cast<T*>(f);
-  } else {
-    fhi = w.fhi.get(c->ncdN());
-    flo = w.flo.get(c->ncdN());
-    REG_CUDA(cudaMemsetAsync(flo, 0, c->ncdN() * sizeof(T), c->s));
+struct BodyForce {
+  reg_ctx* c;
+  double* f;
+  T* hi;
+  T* lo = nullptr;
+  ForceNodes<T> F;
+  BodyForce(reg_ctx* c_, double* f_) : c(c_), f(f_) {
+    Work<T>& w = work<T>(c);
+    const long n = c->ncdN();
+    if (sizeof(T) == sizeof(double)) {
+      hi = reinterpret_cast<T*>(f);
+    } else {
+      hi = w.fhi.get(n);
+      lo = w.flo.get(n);
+      REG_CUDA(cudaMemsetAsync(lo, 0, n * sizeof(T), c->s));
+    }
+    REG_CUDA(cudaMemsetAsync(hi, 0, n * sizeof(T), c->s));
   }
-  REG_CUDA(cudaMemsetAsync(fhi, 0, c->ncdN() * sizeof(T), c->s));
+  // + b_l(t_jA) wA yA gA
+  void add(const T* y, const T* g, int j, double wgt) {
+    const int k = F.count++;
+    const Coefs a = c->basis_at_node(j, wgt);
+    for (int l = 0; l < c->n_c; ++l) F.cA[k][l] = (T)a.c[l];
+    F.yA[k] = y;
+    F.gA[k] = g;
+    F.yB[k] = F.gB[k] = F.yC[k] = F.gC[k] = nullptr;
+  }
+  // a second term of the same entry, with its own weight
+  void also(const T* y, const T* g, int j, double wgt) {
+    const int k = F.count - 1;
+    const Coefs a = c->basis_at_node(j, wgt);
+    for (int l = 0; l < c->n_c; ++l) F.cB[k][l] = (T)a.c[l];
+    F.yB[k] = y;
+    F.gB[k] = g;
+  }
+  // a second product under the entry's weight
+  void with(const T* y, const T* g) {
+    F.yC[F.count - 1] = y;
+    F.gC[F.count - 1] = g;
+  }
+  void flush() {
+    force_acc<T>(hi, lo, F, c->n_c, c->d, c->N(), c->s);
+    F.count = 0;
+  }
+  void finish() {
+    flush();
+    if (lo)
+      pair_to_double(reinterpret_cast<const float*>(hi), reinterpret_cast<const float*>(lo), f, c->ncdN(), c->s);
+  }
+};
+
+// slot k of a ring of kForceNodes + 1 fields
+template <typename T>
+T* ring_slot(T* ring, int k, long stride) {
+  return ring + (long)(k % (kForceNodes + 1)) * stride;
+}
+
+// Adjoint solve (Eq. first-order-adjoint) backward from lam (in w.lam at n_t),
+// accumulating the body force f_l = int b_l lam grad m dt into f (double): the
+// trapezoid term of every node, or the two stage terms per step of the
+// discrete adjoint. lam (and the predictors of the discrete adjoint) are kept
+// for the nodes whose force is still to be added. Returns lam_0.
+template <typename T>
+const T* adjoint_solve(reg_ctx* c, const T* vcoef, double* f) {
+  Work<T>& w = work<T>(c);
+  const long N = c->N();
+  const double hd = c->h();
+  T* acc = w.acc.get(N);
+  T* ring = w.lamR.get((size_t)(kForceNodes + 1) * N);
+  T* yhs = c->quad ? w.yhR.get((size_t)(kForceNodes + 1) * N) : w.yh.get(N);
+  BodyForce<T> bf(c, f);
+  const T* lam = w.lam.p;
+  int k = 0;  // ring slots used
   const int K = c->ckpt > 0 ? c->ckpt : c->n_t;
   for (int seg = (c->n_t - 1) / K; seg >= 0; --seg) {
     int j0 = seg * K, j1 = j0 + K;
     int base = 0;
     if (c->ckpt > 0) {
+      bf.flush();  // the state gradients are about to be overwritten
       recompute_segment<T>(c, vcoef, j0, j1);
       base = j0;
     }
+    NodeVel<T> v(c, vcoef, w.va, w.vb);
     for (int j = j1 - 1; j >= j0; --j) {
-      fused::DivEpi<T> e{};
-      e.f_hi = fhi;
-      e.f_lo = flo;
-      e.nc = c->n_c;
-      e.d = c->d;
-      e.N = N;
+      T* yh = c->quad ? ring_slot(yhs, k, N) : yhs;
+      T* next = ring_slot(ring, k++, N);
+      divh<T>(c, lam, v.get(j + 1), lam, yh, acc, 1);
+      divh<T>(c, yh, v.get(j), acc, next, nullptr, 2);
       if (!c->quad) {
-        e.gmA = gm_slot<T>(c, j + 1, base);
-        Coefs a = c->basis_at_node(j + 1, c->trap_w(j + 1));
-        for (int l = 0; l < c->n_c; ++l) e.cA[l] = (T)a.c[l];
+        bf.add(lam, gm_slot<T>(c, j + 1, base), j + 1, c->trap_w(j + 1));
       } else {
-        e.gmA = gmh_slot<T>(c, j + 1, base);
-        e.gmB = gm_slot<T>(c, j, base);
-        Coefs a = c->basis_at_node(j + 1, 0.5 * hd), b = c->basis_at_node(j, 0.5 * hd);
-        for (int l = 0; l < c->n_c; ++l) {
-          e.cA[l] = (T)a.c[l];
-          e.cB[l] = (T)b.c[l];
-        }
+        bf.add(lam, gmh_slot<T>(c, j + 1, base), j + 1, 0.5 * hd);
+        bf.also(yh, gm_slot<T>(c, j, base), j, 0.5 * hd);
       }
-      divh<T>(c, lam, vel_node<T>(c, vcoef, j + 1, vb), lam, yh, acc, 1, e);
-      divh<T>(c, yh, vel_node<T>(c, vcoef, j, va), acc, lam, nullptr, 2);
+      lam = next;
+      if (bf.F.count == kForceNodes) bf.flush();
     }
-    if (j0 == 0 && !c->quad)
-      force_acc<T>(fhi, flo, lam, gm_slot<T>(c, 0, base), c->basis_at_node(0, c->trap_w(0)), c->n_c, c->d, N, c->s);
+    if (j0 == 0 && !c->quad) bf.add(lam, gm_slot<T>(c, 0, base), 0, c->trap_w(0));
   }
-  if (flo) pair_to_double(reinterpret_cast<const float*>(fhi), reinterpret_cast<const float*>(flo), f, c->ncdN(), c->s);
+  bf.finish();
+  return lam;
 }
 
 // Full Newton incremental adjoint (Eq. sec-order-iadj / sec-order-icontrol,
@@ -498,72 +553,68 @@ template <typename T>
 void newton_adjoint(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
   Work<T>& w = work<T>(c);
   const long N = c->N(), dN = c->dN();
-  T* lt = w.lam.p;  // lam~
+  const size_t slots = kForceNodes + 1;
   T* yh = w.yh.get(N);
   T* acc = w.acc.get(N);
-  T* lam = w.lamN.get(N);
   T* yh2 = w.yh2.get(N);
   T* acc2 = w.acc2.get(N);
   T* sA = w.st0.get(N);
   T* sB = w.st1.get(N);
-  T* Gt = w.Gt.get(dN);
-  T* va = w.va.get(dN);
-  T* vb = w.vb.get(dN);
-  T* wa = w.wa.get(dN);
+  T* ringT = w.lamR.get(slots * N);  // lam~
+  T* ringL = w.lamN.get(slots * N);  // lam
+  T* Gt = w.Gt.get(slots * dN);
   const T* mtil = w.mtil.p;
-  T* fhi;
-  T* flo = nullptr;
-  if (sizeof(T) == sizeof(double)) {
-    fhi = reinterpret_cast<T*>(f);
-  } else {
-    fhi = w.fhi.get(c->ncdN());
-    flo = w.flo.get(c->ncdN());
-    REG_CUDA(cudaMemsetAsync(flo, 0, c->ncdN() * sizeof(T), c->s));
-  }
-  REG_CUDA(cudaMemsetAsync(fhi, 0, c->ncdN() * sizeof(T), c->s));
+  BodyForce<T> bf(c, f);
+  const T* lt = w.lam.p;
   // lam_1 = m_R - m_1 and the source at t_1
-  lincomb_t<T>((T)1, w.mR.p, (T)-1, w.m1.p, lam, N, c->s);
-  divh<T>(c, lam, vel_node<T>(c, wcoef, c->n_t, wa), nullptr, sB, nullptr, 0);
+  T* lam1 = ring_slot(ringL, kForceNodes, N);
+  lincomb_t<T>((T)1, w.mR.p, (T)-1, w.m1.p, lam1, N, c->s);
+  const T* lam = lam1;
+  NodeVel<T> vt(c, wcoef, w.wa, w.wb);
+  divh<T>(c, lam, vt.get(c->n_t), nullptr, sB, nullptr, 0);
+  int k = 0;
   const int K = c->ckpt > 0 ? c->ckpt : c->n_t;
   for (int seg = (c->n_t - 1) / K; seg >= 0; --seg) {
     int j0 = seg * K, j1 = j0 + K;
     int base = 0;
     if (c->ckpt > 0) {
+      bf.flush();
       recompute_segment<T>(c, vcoef, j0, j1);
       base = j0;
     }
+    NodeVel<T> v(c, vcoef, w.va, w.vb);
     for (int j = j1 - 1; j >= j0; --j) {
-      // incremental stage 1 at t_{j+1}, with the force of node j+1
-      grad_fused<T>(c, mtil + (long)(j + 1) * N, Gt);
+      T* gt = ring_slot(Gt, k, dN);
+      T* lt2 = ring_slot(ringT, k, N);
+      T* lam2 = ring_slot(ringL, k, N);
+      ++k;
+      // force of node j+1
+      grad_fused<T>(c, mtil + (long)(j + 1) * N, gt);
+      bf.add(lt, gm_slot<T>(c, j + 1, base), j + 1, c->trap_w(j + 1));
+      bf.with(lam, gt);
+      // incremental stage 1 at t_{j+1}
       fused::DivEpi<T> e{};
-      e.f_hi = fhi;
-      e.f_lo = flo;
-      e.nc = c->n_c;
-      e.d = c->d;
-      e.N = N;
-      e.gmA = gm_slot<T>(c, j + 1, base);
-      e.gmC = Gt;
-      e.yC = lam;
-      Coefs a = c->basis_at_node(j + 1, c->trap_w(j + 1));
-      for (int l = 0; l < c->n_c; ++l) e.cA[l] = (T)a.c[l];
       e.src = sB;
-      const T* vB = vel_node<T>(c, vcoef, j + 1, vb);
-      const T* vA = vel_node<T>(c, vcoef, j, va);
+      const T* vB = v.get(j + 1);
       divh<T>(c, lt, vB, lt, yh, acc, 1, e);
       // adjoint step lam_{j+1} -> lam_j
       divh<T>(c, lam, vB, lam, yh2, acc2, 1);
-      divh<T>(c, yh2, vA, acc2, lam, nullptr, 2);
+      const T* vA = v.get(j);
+      divh<T>(c, yh2, vA, acc2, lam2, nullptr, 2);
       // source at t_j, then incremental stage 2
-      divh<T>(c, lam, vel_node<T>(c, wcoef, j, wa), nullptr, sA, nullptr, 0);
+      divh<T>(c, lam2, vt.get(j), nullptr, sA, nullptr, 0);
       fused::DivEpi<T> e2{};
       e2.src = sA;
-      divh<T>(c, yh, vA, acc, lt, nullptr, 2, e2);
+      divh<T>(c, yh, vA, acc, lt2, nullptr, 2, e2);
       std::swap(sA, sB);  // the source at t_j is the next step's source at t_{j+1}
+      lt = lt2;
+      lam = lam2;
+      if (bf.F.count == kForceNodes) bf.flush();
     }
     if (j0 == 0)  // node 0: m~_0 = 0, so only the Gauss-Newton term
-      force_acc<T>(fhi, flo, lt, gm_slot<T>(c, 0, base), c->basis_at_node(0, c->trap_w(0)), c->n_c, c->d, N, c->s);
+      bf.add(lt, gm_slot<T>(c, 0, base), 0, c->trap_w(0));
   }
-  if (flo) pair_to_double(reinterpret_cast<const float*>(fhi), reinterpret_cast<const float*>(flo), f, c->ncdN(), c->s);
+  bf.finish();
 }
 
 // Incremental state solve forward from 0 (Eq. gauss-newton, first line), then
@@ -579,10 +630,7 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
   T* y = w.lam.get(N);  // the incremental state ends up as -lam~_1 in place
   T* yh = w.yh.get(N);
   T* acc = w.acc.get(N);
-  T* va = w.va.get(dN);
-  T* vb = w.vb.get(dN);
-  T* wa = w.wa.get(dN);
-  T* wb = w.wb.get(dN);
+  NodeVel<T> v(c, vcoef, w.va, w.vb), vt(c, wcoef, w.wa, w.wb);
   const bool use_src = !c->quad;
   const int K = c->ckpt > 0 ? c->ckpt : c->n_t;
   T* mtil = nullptr;
@@ -593,7 +641,7 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
   if (use_src && c->ckpt == 0) {
     T* src = w.src.get((size_t)(c->n_t + 1) * N);
     for (int j = 0; j <= c->n_t; ++j)
-      dot_fields<T>(gm_slot<T>(c, j, 0), vel_node<T>(c, wcoef, j, wa), src + (long)j * N, c->d, N, c->s);
+      dot_fields<T>(gm_slot<T>(c, j, 0), vt.get(j), src + (long)j * N, c->d, N, c->s);
   }
   if (use_src && c->ckpt > 0 && c->d == 3) {
     // Checkpointed 3D sweep: the state re-advance and the incremental sweep
@@ -611,8 +659,8 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
       REG_CUDA(cudaMemcpyAsync(m, w.ck.p + (long)(j0 / c->ckpt) * N, N * sizeof(T), cudaMemcpyDeviceToDevice,
                                c->s));
       for (int j = j0; j < j1; ++j) {
-        const T* vA = vel_node<T>(c, vcoef, j, va);
-        const T* wA = vel_node<T>(c, wcoef, j, wa);
+        const T* vA = v.get(j);
+        const T* wA = vt.get(j);
         fused::AdvEpi<T> sA = adv_epi<T>(c, vA, m, yhS, accS, 1, nullptr, wA, sj);
         if (j == 0) {
           adv<T>(c, m, vA, nullptr, nullptr, m, yhS, accS, nullptr, 1, nullptr, wA, sj);
@@ -623,7 +671,7 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
           if (mtil)
             REG_CUDA(cudaMemcpyAsync(mtil + (long)j * N, y, N * sizeof(T), cudaMemcpyDeviceToDevice, c->s));
         }
-        const T* vB = vel_node<T>(c, vcoef, j + 1, vb);
+        const T* vB = v.get(j + 1);
         if (j == 0) {
           adv<T>(c, yhS, vB, nullptr, nullptr, accS, m, nullptr, nullptr, 2);
           lincomb_t<T>(-h, sj, (T)0, nullptr, yh, N, c->s);
@@ -636,9 +684,9 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
       }
     }
     // the source at t_{n_t} from the final state, and the last incremental stage 2
-    const T* vN = vel_node<T>(c, vcoef, c->n_t, va);
-    fused::AdvEpi<T> sN = adv_epi<T>(c, nullptr, nullptr, nullptr, nullptr, 1, nullptr,
-                                     vel_node<T>(c, wcoef, c->n_t, wa), sj);
+    const T* vN = v.get(c->n_t);
+    fused::AdvEpi<T> sN = adv_epi<T>(c, nullptr, nullptr, nullptr, nullptr, 1, nullptr, vt.get(c->n_t),
+                                     sj);
     fused::AdvEpi<T> iN = adv_epi<T>(c, vN, acc, y, nullptr, 2);
     iN.src_from_a = 1;
     adv2<T>(c, m, sN, yh, iN);
@@ -652,9 +700,10 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
       if (use_src) recompute_segment_src<T>(c, vcoef, wcoef, j0, j1);
       else recompute_segment<T>(c, vcoef, j0, j1);
       base = j0;
+      v = NodeVel<T>(c, vcoef, w.va, w.vb);  // the re-advance used the same buffers
+      vt = NodeVel<T>(c, wcoef, w.wa, w.wb);
     }
     for (int j = j0; j < j1; ++j) {
-      const T* vA = vel_node<T>(c, vcoef, j, va);
       if (use_src) {
         const T* s1 = w.src.p + (long)(j - base) * N;
         const T* s2 = w.src.p + (long)(j + 1 - base) * N;
@@ -662,22 +711,21 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
           lincomb_t<T>(-h, s1, (T)0, nullptr, yh, N, c->s);
           lincomb_t<T>((T)(-0.5) * h, s1, (T)0, nullptr, acc, N, c->s);
         } else {
-          adv<T>(c, y, vA, nullptr, nullptr, y, yh, acc, nullptr, 1, s1);
+          adv<T>(c, y, v.get(j), nullptr, nullptr, y, yh, acc, nullptr, 1, s1);
         }
-        adv<T>(c, yh, vel_node<T>(c, vcoef, j + 1, vb), nullptr, nullptr, acc, y, nullptr, nullptr, 2, s2);
+        adv<T>(c, yh, v.get(j + 1), nullptr, nullptr, acc, y, nullptr, nullptr, 2, s2);
         if (mtil)
           REG_CUDA(cudaMemcpyAsync(mtil + (long)(j + 1) * N, y, N * sizeof(T), cudaMemcpyDeviceToDevice, c->s));
       } else {
         const T* g1 = gm_slot<T>(c, j, base);
         const T* g2 = gmh_slot<T>(c, j + 1, base);
-        const T* wA = vel_node<T>(c, wcoef, j, wa);
+        const T* wA = vt.get(j);
         if (j == 0) {
-          transport_stage1<T>(nullptr, vA, g1, wA, nullptr, h, yh, acc, c->d, N, c->s);
+          transport_stage1<T>(nullptr, v.get(j), g1, wA, nullptr, h, yh, acc, c->d, N, c->s);
         } else {
-          adv<T>(c, y, vA, g1, wA, y, yh, acc, nullptr, 1);
+          adv<T>(c, y, v.get(j), g1, wA, y, yh, acc, nullptr, 1);
         }
-        adv<T>(c, yh, vel_node<T>(c, vcoef, j + 1, vb), g2, vel_node<T>(c, wcoef, j + 1, wb), acc, y, nullptr,
-               nullptr, 2);
+        adv<T>(c, yh, v.get(j + 1), g2, vt.get(j + 1), acc, y, nullptr, nullptr, 2);
       }
     }
   }
@@ -825,7 +873,7 @@ size_t graph_signature(reg_ctx* c) {
                         c->w64.acc2.p, c->w32.acc2.p, c->w64.st0.p,  c->w32.st0.p,  c->w64.st1.p,  c->w32.st1.p,
                         c->w64.Gt.p,   c->w32.Gt.p,   c->w64.gx2.p,  c->w32.gx2.p,  c->w64.gy2.p,  c->w32.gy2.p,
                         c->w64.yhS.p,  c->w32.yhS.p,  c->w64.accS.p, c->w32.accS.p,
-                        c->w64.srcS.p, c->w32.srcS.p};
+                        c->w64.srcS.p, c->w32.srcS.p, c->w64.lamR.p, c->w32.lamR.p, c->w64.yhR.p,  c->w32.yhR.p};
   size_t h = 1469598103934665603ull;
   for (const void* p : ptrs) h = (h ^ (size_t)p) * 1099511628211ull;
   // and the settings that change what the matvec computes
@@ -891,7 +939,7 @@ double cfl(reg_ctx* c, const double* v) {
   for (int j = 0; j < nodes; ++j) {
     const double* vj = v;
     if (c->n_c > 1) {
-      vel_at<double, double>(v, c->n_c, c->basis_at_node(j), vt, dN, c->s);
+      vel_at<double>(v, c->n_c, c->basis_at_node(j), vt, dN, c->s);
       vj = vt;
     }
     for (int i = 0; i < c->d; ++i) {
@@ -927,8 +975,8 @@ double* defgrad(reg_ctx* c, const double* v, int substeps) {
       const double* gg = gvl;
       if (nc > 1) {
         Coefs b = basis_at(c, t);
-        vel_at<double, double>(v, nc, b, vt, dN, c->s);
-        vel_at<double, double>(gvl, nc, b, gvt, ddN, c->s);
+        vel_at<double>(v, nc, b, vt, dN, c->s);
+        vel_at<double>(gvl, nc, b, gvt, ddN, c->s);
         vv = vt;
         gg = gvt;
       }
@@ -1018,14 +1066,13 @@ void displacement(reg_ctx* c, const double* v, double* u) {
   const long N = c->N(), dN = c->dN();
   double* yh = w.yh.get(N);
   double* acc = w.acc.get(N);
-  double* va = w.va.get(dN);
-  double* vb = w.vb.get(dN);
+  NodeVel<double> nv(c, v, w.va, w.vb);
   double* s1 = c->disp_src.get(2 * N);
   double* s2 = s1 + N;
   REG_CUDA(cudaMemsetAsync(u, 0, dN * sizeof(double), c->s));
   for (int j = 0; j < c->n_t; ++j) {
-    const double* vA = vel_node<double>(c, v, j, va);
-    const double* vB = vel_node<double>(c, v, j + 1, vb);
+    const double* vA = nv.get(j);
+    const double* vB = nv.get(j + 1);
     for (int i = 0; i < c->d; ++i) {
       double* ui = u + (long)i * N;
       lincomb_t<double>(-1.0, vA + (long)i * N, 0.0, nullptr, s1, N, c->s);
@@ -1483,7 +1530,7 @@ void cfl_seg(reg_ctx* c, const double* v, std::vector<double>& out) {
   for (int j = 0; j < nodes; ++j) {
     const double* vj = v;
     if (c->n_c > 1) {
-      vel_at<double, double>(v, c->n_c, c->basis_at_node(j), vt, dN, c->s);
+      vel_at<double>(v, c->n_c, c->basis_at_node(j), vt, dN, c->s);
       vj = vt;
     }
     for (int i = 0; i < c->d; ++i) {
@@ -2235,7 +2282,7 @@ reg_status reg_transport_adjoint(reg_ctx* ctx, const double* v, const double* m0
   Work<double>& w = c_->w64;
   lincomb_t<double>(-1.0, Gd, 0.0, nullptr, w.lam.get(N), N, c_->s);  // lam_1 = -G
   double* f = c_->f.get(c_->ncdN());
-  adjoint_solve<double>(c_, vc, f);
+  const double* lam0 = adjoint_solve<double>(c_, vc, f);
   if (grad_v) {
     Output o(c_, grad_v, c_->ncdN(), c_->stage_out);
     REG_CUDA(cudaMemcpyAsync(o.dev, f, c_->ncdN() * sizeof(double), cudaMemcpyDeviceToDevice, c_->s));
@@ -2243,7 +2290,7 @@ reg_status reg_transport_adjoint(reg_ctx* ctx, const double* v, const double* m0
   }
   if (grad_m0) {
     Output o(c_, grad_m0, N, c_->stage_out);
-    lincomb_t<double>(-1.0, w.lam.p, 0.0, nullptr, o.dev, N, c_->s);
+    lincomb_t<double>(-1.0, lam0, 0.0, nullptr, o.dev, N, c_->s);
     o.finish();
   }
   REG_CUDA(cudaStreamSynchronize(c_->s));

@@ -7,7 +7,7 @@
 //   rows     the derivative along the contiguous last axis, and with it the
 //            stage's pointwise epilogue, which reads the column derivatives:
 //     advection  k = -v . grad u [- grad m . v~], Heun update, optional store of grad u
-//     divergence k = div(v lam),                  Heun update, body-force accumulation
+//     divergence k = div(v lam),                  Heun update
 // Both work on real fields: two neighbouring real lines form one complex line
 // (line.cuh). Spectra are never stored.
 #pragma once
@@ -40,13 +40,9 @@ struct AdvEpi {
 };
 
 // Epilogue parameters of the divergence stage (adjoint / incremental adjoint).
-// Stage 1 can also accumulate the body force f_l,i += cA_l y gmA_i (+ cB_l out1
-// gmB_i): the trapezoid term of node j+1, or the two stage terms of the
-// discrete adjoint. The accumulator is f_hi (+ f_lo) with layout [n_c][d][N];
-// with f_lo set, (f_hi, f_lo) is a compensated pair (exact two-sum per add).
 // Stage 0 only evaluates: out1 = div(v lam) (+ src). src (optional) is added
 // to the divergence (the div(v~ lam) source of the full Newton incremental
-// adjoint). gmC/yC (optional) add the Newton force term cA_l yC gmC_i.
+// adjoint).
 template <typename T>
 struct DivEpi {
   const T* y;  // stage 1: lam_{j+1}; stage 2: acc
@@ -54,16 +50,7 @@ struct DivEpi {
   T* out2;
   T h;
   int stage;
-  T* f_hi;          // null: no force accumulation
-  T* f_lo;          // null: plain accumulation into f_hi
-  const T* gmA;     // d fields at stride N
-  const T* gmB;     // d fields or null
-  T cA[16], cB[16]; // per-coefficient weights
-  int nc, d;
-  long N;
-  const T* src;     // added to the divergence
-  const T* gmC;     // d fields or null
-  const T* yC;
+  const T* src;  // added to the divergence
 };
 
 // Advection epilogue on the point pair q with the gradient components g[0..D)
@@ -117,21 +104,21 @@ __device__ __forceinline__ cx<T> adv_point(const AdvEpi<T>& e, const cx<T>* g, l
     }
   }
   C r1;
+  const T h2 = (T)0.5 * e.h;
   if (e.stage == 1) {
     C yv = e.y ? reinterpret_cast<const C*>(e.y)[q] : mk<C>(0, 0);
     r1 = mk<C>(yv.x + e.h * k0, yv.y + e.h * k1);
-    reinterpret_cast<C*>(e.out2)[q] = mk<C>(yv.x + (T)0.5 * e.h * k0, yv.y + (T)0.5 * e.h * k1);
+    reinterpret_cast<C*>(e.out2)[q] = mk<C>(yv.x + h2 * k0, yv.y + h2 * k1);
   } else {
     C yv = reinterpret_cast<const C*>(e.y)[q];
-    r1 = mk<C>(yv.x + (T)0.5 * e.h * k0, yv.y + (T)0.5 * e.h * k1);
+    r1 = mk<C>(yv.x + h2 * k0, yv.y + h2 * k1);
   }
   reinterpret_cast<C*>(e.out1)[q] = r1;
   return so;
 }
 
-// Divergence epilogue on the point pair q with the divergence value k (scaled,
-// real space): Heun stage update and, in stage 1, the optional body-force
-// accumulation (see DivEpi).
+// Divergence epilogue on the point pair q with the divergence value k: Heun
+// stage update.
 template <typename T>
 __device__ __forceinline__ void div_point(const DivEpi<T>& dv, cx<T> k, long q) {
   using C = cx<T>;
@@ -144,61 +131,12 @@ __device__ __forceinline__ void div_point(const DivEpi<T>& dv, cx<T> k, long q) 
     return;
   }
   C yv = reinterpret_cast<const C*>(dv.y)[q];
-  if (dv.stage != 1) {
-    reinterpret_cast<C*>(dv.out1)[q] = mk<C>(yv.x + (T)0.5 * dv.h * k.x, yv.y + (T)0.5 * dv.h * k.y);
-    return;
-  }
-  C o1 = mk<C>(yv.x + dv.h * k.x, yv.y + dv.h * k.y);
-  reinterpret_cast<C*>(dv.out1)[q] = o1;
-  reinterpret_cast<C*>(dv.out2)[q] = mk<C>(yv.x + (T)0.5 * dv.h * k.x, yv.y + (T)0.5 * dv.h * k.y);
-  if (!dv.f_hi) return;
-  // products of the point pair with every component, then per coefficient
-  // all loads before any store
-  C ta[3], tb[3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    ta[i] = tb[i] = mk<C>(0, 0);
-    if (i < dv.d) {
-      C ga = reinterpret_cast<const C*>(dv.gmA + i * dv.N)[q];
-      ta[i] = mk<C>(yv.x * ga.x, yv.y * ga.y);
-      if (dv.gmC) {
-        C gc = reinterpret_cast<const C*>(dv.gmC + i * dv.N)[q];
-        C yc = reinterpret_cast<const C*>(dv.yC)[q];
-        ta[i] = mk<C>(ta[i].x + yc.x * gc.x, ta[i].y + yc.y * gc.y);
-      }
-      if (dv.gmB) {
-        C gb = reinterpret_cast<const C*>(dv.gmB + i * dv.N)[q];
-        tb[i] = mk<C>(o1.x * gb.x, o1.y * gb.y);
-      }
-    }
-  }
-  for (int l = 0; l < dv.nc; ++l) {
-    C hi[3], lo[3];
-    C* Hf = reinterpret_cast<C*>(dv.f_hi + (long)l * dv.d * dv.N);
-    C* Lo = dv.f_lo ? reinterpret_cast<C*>(dv.f_lo + (long)l * dv.d * dv.N) : nullptr;
-    const long hN = dv.N / 2;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-      if (i < dv.d) {
-        hi[i] = Hf[i * hN + q];
-        lo[i] = Lo ? Lo[i * hN + q] : mk<C>(0, 0);
-      }
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-      if (i < dv.d) {
-        T t0 = dv.cA[l] * ta[i].x + dv.cB[l] * tb[i].x;
-        T t1 = dv.cA[l] * ta[i].y + dv.cB[l] * tb[i].y;
-        if (Lo) {
-          C h = hi[i];
-          T s0 = h.x + t0, b0 = s0 - h.x, s1 = h.y + t1, b1 = s1 - h.y;
-          lo[i].x += (h.x - (s0 - b0)) + (t0 - b0);
-          lo[i].y += (h.y - (s1 - b1)) + (t1 - b1);
-          Hf[i * hN + q] = mk<C>(s0, s1);
-          Lo[i * hN + q] = lo[i];
-        } else {
-          Hf[i * hN + q] = mk<C>(hi[i].x + t0, hi[i].y + t1);
-        }
-      }
+  const T h2 = (T)0.5 * dv.h;
+  if (dv.stage == 1) {
+    reinterpret_cast<C*>(dv.out1)[q] = mk<C>(yv.x + dv.h * k.x, yv.y + dv.h * k.y);
+    reinterpret_cast<C*>(dv.out2)[q] = mk<C>(yv.x + h2 * k.x, yv.y + h2 * k.y);
+  } else {
+    reinterpret_cast<C*>(dv.out1)[q] = mk<C>(yv.x + h2 * k.x, yv.y + h2 * k.y);
   }
 }
 

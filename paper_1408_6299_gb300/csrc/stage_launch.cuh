@@ -221,8 +221,7 @@ void div_stage_impl(Spectral<T>& sp, const T* lam, const T* a, const DivEpi<T>& 
   r.gy[0] = g.d == 3 ? ky : nullptr;
   r.dv = e;
   r.nrows = g.rows;
-  double f = 2 + g.d - 1 + (e.stage && e.y != lam ? 1 : 0) + (e.stage == 1 ? 2 : 1) + (e.src ? 1 : 0);
-  if (e.f_hi) f += g.d * (e.gmB ? 2 : 1) + (e.gmC ? g.d + 1 : 0) + 2.0 * e.nc * g.d * (e.f_lo ? 2 : 1);
+  const double f = 2 + g.d - 1 + (e.stage && e.y != lam ? 1 : 0) + (e.stage == 1 ? 2 : 1) + (e.src ? 1 : 0);
   run_rows<T, EPI_DIV>(sp, r, f * N * sizeof(T), s);
 }
 
