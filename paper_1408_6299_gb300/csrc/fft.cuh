@@ -100,136 +100,4 @@ template <typename T> struct Dft<T, 1> {
   static __device__ __forceinline__ void run(cx<T>*) {}
 };
 
-// ---------------------------------------------------------------------------
-// Radix plans: L = R0 * R1 * ...; stage s has Ns = R0*...*R_{s-1}.
-// ---------------------------------------------------------------------------
-template <int L> struct Plan;
-template <> struct Plan<2> { static constexpr int S = 1; static constexpr int R[3] = {2, 1, 1}; };
-template <> struct Plan<4> { static constexpr int S = 1; static constexpr int R[3] = {4, 1, 1}; };
-template <> struct Plan<8> { static constexpr int S = 1; static constexpr int R[3] = {8, 1, 1}; };
-template <> struct Plan<16> { static constexpr int S = 1; static constexpr int R[3] = {16, 1, 1}; };
-template <> struct Plan<32> { static constexpr int S = 2; static constexpr int R[3] = {8, 4, 1}; };
-template <> struct Plan<64> { static constexpr int S = 2; static constexpr int R[3] = {8, 8, 1}; };
-template <> struct Plan<128> { static constexpr int S = 2; static constexpr int R[3] = {16, 8, 1}; };
-template <> struct Plan<256> { static constexpr int S = 2; static constexpr int R[3] = {16, 16, 1}; };
-template <> struct Plan<512> { static constexpr int S = 3; static constexpr int R[3] = {8, 8, 8}; };
-
-// Real floating-point operations of Dft<T,R>::run: two half-size DFTs, R
-// complex additions and one complex multiplication (6 operations) per
-// constant twiddle that is not a multiple of -i.
-__host__ __device__ constexpr double dft_flops(int R) {
-  if (R <= 1) return 0.0;
-  int general = 0;
-  for (int k = 0; k < R / 2; ++k)
-    if (((k * 16 / R) % 16) % 4 != 0) ++general;
-  return 2.0 * dft_flops(R / 2) + 2.0 * R + 6.0 * general;
-}
-
-// Real floating-point operations of one forward transform of length L along
-// the radix plan: the butterflies of every stage and the complex twiddle
-// multiplications between stages (counted for every stage after the first,
-// trivial table entries included, as the kernels execute them).
-template <int L>
-constexpr double fft_flops() {
-  using P = Plan<L>;
-  double f = 0.0;
-  for (int s = 0; s < P::S; ++s) {
-    f += (double)(L / P::R[s]) * dft_flops(P::R[s]);
-    if (s > 0) f += (double)(L / P::R[s]) * (P::R[s] - 1) * 6.0;
-  }
-  return f;
-}
-
-// Offset of stage s's twiddle block inside the table of length L. Stage s
-// (radix R, Ns previous) stores W_{Ns R}^{r k} at [r*Ns + k], r < R, k < Ns.
-// Stage 0 needs none.
-__host__ __device__ constexpr int stage_tw_offset(int L, int s) {
-  // blocks of stages 1..s-1 come first; each block of stage t has R_t*Ns_t = Ns_{t+1} entries
-  int off = 0, ns = 1;
-  int r[3] = {0, 0, 0};
-  if (L == 2) { r[0] = 2; }
-  else if (L == 4) { r[0] = 4; }
-  else if (L == 8) { r[0] = 8; }
-  else if (L == 16) { r[0] = 16; }
-  else if (L == 32) { r[0] = 8; r[1] = 4; }
-  else if (L == 64) { r[0] = 8; r[1] = 8; }
-  else if (L == 128) { r[0] = 16; r[1] = 8; }
-  else if (L == 256) { r[0] = 16; r[1] = 16; }
-  else if (L == 512) { r[0] = 8; r[1] = 8; r[2] = 8; }
-  for (int t = 0; t < s; ++t) {
-    if (t > 0) off += ns * r[t];
-    ns *= r[t];
-  }
-  return off;
-}
-
-// Padded shared-memory index: one spare slot after every 16 elements keeps
-// strided stage stores free of bank conflicts for 8- and 16-byte elements.
-__device__ __forceinline__ int pad16(int i) { return i + (i >> 4); }
-__host__ __device__ constexpr int padded_len(int n) { return n + n / 16; }
-
-// One forward radix-R Stockham stage (natural order in, natural order out),
-// in place in shared memory, on B sequences of length L.
-//   element j of sequence b lives at buf[b*bs + pad16(j)] (ROWS layout) or at
-//   buf[j*bs + b] (COLS layout, bs = number of columns; neighbouring threads
-//   take neighbouring columns, so no padding is needed there).
-// Every thread loads all its butterflies into registers, the block
-// synchronises, then the results are stored; a second barrier follows.
-template <typename T, int L, int R, int NS, bool COLS, int NT, int B>
-__device__ __forceinline__ void stockham_stage(cx<T>* buf, int bs, const cx<T>* __restrict__ tw) {
-  constexpr int Q = L / R;  // butterflies per sequence
-  constexpr int tasks = B * Q;
-  constexpr int MAXT = (tasks + NT - 1) / NT;  // butterflies held per thread
-  cx<T> v[MAXT][R];
-  int nmine = 0;
-#pragma unroll
-  for (int it = 0; it < MAXT; ++it) {
-    int t = threadIdx.x + it * NT;
-    if (t < tasks) {
-      int b = COLS ? (t % B) : (t / Q);
-      int j = COLS ? (t / B) : (t % Q);
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        int e = j + r * Q;
-        v[it][r] = COLS ? buf[e * bs + b] : buf[b * bs + pad16(e)];
-      }
-      if constexpr (NS > 1) {
-        int k = j % NS;
-#pragma unroll
-        for (int r = 1; r < R; ++r) v[it][r] = cmul(v[it][r], __ldg(&tw[r * NS + k]));
-      }
-      Dft<T, R>::run(v[it]);
-      nmine = it + 1;
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int it = 0; it < MAXT; ++it) {
-    if (it < nmine) {
-      int t = threadIdx.x + it * NT;
-      int b = COLS ? (t % B) : (t / Q);
-      int j = COLS ? (t / B) : (t % Q);
-      int base = (j / NS) * NS * R + (j % NS);
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        int e = base + r * NS;
-        if (COLS) buf[e * bs + b] = v[it][r];
-        else buf[b * bs + pad16(e)] = v[it][r];
-      }
-    }
-  }
-  __syncthreads();
-}
-
-// Full forward FFT of length L on B (compile-time) sequences held in shared memory.
-// tw: device table for length L (stage blocks, see stage_tw_offset).
-template <typename T, int L, bool COLS, int NT, int B>
-__device__ __forceinline__ void smem_fft(cx<T>* buf, int bs, const cx<T>* __restrict__ tw) {
-  using P = Plan<L>;
-  constexpr int R0 = P::R[0], R1 = P::R[1], R2 = P::R[2];
-  stockham_stage<T, L, R0, 1, COLS, NT, B>(buf, bs, tw);
-  if constexpr (P::S > 1) stockham_stage<T, L, R1, R0, COLS, NT, B>(buf, bs, tw + stage_tw_offset(L, 1));
-  if constexpr (P::S > 2) stockham_stage<T, L, R2, R0 * R1, COLS, NT, B>(buf, bs, tw + stage_tw_offset(L, 2));
-}
-
 }  // namespace reg

@@ -146,13 +146,23 @@ struct LineFixed {
 };
 
 template <int L>
-constexpr int fx_headroom() {
+__host__ __device__ constexpr int fx_headroom() {
   return L == 512 ? 60 : 61;
 }
 
 // the largest magnitude of a pair, as the high word of a double (ordered as an unsigned number)
 __device__ __forceinline__ unsigned fx_mag(double2 x) {
   return max((unsigned)__double2hiint(x.x) & 0x7fffffffu, (unsigned)__double2hiint(x.y) & 0x7fffffffu);
+}
+
+// |x| + |y| to about 2^-20, for magnitudes from 2^-126 to 2^100 (smaller ones
+// count as zero), from the high words alone
+__device__ __forceinline__ float fx_l1(double2 x) {
+  auto f = [](double v) {
+    const int h = min(__double2hiint(v) & 0x7fffffff, (1023 + 100) << 20);
+    return __int_as_float(max(h - (896 << 20), 0) << 3);
+  };
+  return f(x.x) + f(x.y);
 }
 
 // Scaling of one line from the high word of its largest magnitude. Lines whose
@@ -163,6 +173,7 @@ struct FxScale {
   static constexpr int S0 = fx_headroom<L>() - ilog2_c(R0), S = fx_headroom<L>() - ilog2_c(L);
   int up, down, low;  // exponent shifts in the high word; smallest exponent that still counts
   bool plain;
+  bool scaled = true;  // the forward stages scale (see Line::forward)
   double pre, post;
   __device__ __forceinline__ explicit FxScale(unsigned mag) {
     pre = post = 1.0;
@@ -200,6 +211,24 @@ struct FxScale {
     if (!plain) x *= post;
     return x;
   }
+  // A line whose sum of magnitudes l1 (see fx_l1) is far below L times its
+  // largest value, as the lines of a decaying spectrum are: no partial sum
+  // exceeds l1, so it is scaled by l1 and its stages do not scale, which keeps
+  // its rounding at one unit of that sum (256 points, spectrum |k|^-1: error
+  // 6e-17 against 4e-16 with the scaling stages and 1.7e-16 in double precision).
+  __device__ __forceinline__ void by_sum(unsigned mag, float l1) {
+    const int e = (int)(mag >> 20);
+    if (e < 1023 - 90 || e > 1023 + 90) return;  // outside fx_l1's range (or inf, NaN)
+    const int h = (int)(__float_as_uint(l1 * 1.0001f) >> 23) - 126 - (e - 1022);  // l1 < 2^(e - 1022 + h)
+    if (h > ilog2_c(L) - 2) return;
+    scaled = false;
+    const int s = fx_headroom<L>() - (h > 0 ? h : 0);
+    up = (s + 1022 - e) * (1 << 20);
+    down = (e - 1022 - s) * (1 << 20);
+    low = (e - 63) * (1 << 20);
+  }
+  // results times 2^n as well
+  __device__ __forceinline__ void times_pow2(int n) { down += n * (1 << 20); }
   __device__ __forceinline__ FxV in(double2 x) const { return {in1(x.x), in1(x.y)}; }
   // the conjugate of z, scaled back
   __device__ __forceinline__ double2 out(FxV z) const { return make_double2(out1(z.x), out1(-z.y)); }

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <functional>
 #include <memory>
 #include <string>
 #include <vector>
@@ -110,8 +111,8 @@ void tune_store(const std::string& key, int choice);
 std::string tune_device_tag();
 
 // Twiddle tables of the line transforms (line.cuh) of one grid's axis lengths,
-// for both plans. kind 0: cx<T> entries; kind 1: paired entries (c, c, s, s)
-// in single precision, fixed-point words in double precision.
+// for both plans. Single precision: kind 0 float2 entries, kind 1 paired
+// entries (c, c, s, s). Double precision: kind 1, fixed-point words.
 template <typename T>
 class LineTables {
  public:
@@ -126,44 +127,47 @@ class LineTables {
   long off_[44];
 };
 
-// Batched power-of-two FFTs and Fourier multipliers on one grid, in precision T.
+// The fixed-point tables of the wide plans of every length 8..512, for callers
+// that place them themselves: byte offsets by log2 L into off; out may be null
+// to query the size in bytes.
+size_t write_wide_tables(unsigned char* out, long* off);
+
+// Fields whose lines, one per group of threads of the wide plan, are fewer
+// threads than this run the narrow plans (line.cuh).
+bool narrow_lines(long wide_threads);
+
+// A grid with its stream and line tables in precision T: what the stages run on.
 template <typename T>
 class Spectral {
  public:
-  using C = cx<T>;
-  Spectral(const Grid& g, cudaStream_t s);
-  // Non-owning engine over device tables laid out as write_tables() lays out
-  // its host image; allocates and copies nothing.
-  Spectral(const Grid& g, cudaStream_t s, C* tables, const long* tw_off, long rc_off);
-  ~Spectral();
-  // Host image of the twiddle tables of every FFT length 4..512 followed by
-  // the real-to-complex tables of every last-axis length 8..512 (double,
-  // interleaved re/im). tw_off[e] / rc_off[e]: complex offset of the tables of
-  // length 2^e. out may be null to query the size; returns complex entries.
-  static long write_tables(double* out, long* tw_off, long* rc_off);
-  Spectral(const Spectral&) = delete;
-  Spectral& operator=(const Spectral&) = delete;
-
+  Spectral(const Grid& g, cudaStream_t s) : g_(g), s_(s), lines_(g) {}
   const Grid& grid() const { return g_; }
   cudaStream_t stream() const { return s_; }
-
-  // real field -> packed spectrum (unnormalised)
-  void fwd(const T* u, C* U);
-  // packed spectrum -> real field (normalised by 1/N); U is overwritten
-  void inv(C* U, T* u);
-  const C* twiddles(int L) const;   // Stockham stage tables for length L
-  const C* rc_twiddles() const;     // exp(-2 pi i k / L_last), k < M
-  const void* line_table(int L, bool narrow, int kind) const { return lines_->get(L, narrow, kind); }
+  const void* line_table(int L, bool narrow, int kind) const { return lines_.get(L, narrow, kind); }
 
  private:
-  void cols(C* U, int axis, bool inverse);
   Grid g_;
   cudaStream_t s_;
-  C* tw_ = nullptr;  // device: tables per length + real/complex table
-  std::unique_ptr<LineTables<T>> lines_;
-  bool owns_ = true;
-  long tw_off_[11] = {0};  // offset of the table of length 2^e
-  long rc_off_ = 0;
+  LineTables<T> lines_;
+};
+
+// Double-precision transforms between real fields and packed half spectra, nf
+// fields at strides N and Nc per call (transform.cu).
+class FieldTransforms {
+ public:
+  using TableFn = std::function<const void*(int L, bool narrow)>;  // fixed-point line tables
+  // tuned: plans by size and autotuned blocks; else the wide plans, nothing measured
+  FieldTransforms(const Grid& g, cudaStream_t s, TableFn tables, bool tuned);
+  void fwd(const double* u, double2* U, int nf) const;  // unnormalised
+  void inv(double2* U, double* u, int nf) const;        // normalised by 1/N; U is overwritten
+
+ private:
+  void cols(double2* U, int axis, int nf, bool inverse) const;
+  bool narrow(int L, long lines) const;
+  Grid g_;
+  cudaStream_t s_;
+  TableFn tables_;
+  bool tuned_;
 };
 
 // ---------------------------------------------------------------------------
@@ -196,13 +200,17 @@ void div_stage(Spectral<T>& sp, const T* lam, const T* a, const fused::DivEpi<T>
 // Fourier-diagonal operators on whole coefficient vectors (FP64), with the
 // DC/Nyquist pairing of the packed last-axis slot 0.
 // ---------------------------------------------------------------------------
+// inv_k2 (device): 1/m for m = 1 .. sum_a (n_a/2)^2 at [m], the reciprocals of
+// every squared wavenumber; null: computed per mode.
+long inv_k2_count(const Grid& g);
+void fill_inv_k2(double* inv_k2, long count, cudaStream_t s);
 // out_l = beta sum_l' Cg[l][l'] a(k) V_l' + (stokes ? K F_l : F_l); F may be null.
 // betas (device, may be null): one beta per stacked problem, replacing beta.
 void spec_tail(const Grid& g, cudaStream_t s, const double2* V, const double2* F, double2* out, int nc,
-               double beta, const double* Cg_dev, int reg, int stokes, const double* betas = nullptr);
+               double beta, const double* Cg_dev, int reg, int stokes, const double* betas, const double* inv_k2);
 // out_l = sum_l' Ci[l][l'] s(k) R_l' with s = 1/(beta a(k)), s = 1 at k = 0.
 void spec_precond(const Grid& g, cudaStream_t s, const double2* R, double2* out, int nc, double beta,
-                  const double* Ci_dev, int reg, const double* betas = nullptr);
+                  const double* Ci_dev, int reg, const double* betas, const double* inv_k2);
 // Gaussian filter exp(-sigma^2 |k|^2 / 2) of one packed FP64 field (out may not alias U)
 void spec_gauss(const Grid& g, cudaStream_t s, double2* U, double2* out, double sigma);
 // trigonometric interpolation of nfields packed FP64 spectra of grid c onto the

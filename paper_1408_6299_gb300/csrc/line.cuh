@@ -67,19 +67,40 @@ __host__ __device__ constexpr int line_ns(int s, bool inv) {
   return n;
 }
 // Offset of stage s's twiddle block in the table of a plan. Stage s >= 1
-// stores W_{Ns R}^{r k} at [r Ns + k]; the forward stages come first, then the
-// inverse ones.
+// stores W_{Ns R}^{r k} at [r Ns + k]. Block 0: the forward stages, block 1: the
+// inverse ones; block 2 (fixed point): the forward stages without their scaling.
+template <class P>
+__host__ __device__ constexpr int line_tw_block(bool inv) {
+  int n = 0;
+  for (int t = 1; t < P::S; ++t) n += line_ns<P>(t, inv) * line_radix<P>(t, inv);
+  return n;
+}
 template <class P>
 __host__ __device__ constexpr int line_tw_offset(int s, bool inv) {
-  int off = 0;
-  if (inv)
-    for (int t = 1; t < P::S; ++t) off += line_ns<P>(t, false) * line_radix<P>(t, false);
+  int off = inv ? line_tw_block<P>(false) : 0;
   for (int t = 1; t < s; ++t) off += line_ns<P>(t, inv) * line_radix<P>(t, inv);
   return off;
 }
-template <class P>
-__host__ __device__ constexpr int line_tw_entries() {
-  return line_tw_offset<P>(P::S, true);
+
+// Real additions and multiplications of one forward transform along the wide
+// plan (radix-2 butterflies, general roots and stage twiddles as 6 each).
+__host__ __device__ constexpr double dft_flops(int R) {
+  if (R <= 1) return 0.0;
+  int general = 0;
+  for (int k = 0; k < R / 2; ++k)
+    if (((k * 16 / R) % 16) % 4 != 0) ++general;
+  return 2.0 * dft_flops(R / 2) + 2.0 * R + 6.0 * general;
+}
+template <int L>
+constexpr double fft_flops() {
+  using P = LinePlan<L, false>;
+  double f = 0.0;
+  for (int s = 0; s < P::S; ++s) {
+    const int r = line_radix<P>(s, false);
+    f += (double)(L / r) * dft_flops(r);
+    if (s > 0) f += (double)(L / r) * (r - 1) * 6.0;
+  }
+  return f;
 }
 
 __host__ __device__ constexpr int ilog2_c(int n) { return n <= 1 ? 0 : 1 + ilog2_c(n / 2); }
@@ -230,7 +251,7 @@ struct Line {
 
   template <int s, bool INV, class Buf, class Sync>
   static __device__ __forceinline__ void stages(V* v, int j, const Buf& buf, const Sync& sync,
-                                                const W* __restrict__ tw) {
+                                                const W* __restrict__ tw, bool scaled = true) {
     constexpr int R = line_radix<P>(s, INV), NS = line_ns<P>(s, INV), Q = L / R, TK = E / R;
     if constexpr (s > 0) {
       const W* t0 = tw + line_tw_offset<P>(s, INV);
@@ -239,7 +260,8 @@ struct Line {
         const int t = j + i * TS;
 #pragma unroll
         for (int r = 0; r < R; ++r) v[i * R + r] = *buf(t + r * Q);
-        if constexpr (!INV) v[i * R] = A::template pass_fwd<R>(v[i * R]);
+        if constexpr (!INV)
+          if (scaled) v[i * R] = A::template pass_fwd<R>(v[i * R]);
 #pragma unroll
         for (int r = 1; r < R; ++r) {
           const W w = __ldg(&t0[r * NS + (t & (NS - 1))]);
@@ -260,17 +282,29 @@ struct Line {
         for (int r = 0; r < R; ++r) *buf(base + r * NS) = v[i * R + r];
       }
       sync();
-      stages<s + 1, INV>(v, j, buf, sync, tw);
+      stages<s + 1, INV>(v, j, buf, sync, tw, scaled);
     }
+  }
+
+  // Forward transform: v as in derivative(), on return v[e] is the value of
+  // frequency(j, e). buf is left with the last exchange (not synchronised).
+  // scaled: fixed-point stages take their inputs times 1/R, as derivative() does.
+  static __device__ __forceinline__ int frequency(int j, int e) {
+    constexpr int R = line_radix<P>(S - 1, false);
+    return j + (e / R) * TS + (e % R) * (L / R);
+  }
+  template <class Buf, class Sync>
+  static __device__ __forceinline__ void forward(V* v, int j, const Buf& buf, const Sync& sync,
+                                                 const W* __restrict__ tw, bool scaled) {
+    stages<0, false>(v, j, buf, sync, scaled ? tw : tw + line_tw_block<P>(false) + line_tw_block<P>(true), scaled);
   }
 
   template <class Buf, class Sync>
   static __device__ __forceinline__ void derivative(V* v, int j, const Buf& buf, const Sync& sync,
                                                     const W* __restrict__ tw) {
     stages<0, false>(v, j, buf, sync, tw);
-    constexpr int R = line_radix<P>(S - 1, false), Q = L / R;
 #pragma unroll
-    for (int e = 0; e < E; ++e) v[e] = A::template deriv<L>(v[e], j + (e / R) * TS + (e % R) * Q);
+    for (int e = 0; e < E; ++e) v[e] = A::template deriv<L>(v[e], frequency(j, e));
     stages<0, true>(v, j, buf, sync, tw);
   }
 };

@@ -1,6 +1,8 @@
 // lines.cu -- twiddle tables of the line transforms (line.cuh, fixed.cuh).
 #include <math.h>
 
+#include <algorithm>
+
 #include "internal.h"
 #include "line.cuh"
 
@@ -46,8 +48,9 @@ template <typename T, int L, bool NARROW>
 void emit(std::vector<unsigned char>& out, int kind) {
   using P = LinePlan<L, NARROW>;
   const Circle& k = circle();
-  for (int inv = 0; inv < 2; ++inv)
+  for (int block = 0; block < (sizeof(T) == 8 ? 3 : 2); ++block)
     for (int s = 1; s < P::S; ++s) {
+      const bool inv = block == 1;
       const int R = line_radix<P>(s, inv), ns = line_ns<P>(s, inv);
       for (int r = 0; r < R; ++r)
         for (int t = 0; t < ns; ++t) {
@@ -59,14 +62,11 @@ void emit(std::vector<unsigned char>& out, int kind) {
           } else if (sizeof(T) == 4) {
             const float2 w = make_float2((float)c, (float)d);
             put(out, &w, sizeof w);
-          } else if (kind == 1) {  // fixed point; the forward stages take 1/R with the twiddle
+          } else {  // fixed point; block 0 takes 1/R with the twiddle
             int4 w;
-            const long double f = inv ? 1.0L : 1.0L / R;
+            const long double f = block == 0 ? 1.0L / R : 1.0L;
             fixed_words(c * f, &w.x, &w.y);
             fixed_words(d * f, &w.z, &w.w);
-            put(out, &w, sizeof w);
-          } else {
-            const double2 w = make_double2((double)c, (double)d);
             put(out, &w, sizeof w);
           }
         }
@@ -97,7 +97,7 @@ LineTables<T>::LineTables(const Grid& g) {
   for (long& o : off_) o = -1;
   for (int a = 0; a < g.d; ++a)
     for (int narrow = 0; narrow < 2; ++narrow)
-      for (int kind = 0; kind < 2; ++kind) {
+      for (int kind = sizeof(T) == 8; kind < 2; ++kind) {
         long& o = off_[table_slot(g.n[a], narrow, kind)];
         if (o >= 0) continue;
         h.resize((h.size() + 15) / 16 * 16);
@@ -116,6 +116,17 @@ template <typename T>
 const void* LineTables<T>::get(int L, bool narrow, int kind) const {
   return dev_ + off_[table_slot(L, narrow, kind)];
 }
+
+size_t write_wide_tables(unsigned char* out, long* off) {
+  std::vector<unsigned char> h;
+  for (int L = 8; L <= 512; L *= 2) {
+    off[ilog2_c(L)] = (long)h.size();
+    emit_any<double>(h, L, false, 1);
+  }
+  if (out) std::copy(h.begin(), h.end(), out);
+  return h.size();
+}
+
 template class LineTables<float>;
 template class LineTables<double>;
 

@@ -38,16 +38,13 @@ constexpr int kMaxDevices = 64;
 struct DeviceState {
   bool ready = false;
   unsigned char* base = nullptr;  // device address of g_precond_scratch
-  long tw_off[11] = {0};
-  long rc_off[11] = {0};
+  long tw_off[11] = {0};  // byte offsets of the tables by log2 of the length
 };
 DeviceState g_dev[kMaxDevices];
 std::mutex g_mu;
 constexpr long kCapacity = (long)((kScratchBytes - kTableBytes - kGramBytes) / (2 * sizeof(double2)));
 
-// host image of the tables (double, interleaved), filled at set-up
-constexpr long kMaxTableEntries = (long)(kTableBytes / 16);
-double g_table_image[2 * kMaxTableEntries];
+unsigned char g_table_image[kTableBytes];  // host image of the tables, filled at set-up
 
 struct GramInverse {
   double c[16 * 16];
@@ -73,10 +70,10 @@ int setup_device(int dev) {
   void* p = nullptr;
   cudaError_t e = cudaGetSymbolAddress(&p, g_precond_scratch);
   if (e != cudaSuccess) return (int)e;
-  long n = Spectral<double>::write_tables(nullptr, S.tw_off, S.rc_off);
-  if (n > kMaxTableEntries) return (int)cudaErrorInvalidValue;
-  Spectral<double>::write_tables(g_table_image, S.tw_off, S.rc_off);
-  e = cudaMemcpy(p, g_table_image, (size_t)n * 16, cudaMemcpyHostToDevice);
+  const size_t n = write_wide_tables(nullptr, S.tw_off);
+  if (n > kTableBytes) return (int)cudaErrorInvalidValue;
+  write_wide_tables(g_table_image, S.tw_off);
+  e = cudaMemcpy(p, g_table_image, n, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return (int)e;
   S.base = (unsigned char*)p;
   S.ready = true;
@@ -151,7 +148,6 @@ reg_status reg_precond_noalloc(int d, const int64_t* n, int n_c, double beta, in
     int st = setup_device(dev);
     if (st != 0) return noalloc_fail(REG_ECUDA, cudaGetErrorString((cudaError_t)st));
     DeviceState& S = g_dev[dev];
-    double2* tables = (double2*)S.base;
     double* Ci = (double*)(S.base + kTableBytes);
     double2* SV = (double2*)(S.base + kTableBytes + kGramBytes);
     double2* SF = SV + ncd * g.Nc;
@@ -161,12 +157,17 @@ reg_status reg_precond_noalloc(int d, const int64_t* n, int n_c, double beta, in
     k_store_gram<<<1, 256, 0, s>>>(Ci, gi, n_c * n_c);
     REG_LAUNCH();
 
-    int e2 = 0;
-    while ((1 << e2) < g.L) ++e2;
-    Spectral<double> sp(g, s, tables, S.tw_off, S.rc_off[e2]);
-    for (long q = 0; q < ncd; ++q) sp.fwd(r + q * g.N, SV + q * g.Nc);
-    spec_precond(g, s, SV, SF, n_c, beta, Ci, reg_type);
-    for (long q = 0; q < ncd; ++q) sp.inv(SF + q * g.Nc, z + q * g.N);
+    const FieldTransforms ft(
+        g, s,
+        [&](int L, bool) {
+          int e2 = 0;
+          while ((1 << e2) < L) ++e2;
+          return S.base + S.tw_off[e2];
+        },
+        false);
+    ft.fwd(r, SV, (int)ncd);
+    spec_precond(g, s, SV, SF, n_c, beta, Ci, reg_type, nullptr, nullptr);
+    ft.inv(SF, z, (int)ncd);
   } catch (const StatusError& e) {
     return noalloc_fail(e.status, e.what);
   } catch (const CudaError& e) {

@@ -133,6 +133,8 @@ struct reg_ctx {
   DBuf<double> Cg_dev, Ci_dev;
 
   std::unique_ptr<Spectral<double>> sp64;
+  std::unique_ptr<FieldTransforms> ft;
+  DBuf<double> ik2;    // reciprocals of the squared wavenumbers (spec_tail, spec_precond)
   std::unique_ptr<Spectral<float>> sp32;
   Work<double> w64;
   Work<float> w32;
@@ -743,6 +745,14 @@ namespace {
 // Fourier-diagonal tail (FP64): out = beta (C (x) A) V + K^gamma F
 // (App. A Eq. control-equation-expansion; Eq. eliminated-control). F may be null.
 // ---------------------------------------------------------------------------
+const double* inv_k2(reg_ctx* c) {
+  if (!c->ik2.p) {
+    const long n = inv_k2_count(c->g);
+    fill_inv_k2(c->ik2.get(n), n, c->s);
+  }
+  return c->ik2.p;
+}
+
 // Without the Leray projection the body force passes the tail unchanged, so it
 // is added in physical space and only V is transformed.
 void tail(reg_ctx* c, const double* V, const double* F, double* out) {
@@ -750,27 +760,24 @@ void tail(reg_ctx* c, const double* V, const double* F, double* out) {
   const int ncd = c->n_c * c->d;
   double2* SV = c->SV.get((size_t)ncd * Nc);
   double2* SF = c->SF.get((size_t)ncd * Nc);
-  Spectral<double>& sp = *c->sp64;
   const bool fspec = F && c->stokes;
-  for (int q = 0; q < ncd; ++q) {
-    sp.fwd(V + q * N, SV + q * Nc);
-    if (fspec) sp.fwd(F + q * N, SF + q * Nc);
-  }
+  c->ft->fwd(V, SV, ncd);
+  if (fspec) c->ft->fwd(F, SF, ncd);
   spec_tail(c->g, c->s, SV, fspec ? SF : nullptr, SF, c->n_c, c->beta, c->Cg_dev.p, c->rtype, c->stokes,
-            c->g.B > 1 ? c->betas_dev.p : nullptr);
-  for (int q = 0; q < ncd; ++q) sp.inv(SF + q * Nc, out + q * N);
+            c->g.B > 1 ? c->betas_dev.p : nullptr, inv_k2(c));
+  c->ft->inv(SF, out, ncd);
   if (F && !fspec) lincomb_t<double>(1.0, out, 1.0, F, out, (long)ncd * N, c->s);
 }
 
 void precond(reg_ctx* c, const double* r, double* z) {
-  const long Nc = c->g.Nc, N = c->N();
+  const long Nc = c->g.Nc;
   const int ncd = c->n_c * c->d;
   double2* SV = c->SV.get((size_t)ncd * Nc);
   double2* SF = c->SF.get((size_t)ncd * Nc);
-  Spectral<double>& sp = *c->sp64;
-  for (int q = 0; q < ncd; ++q) sp.fwd(r + q * N, SV + q * Nc);
-  spec_precond(c->g, c->s, SV, SF, c->n_c, c->beta, c->Ci_dev.p, c->rtype, c->g.B > 1 ? c->betas_dev.p : nullptr);
-  for (int q = 0; q < ncd; ++q) sp.inv(SF + q * Nc, z + q * N);
+  c->ft->fwd(r, SV, ncd);
+  spec_precond(c->g, c->s, SV, SF, c->n_c, c->beta, c->Ci_dev.p, c->rtype, c->g.B > 1 ? c->betas_dev.p : nullptr,
+               inv_k2(c));
+  c->ft->inv(SF, z, ncd);
 }
 
 double* red(reg_ctx* c) { return c->red.get(reduce_scratch_doubles()); }
@@ -1024,13 +1031,13 @@ void detF_refined(reg_ctx* c, const double* v, int substeps, int refine, double 
   }
   std::unique_ptr<reg_ctx> f(create_ctx(c->d, nf, c->n_t, c->n_c, c->beta, c->rtype, c->stokes, REG_FP64, 0, c->s, 1));
   const int ncd = c->n_c * c->d;
-  const long N = c->N(), Nc = c->g.Nc;
+  const long Nc = c->g.Nc;
   double2* P = c->SV.get((size_t)ncd * Nc);
-  for (int q = 0; q < ncd; ++q) c->sp64->fwd(v + q * N, P + q * Nc);
+  c->ft->fwd(v, P, ncd);
   double2* Q = f->SV.get((size_t)ncd * f->g.Nc);
   spec_upsample(c->g, f->g, c->s, P, Q, ncd);
   double* vf = f->vlin.get(f->ncdN());
-  for (int q = 0; q < ncd; ++q) f->sp64->inv(Q + q * f->g.Nc, vf + q * f->N());
+  f->ft->inv(Q, vf, ncd);
   detF(f.get(), vf, substeps, st, det_out);
   REG_CUDA(cudaStreamSynchronize(c->s));  // the fine context's buffers are freed on return
 }
@@ -1053,9 +1060,9 @@ void smooth(reg_ctx* c, double sigma, const double* in, double* out) {
   const long Nc = c->g.Nc;
   double2* S = c->SV.get((size_t)c->n_c * c->d * Nc);
   double2* T = c->SF.get((size_t)c->n_c * c->d * Nc);
-  c->sp64->fwd(in, S);
+  c->ft->fwd(in, S, 1);
   spec_gauss(c->g, c->s, S, T, sigma);
-  c->sp64->inv(T, out);
+  c->ft->inv(T, out, 1);
 }
 
 // Deformation map (App. D Eq. displacement): du_i/dt = -v . grad u_i + v_i,
@@ -2115,6 +2122,8 @@ reg_ctx* create_ctx(int d, const int64_t* n, int n_t, int n_c, double beta, int 
   REG_CUDA(cudaMemcpy(c->Cg_dev.get(n_c * n_c), c->Cg.data(), n_c * n_c * sizeof(double), cudaMemcpyHostToDevice));
   REG_CUDA(cudaMemcpy(c->Ci_dev.get(n_c * n_c), c->Ci.data(), n_c * n_c * sizeof(double), cudaMemcpyHostToDevice));
   c->sp64.reset(new Spectral<double>(g, c->s));
+  c->ft.reset(new FieldTransforms(
+      g, c->s, [c](int L, bool narrow) { return c->sp64->line_table(L, narrow, 1); }, true));
   if (precision == REG_MIXED) c->sp32.reset(new Spectral<float>(g, c->s));
   return holder.release();
 }

@@ -1,287 +1,231 @@
-// spectral.cu -- FFT passes and Fourier multipliers of the pseudospectral
-// discretisation (Mang & Biros, Sec. 3.3.1 Fourier collocation; Sec. 3.3.3 the
-// spectral inverse of beta*A; Sec. 3.3.4 / App. B the Leray projection K).
+// spectral.cu -- Fourier multipliers of the pseudospectral discretisation
+// (Mang & Biros, Sec. 3.3.3 the spectral inverse of beta*A; Sec. 3.3.4 / App. B
+// the Leray projection K), on packed half spectra, and the launch accounting.
 //
-// A d-dimensional real transform is one row pass (packed real-to-complex
-// along the contiguous last axis) followed by one strided complex pass per
-// remaining axis. The packed layout stores the DC and Nyquist columns of the
-// last axis together in slot 0 (see Grid in internal.h); derivative and
-// Leray multipliers treat both halves alike (their last-axis wavenumber is 0
-// for both), while multipliers depending on |k| (A and its inverse) pair the
-// mode k' with -k' to act on the two halves separately.
+// The packed layout stores the DC and Nyquist columns of the last axis
+// together in slot 0 (see Grid in internal.h); Leray multipliers treat both
+// halves alike (their last-axis wavenumber is 0 for both), while multipliers
+// depending on |k| (A and its inverse) pair the mode k' with -k' to act on the
+// two halves separately.
+//
+// The kernels are bound by memory only if they stay off the double-precision
+// unit (two operations per clock and SM): wavenumbers and |k|^2 are integers,
+// and the reciprocals of |k|^2 (one of sum (n_a/2)^2 values) come from a table.
 #include <math.h>
 
 #include <algorithm>
 #include <atomic>
 #include <stdexcept>
 
-#include "tune.h"
+#include "internal.h"
 
 namespace reg {
 
 namespace {
 
-constexpr int kThreads = 256;
-
-__host__ __device__ inline long kfull(long j, long n) { return j < n / 2 ? j : j - n; }
-__host__ __device__ inline long kmask(long j, long n) { return j == n / 2 ? 0 : kfull(j, n); }
-
-// ---------------------------------------------------------------------------
-// Row pass: real rows of length L -> packed complex rows of M = L/2.
-// A real row read as M complex values z_j = x_{2j} + i x_{2j+1} is transformed
-// by an M-point FFT Z; then X_k = E_k + W_L^k O_k with E = (Z_k + conj Z_{M-k})/2,
-// O = (Z_k - conj Z_{M-k})/(2i). Slot 0 receives X_0 + i X_M.
-// ---------------------------------------------------------------------------
-template <typename T, int L, int RB>
-__global__ void __launch_bounds__(kThreads) k_rows_r2c(const T* __restrict__ in, cx<T>* __restrict__ out, long nrows,
-                                                        const cx<T>* __restrict__ tw,
-                                                        const cx<T>* __restrict__ twrc) {
-  using C = cx<T>;
-  constexpr int M = L / 2;
-  constexpr int RS = padded_len(M);
-  __shared__ C buf[RB * RS];
-  const long row0 = (long)blockIdx.x * RB;
-  const C* src = reinterpret_cast<const C*>(in);
-  for (int e = threadIdx.x; e < RB * M; e += kThreads) {
-    int r = e / M, j = e % M;
-    long row = row0 + r;
-    C z = mk<C>(0, 0);
-    if (row < nrows) z = src[row * M + j];
-    buf[r * RS + pad16(j)] = z;
-  }
-  __syncthreads();
-  smem_fft<T, M, false, kThreads, RB>(buf, RS, tw);
-  constexpr int H = M / 2 + 1;
-  for (int e = threadIdx.x; e < RB * H; e += kThreads) {
-    int r = e / H, k = e % H;
-    long row = row0 + r;
-    if (row >= nrows) continue;
-    C* o = out + row * M;
-    if (k == 0) {
-      C z0 = buf[r * RS];
-      o[0] = mk<C>(z0.x + z0.y, z0.x - z0.y);
-    } else {
-      C zk = buf[r * RS + pad16(k)], zm = buf[r * RS + pad16(M - k)];
-      C E = cscale(cadd(zk, cconj(zm)), (T)0.5);
-      C Od = cscale(cmul_mi(csub(zk, cconj(zm))), (T)0.5);
-      C t = cmul(__ldg(&twrc[k]), Od);
-      o[k] = cadd(E, t);
-      if (k != M - k) o[M - k] = cconj(csub(E, t));
-    }
-  }
-}
-
-// Inverse of the row pass, normalised by 1/L.
-template <typename T, int L, int RB>
-__global__ void __launch_bounds__(kThreads) k_rows_c2r(const cx<T>* __restrict__ in, T* __restrict__ out, long nrows,
-                                                        const cx<T>* __restrict__ tw,
-                                                        const cx<T>* __restrict__ twrc) {
-  using C = cx<T>;
-  constexpr int M = L / 2;
-  constexpr int RS = padded_len(M);
-  __shared__ C buf[RB * RS];
-  const long row0 = (long)blockIdx.x * RB;
-  for (int e = threadIdx.x; e < RB * M; e += kThreads) {
-    int r = e / M, j = e % M;
-    long row = row0 + r;
-    C z = mk<C>(0, 0);
-    if (row < nrows) z = in[row * M + j];
-    buf[r * RS + pad16(j)] = z;
-  }
-  __syncthreads();
-  constexpr int H = M / 2 + 1;
-  for (int e = threadIdx.x; e < RB * H; e += kThreads) {
-    int r = e / H, k = e % H;
-    if (k == 0) {
-      C p = buf[r * RS];
-      // X_0 = p.x, X_M = p.y; E_0 = (X_0+X_M)/2, O_0 = (X_0-X_M)/2
-      C z0 = mk<C>((p.x + p.y) * (T)0.5, (p.x - p.y) * (T)0.5);
-      buf[r * RS] = cconj(z0);
-    } else {
-      C xk = buf[r * RS + pad16(k)], xm = buf[r * RS + pad16(M - k)];
-      C E = cscale(cadd(xk, cconj(xm)), (T)0.5);
-      C Od = cscale(cmul(csub(xk, cconj(xm)), cconj(__ldg(&twrc[k]))), (T)0.5);
-      // Z_k = E + i O, Z_{M-k} = conj(E) + i conj(O); stored conjugated for the inverse
-      C zk = mk<C>(E.x - Od.y, E.y + Od.x);
-      C zm = mk<C>(E.x + Od.y, -E.y + Od.x);
-      buf[r * RS + pad16(k)] = cconj(zk);
-      if (k != M - k) buf[r * RS + pad16(M - k)] = cconj(zm);
-    }
-  }
-  __syncthreads();
-  smem_fft<T, M, false, kThreads, RB>(buf, RS, tw);
-  C* dst = reinterpret_cast<C*>(out);
-  const T s = (T)1 / (T)M;
-  for (int e = threadIdx.x; e < RB * M; e += kThreads) {
-    int r = e / M, j = e % M;
-    long row = row0 + r;
-    if (row >= nrows) continue;
-    C z = buf[r * RS + pad16(j)];
-    dst[row * M + j] = mk<C>(z.x * s, -z.y * s);
-  }
-}
-
-// Strided complex pass along one axis: element j of pencil (outer, inner) at
-// data[outer*L*s + j*s + inner]. A block takes TC neighbouring inner indices.
-template <typename T, int L, int TC>
-__global__ void __launch_bounds__(kThreads) k_cols(cx<T>* __restrict__ data, long s, const cx<T>* __restrict__ tw,
-                                                    int inverse) {
-  using C = cx<T>;
-  __shared__ C buf[L * TC];
-  C* base = data + (long)blockIdx.y * L * s + (long)blockIdx.x * TC;
-  for (int e = threadIdx.x; e < L * TC; e += kThreads) {
-    int j = e / TC, c = e % TC;
-    C z = base[(long)j * s + c];
-    buf[j * TC + c] = inverse ? cconj(z) : z;
-  }
-  __syncthreads();
-  smem_fft<T, L, true, kThreads, TC>(buf, TC, tw);
-  const T sc = (T)1 / (T)L;
-  for (int e = threadIdx.x; e < L * TC; e += kThreads) {
-    int j = e / TC, c = e % TC;
-    C z = buf[j * TC + c];
-    base[(long)j * s + c] = inverse ? mk<C>(z.x * sc, -z.y * sc) : z;
-  }
-}
+__host__ __device__ inline int kfull(int j, int n) { return j < n / 2 ? j : j - n; }
+__host__ __device__ inline int kmask(int j, int n) { return j == n / 2 ? 0 : kfull(j, n); }
 
 // mode index q of the packed spectrum -> per-axis indices (last = slot)
 struct ModeIdx {
-  long j[3];
+  int j[3];
 };
-__device__ inline ModeIdx decode(long q, int d, const int* n, int M) {
-  ModeIdx m;
-  m.j[d - 1] = q % M;
-  long rest = q / M;
-  for (int a = d - 2; a >= 0; --a) {
-    m.j[a] = rest % n[a];
-    rest /= n[a];
-  }
-  return m;
-}
 struct GridArgs {
   int d;
   int n[3];
   int M;
   long Nc;   // all stacked problems
-  long Nc1;  // one problem
+  long Nc1;  // one problem (a power of two)
+  int lg1;   // log2 Nc1
 };
-// index of -k' on the slot-0 plane of the problem that holds mode q
+__device__ inline ModeIdx decode(long q, const GridArgs& g) {
+  ModeIdx m;
+  int r = (int)(q & (g.Nc1 - 1));
+  m.j[g.d - 1] = r & (g.M - 1);
+  r /= g.M;
+  for (int a = g.d - 2; a >= 0; --a) {
+    m.j[a] = r & (g.n[a] - 1);
+    r /= g.n[a];
+  }
+  return m;
+}
+// index of -k' on the slot-0 plane of the problem that holds mode q0
 __device__ inline long encode_neg(long q0, const ModeIdx& m, const GridArgs& g) {
-  long q = 0;
-  for (int a = 0; a < g.d - 1; ++a) q = q * g.n[a] + ((g.n[a] - m.j[a]) % g.n[a]);
-  return (q0 / g.Nc1) * g.Nc1 + q * g.M;
+  int q = 0;
+  for (int a = 0; a < g.d - 1; ++a) q = q * g.n[a] + ((g.n[a] - m.j[a]) & (g.n[a] - 1));
+  return (q0 & ~(g.Nc1 - 1)) + (long)q * g.M;
 }
-__device__ inline double masked_k(const ModeIdx& m, const GridArgs& g, int a) {
-  if (a == g.d - 1) return (double)m.j[a];  // slot 0 -> 0 for both DC and Nyquist halves
-  return (double)kmask(m.j[a], g.n[a]);
+__device__ inline int masked_k(const ModeIdx& m, const GridArgs& g, int a) {
+  if (a == g.d - 1) return m.j[a];  // slot 0 -> 0 for both DC and Nyquist halves
+  return kmask(m.j[a], g.n[a]);
 }
-
 // |k|^2 over the leading axes (full wavenumbers, Nyquist kept)
-__device__ inline double lead_k2(const ModeIdx& m, const GridArgs& g) {
-  double kk = 0;
+__device__ inline int lead_k2(const ModeIdx& m, const GridArgs& g) {
+  int kk = 0;
   for (int a = 0; a < g.d - 1; ++a) {
-    double k = (double)kfull(m.j[a], g.n[a]);
+    const int k = kfull(m.j[a], g.n[a]);
     kk += k * k;
   }
   return kk;
 }
-__device__ inline double sym_pow(double kk, int reg) { return reg == 1 ? kk : kk * kk; }
+// |k|^2 or |k|^4 (exact: |k|^2 <= 3 256^2) and its reciprocal
+__device__ inline double sym_pow(int kk, int reg) { return (double)(reg == 1 ? (long long)kk : (long long)kk * kk); }
+__device__ inline double inv_pow(int kk, int reg, const double* __restrict__ inv_k2) {
+  const double r = inv_k2 ? __ldg(&inv_k2[kk]) : 1.0 / (double)kk;
+  return reg == 1 ? r : r * r;
+}
 
 constexpr int kMaxNc = 16;
 
-__global__ void k_spec_tail(const double2* __restrict__ V, const double2* __restrict__ F, double2* __restrict__ out,
-                            GridArgs g, int nc, double beta, const double* __restrict__ Cg, int reg, int stokes,
-                            const double* __restrict__ betas) {
-  long q = (long)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void k_inv_k2(double* t, long n) {
+  const long m = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (m < n) t[m] = m ? 1.0 / (double)m : 0.0;
+}
+
+// NC: n_c where it is 1, 2 or 3 (the coefficients of a component then stay in
+// registers), else 0.
+template <int NC>
+__global__ void __launch_bounds__(256) k_spec_tail(const double2* __restrict__ V, const double2* __restrict__ F,
+                                                   double2* __restrict__ out, GridArgs g, int nc_, double beta,
+                                                   const double* __restrict__ Cg, int reg, int stokes,
+                                                   const double* __restrict__ betas,
+                                                   const double* __restrict__ inv_k2) {
+  const long q = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= g.Nc) return;
-  if (betas) beta = betas[q / g.Nc1];
-  const int d = g.d;
+  if (betas) beta = betas[q >> g.lg1];
+  const int d = g.d, nc = NC ? NC : nc_;
   const long Nc = g.Nc;
-  ModeIdx m = decode(q, d, g.n, g.M);
-  double kk = lead_k2(m, g);
-  long kz = m.j[d - 1];
-  double alpha, delta;
+  const ModeIdx m = decode(q, g);
+  const int kk = lead_k2(m, g), kz = m.j[d - 1];
+  double alpha, delta = 0.0;
   long qn = q;
   if (kz == 0) {
-    double a0 = sym_pow(kk, reg), aN = sym_pow(kk + 0.25 * (double)g.n[d - 1] * g.n[d - 1], reg);
-    alpha = 0.5 * (a0 + aN);
-    delta = 0.5 * (a0 - aN);
+    const double a0 = sym_pow(kk, reg), aN = sym_pow(kk + g.M * g.M, reg);
+    alpha = 0.5 * beta * (a0 + aN);
+    delta = 0.5 * beta * (a0 - aN);
     qn = encode_neg(q, m, g);
   } else {
-    alpha = sym_pow(kk + (double)kz * kz, reg);
-    delta = 0.0;
+    alpha = beta * sym_pow(kk + kz * kz, reg);
   }
   // masked wavenumber for K
-  double kt[3], kt2 = 0;
-  for (int a = 0; a < d; ++a) {
-    kt[a] = masked_k(m, g, a);
-    kt2 += kt[a] * kt[a];
-  }
-  for (int l = 0; l < nc; ++l) {
-    double2 proj[3];
-    if (F) {
-      double dr = 0, di = 0;
-      for (int i = 0; i < d; ++i) {
-        double2 f = F[(l * d + i) * Nc + q];
-        proj[i] = f;
-        dr += kt[i] * f.x;
-        di += kt[i] * f.y;
-      }
-      if (stokes && kt2 > 0)
-        for (int i = 0; i < d; ++i) proj[i] = make_double2(proj[i].x - kt[i] * dr / kt2, proj[i].y - kt[i] * di / kt2);
-    } else {
-      for (int i = 0; i < d; ++i) proj[i] = make_double2(0, 0);
+  int kt[3], kt2 = 0;
+  if (F && stokes)
+    for (int a = 0; a < d; ++a) {
+      kt[a] = masked_k(m, g, a);
+      kt2 += kt[a] * kt[a];
     }
-    for (int i = 0; i < d; ++i) {
-      double sr = 0, si = 0;
-      for (int lp = 0; lp < nc; ++lp) {
-        double c = Cg[l * nc + lp];
-        double2 v = V[(lp * d + i) * Nc + q];
-        double2 vn = V[(lp * d + i) * Nc + qn];
-        // alpha v + delta conj(vn)
-        sr += c * (alpha * v.x + delta * vn.x);
-        si += c * (alpha * v.y - delta * vn.y);
+  auto reg_term = [&](int i, int l, const double2* v, const double2* vn) {
+    double2 s = make_double2(0, 0), n = make_double2(0, 0);
+    for (int lp = 0; lp < nc; ++lp) {
+      const double c = __ldg(&Cg[l * nc + lp]);
+      if (c == 0.0) continue;  // odd pairs of Chebyshev polynomials are orthogonal
+      const double2 x = NC ? v[lp] : V[(lp * d + i) * Nc + q];
+      s.x += c * x.x;
+      s.y += c * x.y;
+      if (kz == 0) {
+        const double2 y = NC ? vn[lp] : V[(lp * d + i) * Nc + qn];
+        n.x += c * y.x;
+        n.y += c * y.y;
       }
-      out[(l * d + i) * Nc + q] = make_double2(beta * sr + proj[i].x, beta * si + proj[i].y);
+    }
+    double2 r = make_double2(alpha * s.x, alpha * s.y);
+    if (kz == 0) r = make_double2(r.x + delta * n.x, r.y - delta * n.y);  // + delta conj(n)
+    return r;
+  };
+  // k . f_l / |k|^2; out may be F, so it is formed before any component of f_l is overwritten
+  auto projection = [&](int l) {
+    double2 p = make_double2(0, 0);
+    if (!(F && stokes && kt2 > 0)) return p;
+    for (int a = 0; a < d; ++a) {
+      const double2 fa = F[(l * d + a) * Nc + q];
+      p.x += (double)kt[a] * fa.x;
+      p.y += (double)kt[a] * fa.y;
+    }
+    const double w = inv_pow(kt2, 1, inv_k2);
+    return make_double2(p.x * w, p.y * w);
+  };
+  auto store = [&](int i, int l, double2 r, double2 p) {
+    if (F) {
+      const double2 f = F[(l * d + i) * Nc + q];
+      r = make_double2(r.x + f.x, r.y + f.y);
+      if (stokes && kt2 > 0) r = make_double2(r.x - (double)kt[i] * p.x, r.y - (double)kt[i] * p.y);
+    }
+    out[(l * d + i) * Nc + q] = r;
+  };
+  if constexpr (NC > 0) {
+    double2 p[NC];
+#pragma unroll
+    for (int l = 0; l < NC; ++l) p[l] = projection(l);
+    for (int i = 0; i < d; ++i) {
+      double2 v[NC], vn[NC];
+#pragma unroll
+      for (int lp = 0; lp < NC; ++lp) {
+        v[lp] = V[(lp * d + i) * Nc + q];
+        vn[lp] = kz == 0 ? V[(lp * d + i) * Nc + qn] : make_double2(0, 0);
+      }
+#pragma unroll
+      for (int l = 0; l < NC; ++l) store(i, l, reg_term(i, l, v, vn), p[l]);
+    }
+  } else {
+    for (int l = 0; l < nc; ++l) {
+      const double2 p = projection(l);
+      for (int i = 0; i < d; ++i) store(i, l, reg_term(i, l, nullptr, nullptr), p);
     }
   }
 }
 
-__global__ void k_spec_precond(const double2* __restrict__ R, double2* __restrict__ out, GridArgs g, int nc,
-                               double beta, const double* __restrict__ Ci, int reg, const double* __restrict__ betas) {
-  long q = (long)blockIdx.x * blockDim.x + threadIdx.x;
+template <int NC>
+__global__ void __launch_bounds__(256) k_spec_precond(const double2* __restrict__ R, double2* __restrict__ out,
+                                                      GridArgs g, int nc_, double beta, const double* __restrict__ Ci,
+                                                      int reg, const double* __restrict__ betas,
+                                                      const double* __restrict__ inv_k2) {
+  const long q = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= g.Nc) return;
-  if (betas) beta = betas[q / g.Nc1];
-  const int d = g.d;
+  if (betas) beta = betas[q >> g.lg1];
+  const int d = g.d, nc = NC ? NC : nc_;
   const long Nc = g.Nc;
-  ModeIdx m = decode(q, d, g.n, g.M);
-  double kk = lead_k2(m, g);
-  long kz = m.j[d - 1];
-  double alpha, delta;
+  const ModeIdx m = decode(q, g);
+  const int kk = lead_k2(m, g), kz = m.j[d - 1];
+  const double ib = 1.0 / beta;
+  double alpha, delta = 0.0;
   long qn = q;
   if (kz == 0) {
-    double a0 = sym_pow(kk, reg), aN = sym_pow(kk + 0.25 * (double)g.n[d - 1] * g.n[d - 1], reg);
-    double s0 = (q % g.Nc1 == 0) ? 1.0 : 1.0 / (beta * a0);  // k = 0: the inverse is replaced by one
-    double sN = 1.0 / (beta * aN);
+    const double s0 = kk == 0 ? 1.0 : ib * inv_pow(kk, reg, inv_k2);  // k = 0: the inverse is replaced by one
+    const double sN = ib * inv_pow(kk + g.M * g.M, reg, inv_k2);
     alpha = 0.5 * (s0 + sN);
     delta = 0.5 * (s0 - sN);
     qn = encode_neg(q, m, g);
   } else {
-    alpha = 1.0 / (beta * sym_pow(kk + (double)kz * kz, reg));
-    delta = 0.0;
+    alpha = ib * inv_pow(kk + kz * kz, reg, inv_k2);
   }
-  for (int l = 0; l < nc; ++l)
-    for (int i = 0; i < d; ++i) {
-      double sr = 0, si = 0;
-      for (int lp = 0; lp < nc; ++lp) {
-        double c = Ci[l * nc + lp];
-        double2 v = R[(lp * d + i) * Nc + q];
-        double2 vn = R[(lp * d + i) * Nc + qn];
-        sr += c * (alpha * v.x + delta * vn.x);
-        si += c * (alpha * v.y - delta * vn.y);
+  for (int i = 0; i < d; ++i) {
+    double2 v[NC ? NC : 1], vn[NC ? NC : 1];
+    if (NC) {
+#pragma unroll
+      for (int lp = 0; lp < NC; ++lp) {
+        v[lp] = R[(lp * d + i) * Nc + q];
+        if (kz == 0) vn[lp] = R[(lp * d + i) * Nc + qn];
       }
-      out[(l * d + i) * Nc + q] = make_double2(sr, si);
     }
+#pragma unroll
+    for (int l = 0; l < nc; ++l) {
+      double2 s = make_double2(0, 0), n = make_double2(0, 0);
+      for (int lp = 0; lp < nc; ++lp) {
+        const double c = NC == 1 ? 1.0 : __ldg(&Ci[l * nc + lp]);  // the 1 x 1 Gram matrix is 1
+        const double2 x = NC ? v[NC ? lp : 0] : R[(lp * d + i) * Nc + q];
+        s.x += c * x.x;
+        s.y += c * x.y;
+        if (kz == 0) {
+          const double2 y = NC ? vn[NC ? lp : 0] : R[(lp * d + i) * Nc + qn];
+          n.x += c * y.x;
+          n.y += c * y.y;
+        }
+      }
+      double2 r = make_double2(alpha * s.x, alpha * s.y);
+      if (kz == 0) r = make_double2(r.x + delta * n.x, r.y - delta * n.y);
+      out[(l * d + i) * Nc + q] = r;
+    }
+  }
 }
 
 // Gaussian filter exp(-sigma^2 |k|^2 / 2) on one packed field (full
@@ -290,9 +234,9 @@ __global__ void k_spec_gauss(double2* __restrict__ U, double2* __restrict__ out,
   long q = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= g.Nc) return;
   const int d = g.d;
-  ModeIdx m = decode(q, d, g.n, g.M);
-  double kk = lead_k2(m, g);
-  long kz = m.j[d - 1];
+  ModeIdx m = decode(q, g);
+  double kk = (double)lead_k2(m, g);
+  int kz = m.j[d - 1];
   double2 v = U[q];
   if (kz == 0) {
     double g0 = exp(-0.5 * s2 * kk), gN = exp(-0.5 * s2 * (kk + 0.25 * (double)g.n[d - 1] * g.n[d - 1]));
@@ -312,120 +256,9 @@ GridArgs args(const Grid& g) {
   a.M = g.M;
   a.Nc = g.Nc;
   a.Nc1 = g.Nc / g.B;
+  a.lg1 = 0;
+  while ((1L << a.lg1) < a.Nc1) ++a.lg1;
   return a;
-}
-
-int ilog2(long n) {
-  int e = 0;
-  while ((1L << e) < n) ++e;
-  return e;
-}
-
-// radix plan mirrored on the host (see Plan<> in fft.cuh)
-std::vector<int> host_plan(int L) {
-  switch (L) {
-    case 2: return {2};
-    case 4: return {4};
-    case 8: return {8};
-    case 16: return {16};
-    case 32: return {8, 4};
-    case 64: return {8, 8};
-    case 128: return {16, 8};
-    case 256: return {16, 16};
-    case 512: return {8, 8, 8};
-  }
-  throw StatusError{1, "unsupported FFT length " + std::to_string(L)};
-}
-
-// Stage tables for length L: for stages s >= 1 (radix R, Ns previous), the
-// entries W_{Ns R}^{r k} at [r*Ns + k], computed in double precision.
-std::vector<double> stage_table(int L) {
-  std::vector<double> t;
-  std::vector<int> R = host_plan(L);
-  int ns = R[0];
-  for (size_t s = 1; s < R.size(); ++s) {
-    for (int r = 0; r < R[s]; ++r)
-      for (int k = 0; k < ns; ++k) {
-        double ang = -2.0 * M_PI * (double)(r * k) / (double)(ns * R[s]);
-        t.push_back(cos(ang));
-        t.push_back(sin(ang));
-      }
-    ns *= R[s];
-  }
-  return t;
-}
-
-template <typename T, int L, int RB>
-void launch_rows(bool inverse, const void* in, void* out, long nrows, const cx<T>* tw, const cx<T>* twrc,
-                 cudaStream_t s) {
-  ProfScope ps(inverse ? KK_ROWS_C2R : KK_ROWS_R2C, s, 2.0 * (double)nrows * L * sizeof(T),
-               (double)nrows * (fft_flops<L / 2>() + 8.0 * (L / 2)));
-  dim3 grid((unsigned)((nrows + RB - 1) / RB));
-  if (!inverse)
-    k_rows_r2c<T, L, RB><<<grid, kThreads, 0, s>>>((const T*)in, (cx<T>*)out, nrows, tw, twrc);
-  else
-    k_rows_c2r<T, L, RB><<<grid, kThreads, 0, s>>>((const cx<T>*)in, (T*)out, nrows, tw, twrc);
-  REG_LAUNCH();
-}
-
-// tune: the autotuner may halve the rows per block of the real-to-complex pass
-template <typename T, int L, int RB>
-void tuned_rows(bool inverse, const void* in, void* out, long nrows, const cx<T>* tw, const cx<T>* twrc,
-                cudaStream_t s, bool tune) {
-  auto run = [&](int v) {
-    if (v == 0) launch_rows<T, L, RB>(inverse, in, out, nrows, tw, twrc, s);
-    else launch_rows<T, L, RB / 2>(inverse, in, out, nrows, tw, twrc, s);
-  };
-  run(!inverse && tune ? tuned_choice("rows_r2c", sizeof(T), L, tune_size(nrows), 2, s, run) : 0);
-}
-
-template <typename T>
-void dispatch_rows(int L, bool inverse, const void* in, void* out, long nrows, const cx<T>* tw,
-                   const cx<T>* twrc, cudaStream_t s, bool tune) {
-  // about 2048 (fp32) / 1024 (fp64) complex values per block
-  constexpr int E = sizeof(T) == 4 ? 2048 : 1024;
-  switch (L) {
-    case 8: return tuned_rows<T, 8, E / 4>(inverse, in, out, nrows, tw, twrc, s, tune);
-    case 16: return tuned_rows<T, 16, E / 8>(inverse, in, out, nrows, tw, twrc, s, tune);
-    case 32: return tuned_rows<T, 32, E / 16>(inverse, in, out, nrows, tw, twrc, s, tune);
-    case 64: return tuned_rows<T, 64, E / 32>(inverse, in, out, nrows, tw, twrc, s, tune);
-    case 128: return tuned_rows<T, 128, E / 64>(inverse, in, out, nrows, tw, twrc, s, tune);
-    case 256: return tuned_rows<T, 256, E / 128>(inverse, in, out, nrows, tw, twrc, s, tune);
-    case 512: return tuned_rows<T, 512, E / 256>(inverse, in, out, nrows, tw, twrc, s, tune);
-  }
-  throw StatusError{1, "unsupported last-axis length " + std::to_string(L)};
-}
-
-template <typename T, int L, int TC>
-void launch_cols(cx<T>* U, long s, long outer, const cx<T>* tw, bool inverse, cudaStream_t st) {
-  ProfScope ps(KK_COLS, st, 2.0 * (double)s * outer * L * sizeof(cx<T>), (double)s * outer * fft_flops<L>());
-  dim3 grid((unsigned)(s / TC), (unsigned)outer);
-  k_cols<T, L, TC><<<grid, kThreads, 0, st>>>(U, s, tw, inverse ? 1 : 0);
-  REG_LAUNCH();
-}
-
-template <typename T, int L>
-void dispatch_cols_tc(cx<T>* U, long s, long outer, const cx<T>* tw, bool inverse, cudaStream_t st) {
-  // tiles of 128-byte column segments (capped so the tile fits 32 KB)
-  constexpr int TCmax0 = sizeof(T) == 4 ? 16 : 8;
-  constexpr int TCmax = (L * TCmax0 * sizeof(cx<T>) > 32768) ? TCmax0 / 2 : TCmax0;
-  if (s >= TCmax) return launch_cols<T, L, TCmax>(U, s, outer, tw, inverse, st);
-  if (s >= 4) return launch_cols<T, L, 4>(U, s, outer, tw, inverse, st);
-  return launch_cols<T, L, 2>(U, s, outer, tw, inverse, st);
-}
-
-template <typename T>
-void dispatch_cols(int L, cx<T>* U, long s, long outer, const cx<T>* tw, bool inverse, cudaStream_t st) {
-  switch (L) {
-    case 8: return dispatch_cols_tc<T, 8>(U, s, outer, tw, inverse, st);
-    case 16: return dispatch_cols_tc<T, 16>(U, s, outer, tw, inverse, st);
-    case 32: return dispatch_cols_tc<T, 32>(U, s, outer, tw, inverse, st);
-    case 64: return dispatch_cols_tc<T, 64>(U, s, outer, tw, inverse, st);
-    case 128: return dispatch_cols_tc<T, 128>(U, s, outer, tw, inverse, st);
-    case 256: return dispatch_cols_tc<T, 256>(U, s, outer, tw, inverse, st);
-    case 512: return dispatch_cols_tc<T, 512>(U, s, outer, tw, inverse, st);
-  }
-  throw StatusError{1, "unsupported axis length " + std::to_string(L)};
 }
 
 unsigned blocks_for(long n, int bs = 256) { return (unsigned)((n + bs - 1) / bs); }
@@ -455,125 +288,45 @@ Grid make_grid(int d, const int64_t* n, int batch) {
   return g;
 }
 
-template <typename T>
-Spectral<T>::Spectral(const Grid& g, cudaStream_t s) : g_(g), s_(s) {
-  // tables for every power of two from 4 to 512 (row half-length and axes)
-  std::vector<double> all;
-  for (int e = 2; e <= 9; ++e) {
-    tw_off_[e] = (long)all.size() / 2;
-    std::vector<double> t = stage_table(1 << e);
-    all.insert(all.end(), t.begin(), t.end());
-  }
-  rc_off_ = (long)all.size() / 2;
-  for (int k = 0; k < g.M; ++k) {
-    double ang = -2.0 * M_PI * (double)k / (double)g.L;
-    all.push_back(cos(ang));
-    all.push_back(sin(ang));
-  }
-  std::vector<T> h(all.size());
-  for (size_t i = 0; i < all.size(); ++i) h[i] = (T)all[i];
-  REG_CUDA(cudaMalloc(&tw_, h.size() * sizeof(T)));
-  REG_CUDA(cudaMemcpy(tw_, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice));
-  lines_.reset(new LineTables<T>(g));
+bool narrow_lines(long wide_threads) {
+  static const long lim = getenv("REG_NARROW") ? atol(getenv("REG_NARROW")) : 152 * 256;
+  return wide_threads < lim;
 }
 
-template <typename T>
-Spectral<T>::Spectral(const Grid& g, cudaStream_t s, C* tables, const long* tw_off, long rc_off)
-    : g_(g), s_(s), tw_(tables), owns_(false) {
-  for (int e = 0; e < 11; ++e) tw_off_[e] = tw_off[e];
-  rc_off_ = rc_off;
+long inv_k2_count(const Grid& g) {
+  long n = 1;
+  for (int a = 0; a < g.d; ++a) n += (long)(g.n[a] / 2) * (g.n[a] / 2);
+  return n;
 }
 
-template <typename T>
-long Spectral<T>::write_tables(double* out, long* tw_off, long* rc_off) {
-  long pos = 0;
-  auto put = [&](double re, double im) {
-    if (out) {
-      out[2 * pos] = re;
-      out[2 * pos + 1] = im;
-    }
-    ++pos;
-  };
-  for (int e = 0; e < 11; ++e) tw_off[e] = rc_off[e] = 0;
-  for (int e = 2; e <= 9; ++e) {
-    int L = 1 << e;
-    tw_off[e] = pos;
-    // the radix plan of Plan<L> (fft.cuh), in a fixed array: no heap use here
-    int R[3] = {L, 1, 1}, S = 1;
-    if (L == 32) { R[0] = 8; R[1] = 4; S = 2; }
-    else if (L == 64) { R[0] = 8; R[1] = 8; S = 2; }
-    else if (L == 128) { R[0] = 16; R[1] = 8; S = 2; }
-    else if (L == 256) { R[0] = 16; R[1] = 16; S = 2; }
-    else if (L == 512) { R[0] = 8; R[1] = 8; R[2] = 8; S = 3; }
-    int ns = R[0];
-    for (int st = 1; st < S; ++st) {
-      for (int r = 0; r < R[st]; ++r)
-        for (int k = 0; k < ns; ++k) {
-          double ang = -2.0 * M_PI * (double)(r * k) / (double)(ns * R[st]);
-          put(cos(ang), sin(ang));
-        }
-      ns *= R[st];
-    }
-  }
-  for (int e = 3; e <= 9; ++e) {
-    int L = 1 << e;
-    rc_off[e] = pos;
-    for (int k = 0; k < L / 2; ++k) {
-      double ang = -2.0 * M_PI * (double)k / (double)L;
-      put(cos(ang), sin(ang));
-    }
-  }
-  return pos;
+void fill_inv_k2(double* inv_k2, long count, cudaStream_t s) {
+  k_inv_k2<<<blocks_for(count), 256, 0, s>>>(inv_k2, count);
+  REG_LAUNCH();
 }
-
-template <typename T>
-Spectral<T>::~Spectral() {
-  if (tw_ && owns_) cudaFree(tw_);
-}
-
-template <typename T>
-const cx<T>* Spectral<T>::twiddles(int L) const {
-  return tw_ + tw_off_[ilog2(L)];
-}
-template <typename T>
-const cx<T>* Spectral<T>::rc_twiddles() const {
-  return tw_ + rc_off_;
-}
-template <typename T>
-void Spectral<T>::cols(C* U, int axis, bool inverse) {
-  long s = g_.M;
-  for (int a = axis + 1; a < g_.d - 1; ++a) s *= g_.n[a];
-  long outer = g_.Nc / (s * g_.n[axis]);
-  dispatch_cols<T>(g_.n[axis], U, s, outer, twiddles(g_.n[axis]), inverse, s_);
-}
-
-template <typename T>
-void Spectral<T>::fwd(const T* u, C* U) {
-  dispatch_rows<T>(g_.L, false, u, U, g_.rows, twiddles(g_.M), rc_twiddles(), s_, owns_);
-  for (int a = g_.d - 2; a >= 0; --a) cols(U, a, false);
-}
-
-template <typename T>
-void Spectral<T>::inv(C* U, T* u) {
-  for (int a = 0; a <= g_.d - 2; ++a) cols(U, a, true);
-  dispatch_rows<T>(g_.L, true, U, u, g_.rows, twiddles(g_.M), rc_twiddles(), s_, owns_);
-}
-
-template class Spectral<float>;
-
-template class Spectral<double>;
 
 void spec_tail(const Grid& g, cudaStream_t s, const double2* V, const double2* F, double2* out, int nc, double beta,
-               const double* Cg_dev, int reg, int stokes, const double* betas) {
+               const double* Cg_dev, int reg, int stokes, const double* betas, const double* inv_k2) {
   if (nc > kMaxNc) throw StatusError{1, "n_c too large"};
-  k_spec_tail<<<blocks_for(g.Nc), 256, 0, s>>>(V, F, out, args(g), nc, beta, Cg_dev, reg, stokes, betas);
-  REG_LAUNCH();
+  auto run = [&](auto k) {
+    k<<<blocks_for(g.Nc), 256, 0, s>>>(V, F, out, args(g), nc, beta, Cg_dev, reg, stokes, betas, inv_k2);
+    REG_LAUNCH();
+  };
+  if (nc == 1) run(k_spec_tail<1>);
+  else if (nc == 2) run(k_spec_tail<2>);
+  else if (nc == 3) run(k_spec_tail<3>);
+  else run(k_spec_tail<0>);
 }
 
 void spec_precond(const Grid& g, cudaStream_t s, const double2* R, double2* out, int nc, double beta,
-                  const double* Ci_dev, int reg, const double* betas) {
-  k_spec_precond<<<blocks_for(g.Nc), 256, 0, s>>>(R, out, args(g), nc, beta, Ci_dev, reg, betas);
-  REG_LAUNCH();
+                  const double* Ci_dev, int reg, const double* betas, const double* inv_k2) {
+  auto run = [&](auto k) {
+    k<<<blocks_for(g.Nc), 256, 0, s>>>(R, out, args(g), nc, beta, Ci_dev, reg, betas, inv_k2);
+    REG_LAUNCH();
+  };
+  if (nc == 1) run(k_spec_precond<1>);
+  else if (nc == 2) run(k_spec_precond<2>);
+  else if (nc == 3) run(k_spec_precond<3>);
+  else run(k_spec_precond<0>);
 }
 
 void spec_gauss(const Grid& g, cudaStream_t s, double2* U, double2* out, double sigma) {
@@ -597,7 +350,7 @@ __global__ void k_spec_upsample(const double2* __restrict__ P, double2* __restri
   const long total = (long)nfields * f.Nc;
   for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
     const long fld = t / f.Nc, q = t % f.Nc;
-    const ModeIdx m = decode(q, f.d, f.n, f.M);
+    const ModeIdx m = decode(q, f);
     bool zero = m.j[f.d - 1] >= c.M;
     long row = 0, nrow = 0;  // coarse row of k' and of -k'
     for (int a = 0; a < f.d - 1 && !zero; ++a) {

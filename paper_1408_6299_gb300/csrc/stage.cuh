@@ -14,8 +14,7 @@
 #include <cuda.h>
 
 #include "internal.h"
-#include "fixed.cuh"
-#include "line.cuh"
+#include "transform.cuh"
 
 namespace reg {
 namespace fused {
@@ -174,27 +173,6 @@ struct ColTile {
   static constexpr int NT = TC * TS;
 };
 
-// the largest mag of the TS threads (c, j), j < TS, of a column; thread c + j TC
-// of the block holds (c, j). red: scratch, free again after the next barrier.
-template <int TC, int TS>
-__device__ __forceinline__ unsigned line_max(unsigned mag, unsigned* red, int c, int j) {
-  if constexpr (TS == 1) {
-    return mag;
-  } else {
-#pragma unroll
-    for (int o = TC; o < 32; o *= 2) mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, o));
-    constexpr int NW = TC >= 32 ? TS : TC * TS / 32;  // partial results per column
-    if constexpr (NW > 1) {
-      red[(TC >= 32 ? j : (int)threadIdx.x / 32) * TC + c] = mag;  // equal values where lanes share a slot
-      __syncthreads();
-#pragma unroll
-      for (int w = 0; w < NW; ++w) mag = max(mag, red[w * TC + c]);
-      __syncthreads();
-    }
-    return mag;
-  }
-}
-
 __device__ __forceinline__ float2 gmul(float2 a, float2 b) { return make_float2(a.x * b.x, a.y * b.y); }
 __device__ __forceinline__ double2 gmul(double2 a, double2 b) { return make_double2(a.x * b.x, a.y * b.y); }
 __device__ __forceinline__ float4 gmul(float4 a, float4 b) {
@@ -329,26 +307,13 @@ __global__ void __launch_bounds__(RowTile<L, NARROW, EPI>::NT) k_rows_line(RowAr
       }
     }
     V v[E];
-    auto sync = [] {
-      if constexpr (TS <= 32) __syncwarp();
-      else asm volatile("bar.sync 1, %0;" ::"n"(Tile::NFFT) : "memory");
-    };
+    const RowSync<TS, Tile::NFFT> sync;
     auto at = [&](int p) { return b + p + (p >> Tile::PADSH); };
     if constexpr (A::SCALED) {
       unsigned mag = 0;
 #pragma unroll
       for (int e = 0; e < E; ++e) mag = max(mag, fx_mag(x[e]));
-#pragma unroll
-      for (int o = 1; o < (TS < 32 ? TS : 32); o *= 2) mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, o));
-      if constexpr (TS > 32) {  // the line's warps exchange their maxima
-        unsigned* red = reinterpret_cast<unsigned*>(b);
-        red[j / 32] = mag;
-        sync();
-#pragma unroll
-        for (int w = 0; w < TS / 32; ++w) mag = max(mag, red[w]);
-        sync();
-      }
-      const FxScale<L, Ln::R0> sc(mag);
+      const FxScale<L, Ln::R0> sc(row_max<TS>(mag, reinterpret_cast<unsigned*>(b), j, sync));
 #pragma unroll
       for (int e = 0; e < E; ++e) v[e] = sc.in(x[e]);
       Ln::derivative(v, j, at, sync, tw);

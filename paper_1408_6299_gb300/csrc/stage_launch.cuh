@@ -20,7 +20,7 @@ struct Arith<float> {
 };
 template <>
 struct Arith<double> {
-  using Main = LineFloat<double>;
+  using Main = LineFixed;
 };
 
 // One derivative pass along a strided axis: out = D_axis in, or D_axis (in mul)
@@ -37,11 +37,6 @@ inline long line_stride(const Grid& g, int axis) {
   long s = g.M;
   for (int a = axis + 1; a < g.d - 1; ++a) s *= g.n[a];
   return s;
-}
-
-inline bool narrow_lines(long threads_wide) {
-  static const long lim = getenv("REG_NARROW") ? atol(getenv("REG_NARROW")) : 152 * 256;
-  return threads_wide < lim;
 }
 
 template <class A, typename T, int L, bool NARROW, bool PROD, int VAR>
