@@ -53,6 +53,25 @@ void count_launch();
 void add_launches(long n);  // kernels launched by a graph replay
 long launch_count();
 
+// Launch of a kernel that begins with chain_enter(): it may be set up while its
+// predecessor on the stream still runs, and waits there for its results. The
+// kernels of a sweep depend on one another and run a few microseconds each on
+// small grids, so the launch gap between them counts.
+template <typename... P, typename... A>
+void chain(void (*kern)(P...), unsigned grid, unsigned block, cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  count_launch();
+  REG_CUDA(cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...));
+}
+
 struct KernelProfiler {
   unsigned mask = 0;
   struct Rec {
@@ -174,11 +193,6 @@ class FieldTransforms {
 // Transport stages (stage.cuh): advection k = -v.grad u [- grad m . v~] and
 // divergence k = div(v lam), each with its Runge-Kutta update in the last pass.
 // ---------------------------------------------------------------------------
-// bounded waits of the TMA column pass that gave up since the last call
-// (per precision; synchronises s)
-int take_tma_timeouts_f32(cudaStream_t s);
-int take_tma_timeouts_f64(cudaStream_t s);
-
 namespace fused {
 template <typename T>
 struct AdvEpi;

@@ -23,6 +23,7 @@ inline unsigned nblk(long n, int bs = 256) {
 }
 
 __global__ void k_vel_at(const double* __restrict__ coef, int nc, Coefs b, double* __restrict__ out, long dN) {
+  chain_enter();
   long x = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= dN) return;
   double s = 0.0;
@@ -38,6 +39,7 @@ struct FloatWeights {
   float hi[16], lo[16];
 };
 __global__ void k_vel_at(const float* __restrict__ coef, int nc, FloatWeights b, float* __restrict__ out, long dN) {
+  chain_enter();
   long x = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= dN) return;
   float s = 0.f, err = 0.f;
@@ -54,6 +56,7 @@ __global__ void k_vel_at(const float* __restrict__ coef, int nc, FloatWeights b,
 
 template <typename S, typename T>
 __global__ void k_convert(const S* __restrict__ in, T* __restrict__ out, long n) {
+  chain_enter();
   long x = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (x < n) out[x] = (T)in[x];
 }
@@ -63,6 +66,7 @@ template <typename T, bool SRC, bool STAGE1>
 __global__ void k_stage(const T* __restrict__ G, const T* __restrict__ vt, const T* __restrict__ gm,
                         const T* __restrict__ wt, const T* __restrict__ y, T h, T* __restrict__ yh,
                         T* __restrict__ acc, int d, long N) {
+  chain_enter();
   long x = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= N) return;
   T k = 0;
@@ -81,6 +85,7 @@ __global__ void k_stage(const T* __restrict__ G, const T* __restrict__ vt, const
 
 template <typename T>
 __global__ void k_dot_fields(const T* __restrict__ a, const T* __restrict__ b, T* __restrict__ out, int d, long N) {
+  chain_enter();
   long x = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= N) return;
   T s = 0;
@@ -98,6 +103,7 @@ __global__ void k_dot_fields(const T* __restrict__ a, const T* __restrict__ b, T
 template <typename T>
 __global__ void __launch_bounds__(256) k_force(T* __restrict__ fhi, T* __restrict__ flo, ForceNodes<T> F, int nc, int d,
                                                long N) {
+  chain_enter();
   using C = cx<T>;
   const int i = blockIdx.x % d;
   const long q = (long)(blockIdx.x / d) * blockDim.x + threadIdx.x;
@@ -148,6 +154,7 @@ __global__ void __launch_bounds__(256) k_force(T* __restrict__ fhi, T* __restric
 
 __global__ void k_pair_to_double(const float* __restrict__ hi, const float* __restrict__ lo, double* __restrict__ out,
                                  long n) {
+  chain_enter();
   long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = (double)hi[i] + (double)lo[i];
 }
@@ -209,17 +216,20 @@ __global__ void k_det(const double* __restrict__ F, double* __restrict__ det, in
 
 template <typename T>
 __global__ void k_lincomb_t(T a, const T* __restrict__ x, T b, const T* __restrict__ y, T* __restrict__ out, long n) {
+  chain_enter();
   long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = a * x[i] + (y ? b * y[i] : (T)0);
 }
 
 __global__ void k_axpby(double a, const double* __restrict__ x, double b, double* __restrict__ y, long n) {
+  chain_enter();
   long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) y[i] = a * x[i] + b * y[i];
 }
 
 __global__ void k_lincomb(double a, const double* __restrict__ x, double b, const double* __restrict__ y,
                           double* __restrict__ out, long n) {
+  chain_enter();
   long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = a * x[i] + b * y[i];
 }
@@ -240,6 +250,7 @@ struct Acc4 {
 template <int OP>
 __global__ void k_reduce(const double* __restrict__ a, const double* __restrict__ b, long n, double center,
                          double* __restrict__ part) {
+  chain_enter();
   __shared__ double sh[4][kRedThreads];
   double s = 0, s2 = 0, mn = DBL_MAX, mx = -DBL_MAX;
   for (long i = (long)blockIdx.x * kRedThreads + threadIdx.x; i < n; i += (long)kRedBlocks * kRedThreads) {
@@ -268,6 +279,7 @@ __global__ void k_reduce(const double* __restrict__ a, const double* __restrict_
 }
 
 __global__ void k_reduce_final(const double* __restrict__ part, double* __restrict__ out) {
+  chain_enter();
   __shared__ double sh[4][kRedThreads];
   double s = 0, s2 = 0, mn = DBL_MAX, mx = -DBL_MAX;
   for (int i = threadIdx.x; i < kRedBlocks; i += kRedThreads) {
@@ -298,8 +310,7 @@ __global__ void k_reduce_final(const double* __restrict__ part, double* __restri
 
 template <>
 void vel_at<double>(const double* coef, int nc, const Coefs& b, double* out, long dN, cudaStream_t s) {
-  k_vel_at<<<nblk(dN), 256, 0, s>>>(coef, nc, b, out, dN);
-  REG_LAUNCH();
+  chain<const double*, int, Coefs, double*, long>(k_vel_at, nblk(dN), 256, s, coef, nc, b, out, dN);
 }
 template <>
 void vel_at<float>(const float* coef, int nc, const Coefs& b, float* out, long dN, cudaStream_t s) {
@@ -308,14 +319,12 @@ void vel_at<float>(const float* coef, int nc, const Coefs& b, float* out, long d
     w.hi[l] = l < nc ? (float)b.c[l] : 0.f;
     w.lo[l] = l < nc ? (float)(b.c[l] - (double)w.hi[l]) : 0.f;
   }
-  k_vel_at<<<nblk(dN), 256, 0, s>>>(coef, nc, w, out, dN);
-  REG_LAUNCH();
+  chain<const float*, int, FloatWeights, float*, long>(k_vel_at, nblk(dN), 256, s, coef, nc, w, out, dN);
 }
 
 template <typename S, typename T>
 void convert(const S* in, T* out, long n, cudaStream_t s) {
-  k_convert<S, T><<<nblk(n), 256, 0, s>>>(in, out, n);
-  REG_LAUNCH();
+  chain(k_convert<S, T>, nblk(n), 256, s, in, out, n);
 }
 template void convert<double, float>(const double*, float*, long, cudaStream_t);
 template void convert<float, double>(const float*, double*, long, cudaStream_t);
@@ -325,15 +334,12 @@ template <typename T>
 void transport_stage1(const T* G, const T* vt, const T* gm, const T* wt, const T* y, T h, T* yh, T* acc, int d,
                       long N, cudaStream_t s) {
   ProfScope ps(KK_STAGE, s, (double)N * sizeof(T) * ((G ? 2 * d : 0) + (gm ? 2 * d : 0) + (y ? 1 : 0) + 2));
-  if (gm) k_stage<T, true, true><<<nblk(N), 256, 0, s>>>(G, vt, gm, wt, y, h, yh, acc, d, N);
-  else k_stage<T, false, true><<<nblk(N), 256, 0, s>>>(G, vt, gm, wt, y, h, yh, acc, d, N);
-  REG_LAUNCH();
+  chain(gm ? k_stage<T, true, true> : k_stage<T, false, true>, nblk(N), 256, s, G, vt, gm, wt, y, h, yh, acc, d, N);
 }
 template <typename T>
 void dot_fields(const T* a, const T* b, T* out, int d, long N, cudaStream_t s) {
   ProfScope ps(KK_STAGE, s, (double)N * sizeof(T) * (2 * d + 1));
-  k_dot_fields<T><<<nblk(N), 256, 0, s>>>(a, b, out, d, N);
-  REG_LAUNCH();
+  chain(k_dot_fields<T>, nblk(N), 256, s, a, b, out, d, N);
 }
 
 template <typename T>
@@ -342,13 +348,11 @@ void force_acc(T* fhi, T* flo, const ForceNodes<T>& F, int nc, int d, long N, cu
   double fields = 2.0 * nc * d * (flo ? 2 : 1);
   for (int k = 0; k < F.count; ++k) fields += (d + 1) * (1 + (F.yB[k] ? 1 : 0) + (F.yC[k] ? 1 : 0));
   ProfScope ps(KK_FORCE, s, (double)N * sizeof(T) * fields);
-  k_force<T><<<nblk(N / 2) * d, 256, 0, s>>>(fhi, flo, F, nc, d, N);
-  REG_LAUNCH();
+  chain(k_force<T>, nblk(N / 2) * d, 256, s, fhi, flo, F, nc, d, N);
 }
 
 void pair_to_double(const float* hi, const float* lo, double* out, long n, cudaStream_t s) {
-  k_pair_to_double<<<nblk(n), 256, 0, s>>>(hi, lo, out, n);
-  REG_LAUNCH();
+  chain(k_pair_to_double, nblk(n), 256, s, hi, lo, out, n);
 }
 
 #define INST(T)                                                                                          \
@@ -362,8 +366,7 @@ INST(double)
 
 template <typename T>
 void lincomb_t(T a, const T* x, T b, const T* y, T* out, long n, cudaStream_t s) {
-  k_lincomb_t<T><<<nblk(n), 256, 0, s>>>(a, x, b, y, out, n);
-  REG_LAUNCH();
+  chain(k_lincomb_t<T>, nblk(n), 256, s, a, x, b, y, out, n);
 }
 template void lincomb_t<float>(float, const float*, float, const float*, float*, long, cudaStream_t);
 template void lincomb_t<double>(double, const double*, double, const double*, double*, long, cudaStream_t);
@@ -386,12 +389,10 @@ void grid_angle_tensor(const double* F, double* angle, int d, long N, cudaStream
   REG_LAUNCH();
 }
 void axpby(double a, const double* x, double b, double* y, long n, cudaStream_t s) {
-  k_axpby<<<nblk(n), 256, 0, s>>>(a, x, b, y, n);
-  REG_LAUNCH();
+  chain(k_axpby, nblk(n), 256, s, a, x, b, y, n);
 }
 void lincomb(double a, const double* x, double b, const double* y, double* out, long n, cudaStream_t s) {
-  k_lincomb<<<nblk(n), 256, 0, s>>>(a, x, b, y, out, n);
-  REG_LAUNCH();
+  chain(k_lincomb, nblk(n), 256, s, a, x, b, y, out, n);
 }
 
 long reduce_scratch_doubles() { return 4L * kRedBlocks + 4; }
@@ -694,15 +695,11 @@ void lincomb_seg(const double* a_dev, const double* x, const double* c_dev, cons
 static double* launch_reduce(int op, const double* a, const double* b, long n, double* scratch, cudaStream_t s,
                              double center = 0.0) {
   double* out = scratch + 4L * kRedBlocks;
-  switch (op) {
-    case RED_DOT: k_reduce<RED_DOT><<<kRedBlocks, kRedThreads, 0, s>>>(a, b, n, 0.0, scratch); break;
-    case RED_SQDIFF: k_reduce<RED_SQDIFF><<<kRedBlocks, kRedThreads, 0, s>>>(a, b, n, 0.0, scratch); break;
-    case RED_MAXABS: k_reduce<RED_MAXABS><<<kRedBlocks, kRedThreads, 0, s>>>(a, b, n, 0.0, scratch); break;
-    default: k_reduce<RED_STATS><<<kRedBlocks, kRedThreads, 0, s>>>(a, b, n, center, scratch); break;
-  }
-  REG_LAUNCH();
-  k_reduce_final<<<1, kRedThreads, 0, s>>>(scratch, out);
-  REG_LAUNCH();
+  auto kern = op == RED_DOT ? k_reduce<RED_DOT>
+                            : (op == RED_SQDIFF ? k_reduce<RED_SQDIFF>
+                                                : (op == RED_MAXABS ? k_reduce<RED_MAXABS> : k_reduce<RED_STATS>));
+  chain(kern, kRedBlocks, kRedThreads, s, a, b, n, center, scratch);
+  chain(k_reduce_final, 1, kRedThreads, s, scratch, out);
   return out;
 }
 

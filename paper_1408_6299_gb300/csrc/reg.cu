@@ -114,6 +114,22 @@ struct Work {
   DBuf<T> mtil, lamN, yh2, acc2, st0, st1, Gt, mR, m1;  // full Newton matvec
 };
 
+// A sweep replayed as a CUDA graph. A sweep is hundreds of dependent launches
+// of a few microseconds on small grids, which the host cannot issue as fast as
+// they run. The first call with a set of buffers and settings (sig) runs
+// plainly: it allocates, tunes, and costs no capture where a context is used
+// once; the second captures, and the graph is replayed while sig holds.
+struct Replay {
+  cudaGraphExec_t exec = nullptr;
+  size_t sig = 0, seen = 0;
+  long kernels = 0;
+  void drop() {
+    if (exec) cudaGraphExecDestroy(exec);
+    exec = nullptr;
+  }
+  ~Replay() { drop(); }
+};
+
 }  // namespace
 
 struct reg_ctx {
@@ -157,13 +173,14 @@ struct reg_ctx {
   // solve vectors
   DBuf<double> sv_g, sv_s, sv_r, sv_z, sv_p, sv_Hp, sv_vt;
   KernelProfiler prof;  // CUDA-event bracketing of launches by kind (off unless enabled)
-  // CUDA graph of the Hessian matvec (contexts with their own stream): the
-  // sweeps and the tail read the direction from gdir and write gout
-  bool graphs = false;
-  cudaGraphExec_t gexec = nullptr;
-  size_t gsig = 0;
-  long gkernels = 0;
-  DBuf<double> gdir, gout;
+  // CUDA graphs of the sweeps (see Replay); they read the velocity from vfix
+  // and the direction from gdir
+  Replay rp_state, rp_store, rp_adj, rp_hess;
+  DBuf<double> vfix, gdir;
+  // a context created on the NULL stream works on a stream of its own, ordered
+  // behind the NULL stream at every call (captures are not allowed there)
+  cudaStream_t own = nullptr;
+  cudaEvent_t own_ev = nullptr;
   // device-driven lockstep loops (stacked problems): per-problem scalars, the
   // control block, and the graphs of the PCG and line-search loops
   DBuf<double> lk;
@@ -173,9 +190,10 @@ struct reg_ctx {
   size_t lk_sig = 0;
   int lk_state = 0;  // 0 not built yet, 1 built, -1 refused (host-driven loops)
   ~reg_ctx() {
-    if (gexec) cudaGraphExecDestroy(gexec);
     if (lk_pcg) cudaGraphExecDestroy(lk_pcg);
     if (lk_ls) cudaGraphExecDestroy(lk_ls);
+    if (own_ev) cudaEventDestroy(own_ev);
+    if (own) cudaStreamDestroy(own);
   }
 
   long N() const { return g.N; }
@@ -422,12 +440,11 @@ const T* gmh_slot(reg_ctx* c, int j, int base) {
   return work<T>(c).gmh.p + (long)(j - base) * c->dN();
 }
 
-// Full state solve from m0 with storage for later sweeps (store-all or checkpoints).
+// Full state solve from the state in w.m with storage for later sweeps (store-all or checkpoints).
 template <typename T>
-void state_solve_store(reg_ctx* c, const T* vcoef, const T* m0) {
+void state_solve_store(reg_ctx* c, const T* vcoef) {
   Work<T>& w = work<T>(c);
   const long N = c->N(), dN = c->dN();
-  REG_CUDA(cudaMemcpyAsync(w.m.get(N), m0, N * sizeof(T), cudaMemcpyDeviceToDevice, c->s));
   if (c->ckpt == 0) {
     state_steps<T>(c, vcoef, 0, c->n_t, w.gm.get((size_t)(c->n_t + 1) * dN),
                    c->quad ? w.gmh.get((size_t)(c->n_t + 1) * dN) : nullptr, 0, nullptr);
@@ -502,9 +519,9 @@ T* ring_slot(T* ring, int k, long stride) {
 // accumulating the body force f_l = int b_l lam grad m dt into f (double): the
 // trapezoid term of every node, or the two stage terms per step of the
 // discrete adjoint. lam (and the predictors of the discrete adjoint) are kept
-// for the nodes whose force is still to be added. Returns lam_0.
+// for the nodes whose force is still to be added; lam_0 ends in slot n_t - 1.
 template <typename T>
-const T* adjoint_solve(reg_ctx* c, const T* vcoef, double* f) {
+void adjoint_solve(reg_ctx* c, const T* vcoef, double* f) {
   Work<T>& w = work<T>(c);
   const long N = c->N();
   const double hd = c->h();
@@ -541,7 +558,6 @@ const T* adjoint_solve(reg_ctx* c, const T* vcoef, double* f) {
     if (j0 == 0 && !c->quad) bf.add(lam, gm_slot<T>(c, 0, base), 0, c->trap_w(0));
   }
   bf.finish();
-  return lam;
 }
 
 // Full Newton incremental adjoint (Eq. sec-order-iadj / sec-order-icontrol,
@@ -789,12 +805,80 @@ double reg_term(reg_ctx* c, const double* v) {
   return 0.5 * c->hd * dot(v, Rv, c->ncdN(), red(c), c->s);
 }
 
+// addresses of every buffer the captured sweeps touch: a change means a graph
+// would read or write stale memory and must be captured again
+size_t graph_signature(reg_ctx* c) {
+  const void* ptrs[] = {c->f.p,        c->SV.p,       c->SF.p,       c->vlin.p,     c->gdir.p,     c->vfix.p,
+                        c->w64.gx.p,   c->w64.gy.p,    c->w64.m.p,    c->w64.yh.p,   c->w64.acc.p,
+                        c->w64.lam.p,  c->w64.va.p,   c->w64.vb.p,   c->w64.wa.p,   c->w64.wb.p,   c->w64.gm.p,
+                        c->w64.gmh.p,  c->w64.ck.p,   c->w32.gx.p,   c->w32.gy.p,    c->w32.m.p,
+                        c->w32.yh.p,   c->w32.acc.p,  c->w32.lam.p,  c->w32.va.p,   c->w32.vb.p,   c->w32.wa.p,
+                        c->w32.wb.p,   c->w32.gm.p,   c->w32.gmh.p,  c->w32.ck.p,   c->w32.vcoef.p, c->w32.wcoef.p,
+                        c->w32.fhi.p,  c->w32.flo.p,  c->w64.G.p,    c->w32.G.p,    c->w64.src.p,  c->w32.src.p,
+                        c->w64.mtil.p, c->w32.mtil.p, c->w64.lamN.p, c->w32.lamN.p, c->w64.yh2.p, c->w32.yh2.p,
+                        c->w64.acc2.p, c->w32.acc2.p, c->w64.st0.p,  c->w32.st0.p,  c->w64.st1.p,  c->w32.st1.p,
+                        c->w64.Gt.p,   c->w32.Gt.p,   c->w64.gx2.p,  c->w32.gx2.p,  c->w64.gy2.p,  c->w32.gy2.p,
+                        c->w64.yhS.p,  c->w32.yhS.p,  c->w64.accS.p, c->w32.accS.p,
+                        c->w64.srcS.p, c->w32.srcS.p, c->w64.lamR.p, c->w32.lamR.p, c->w64.yhR.p,  c->w32.yhR.p};
+  size_t h = 1469598103934665603ull;
+  for (const void* p : ptrs) h = (h ^ (size_t)p) * 1099511628211ull;
+  // and the settings that change what the sweeps compute
+  const uint64_t modes[] = {(uint64_t)c->hess, (uint64_t)c->quad, (uint64_t)c->prec, (uint64_t)c->n_t};
+  for (uint64_t m : modes) h = (h ^ (size_t)m) * 1099511628211ull;
+  return h;
+}
+
+// Runs body, a sequence of launches on the context's stream whose arguments
+// depend on the signature alone, as a graph where it repeats (see Replay).
+template <typename Body>
+void replay(reg_ctx* c, Replay& g, Body body) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (c->s) REG_CUDA(cudaStreamIsCapturing(c->s, &cs));
+  if (!c->s || c->prof.mask || cs != cudaStreamCaptureStatusNone) return body();  // timed by kernel, or inside a capture
+  const size_t sig = graph_signature(c);
+  if (!g.exec || g.sig != sig) {
+    g.drop();
+    if (g.seen != sig) {
+      body();
+      g.seen = graph_signature(c);
+      return;
+    }
+    const long l0 = launch_count();
+    cudaGraph_t graph = nullptr;
+    REG_CUDA(cudaStreamBeginCapture(c->s, cudaStreamCaptureModeThreadLocal));
+    try {
+      body();
+    } catch (...) {
+      cudaStreamEndCapture(c->s, &graph);
+      if (graph) cudaGraphDestroy(graph);
+      throw;
+    }
+    REG_CUDA(cudaStreamEndCapture(c->s, &graph));
+    const cudaError_t e = cudaGraphInstantiate(&g.exec, graph, 0);
+    cudaGraphDestroy(graph);
+    REG_CUDA(e);
+    g.kernels = launch_count() - l0;
+    add_launches(-g.kernels);
+    g.sig = sig;
+  }
+  REG_CUDA(cudaGraphLaunch(g.exec, c->s));
+  add_launches(g.kernels);
+}
+
+// m_1 of the state solve from w.m under v, left in w.m
+void state_solve(reg_ctx* c, const double* v) {
+  double* vf = c->vfix.get(c->ncdN());
+  c->w64.m.get(c->N());
+  REG_CUDA(cudaMemcpyAsync(vf, v, c->ncdN() * sizeof(double), cudaMemcpyDeviceToDevice, c->s));
+  replay(c, c->rp_state, [&] { state_steps<double>(c, vf, 0, c->n_t, nullptr, nullptr, 0, nullptr); });
+}
+
 void objective(reg_ctx* c, const double* v, double parts[2]) {
   if (!c->have_images) throw StatusError{REG_EINVAL, "reg_set_images has not been called"};
   const long N = c->N();
   Work<double>& w = c->w64;
   REG_CUDA(cudaMemcpyAsync(w.m.get(N), c->mT.p, N * sizeof(double), cudaMemcpyDeviceToDevice, c->s));
-  state_steps<double>(c, v, 0, c->n_t, nullptr, nullptr, 0, nullptr);
+  state_solve(c, v);
   parts[0] = 0.5 * c->hd * sqdiff(c->mR.p, w.m.p, N, red(c), c->s);
   parts[1] = reg_term(c, v);
 }
@@ -824,7 +908,8 @@ void set_point(reg_ctx* c, const double* v) {
   if (!c->have_images) throw StatusError{REG_EINVAL, "reg_set_images has not been called"};
   c->ready = false;
   REG_CUDA(cudaMemcpyAsync(c->vlin.get(c->ncdN()), v, c->ncdN() * sizeof(double), cudaMemcpyDeviceToDevice, c->s));
-  state_solve_store<double>(c, c->vlin.p, c->mT.p);
+  REG_CUDA(cudaMemcpyAsync(c->w64.m.get(c->N()), c->mT.p, c->N() * sizeof(double), cudaMemcpyDeviceToDevice, c->s));
+  replay(c, c->rp_store, [&] { state_solve_store<double>(c, c->vlin.p); });
   if (c->hess == REG_HESS_NEWTON) {  // m_1 and m_R for the adjoint inside the Newton matvec
     const long N = c->N();
     REG_CUDA(cudaMemcpyAsync(c->w64.m1.get(N), c->w64.m.p, N * sizeof(double), cudaMemcpyDeviceToDevice, c->s));
@@ -845,7 +930,7 @@ void gradient(reg_ctx* c, const double* v, double* g, double parts[2]) {
   parts[0] = 0.5 * c->hd * sqdiff(c->mR.p, w.m.p, N, red(c), c->s);
   lincomb_t<double>(1.0, c->mR.p, -1.0, w.m.p, w.lam.get(N), N, c->s);  // lam_1 = m_R - m_1
   double* f = c->f.get(c->ncdN());
-  adjoint_solve<double>(c, c->vlin.p, f);
+  replay(c, c->rp_adj, [&] { adjoint_solve<double>(c, c->vlin.p, f); });
   tail(c, c->vlin.p, f, g);
   parts[1] = reg_term(c, c->vlin.p);
   check_finite(parts[0] + parts[1], "objective");
@@ -855,81 +940,23 @@ void gradient(reg_ctx* c, const double* v, double* g, double parts[2]) {
 }
 
 void hessvec_body(reg_ctx* c, const double* vt, double* out) {
-  double* f = c->f.get(c->ncdN());
+  const long n = c->ncdN();
+  double* f = c->f.get(n);
   if (c->prec == REG_FP64) {
-    gn_sweeps<double>(c, c->vlin.p, vt, f);
+    double* w = c->gdir.get(n);
+    REG_CUDA(cudaMemcpyAsync(w, vt, n * sizeof(double), cudaMemcpyDeviceToDevice, c->s));
+    replay(c, c->rp_hess, [&] { gn_sweeps<double>(c, c->vlin.p, w, f); });
   } else {
-    float* w32 = c->w32.wcoef.get(c->ncdN());
-    convert<double, float>(vt, w32, c->ncdN(), c->s);
-    gn_sweeps<float>(c, c->w32.vcoef.p, w32, f);
+    float* w32 = c->w32.wcoef.get(n);
+    convert<double, float>(vt, w32, n, c->s);
+    replay(c, c->rp_hess, [&] { gn_sweeps<float>(c, c->w32.vcoef.p, w32, f); });
   }
   tail(c, vt, f, out);
 }
 
-// addresses of every buffer the captured matvec touches: a change means the
-// graph would read or write stale memory and must be captured again
-size_t graph_signature(reg_ctx* c) {
-  const void* ptrs[] = {c->f.p,        c->SV.p,       c->SF.p,       c->vlin.p,     c->gdir.p,     c->gout.p,
-                        c->w64.gx.p,   c->w64.gy.p,    c->w64.m.p,    c->w64.yh.p,   c->w64.acc.p,
-                        c->w64.lam.p,  c->w64.va.p,   c->w64.vb.p,   c->w64.wa.p,   c->w64.wb.p,   c->w64.gm.p,
-                        c->w64.gmh.p,  c->w64.ck.p,   c->w32.gx.p,   c->w32.gy.p,    c->w32.m.p,
-                        c->w32.yh.p,   c->w32.acc.p,  c->w32.lam.p,  c->w32.va.p,   c->w32.vb.p,   c->w32.wa.p,
-                        c->w32.wb.p,   c->w32.gm.p,   c->w32.gmh.p,  c->w32.ck.p,   c->w32.vcoef.p, c->w32.wcoef.p,
-                        c->w32.fhi.p,  c->w32.flo.p,  c->w64.G.p,    c->w32.G.p,    c->w64.src.p,  c->w32.src.p,
-                        c->w64.mtil.p, c->w32.mtil.p, c->w64.lamN.p, c->w32.lamN.p, c->w64.yh2.p, c->w32.yh2.p,
-                        c->w64.acc2.p, c->w32.acc2.p, c->w64.st0.p,  c->w32.st0.p,  c->w64.st1.p,  c->w32.st1.p,
-                        c->w64.Gt.p,   c->w32.Gt.p,   c->w64.gx2.p,  c->w32.gx2.p,  c->w64.gy2.p,  c->w32.gy2.p,
-                        c->w64.yhS.p,  c->w32.yhS.p,  c->w64.accS.p, c->w32.accS.p,
-                        c->w64.srcS.p, c->w32.srcS.p, c->w64.lamR.p, c->w32.lamR.p, c->w64.yhR.p,  c->w32.yhR.p};
-  size_t h = 1469598103934665603ull;
-  for (const void* p : ptrs) h = (h ^ (size_t)p) * 1099511628211ull;
-  // and the settings that change what the matvec computes
-  uint64_t bb;
-  std::memcpy(&bb, &c->beta, sizeof bb);
-  const uint64_t modes[] = {bb, (uint64_t)c->hess, (uint64_t)c->quad, (uint64_t)c->prec, (uint64_t)c->n_t};
-  for (uint64_t m : modes) h = (h ^ (size_t)m) * 1099511628211ull;
-  return h;
-}
-
 void hessvec(reg_ctx* c, const double* vt, double* out) {
   if (!c->ready) throw StatusError{REG_ENOTREADY, "no linearisation point: call reg_gradient or reg_linearize first"};
-  if (!c->graphs || !c->s || c->prof.mask) {
-    hessvec_body(c, vt, out);
-    return;
-  }
-  const long n = c->ncdN();
-  double* gvt = c->gdir.get(n);
-  double* gout = c->gout.get(n);
-  if (!c->gexec || graph_signature(c) != c->gsig) {
-    if (c->gexec) {
-      cudaGraphExecDestroy(c->gexec);
-      c->gexec = nullptr;
-    }
-    // one ordinary run allocates every buffer (and tunes the passes) first
-    REG_CUDA(cudaMemcpyAsync(gvt, vt, n * sizeof(double), cudaMemcpyDeviceToDevice, c->s));
-    hessvec_body(c, gvt, gout);
-    REG_CUDA(cudaStreamSynchronize(c->s));
-    long l0 = launch_count();
-    cudaGraph_t graph = nullptr;
-    REG_CUDA(cudaStreamBeginCapture(c->s, cudaStreamCaptureModeThreadLocal));
-    try {
-      hessvec_body(c, gvt, gout);
-    } catch (...) {
-      cudaStreamEndCapture(c->s, &graph);
-      if (graph) cudaGraphDestroy(graph);
-      throw;
-    }
-    REG_CUDA(cudaStreamEndCapture(c->s, &graph));
-    cudaError_t e = cudaGraphInstantiate(&c->gexec, graph, 0);
-    cudaGraphDestroy(graph);
-    REG_CUDA(e);
-    c->gkernels = launch_count() - l0;
-    c->gsig = graph_signature(c);
-  }
-  REG_CUDA(cudaMemcpyAsync(gvt, vt, n * sizeof(double), cudaMemcpyDeviceToDevice, c->s));
-  REG_CUDA(cudaGraphLaunch(c->gexec, c->s));
-  add_launches(c->gkernels);
-  REG_CUDA(cudaMemcpyAsync(out, gout, n * sizeof(double), cudaMemcpyDeviceToDevice, c->s));
+  hessvec_body(c, vt, out);
 }
 
 Coefs basis_at(const reg_ctx* c, double t) {
@@ -1494,7 +1521,7 @@ void objective_seg(reg_ctx* c, const double* v, std::vector<double>& dist, std::
   const long N = c->N();
   Work<double>& w = c->w64;
   REG_CUDA(cudaMemcpyAsync(w.m.get(N), c->mT.p, N * sizeof(double), cudaMemcpyDeviceToDevice, c->s));
-  state_steps<double>(c, v, 0, c->n_t, nullptr, nullptr, 0, nullptr);
+  state_solve(c, v);
   Seg one(c, 1), vec(c, c->n_c * c->d);
   dist.resize(c->g.B);
   seg_sqdiff(c->mR.p, w.m.p, 1, c->g.B, c->g.N1, one.scr, c->s, dist.data());
@@ -1515,7 +1542,7 @@ void gradient_seg(reg_ctx* c, const double* v, double* g, std::vector<double>& d
   for (double& x : dist) x *= 0.5 * c->hd;
   lincomb_t<double>(1.0, c->mR.p, -1.0, w.m.p, w.lam.get(N), N, c->s);
   double* f = c->f.get(c->ncdN());
-  adjoint_solve<double>(c, c->vlin.p, f);
+  replay(c, c->rp_adj, [&] { adjoint_solve<double>(c, c->vlin.p, f); });
   tail(c, c->vlin.p, f, g);
   double* Rv = c->tmpB.get(c->ncdN());
   tail(c, c->vlin.p, nullptr, Rv);
@@ -2058,10 +2085,11 @@ void reg::set_thread_error(const std::string& msg) { g_create_error = msg; }
 
 namespace {
 
-// a tile copy of the TMA column pass that never landed leaves garbage: fail the call
-void check_copies(reg_ctx* c) {
-  if (take_tma_timeouts_f32(c->s) + take_tma_timeouts_f64(c->s) > 0)
-    throw StatusError{REG_ETIMEOUT, "a tile copy of the column pass timed out"};
+// a context on the NULL stream: its own stream waits for what the NULL stream holds
+void behind_null_stream(reg_ctx* c) {
+  if (!c->own) return;
+  REG_CUDA(cudaEventRecord(c->own_ev, nullptr));
+  REG_CUDA(cudaStreamWaitEvent(c->own, c->own_ev, 0));
 }
 
 reg_status fail(reg_ctx* c, int st, const std::string& msg) {
@@ -2077,9 +2105,9 @@ reg_status fail(reg_ctx* c, int st, const std::string& msg) {
   reg_ctx* c_ = (ctx);                                          \
   c_->err.clear();                                              \
   tl_prof = c_->prof.mask ? &c_->prof : nullptr;                \
-  try {
+  try {                                                         \
+    behind_null_stream(c_);
 #define API_END                                                                                       \
-  check_copies(c_);                                                                                   \
   }                                                                                                   \
   catch (const StatusError& e) {                                                                      \
     return fail(c_, e.status, e.what);                                                                \
@@ -2111,7 +2139,11 @@ reg_ctx* create_ctx(int d, const int64_t* n, int n_t, int n_c, double beta, int 
   c->prec = precision;
   c->ckpt = ckpt_every;
   c->s = (cudaStream_t)cuda_stream;
-  c->graphs = c->s != nullptr;  // a context with its own stream replays its matvec as a CUDA graph
+  if (!c->s) {
+    REG_CUDA(cudaEventCreateWithFlags(&c->own_ev, cudaEventDisableTiming));
+    REG_CUDA(cudaStreamCreateWithFlags(&c->own, cudaStreamNonBlocking));
+    c->s = c->own;
+  }
   for (int i = 0; i < d; ++i) c->hd *= 2.0 * M_PI / g.n[i];
   c->bnode.resize((size_t)(n_t + 1) * n_c);
   for (int j = 0; j <= n_t; ++j) cheb_values(n_c, (double)j / n_t, &c->bnode[(size_t)j * n_c]);
@@ -2271,7 +2303,7 @@ reg_status reg_transport(reg_ctx* ctx, const double* v, const double* m0, double
   Output o(c_, m1, N, c_->stage_out);
   Work<double>& w = c_->w64;
   REG_CUDA(cudaMemcpyAsync(w.m.get(N), md, N * sizeof(double), cudaMemcpyDeviceToDevice, c_->s));
-  state_steps<double>(c_, vd, 0, c_->n_t, nullptr, nullptr, 0, nullptr);
+  state_solve(c_, vd);
   REG_CUDA(cudaMemcpyAsync(o.dev, w.m.p, N * sizeof(double), cudaMemcpyDeviceToDevice, c_->s));
   o.finish();
   API_END
@@ -2285,13 +2317,15 @@ reg_status reg_transport_adjoint(reg_ctx* ctx, const double* v, const double* m0
   const double* md = input_ptr(c_, m0, N, 1);
   const double* Gd = input_ptr(c_, G, N, 2);
   c_->ready = false;  // the stored state now belongs to (v, m0)
-  double* vc = c_->tmpA.get(c_->ncdN());
+  double* vc = c_->vlin.get(c_->ncdN());
   REG_CUDA(cudaMemcpyAsync(vc, vd, c_->ncdN() * sizeof(double), cudaMemcpyDeviceToDevice, c_->s));
-  state_solve_store<double>(c_, vc, md);
   Work<double>& w = c_->w64;
+  REG_CUDA(cudaMemcpyAsync(w.m.get(N), md, N * sizeof(double), cudaMemcpyDeviceToDevice, c_->s));
+  replay(c_, c_->rp_store, [&] { state_solve_store<double>(c_, vc); });
   lincomb_t<double>(-1.0, Gd, 0.0, nullptr, w.lam.get(N), N, c_->s);  // lam_1 = -G
   double* f = c_->f.get(c_->ncdN());
-  const double* lam0 = adjoint_solve<double>(c_, vc, f);
+  replay(c_, c_->rp_adj, [&] { adjoint_solve<double>(c_, vc, f); });
+  const double* lam0 = ring_slot(w.lamR.p, c_->n_t - 1, N);  // where the last step left lam_0
   if (grad_v) {
     Output o(c_, grad_v, c_->ncdN(), c_->stage_out);
     REG_CUDA(cudaMemcpyAsync(o.dev, f, c_->ncdN() * sizeof(double), cudaMemcpyDeviceToDevice, c_->s));

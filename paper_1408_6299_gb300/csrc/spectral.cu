@@ -90,6 +90,7 @@ __global__ void __launch_bounds__(256) k_spec_tail(const double2* __restrict__ V
                                                    const double* __restrict__ Cg, int reg, int stokes,
                                                    const double* __restrict__ betas,
                                                    const double* __restrict__ inv_k2) {
+  chain_enter();
   const long q = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= g.Nc) return;
   if (betas) beta = betas[q >> g.lg1];
@@ -179,6 +180,7 @@ __global__ void __launch_bounds__(256) k_spec_precond(const double2* __restrict_
                                                       GridArgs g, int nc_, double beta, const double* __restrict__ Ci,
                                                       int reg, const double* __restrict__ betas,
                                                       const double* __restrict__ inv_k2) {
+  chain_enter();
   const long q = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= g.Nc) return;
   if (betas) beta = betas[q >> g.lg1];
@@ -308,8 +310,7 @@ void spec_tail(const Grid& g, cudaStream_t s, const double2* V, const double2* F
                const double* Cg_dev, int reg, int stokes, const double* betas, const double* inv_k2) {
   if (nc > kMaxNc) throw StatusError{1, "n_c too large"};
   auto run = [&](auto k) {
-    k<<<blocks_for(g.Nc), 256, 0, s>>>(V, F, out, args(g), nc, beta, Cg_dev, reg, stokes, betas, inv_k2);
-    REG_LAUNCH();
+    chain(k, blocks_for(g.Nc), 256, s, V, F, out, args(g), nc, beta, Cg_dev, reg, stokes, betas, inv_k2);
   };
   if (nc == 1) run(k_spec_tail<1>);
   else if (nc == 2) run(k_spec_tail<2>);
@@ -320,8 +321,7 @@ void spec_tail(const Grid& g, cudaStream_t s, const double2* V, const double2* F
 void spec_precond(const Grid& g, cudaStream_t s, const double2* R, double2* out, int nc, double beta,
                   const double* Ci_dev, int reg, const double* betas, const double* inv_k2) {
   auto run = [&](auto k) {
-    k<<<blocks_for(g.Nc), 256, 0, s>>>(R, out, args(g), nc, beta, Ci_dev, reg, betas, inv_k2);
-    REG_LAUNCH();
+    chain(k, blocks_for(g.Nc), 256, s, R, out, args(g), nc, beta, Ci_dev, reg, betas, inv_k2);
   };
   if (nc == 1) run(k_spec_precond<1>);
   else if (nc == 2) run(k_spec_precond<2>);

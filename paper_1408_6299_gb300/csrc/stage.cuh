@@ -11,8 +11,6 @@
 // Both work on real fields: two neighbouring real lines form one complex line
 // (line.cuh). Spectra are never stored.
 #pragma once
-#include <cuda.h>
-
 #include "internal.h"
 #include "transform.cuh"
 
@@ -182,6 +180,7 @@ __device__ __forceinline__ float4 gmul(float4 a, float4 b) {
 template <class A, typename T, int L, bool NARROW, bool PROD, int VAR>
 __global__ void __launch_bounds__(ColTile<A, L, NARROW, VAR>::NT) k_cols_line(ColJobs<T> J,
                                                                           const typename A::W* __restrict__ tw) {
+  chain_enter(sizeof(T) == 4);
   using Tile = ColTile<A, L, NARROW, VAR>;
   using Ln = Line<A, L, NARROW>;
   using V = typename A::V;
@@ -275,6 +274,7 @@ struct RowTile {
 template <class A, typename T, int L, bool NARROW, int EPI>
 __global__ void __launch_bounds__(RowTile<L, NARROW, EPI>::NT) k_rows_line(RowArgs<T> a,
                                                                             const typename A::W* __restrict__ tw) {
+  chain_enter(sizeof(T) == 4);
   using Tile = RowTile<L, NARROW, EPI>;
   using Ln = Line<A, L, NARROW>;
   using V = typename A::V;
@@ -376,53 +376,6 @@ __global__ void __launch_bounds__(RowTile<L, NARROW, EPI>::NT) k_rows_line(RowAr
       div_point<T>(a.dv, k, q);
     }
   }
-}
-
-// ---------------------------------------------------------------------------
-// Bounded waits on tensor copies
-// ---------------------------------------------------------------------------
-static __device__ int g_tma_timeouts;
-
-__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_addr(bar)), "r"(bytes)
-               : "memory");
-}
-// wait for the phase with parity `parity`; false when the bound runs out
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, int tries = 1 << 20) {
-  for (int i = 0; i < tries; ++i) {
-    unsigned done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(smem_addr(bar)), "r"(parity)
-        : "memory");
-    if (done) return true;
-  }
-  return false;
-}
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n" ::
-          "r"(smem_addr(dst)),
-      "l"(map), "r"(x), "r"(y), "r"(smem_addr(bar))
-      : "memory");
-}
-
-// Failure-path check: one block waits on an mbarrier that nothing completes,
-// gives up after `tries` polls and counts the timeout as the column pass does.
-static __global__ void k_wait_timeout_probe(int tries) {
-  __shared__ __align__(8) uint64_t bar;
-  if (threadIdx.x == 0) {
-    mbar_init(&bar, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-  }
-  __syncthreads();
-  if (!__syncthreads_and(mbar_wait(&bar, 0, tries)) && threadIdx.x == 0) atomicAdd(&g_tma_timeouts, 1);
 }
 
 }  // namespace fused

@@ -57,9 +57,8 @@ void cols_launch(const Spectral<T>& sp, const ColJob<T>* jobs, int nj, cudaStrea
   J.start[nj] = nj * per;
   ProfScope ps(KK_COLS, st, (double)nj * g.N * sizeof(T) * (PROD ? 3.0 : 2.0),
                (double)nj * g.Nc / L * (2.0 * fft_flops<L>() + 2.0 * L));
-  k_cols_line<A, T, L, NARROW, PROD, VAR><<<(unsigned)(nj * per), Tile::NT, 0, st>>>(
-      J, static_cast<const typename A::W*>(sp.line_table(L, NARROW, A::TABLE)));
-  REG_LAUNCH();
+  chain(k_cols_line<A, T, L, NARROW, PROD, VAR>, (unsigned)(nj * per), Tile::NT, st, J,
+        static_cast<const typename A::W*>(sp.line_table(L, NARROW, A::TABLE)));
 }
 
 // Fields up to 16 MB live in L2 between the passes, as in the trials; larger
@@ -123,9 +122,8 @@ void rows_L(const Spectral<T>& sp, const RowArgs<T>& a, double bytes, cudaStream
     constexpr bool NARROW = decltype(narrow)::value;
     using Tile = RowTile<L, NARROW, EPI>;
     const unsigned grid = (unsigned)((a.nrows + Tile::ROWS - 1) / Tile::ROWS);
-    k_rows_line<A, T, L, NARROW, EPI><<<grid, Tile::NT, 0, st>>>(
-        a, static_cast<const typename A::W*>(sp.line_table(L, NARROW, A::TABLE)));
-    REG_LAUNCH();
+    chain(k_rows_line<A, T, L, NARROW, EPI>, grid, Tile::NT, st, a,
+          static_cast<const typename A::W*>(sp.line_table(L, NARROW, A::TABLE)));
   };
   if (narrow_lines(a.nrows / 2 * NF * LinePlan<L, false>::TS)) go(std::true_type{});
   else go(std::false_type{});

@@ -25,6 +25,7 @@ __global__ void __launch_bounds__(FieldRows<L, NARROW, VAR>::NT) k_field_rows_fw
                                                                                    double2* __restrict__ out,
                                                                                    long nrows,
                                                                                    const int4* __restrict__ tw) {
+  chain_enter();
   using F = FieldRows<L, NARROW, VAR>;
   using Ln = Line<LineFixed, L, NARROW>;
   constexpr int E = Ln::E, TS = F::TS, M = L / 2;
@@ -80,6 +81,7 @@ template <int L, bool NARROW>
 __global__ void __launch_bounds__(FieldRows<L, NARROW, 0>::NT) k_field_rows_inv(const double2* __restrict__ in,
                                                                                  double* __restrict__ out, long nrows,
                                                                                  const int4* __restrict__ tw) {
+  chain_enter();
   using F = FieldRows<L, NARROW, 0>;
   using Ln = Line<LineFixed, L, NARROW>;
   constexpr int E = Ln::E, TS = F::TS, M = L / 2;
@@ -136,6 +138,7 @@ struct FieldCols {
 template <int L, bool NARROW, bool INV>
 __global__ void __launch_bounds__(FieldCols<L, NARROW>::NT) k_field_cols(double2* __restrict__ data, int ls, long n,
                                                                           const int4* __restrict__ tw) {
+  chain_enter();
   using F = FieldCols<L, NARROW>;
   using Ln = Line<LineFixed, L, NARROW>;
   constexpr int E = Ln::E, TC = F::TC;
@@ -211,9 +214,8 @@ void FieldTransforms::cols(double2* U, int axis, int nf, bool inverse) const {
       using F = FieldCols<L, NW>;
       const int4* tw = static_cast<const int4*>(tables_(L, NW));
       const unsigned grid = (unsigned)((n + F::TC - 1) / F::TC);
-      if (inverse) k_field_cols<L, NW, true><<<grid, F::NT, 0, s_>>>(U, ilog2_c((int)s), n, tw);
-      else k_field_cols<L, NW, false><<<grid, F::NT, 0, s_>>>(U, ilog2_c((int)s), n, tw);
-      REG_LAUNCH();
+      chain(inverse ? k_field_cols<L, NW, true> : k_field_cols<L, NW, false>, grid, F::NT, s_, U, ilog2_c((int)s), n,
+            tw);
     });
   });
 }
@@ -231,10 +233,9 @@ void FieldTransforms::fwd(const double* u, double2* U, int nf) const {
         using F1 = FieldRows<L, NW, 1>;
         const long lines = rows / 2;
         if (var == 0)
-          k_field_rows_fwd<L, NW, 0><<<(unsigned)((lines + F0::NSEQ - 1) / F0::NSEQ), F0::NT, 0, s_>>>(u, U, rows, tw);
+          chain(k_field_rows_fwd<L, NW, 0>, (unsigned)((lines + F0::NSEQ - 1) / F0::NSEQ), F0::NT, s_, u, U, rows, tw);
         else
-          k_field_rows_fwd<L, NW, 1><<<(unsigned)((lines + F1::NSEQ - 1) / F1::NSEQ), F1::NT, 0, s_>>>(u, U, rows, tw);
-        REG_LAUNCH();
+          chain(k_field_rows_fwd<L, NW, 1>, (unsigned)((lines + F1::NSEQ - 1) / F1::NSEQ), F1::NT, s_, u, U, rows, tw);
       };
       run(tuned_ ? tuned_choice("rows_r2c", sizeof(double), L, tune_size(rows), 2, s_, run) : 0);
     });
@@ -251,9 +252,8 @@ void FieldTransforms::inv(double2* U, double* u, int nf) const {
     by_plan(narrow(L, rows / 2), [&](auto nw) {
       constexpr bool NW = decltype(nw)::value;
       using F = FieldRows<L, NW, 0>;
-      k_field_rows_inv<L, NW><<<(unsigned)((rows / 2 + F::NSEQ - 1) / F::NSEQ), F::NT, 0, s_>>>(
-          U, u, rows, static_cast<const int4*>(tables_(L, NW)));
-      REG_LAUNCH();
+      chain(k_field_rows_inv<L, NW>, (unsigned)((rows / 2 + F::NSEQ - 1) / F::NSEQ), F::NT, s_, U, u, rows,
+            static_cast<const int4*>(tables_(L, NW)));
     });
   });
 }
