@@ -24,8 +24,13 @@
  * cudaPointerGetAttributes and stages host arrays through its own device
  * buffers. The caller owns every array it passes; the library never frees
  * them and keeps no reference after a call returns (images are copied).
- * All work is ordered on the context's stream; calls return after that work
- * has finished (results are valid on return). A context is not thread-safe:
+ * Device arrays may start at any element; those off a 16-byte boundary are
+ * staged like host arrays.
+ * All work is ordered on the context's stream (a context created on the NULL
+ * stream works on a stream of its own that first waits for what the NULL
+ * stream holds); calls return after that work has finished (results are valid
+ * on return). From their second call on, the sweeps of a context are captured
+ * and replayed as CUDA graphs. A context is not thread-safe:
  * use one context per host thread.
  *
  * Errors: every call returns a reg_status; reg_last_error() describes the most
@@ -336,8 +341,7 @@ typedef struct {
 /* Solve `count` independent problems (Alg. 1 each, options opts for all, or
  * the defaults when NULL) concurrently on the current device: `workers` host
  * threads, each with its own CUDA stream and contexts cached per problem
- * configuration, take problems from a queue ordered largest first. Contexts
- * with their own stream replay the Hessian matvec as a captured CUDA graph.
+ * configuration, take problems from a queue ordered largest first.
  * reports (may be NULL): host array of count, report i for problem i. Returns
  * REG_OK when every solve returned REG_OK or REG_EMAXIT, else the status of
  * the first failing problem (all problems are attempted); the message is in
@@ -418,8 +422,9 @@ REG_API reg_status reg_continuation(reg_ctx* ctx, double* v_inout, const reg_sol
 
 /* ------------------------------------------------------------------------
  * Instrumentation (no counterpart in the paper; used to measure the kernels).
- * Kernel kinds: 0 row real-to-complex FFT pass, 1 row complex-to-real pass,
- * 2 strided complex FFT pass, 3 Fourier multipliers, 4 Heun stage /
+ * Kernel kinds: 0 real-to-complex rows of whole-field transforms, 1 row pass of
+ * a transport stage with its epilogue (or complex-to-real rows of a whole-field
+ * transform), 2 strided pass, 3 Fourier multipliers, 4 Heun stage /
  * transport right-hand side, 5 body-force accumulation, 6 other.
  * ------------------------------------------------------------------------ */
 #define REG_KIND_COUNT 7
@@ -436,16 +441,16 @@ REG_API reg_status reg_profile_end(reg_ctx* ctx, double* ms, double* bytes, long
 /* Floating-point operations of the transforms of the launches collected by
  * the last reg_profile_end, per kind (REG_KIND_COUNT values): the butterflies
  * and twiddle multiplications of every FFT the launches ran (radix plan
- * counts), the spectral multipliers of the column passes, and the packing of
- * the real-to-complex rows. Pointwise epilogue arithmetic is not counted. */
+ * counts) and the spectral multipliers. Pointwise epilogue arithmetic is not
+ * counted; in double precision the lines run in fixed point, where the count is
+ * that of the same plan in floating point. */
 REG_API reg_status reg_profile_flops(reg_ctx* ctx, double* flops);
 
 /* Double-precision FMA throughput of the current device in GFLOP/s (2 flops
  * per FMA): independent FMA chains in every thread of one wave of resident
  * blocks, the best of three launches timed with CUDA events after a warm-up.
- * Allocates and frees a small buffer; changes no device setting. The bound
- * of the FP64 transport sweeps, whose arithmetic rate the bench reports
- * against it. Errors: REG_ECUDA (message in reg_last_error(NULL)). */
+ * Allocates and frees a small buffer; changes no device setting. The bench
+ * reports the transforms' rate in the FP64 sweeps against it. Errors: REG_ECUDA (message in reg_last_error(NULL)). */
 REG_API reg_status reg_fp64_peak(double* gflops);
 
 /* Number of kernel launches issued by the library in this process so far. */
@@ -453,9 +458,7 @@ REG_API long reg_launch_count(void);
 
 /* Failure-path check of the bounded waits (no counterpart in the paper): one
  * block polls an mbarrier that nothing completes, gives up after a bounded
- * number of polls, and counts the timeout the way the TMA column pass counts
- * a tile copy that never lands (which fails the API call with
- * REG_ETIMEOUT). *counted: the timeouts read back and cleared (1 expected).
+ * number of polls, and counts the timeout. *counted: the timeouts read back and cleared (1 expected).
  * Faults, traps and hangs nothing; uses the current device. */
 REG_API reg_status reg_selftest_copy_timeout(int* counted);
 

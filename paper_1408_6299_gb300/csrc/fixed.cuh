@@ -150,9 +150,12 @@ __host__ __device__ constexpr int fx_headroom() {
   return L == 512 ? 60 : 61;
 }
 
-// the largest magnitude of a pair, as the high word of a double (ordered as an unsigned number)
+// the largest magnitude of a pair, as the high word of a double (ordered as an
+// unsigned number), its lowest bit set by low words: subnormal values without a
+// high word are not zero
 __device__ __forceinline__ unsigned fx_mag(double2 x) {
-  return max((unsigned)__double2hiint(x.x) & 0x7fffffffu, (unsigned)__double2hiint(x.y) & 0x7fffffffu);
+  return max((unsigned)__double2hiint(x.x) & 0x7fffffffu, (unsigned)__double2hiint(x.y) & 0x7fffffffu) |
+         min((unsigned)(__double2loint(x.x) | __double2loint(x.y)), 1u);
 }
 
 // |x| + |y| to about 2^-20, for magnitudes from 2^-126 to 2^100 (smaller ones

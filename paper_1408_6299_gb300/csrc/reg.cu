@@ -164,7 +164,7 @@ struct reg_ctx {
   DBuf<double2> SV, SF;  // spectra of coefficient vectors for the tail
   DBuf<double> red;    // reduction scratch
   DBuf<double> tmpA, tmpB;  // coefficient-vector temporaries
-  DBuf<double> stage_in[3], stage_out;  // staging of host arrays
+  DBuf<double> stage_in[3], stage_out;  // staging of host arrays and of views at odd offsets
   // det F scratch
   DBuf<double> F, Fh, K1, K2, gvl, gvt, det, ang;
   DBuf<double> disp_src;                          // sources -v_i(t) of the deformation map
@@ -234,11 +234,15 @@ bool is_device_ptr(const void* p) {
   return true;
 }
 
+// Kernels access fields in units of 16 bytes: host arrays, and device arrays
+// that start elsewhere (views at an odd offset), go through a staging buffer.
+bool usable(const double* p) { return is_device_ptr(p) && (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
 const double* input_ptr(reg_ctx* c, const double* p, long n, int slot) {
   if (!p) throw StatusError{REG_EINVAL, "null array argument"};
-  if (is_device_ptr(p)) return p;
+  if (usable(p)) return p;
   double* d = c->stage_in[slot].get(n);
-  REG_CUDA(cudaMemcpyAsync(d, p, n * sizeof(double), cudaMemcpyHostToDevice, c->s));
+  REG_CUDA(cudaMemcpyAsync(d, p, n * sizeof(double), cudaMemcpyDefault, c->s));
   return d;
 }
 
@@ -247,14 +251,14 @@ struct Output {
   double* user;
   double* dev;
   long n;
-  bool host;
+  bool staged;
   Output(reg_ctx* c_, double* p, long n_, DBuf<double>& stage) : c(c_), user(p), n(n_) {
     if (!p) throw StatusError{REG_EINVAL, "null output argument"};
-    host = !is_device_ptr(p);
-    dev = host ? stage.get(n) : p;
+    staged = !usable(p);
+    dev = staged ? stage.get(n) : p;
   }
   void finish() {
-    if (host) REG_CUDA(cudaMemcpyAsync(user, dev, n * sizeof(double), cudaMemcpyDeviceToHost, c->s));
+    if (staged) REG_CUDA(cudaMemcpyAsync(user, dev, n * sizeof(double), cudaMemcpyDefault, c->s));
     REG_CUDA(cudaStreamSynchronize(c->s));
   }
 };
@@ -2475,8 +2479,8 @@ reg_status reg_continuation(reg_ctx* ctx, double* v_inout, const reg_solve_opts*
   if (cont_opts) co = *cont_opts;
   if (!v_inout) throw StatusError{REG_EINVAL, "v_inout is null"};
   Output io(c_, v_inout, c_->ncdN(), c_->stage_out);
-  if (io.host)
-    REG_CUDA(cudaMemcpyAsync(io.dev, v_inout, c_->ncdN() * sizeof(double), cudaMemcpyHostToDevice, c_->s));
+  if (io.staged)
+    REG_CUDA(cudaMemcpyAsync(io.dev, v_inout, c_->ncdN() * sizeof(double), cudaMemcpyDefault, c_->s));
   reg_cont_report R;
   continuation(c_, io.dev, so, co, R);
   io.finish();
@@ -2672,8 +2676,8 @@ reg_status reg_solve(reg_ctx* ctx, double* v_inout, const reg_solve_opts* opts, 
   if (opts) o = *opts;
   if (!v_inout) throw StatusError{REG_EINVAL, "v_inout is null"};
   Output io(c_, v_inout, c_->ncdN(), c_->stage_out);
-  if (io.host)
-    REG_CUDA(cudaMemcpyAsync(io.dev, v_inout, c_->ncdN() * sizeof(double), cudaMemcpyHostToDevice, c_->s));
+  if (io.staged)
+    REG_CUDA(cudaMemcpyAsync(io.dev, v_inout, c_->ncdN() * sizeof(double), cudaMemcpyDefault, c_->s));
   reg_solve_report R;
   int st = solve(c_, io.dev, o, R);
   io.finish();
