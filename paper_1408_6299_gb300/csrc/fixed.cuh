@@ -174,7 +174,7 @@ __device__ __forceinline__ float fx_l1(double2 x) {
 template <int L, int R0>
 struct FxScale {
   static constexpr int S0 = fx_headroom<L>() - ilog2_c(R0), S = fx_headroom<L>() - ilog2_c(L);
-  int up, down, low;  // exponent shifts in the high word; smallest exponent that still counts
+  int right, down;  // in1: shift of a value with exponent field 0; exponent shift of the results (high word)
   bool plain;
   bool scaled = true;  // the forward stages scale (see Line::forward)
   double pre, post;
@@ -195,22 +195,41 @@ struct FxScale {
         e = __double2hiint(m * pre) >> 20;
       }
     }
-    up = (S0 + 1022 - e) * (1 << 20);
+    right = 63 - S0 + e;
     down = (e - 1022 - S) * (1 << 20);
-    low = (e - 62) * (1 << 20);
   }
+  // Conversions in integer arithmetic: the double-precision unit converts two
+  // values per clock and SM, and the epilogues need it. Rounded to nearest.
   __device__ __forceinline__ long long in1(double x) const {
     if (!plain) {
       if (pre == 0.0) return 0;
       x *= pre;
     }
     const int hi = __double2hiint(x);
-    if ((hi & 0x7ff00000) < low) return 0;  // below half a unit
-    return __double2ll_rn(__hiloint2double(hi + up, __double2loint(x)));
+    const unsigned lo = (unsigned)__double2loint(x);
+    // the 53-bit significand times 2^10, shifted right by r >= 1; r counts up for smaller values
+    const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+    const unsigned long long m = ((unsigned long long)__funnelshift_l(lo, mh, 10) << 32) | (lo << 10);
+    const int r = right - ((hi >> 20) & 0x7ff);
+    const unsigned long long v = ((r > 64 ? 0ull : m >> (r - 1)) + 1) >> 1;
+    const long long sign = (long long)(hi >> 31);
+    return (long long)(v ^ (unsigned long long)sign) - sign;
   }
   __device__ __forceinline__ double out1(long long r) const {
     const double d = __ll2double_rn(r);
     double x = r == 0 ? 0.0 : __hiloint2double(__double2hiint(d) + down, __double2loint(d));
+    if (!plain) x *= post;
+    return x;
+  }
+  __device__ __forceinline__ double out1i(long long r) const {
+    const long long sign = r >> 63;
+    const unsigned long long a = (unsigned long long)((r ^ sign) - sign);
+    const int lz = __clzll((long long)a);
+    // leading one at bit 62, rounded at bit 10; a carry moves into the exponent by itself
+    const unsigned long long n = ((a << lz) >> 1) + 0x200;
+    const unsigned hi = (unsigned)(n >> 42) + (unsigned)((1085 - lz) * (1 << 20) + down);
+    const unsigned lo = __funnelshift_r((unsigned)n, (unsigned)(n >> 32), 10);
+    double x = r == 0 ? 0.0 : __hiloint2double((int)(hi | ((unsigned)(sign >> 32) & 0x80000000u)), (int)lo);
     if (!plain) x *= post;
     return x;
   }
@@ -226,15 +245,15 @@ struct FxScale {
     if (h > ilog2_c(L) - 2) return;
     scaled = false;
     const int s = fx_headroom<L>() - (h > 0 ? h : 0);
-    up = (s + 1022 - e) * (1 << 20);
+    right = 63 - s + e;
     down = (e - 1022 - s) * (1 << 20);
-    low = (e - 63) * (1 << 20);
   }
   // results times 2^n as well
   __device__ __forceinline__ void times_pow2(int n) { down += n * (1 << 20); }
   __device__ __forceinline__ FxV in(double2 x) const { return {in1(x.x), in1(x.y)}; }
-  // the conjugate of z, scaled back
+  // the conjugate of z, scaled back; out converts on the double-precision unit, outi on the integer one
   __device__ __forceinline__ double2 out(FxV z) const { return make_double2(out1(z.x), out1(-z.y)); }
+  __device__ __forceinline__ double2 outi(FxV z) const { return make_double2(out1i(z.x), out1i(-z.y)); }
 };
 
 }  // namespace reg

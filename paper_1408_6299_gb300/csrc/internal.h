@@ -56,18 +56,21 @@ long launch_count();
 // Launch of a kernel that begins with chain_enter(): it may be set up while its
 // predecessor on the stream still runs, and waits there for its results. The
 // kernels of a sweep depend on one another and run a few microseconds each on
-// small grids, so the launch gap between them counts.
+// small grids, so the launch gap between them counts. (Behind a join of two
+// streams the launch is an ordinary one: tl_plain_launch.)
+extern thread_local bool tl_plain_launch;
 template <typename... P, typename... A>
-void chain(void (*kern)(P...), unsigned grid, unsigned block, cudaStream_t s, A&&... args) {
+void chain(void (*kern)(P...), dim3 grid, unsigned block, cudaStream_t s, A&&... args) {
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(block);
   cfg.stream = s;
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = tl_plain_launch ? 0 : 1;
+  tl_plain_launch = false;
   count_launch();
   REG_CUDA(cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...));
 }
@@ -151,22 +154,50 @@ class LineTables {
 // to query the size in bytes.
 size_t write_wide_tables(unsigned char* out, long* off);
 
-// Fields whose lines, one per group of threads of the wide plan, are fewer
-// threads than this run the narrow plans (line.cuh).
-bool narrow_lines(long wide_threads);
+// Whether lines that take so many threads on the wide plan run the narrow one
+// (line.cuh) instead: below two warps (single precision: four) per scheduler
+// of the 152 SMs, where a pass lasts as long as one thread's serial work. Both
+// sides measured: 128^2 gradient 5600 us wide, 2170 narrow; 128^3 gradient 42.7
+// ms wide, 61.9 narrow; 128^3 mixed matvec, checkpoints every 8: 16.5 ms at the
+// lower limit for both precisions, 12.6 at this one, 14.1 at twice this one.
+inline bool narrow_lines(long wide_threads, int size) { return wide_threads < 152L * (size == 8 ? 256 : 512); }
 
 // A grid with its stream and line tables in precision T: what the stages run on.
 template <typename T>
 class Spectral {
  public:
   Spectral(const Grid& g, cudaStream_t s) : g_(g), s_(s), lines_(g) {}
+  ~Spectral() {
+    if (fork_ev_) cudaEventDestroy(fork_ev_);
+    if (join_ev_) cudaEventDestroy(join_ev_);
+    if (aux_) cudaStreamDestroy(aux_);
+  }
+  Spectral(const Spectral&) = delete;
+  Spectral& operator=(const Spectral&) = delete;
+  // a second stream for launches that do not depend on one another: fork()
+  // orders it behind the stream, join() the stream behind it
+  cudaStream_t fork() {
+    if (!aux_) {
+      REG_CUDA(cudaEventCreateWithFlags(&fork_ev_, cudaEventDisableTiming));
+      REG_CUDA(cudaEventCreateWithFlags(&join_ev_, cudaEventDisableTiming));
+      REG_CUDA(cudaStreamCreateWithFlags(&aux_, cudaStreamNonBlocking));
+    }
+    REG_CUDA(cudaEventRecord(fork_ev_, s_));
+    REG_CUDA(cudaStreamWaitEvent(aux_, fork_ev_, 0));
+    return aux_;
+  }
+  void join() {
+    REG_CUDA(cudaEventRecord(join_ev_, aux_));
+    REG_CUDA(cudaStreamWaitEvent(s_, join_ev_, 0));
+  }
   const Grid& grid() const { return g_; }
   cudaStream_t stream() const { return s_; }
   const void* line_table(int L, bool narrow, int kind) const { return lines_.get(L, narrow, kind); }
 
  private:
   Grid g_;
-  cudaStream_t s_;
+  cudaStream_t s_, aux_ = nullptr;
+  cudaEvent_t fork_ev_ = nullptr, join_ev_ = nullptr;
   LineTables<T> lines_;
 };
 

@@ -246,15 +246,52 @@ struct Line {
   static constexpr int E = P::E, TS = P::TS, S = P::S;
   static constexpr int R0 = P::R(0), Q0 = L / R0;
 
+  // Twiddles a thread uses in derivative(), in the order of use: forward stages
+  // s >= 1, then inverse ones. Narrow kernels load them into registers before
+  // they wait for their predecessor: a stage would otherwise begin with a miss
+  // to L2, as L1 is empty when a kernel starts.
+  static constexpr bool PRELOAD = NARROW;
+  __host__ __device__ static constexpr int tw_index(int s, bool inv) {
+    int n = 0;
+    for (int b = 0; b < 2; ++b)
+      for (int t = 1; t < S; ++t) {
+        if ((inv ? 1 : 0) == b && t == s) return n;
+        const int R = b ? P::R(S - 1 - t) : P::R(t);
+        n += E / R * (R - 1);
+      }
+    return n;
+  }
+  static constexpr int NTW = PRELOAD ? tw_index(S, true) : 0;
+  template <int s, bool INV>
+  static __device__ __forceinline__ void load_stage(W* w, int j, const W* __restrict__ tw) {
+    if constexpr (s < S) {
+      constexpr int R = line_radix<P>(s, INV), NS = line_ns<P>(s, INV), TK = E / R;
+      const W* t0 = tw + line_tw_offset<P>(s, INV);
+#pragma unroll
+      for (int i = 0; i < TK; ++i)
+#pragma unroll
+        for (int r = 1; r < R; ++r)
+          w[tw_index(s, INV) + i * (R - 1) + r - 1] = __ldg(&t0[r * NS + ((j + i * TS) & (NS - 1))]);
+      load_stage<s + 1, INV>(w, j, tw);
+    }
+  }
+  static __device__ __forceinline__ void preload(W* w, int j, const W* __restrict__ tw) {
+    if constexpr (PRELOAD) {
+      load_stage<1, false>(w, j, tw);
+      load_stage<1, true>(w, j, tw);
+    }
+  }
+
   // position of v[i * R0 + r]
   static __device__ __forceinline__ int position(int j, int e) { return j + (e / R0) * TS + (e % R0) * Q0; }
 
-  template <int s, bool INV, class Buf, class Sync>
-  static __device__ __forceinline__ void stages(V* v, int j, const Buf& buf, const Sync& sync,
-                                                const W* __restrict__ tw, bool scaled = true) {
+  // PRE: tw is the thread's preloaded array
+  template <int s, bool INV, bool PRE, class Buf, class Sync>
+  static __device__ __forceinline__ void stages(V* v, int j, const Buf& buf, const Sync& sync, const W* tw,
+                                                bool scaled = true) {
     constexpr int R = line_radix<P>(s, INV), NS = line_ns<P>(s, INV), Q = L / R, TK = E / R;
     if constexpr (s > 0) {
-      const W* t0 = tw + line_tw_offset<P>(s, INV);
+      const W* t0 = tw + (PRE ? 0 : line_tw_offset<P>(s, INV));
 #pragma unroll
       for (int i = 0; i < TK; ++i) {
         const int t = j + i * TS;
@@ -264,7 +301,9 @@ struct Line {
           if (scaled) v[i * R] = A::template pass_fwd<R>(v[i * R]);
 #pragma unroll
         for (int r = 1; r < R; ++r) {
-          const W w = __ldg(&t0[r * NS + (t & (NS - 1))]);
+          W w;
+          if constexpr (PRE) w = t0[tw_index(s, INV) + i * (R - 1) + r - 1];
+          else w = __ldg(&t0[r * NS + (t & (NS - 1))]);
           if constexpr (INV) v[i * R + r] = A::twiddle_inv(v[i * R + r], w);
           else v[i * R + r] = A::template twiddle_fwd<R>(v[i * R + r], w);
         }
@@ -282,7 +321,7 @@ struct Line {
         for (int r = 0; r < R; ++r) *buf(base + r * NS) = v[i * R + r];
       }
       sync();
-      stages<s + 1, INV>(v, j, buf, sync, tw, scaled);
+      stages<s + 1, INV, PRE>(v, j, buf, sync, tw, scaled);
     }
   }
 
@@ -294,18 +333,18 @@ struct Line {
     return j + (e / R) * TS + (e % R) * (L / R);
   }
   template <class Buf, class Sync>
-  static __device__ __forceinline__ void forward(V* v, int j, const Buf& buf, const Sync& sync,
-                                                 const W* __restrict__ tw, bool scaled) {
-    stages<0, false>(v, j, buf, sync, scaled ? tw : tw + line_tw_block<P>(false) + line_tw_block<P>(true), scaled);
+  static __device__ __forceinline__ void forward(V* v, int j, const Buf& buf, const Sync& sync, const W* tw,
+                                                 bool scaled) {
+    stages<0, false, false>(v, j, buf, sync, scaled ? tw : tw + line_tw_block<P>(false) + line_tw_block<P>(true), scaled);
   }
 
+  // tw: the table, or the array preload() filled (PRELOAD plans)
   template <class Buf, class Sync>
-  static __device__ __forceinline__ void derivative(V* v, int j, const Buf& buf, const Sync& sync,
-                                                    const W* __restrict__ tw) {
-    stages<0, false>(v, j, buf, sync, tw);
+  static __device__ __forceinline__ void derivative(V* v, int j, const Buf& buf, const Sync& sync, const W* tw) {
+    stages<0, false, PRELOAD>(v, j, buf, sync, tw);
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = A::template deriv<L>(v[e], frequency(j, e));
-    stages<0, true>(v, j, buf, sync, tw);
+    stages<0, true, PRELOAD>(v, j, buf, sync, tw);
   }
 };
 

@@ -11,6 +11,8 @@
 // together with the Runge-Kutta combination.
 #include <float.h>
 
+#include <type_traits>
+
 #include "pointwise.h"
 
 namespace reg {
@@ -22,36 +24,65 @@ inline unsigned nblk(long n, int bs = 256) {
   return (unsigned)(b < 1 ? 1 : b);
 }
 
-__global__ void k_vel_at(const double* __restrict__ coef, int nc, Coefs b, double* __restrict__ out, long dN) {
-  chain_enter();
-  long x = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= dN) return;
-  double s = 0.0;
-  for (int l = 0; l < nc; ++l) s += b.c[l] * coef[l * dN + x];
-  out[x] = s;
-}
-
-// The single-precision combination, accurate to the last bit without the
-// double-precision unit (two operations per clock and SM; 16 us for 64^3 with
-// three coefficients that way): every weight is a pair of floats, products
-// and sums keep their rounding errors, and the sum is rounded once.
-struct FloatWeights {
-  float hi[16], lo[16];
+// Sixteen bytes of a field per thread and access
+template <typename T>
+struct alignas(16) Quad {
+  static constexpr int W = 16 / sizeof(T);
+  T v[W];
 };
-__global__ void k_vel_at(const float* __restrict__ coef, int nc, FloatWeights b, float* __restrict__ out, long dN) {
+template <typename T>
+struct One {
+  static constexpr int W = 1;
+  T v[1];
+};
+
+// Weights of a velocity combination. In single precision every weight is a
+// pair of floats: products and sums keep their rounding errors and the sum is
+// rounded once, accurate to the last bit without the double-precision unit
+// (two operations per clock and SM).
+template <typename T>
+struct NodeWeights {
+  T hi[16], lo[16];
+};
+// NC: n_c where it is 2, 3 or 4 (the loads of a point are then issued
+// together: 64^3 with three coefficients 16 -> 4 us), else 0. VEC: 16-byte
+// accesses, else single values (callers' arrays may be offset views).
+template <typename T, int NC, bool VEC>
+__global__ void __launch_bounds__(128) k_vel_at(const T* __restrict__ coef, int nc_, NodeWeights<T> b,
+                                                T* __restrict__ out, long dN) {
   chain_enter();
-  long x = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= dN) return;
-  float s = 0.f, err = 0.f;
-  for (int l = 0; l < nc; ++l) {
-    const float c = coef[l * dN + x];
-    const float p = __fmul_rn(b.hi[l], c);
-    err += fmaf(b.hi[l], c, -p) + b.lo[l] * c;
-    const float t = __fadd_rn(s, p), z = __fsub_rn(t, s);
-    err += __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z));
-    s = t;
+  using Q = std::conditional_t<VEC, Quad<T>, One<T>>;
+  const int nc = NC ? NC : nc_;
+  const long x = (long)blockIdx.x * blockDim.x + threadIdx.x, n = dN / Q::W;
+  if (x >= n) return;
+  const Q* c = reinterpret_cast<const Q*>(coef) + x;
+  Q v[NC ? NC : 1];
+  if (NC) {
+#pragma unroll
+    for (int l = 0; l < NC; ++l) v[l] = c[l * n];
   }
-  out[x] = s + err;
+  Q s{}, err{};
+#pragma unroll
+  for (int l = 0; l < nc; ++l) {
+    if (!NC) v[0] = c[l * n];
+    const Q u = v[NC ? l : 0];
+#pragma unroll
+    for (int w = 0; w < Q::W; ++w) {
+      if constexpr (sizeof(T) == 8) {
+        s.v[w] += b.hi[l] * u.v[w];
+      } else {
+        const float p = __fmul_rn(b.hi[l], u.v[w]);
+        const float e = fmaf(b.hi[l], u.v[w], -p) + b.lo[l] * u.v[w];
+        const float t = __fadd_rn(s.v[w], p), z = __fsub_rn(t, s.v[w]);
+        err.v[w] += e + __fadd_rn(__fsub_rn(s.v[w], __fsub_rn(t, z)), __fsub_rn(p, z));
+        s.v[w] = t;
+      }
+    }
+  }
+  if (sizeof(T) == 4)
+#pragma unroll
+    for (int w = 0; w < Q::W; ++w) s.v[w] += err.v[w];
+  reinterpret_cast<Q*>(out)[x] = s;
 }
 
 template <typename S, typename T>
@@ -83,72 +114,92 @@ __global__ void k_stage(const T* __restrict__ G, const T* __restrict__ vt, const
   }
 }
 
+// out_k = sum_i a_{k,i} b_i for the nodes k = blockIdx.y
 template <typename T>
 __global__ void k_dot_fields(const T* __restrict__ a, const T* __restrict__ b, T* __restrict__ out, int d, long N) {
   chain_enter();
   long x = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= N) return;
+  a += blockIdx.y * d * N;
   T s = 0;
   for (int i = 0; i < d; ++i) s += a[i * N + x] * b[i * N + x];
-  out[x] = s;
+  out[blockIdx.y * N + x] = s;
 }
 
 // Body force of a group of time nodes. Adding each node's term inside the
 // adjoint stage reads and writes the accumulator (n_c d fields, twice that for
 // a compensated pair) at every step; here the nodes of a group share one read
 // and one write of it, and the terms are added in the same order. Bound by
-// the reads of the state gradients. A thread takes one component of a point
-// pair; the blocks of the d components of the same points are neighbours, so
-// they find y in L2.
-template <typename T>
-__global__ void __launch_bounds__(256) k_force(T* __restrict__ fhi, T* __restrict__ flo, ForceNodes<T> F, int nc, int d,
+// the reads of the state gradients. A thread takes 16 bytes of a field, one
+// component (SPLIT; the blocks of the d components of the same points are
+// neighbours, so they find y in L2: small grids) or all of them.
+template <typename T, bool SPLIT>
+__global__ void __launch_bounds__(128) k_force(T* __restrict__ fhi, T* __restrict__ flo, ForceNodes<T> F, int nc, int d,
                                                long N) {
   chain_enter();
-  using C = cx<T>;
-  const int i = blockIdx.x % d;
-  const long q = (long)(blockIdx.x / d) * blockDim.x + threadIdx.x;
-  if (q >= N / 2) return;
-  auto ld = [&](const T* p) { return reinterpret_cast<const C*>(p)[q]; };
-  C ta[kForceNodes], tb[kForceNodes];
+  using Q = Quad<T>;
+  constexpr int W = Q::W;
+  const long q = (long)(SPLIT ? blockIdx.x / d : blockIdx.x) * blockDim.x + threadIdx.x;
+  if (q >= N / W) return;
+  auto ld = [&](const T* p) { return reinterpret_cast<const Q*>(p)[q]; };
+  auto lds = [&](const T* p) {  // read once
+    union {
+      float4 f;
+      Q q;
+    } u;
+    u.f = __ldcs(reinterpret_cast<const float4*>(p) + q);
+    return u.q;
+  };
+  Q y[kForceNodes];
 #pragma unroll
-  for (int k = 0; k < kForceNodes; ++k) {
-    ta[k] = tb[k] = mk<C>(0, 0);
-    if (k < F.count) {
-      const C y = ld(F.yA[k]), g = ld(F.gA[k] + i * N);
-      ta[k] = mk<C>(y.x * g.x, y.y * g.y);
-      if (F.yC[k]) {
-        const C yc = ld(F.yC[k]), gc = ld(F.gC[k] + i * N);
-        ta[k] = mk<C>(ta[k].x + yc.x * gc.x, ta[k].y + yc.y * gc.y);
-      }
-      if (F.yB[k]) {
-        const C yb = ld(F.yB[k]), gb = ld(F.gB[k] + i * N);
-        tb[k] = mk<C>(yb.x * gb.x, yb.y * gb.y);
-      }
-    }
-  }
-  for (int l = 0; l < nc; ++l) {
-    const long o = ((long)l * d + i) * (N / 2) + q;
-    C h = reinterpret_cast<C*>(fhi)[o];
-    C e = flo ? reinterpret_cast<C*>(flo)[o] : mk<C>(0, 0);
+  for (int k = 0; k < kForceNodes; ++k)
+    if (k < F.count) y[k] = ld(F.yA[k]);
+  const int i0 = SPLIT ? blockIdx.x % d : 0, i1 = SPLIT ? i0 + 1 : d;
+  for (int i = i0; i < i1; ++i) {
+    Q ta[kForceNodes];
 #pragma unroll
-    for (int k = 0; k < kForceNodes; ++k) {
-      if (k >= F.count) break;
-      T t0 = F.cA[k][l] * ta[k].x, t1 = F.cA[k][l] * ta[k].y;
-      if (F.yB[k]) {
-        t0 += F.cB[k][l] * tb[k].x;
-        t1 += F.cB[k][l] * tb[k].y;
+    for (int k = 0; k < kForceNodes; ++k)
+      if (k < F.count) ta[k] = lds(F.gA[k] + i * N);
+#pragma unroll
+    for (int k = 0; k < kForceNodes; ++k)
+      if (k < F.count) {
+#pragma unroll
+        for (int w = 0; w < W; ++w) ta[k].v[w] = y[k].v[w] * ta[k].v[w];
+        if (F.yC[k]) {
+          const Q yc = ld(F.yC[k]), gc = ld(F.gC[k] + i * N);
+#pragma unroll
+          for (int w = 0; w < W; ++w) ta[k].v[w] += yc.v[w] * gc.v[w];
+        }
       }
-      if (flo) {
-        const T s0 = h.x + t0, b0 = s0 - h.x, s1 = h.y + t1, b1 = s1 - h.y;
-        e.x += (h.x - (s0 - b0)) + (t0 - b0);
-        e.y += (h.y - (s1 - b1)) + (t1 - b1);
-        h = mk<C>(s0, s1);
-      } else {
-        h = mk<C>(h.x + t0, h.y + t1);
+    for (int l = 0; l < nc; ++l) {
+      const long o = ((long)l * d + i) * (N / W) + q;
+      Q h = reinterpret_cast<Q*>(fhi)[o], e;
+      if (flo) e = reinterpret_cast<Q*>(flo)[o];
+#pragma unroll
+      for (int k = 0; k < kForceNodes; ++k) {
+        if (k >= F.count) break;
+        Q t;
+#pragma unroll
+        for (int w = 0; w < W; ++w) t.v[w] = F.cA[k][l] * ta[k].v[w];
+        if (F.yB[k]) {
+          const Q yb = ld(F.yB[k]), gb = ld(F.gB[k] + i * N);
+#pragma unroll
+          for (int w = 0; w < W; ++w) t.v[w] += F.cB[k][l] * (yb.v[w] * gb.v[w]);
+        }
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+          if (flo) {
+            const T s = h.v[w] + t.v[w], b = s - h.v[w];
+            e.v[w] += (h.v[w] - (s - b)) + (t.v[w] - b);
+            h.v[w] = s;
+          } else {
+            h.v[w] += t.v[w];
+          }
+        }
       }
+      reinterpret_cast<Q*>(fhi)[o] = h;
+      if (flo) reinterpret_cast<Q*>(flo)[o] = e;
     }
-    reinterpret_cast<C*>(fhi)[o] = h;
-    if (flo) reinterpret_cast<C*>(flo)[o] = e;
   }
 }
 
@@ -308,19 +359,21 @@ __global__ void k_reduce_final(const double* __restrict__ part, double* __restri
 
 }  // namespace
 
-template <>
-void vel_at<double>(const double* coef, int nc, const Coefs& b, double* out, long dN, cudaStream_t s) {
-  chain<const double*, int, Coefs, double*, long>(k_vel_at, nblk(dN), 256, s, coef, nc, b, out, dN);
-}
-template <>
-void vel_at<float>(const float* coef, int nc, const Coefs& b, float* out, long dN, cudaStream_t s) {
-  FloatWeights w;
+template <typename T>
+void vel_at(const T* coef, int nc, const Coefs& b, T* out, long dN, cudaStream_t s) {
+  NodeWeights<T> w;
   for (int l = 0; l < 16; ++l) {
-    w.hi[l] = l < nc ? (float)b.c[l] : 0.f;
-    w.lo[l] = l < nc ? (float)(b.c[l] - (double)w.hi[l]) : 0.f;
+    w.hi[l] = l < nc ? (T)b.c[l] : (T)0;
+    w.lo[l] = l < nc ? (T)(b.c[l] - (double)w.hi[l]) : (T)0;
   }
-  chain<const float*, int, FloatWeights, float*, long>(k_vel_at, nblk(dN), 256, s, coef, nc, w, out, dN);
+  const bool vec = ((reinterpret_cast<uintptr_t>(coef) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
+  auto kern = !vec ? k_vel_at<T, 0, false>
+                   : (nc == 2 ? k_vel_at<T, 2, true>
+                              : (nc == 3 ? k_vel_at<T, 3, true> : (nc == 4 ? k_vel_at<T, 4, true> : k_vel_at<T, 0, true>)));
+  chain(kern, nblk(vec ? dN / Quad<T>::W : dN, 128), 128, s, coef, nc, w, out, dN);
 }
+template void vel_at<float>(const float*, int, const Coefs&, float*, long, cudaStream_t);
+template void vel_at<double>(const double*, int, const Coefs&, double*, long, cudaStream_t);
 
 template <typename S, typename T>
 void convert(const S* in, T* out, long n, cudaStream_t s) {
@@ -337,9 +390,11 @@ void transport_stage1(const T* G, const T* vt, const T* gm, const T* wt, const T
   chain(gm ? k_stage<T, true, true> : k_stage<T, false, true>, nblk(N), 256, s, G, vt, gm, wt, y, h, yh, acc, d, N);
 }
 template <typename T>
-void dot_fields(const T* a, const T* b, T* out, int d, long N, cudaStream_t s) {
-  ProfScope ps(KK_STAGE, s, (double)N * sizeof(T) * (2 * d + 1));
-  chain(k_dot_fields<T>, nblk(N), 256, s, a, b, out, d, N);
+void dot_fields(const T* a, const T* b, T* out, int d, long N, int nodes, cudaStream_t s) {
+  ProfScope ps(KK_STAGE, s, (double)nodes * N * sizeof(T) * (2 * d + 1));
+  for (int k = 0; k < nodes; k += 65535)  // grid.y is limited to 65535
+    chain(k_dot_fields<T>, dim3(nblk(N), (unsigned)(nodes - k < 65535 ? nodes - k : 65535)), 256, s, a + (long)k * d * N, b,
+          out + (long)k * N, d, N);
 }
 
 template <typename T>
@@ -348,7 +403,10 @@ void force_acc(T* fhi, T* flo, const ForceNodes<T>& F, int nc, int d, long N, cu
   double fields = 2.0 * nc * d * (flo ? 2 : 1);
   for (int k = 0; k < F.count; ++k) fields += (d + 1) * (1 + (F.yB[k] ? 1 : 0) + (F.yC[k] ? 1 : 0));
   ProfScope ps(KK_FORCE, s, (double)N * sizeof(T) * fields);
-  chain(k_force<T>, nblk(N / 2) * d, 256, s, fhi, flo, F, nc, d, N);
+  const long n = N / Quad<T>::W;
+  // double precision is bound by its unit: more threads up to larger grids
+  if (n * d <= 152L * (sizeof(T) == 8 ? 16384 : 2048)) chain(k_force<T, true>, nblk(n, 128) * d, 128, s, fhi, flo, F, nc, d, N);
+  else chain(k_force<T, false>, nblk(n, 128), 128, s, fhi, flo, F, nc, d, N);
 }
 
 void pair_to_double(const float* hi, const float* lo, double* out, long n, cudaStream_t s) {
@@ -358,7 +416,7 @@ void pair_to_double(const float* hi, const float* lo, double* out, long n, cudaS
 #define INST(T)                                                                                          \
   template void transport_stage1<T>(const T*, const T*, const T*, const T*, const T*, T, T*, T*, int, long, \
                                     cudaStream_t);                                                       \
-  template void dot_fields<T>(const T*, const T*, T*, int, long, cudaStream_t);                             \
+  template void dot_fields<T>(const T*, const T*, T*, int, long, int, cudaStream_t);                             \
   template void force_acc<T>(T*, T*, const ForceNodes<T>&, int, int, long, cudaStream_t);
 INST(float)
 INST(double)

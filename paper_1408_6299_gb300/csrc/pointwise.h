@@ -22,9 +22,9 @@ void convert(const S* in, T* out, long n, cudaStream_t s);
 template <typename T>
 void transport_stage1(const T* G, const T* vt, const T* gm, const T* wt, const T* y, T h, T* yh, T* acc, int d,
                       long N, cudaStream_t s);
-// out = sum_i a_i b_i (d fields at stride N)
+// out_k = sum_i a_{k,i} b_i (d fields at stride N) for `nodes` consecutive groups a_k
 template <typename T>
-void dot_fields(const T* a, const T* b, T* out, int d, long N, cudaStream_t s);
+void dot_fields(const T* a, const T* b, T* out, int d, long N, int nodes, cudaStream_t s);
 // Body force of up to kForceNodes time nodes (see ForceNodes):
 //   f[l][i] += cA_l (yA gA_i + yC gC_i) + cB_l yB gB_i   for every node in order,
 // a plain sum into fhi (flo null) or a compensated (fhi, flo) pair of precision T

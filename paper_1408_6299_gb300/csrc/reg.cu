@@ -662,8 +662,12 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
   }
   if (use_src && c->ckpt == 0) {
     T* src = w.src.get((size_t)(c->n_t + 1) * N);
-    for (int j = 0; j <= c->n_t; ++j)
-      dot_fields<T>(gm_slot<T>(c, j, 0), vt.get(j), src + (long)j * N, c->d, N, c->s);
+    if (c->n_c == 1) {  // one direction for all nodes: one launch
+      dot_fields<T>(gm_slot<T>(c, 0, 0), vt.get(0), src, c->d, N, c->n_t + 1, c->s);
+    } else {
+      for (int j = 0; j <= c->n_t; ++j)
+        dot_fields<T>(gm_slot<T>(c, j, 0), vt.get(j), src + (long)j * N, c->d, N, 1, c->s);
+    }
   }
   if (use_src && c->ckpt > 0 && c->d == 3) {
     // Checkpointed 3D sweep: the state re-advance and the incremental sweep

@@ -290,11 +290,6 @@ Grid make_grid(int d, const int64_t* n, int batch) {
   return g;
 }
 
-bool narrow_lines(long wide_threads) {
-  static const long lim = getenv("REG_NARROW") ? atol(getenv("REG_NARROW")) : 152 * 256;
-  return wide_threads < lim;
-}
-
 long inv_k2_count(const Grid& g) {
   long n = 1;
   for (int a = 0; a < g.d; ++a) n += (long)(g.n[a] / 2) * (g.n[a] / 2);
@@ -398,6 +393,7 @@ void add_launches(long n) { g_launches.fetch_add(n, std::memory_order_relaxed); 
 long launch_count() { return g_launches.load(std::memory_order_relaxed); }
 
 thread_local KernelProfiler* tl_prof = nullptr;
+thread_local bool tl_plain_launch = false;
 
 KernelProfiler::~KernelProfiler() {
   for (auto& r : recs) {

@@ -50,6 +50,19 @@ struct DivEpi {
   const T* src;  // added to the divergence
 };
 
+// Accesses that are not repeated before the next stage: first to leave the
+// caches, so that the differentiated field and the derivative along the second
+// axis, which the next pass reads, stay in L2 (256^3 mixed matvec 176.4 -> 173.8
+// ms, 128^3 FP64 gradient 47.6 -> 45.2 ms).
+template <typename C>
+__device__ __forceinline__ C ld_stream(const C* p) {
+  return __ldcs(p);
+}
+template <typename C>
+__device__ __forceinline__ void st_stream(C* p, C v) {
+  __stcs(p, v);
+}
+
 // Advection epilogue on the point pair q with the gradient components g[0..D)
 // (-a.g [- source], Heun update, optional keep of g or of g.sw). srcv, when
 // given, is the source value instead of e.src. Returns the Sout value.
@@ -62,24 +75,24 @@ __device__ __forceinline__ cx<T> adv_point(const AdvEpi<T>& e, const cx<T>* g, l
   C so = mk<C>(0, 0);
   if (e.G[0]) {
 #pragma unroll
-    for (int f = 0; f < D; ++f) reinterpret_cast<C*>(e.G[f])[q] = g[f];
+    for (int f = 0; f < D; ++f) st_stream(reinterpret_cast<C*>(e.G[f]) + q, g[f]);
   }
   if (e.Sout) {
     T s0 = 0, s1 = 0;
 #pragma unroll
     for (int f = 0; f < D; ++f) {
-      C w = reinterpret_cast<const C*>(e.sw[f])[q];
+      C w = ld_stream(reinterpret_cast<const C*>(e.sw[f]) + q);
       s0 += g[f].x * w.x;
       s1 += g[f].y * w.y;
     }
     so = mk<C>(s0, s1);
-    reinterpret_cast<C*>(e.Sout)[q] = so;
+    st_stream(reinterpret_cast<C*>(e.Sout) + q, so);
   }
   if (!e.out1) return so;
   T k0 = 0, k1 = 0;
 #pragma unroll
   for (int f = 0; f < D; ++f) {
-    C a = av_in ? av_in[f] : reinterpret_cast<const C*>(e.a[f])[q];
+    C a = av_in ? av_in[f] : ld_stream(reinterpret_cast<const C*>(e.a[f]) + q);
     if (av_out) av_out[f] = a;
     k0 -= a.x * g[f].x;
     k1 -= a.y * g[f].y;
@@ -88,14 +101,14 @@ __device__ __forceinline__ cx<T> adv_point(const AdvEpi<T>& e, const cx<T>* g, l
     k0 -= srcv->x;
     k1 -= srcv->y;
   } else if (e.src) {
-    C sv = reinterpret_cast<const C*>(e.src)[q];
+    C sv = ld_stream(reinterpret_cast<const C*>(e.src) + q);
     k0 -= sv.x;
     k1 -= sv.y;
   } else if (e.gm[0]) {
 #pragma unroll
     for (int f = 0; f < D; ++f) {
-      C gm = reinterpret_cast<const C*>(e.gm[f])[q];
-      C w = reinterpret_cast<const C*>(e.w[f])[q];
+      C gm = ld_stream(reinterpret_cast<const C*>(e.gm[f]) + q);
+      C w = ld_stream(reinterpret_cast<const C*>(e.w[f]) + q);
       k0 -= gm.x * w.x;
       k1 -= gm.y * w.y;
     }
@@ -103,11 +116,11 @@ __device__ __forceinline__ cx<T> adv_point(const AdvEpi<T>& e, const cx<T>* g, l
   C r1;
   const T h2 = (T)0.5 * e.h;
   if (e.stage == 1) {
-    C yv = e.y ? reinterpret_cast<const C*>(e.y)[q] : mk<C>(0, 0);
+    C yv = e.y ? ld_stream(reinterpret_cast<const C*>(e.y) + q) : mk<C>(0, 0);
     r1 = mk<C>(yv.x + e.h * k0, yv.y + e.h * k1);
-    reinterpret_cast<C*>(e.out2)[q] = mk<C>(yv.x + h2 * k0, yv.y + h2 * k1);
+    st_stream(reinterpret_cast<C*>(e.out2) + q, mk<C>(yv.x + h2 * k0, yv.y + h2 * k1));
   } else {
-    C yv = reinterpret_cast<const C*>(e.y)[q];
+    C yv = ld_stream(reinterpret_cast<const C*>(e.y) + q);
     r1 = mk<C>(yv.x + h2 * k0, yv.y + h2 * k1);
   }
   reinterpret_cast<C*>(e.out1)[q] = r1;
@@ -120,18 +133,18 @@ template <typename T>
 __device__ __forceinline__ void div_point(const DivEpi<T>& dv, cx<T> k, long q) {
   using C = cx<T>;
   if (dv.src) {
-    C sv = reinterpret_cast<const C*>(dv.src)[q];
+    C sv = ld_stream(reinterpret_cast<const C*>(dv.src) + q);
     k = mk<C>(k.x + sv.x, k.y + sv.y);
   }
   if (dv.stage == 0) {
     reinterpret_cast<C*>(dv.out1)[q] = k;
     return;
   }
-  C yv = reinterpret_cast<const C*>(dv.y)[q];
+  C yv = ld_stream(reinterpret_cast<const C*>(dv.y) + q);
   const T h2 = (T)0.5 * dv.h;
   if (dv.stage == 1) {
     reinterpret_cast<C*>(dv.out1)[q] = mk<C>(yv.x + dv.h * k.x, yv.y + dv.h * k.y);
-    reinterpret_cast<C*>(dv.out2)[q] = mk<C>(yv.x + h2 * k.x, yv.y + h2 * k.y);
+    st_stream(reinterpret_cast<C*>(dv.out2) + q, mk<C>(yv.x + h2 * k.x, yv.y + h2 * k.y));
   } else {
     reinterpret_cast<C*>(dv.out1)[q] = mk<C>(yv.x + h2 * k.x, yv.y + h2 * k.y);
   }
@@ -153,18 +166,20 @@ struct ColJobs {
   int start[kColJobs + 1];  // first block of each job; start[nj] = all blocks
   int nj;
   int n;
+  int stream[kColJobs];  // write out past the cache (axis-0 passes)
 };
 
-// Threads of a block: TS along a line times TC neighbouring lines (128-byte
-// row segments where the block allows it). VAR: 0, or 1 for the other block
-// size the autotuner may choose; both give the same bits.
+// Threads of a block: TS along a line times TC neighbouring lines. VAR: 0, or 1
+// for the other block size the autotuner may choose; both give the same bits.
+// Wide: 128-byte row segments where the block allows it. Narrow: one warp or
+// one line (the most blocks; against four lines 512^2 FP64 transport 6370 ->
+// 4700 us, 128^2 mixed matvec 670 -> 613), or four lines and at least 128 threads.
 template <class A, int L, bool NARROW, int VAR>
 struct ColTile {
   static constexpr int TS = LinePlan<L, NARROW>::TS;
   static constexpr int LINE = L * (int)sizeof(typename A::V);  // shared bytes of a line
-  static constexpr int NT0 = (NARROW ? 64 : (sizeof(typename A::V) == 8 ? 256 : 128)) * (VAR ? (NARROW ? 2 : 1) : 1) /
-                             (VAR && !NARROW ? 2 : 1);
-  static constexpr int MINTC = NARROW ? 4 : (VAR ? 4 : 8);
+  static constexpr int NT0 = NARROW ? (VAR ? 128 : 32) : (sizeof(typename A::V) == 8 ? 256 : 128) / (VAR ? 2 : 1);
+  static constexpr int MINTC = NARROW ? (VAR ? 4 : 1) : (VAR ? 4 : 8);
   static constexpr int TC1 = NT0 / TS < MINTC ? MINTC : NT0 / TS;
   static constexpr int fit(int tc) { return tc * LINE <= 49152 ? tc : fit(tc / 2); }  // 48 KB of shared memory
   static constexpr int TC = fit(TC1);
@@ -180,19 +195,23 @@ __device__ __forceinline__ float4 gmul(float4 a, float4 b) {
 template <class A, typename T, int L, bool NARROW, bool PROD, int VAR>
 __global__ void __launch_bounds__(ColTile<A, L, NARROW, VAR>::NT) k_cols_line(ColJobs<T> J,
                                                                           const typename A::W* __restrict__ tw) {
-  chain_enter(sizeof(T) == 4);
   using Tile = ColTile<A, L, NARROW, VAR>;
   using Ln = Line<A, L, NARROW>;
+  typename A::W pre[Ln::NTW + 1];
+  Ln::preload(pre, threadIdx.x / Tile::TC, tw);
+  const typename A::W* twd = Ln::PRELOAD ? pre : tw;
+  chain_enter(sizeof(T) == 4);
   using V = typename A::V;
   using G = typename A::G;
   constexpr int E = Ln::E, TC = Tile::TC;
   __shared__ V buf[L * TC];
-  int q = 0;
+  int q = 0, tile = blockIdx.x;
 #pragma unroll
   for (int k = 1; k < kColJobs; ++k)
-    if (k < J.nj && (int)blockIdx.x >= J.start[k]) q = k;
+    if (k < J.nj && tile >= J.start[k]) q = k;
+  tile -= J.start[q];
   const int c = threadIdx.x % TC, j = threadIdx.x / TC;
-  const int line = ((int)blockIdx.x - J.start[q]) * TC + c;
+  const int line = tile * TC + c;
   const int ls = J.log2s[q];
   const long s = 1L << ls;
   const long off = ((long)(line >> ls) * L << ls) + (line & (int)(s - 1));
@@ -201,7 +220,8 @@ __global__ void __launch_bounds__(ColTile<A, L, NARROW, VAR>::NT) k_cols_line(Co
   {
     const G* in = reinterpret_cast<const G*>(J.in[q]) + off;
 #pragma unroll
-    for (int e = 0; e < E; ++e) x[e] = ok ? in[Ln::position(j, e) * s] : G{};
+    for (int e = 0; e < E; ++e)
+      x[e] = ok ? (PROD ? ld_stream(in + Ln::position(j, e) * s) : in[Ln::position(j, e) * s]) : G{};
     if constexpr (PROD) {
       const G* mul = reinterpret_cast<const G*>(J.mul[q]) + off;
 #pragma unroll
@@ -220,17 +240,20 @@ __global__ void __launch_bounds__(ColTile<A, L, NARROW, VAR>::NT) k_cols_line(Co
     const FxScale<L, Ln::R0> sc(line_max<TC, Tile::TS>(mag, reinterpret_cast<unsigned*>(buf), c, j));
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = sc.in(x[e]);
-    Ln::derivative(v, j, at, sync, tw);
+    Ln::derivative(v, j, at, sync, twd);
     if (!ok) return;
 #pragma unroll
     for (int e = 0; e < E; ++e) out[Ln::position(j, e) * s] = sc.out(v[e]);
   } else {
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = A::in(x[e]);
-    Ln::derivative(v, j, at, sync, tw);
+    Ln::derivative(v, j, at, sync, twd);
     if (!ok) return;
 #pragma unroll
-    for (int e = 0; e < E; ++e) out[Ln::position(j, e) * s] = A::out(v[e]);
+    for (int e = 0; e < E; ++e) {
+      if (J.stream[q]) st_stream(out + Ln::position(j, e) * s, A::out(v[e]));
+      else out[Ln::position(j, e) * s] = A::out(v[e]);
+    }
   }
 }
 
@@ -250,6 +273,7 @@ struct RowArgs {
   AdvEpi<T> adv, advB;
   DivEpi<T> dv;
   long nrows;
+  int rev;  // blocks take the rows from the last one
 };
 
 // Rows r and r + 1 (r even) form one complex line. A block holds NSEQ lines;
@@ -274,14 +298,17 @@ struct RowTile {
 template <class A, typename T, int L, bool NARROW, int EPI>
 __global__ void __launch_bounds__(RowTile<L, NARROW, EPI>::NT) k_rows_line(RowArgs<T> a,
                                                                             const typename A::W* __restrict__ tw) {
-  chain_enter(sizeof(T) == 4);
   using Tile = RowTile<L, NARROW, EPI>;
   using Ln = Line<A, L, NARROW>;
+  typename A::W pre[Ln::NTW + 1];
+  if (Tile::NFFT == Tile::NT || threadIdx.x < Tile::NFFT) Ln::preload(pre, threadIdx.x % Tile::TS, tw);
+  const typename A::W* twd = Ln::PRELOAD ? pre : tw;
+  chain_enter(sizeof(T) == 4);
   using V = typename A::V;
   using C = cx<T>;
   constexpr int E = Ln::E, TS = Tile::TS, RS = Tile::RS, NF = Tile::NF, M = L / 2;
   __shared__ __align__(16) V buf[Tile::NSEQ * RS];
-  const long row0 = (long)blockIdx.x * Tile::ROWS;
+  const long row0 = (long)(a.rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * Tile::ROWS;
   if (Tile::NFFT == Tile::NT || threadIdx.x < Tile::NFFT) {
     const int seq = threadIdx.x / TS, j = threadIdx.x % TS;
     const long row = row0 + seq / NF * 2;
@@ -316,13 +343,13 @@ __global__ void __launch_bounds__(RowTile<L, NARROW, EPI>::NT) k_rows_line(RowAr
       const FxScale<L, Ln::R0> sc(row_max<TS>(mag, reinterpret_cast<unsigned*>(b), j, sync));
 #pragma unroll
       for (int e = 0; e < E; ++e) v[e] = sc.in(x[e]);
-      Ln::derivative(v, j, at, sync, tw);
+      Ln::derivative(v, j, at, sync, twd);
 #pragma unroll
-      for (int e = 0; e < E; ++e) x[e] = sc.out(v[e]);
+      for (int e = 0; e < E; ++e) x[e] = sc.outi(v[e]);
     } else {
 #pragma unroll
       for (int e = 0; e < E; ++e) v[e] = A::in(x[e]);
-      Ln::derivative(v, j, at, sync, tw);
+      Ln::derivative(v, j, at, sync, twd);
 #pragma unroll
       for (int e = 0; e < E; ++e) x[e] = A::out(v[e]);
     }
@@ -353,21 +380,22 @@ __global__ void __launch_bounds__(RowTile<L, NARROW, EPI>::NT) k_rows_line(RowAr
       return reinterpret_cast<const C*>(ra)[jj];
     };
     auto ld = [&](const T* p) { return reinterpret_cast<const C*>(p)[q]; };
+    auto lds = [&](const T* p) { return ld_stream(reinterpret_cast<const C*>(p) + q); };
     if constexpr (EPI == EPI_ADV2) {
-      const C g[2] = {ld(a.gx[0]), dlast(0)};
+      const C g[2] = {lds(a.gx[0]), dlast(0)};
       adv_point<T, 2>(a.adv, g, q, nullptr);
     } else if constexpr (EPI == EPI_ADV3) {
-      const C g[3] = {ld(a.gx[0]), ld(a.gy[0]), dlast(0)};
+      const C g[3] = {lds(a.gx[0]), ld(a.gy[0]), dlast(0)};
       adv_point<T, 3>(a.adv, g, q, nullptr);
     } else if constexpr (EPI == EPI_ADV33) {
-      const C g[3] = {ld(a.gx[0]), ld(a.gy[0]), dlast(0)};
-      const C h[3] = {ld(a.gx[1]), ld(a.gy[1]), dlast(1)};
+      const C g[3] = {lds(a.gx[0]), ld(a.gy[0]), dlast(0)};
+      const C h[3] = {lds(a.gx[1]), ld(a.gy[1]), dlast(1)};
       C av[3];
       const C sa = adv_point<T, 3>(a.adv, g, q, nullptr, nullptr, av);
       adv_point<T, 3>(a.advB, h, q, a.advB.src_from_a ? &sa : nullptr, a.advB.a_from_a ? av : nullptr);
     } else {
       C k = dlast(0);
-      const C x = ld(a.gx[0]);
+      const C x = lds(a.gx[0]);
       k = mk<C>(k.x + x.x, k.y + x.y);
       if (a.gy[0]) {
         const C y = ld(a.gy[0]);

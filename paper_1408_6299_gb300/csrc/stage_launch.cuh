@@ -1,8 +1,6 @@
 // stage_launch.cuh -- host launchers of the transport stages (stage.cuh),
 // instantiated per precision by the stage_*.cu files.
 #pragma once
-#include <stdlib.h>
-
 #include <type_traits>
 
 #include "stage.cuh"
@@ -51,6 +49,7 @@ void cols_launch(const Spectral<T>& sp, const ColJob<T>* jobs, int nj, cudaStrea
     J.in[q] = jobs[q].in;
     J.mul[q] = jobs[q].mul;
     J.out[q] = jobs[q].out;
+    J.stream[q] = jobs[q].axis == 0;
     J.log2s[q] = ilog2_c((int)(line_stride(g, jobs[q].axis) / A::CW));
     J.start[q] = q * per;
   }
@@ -61,8 +60,9 @@ void cols_launch(const Spectral<T>& sp, const ColJob<T>* jobs, int nj, cudaStrea
         static_cast<const typename A::W*>(sp.line_table(L, NARROW, A::TABLE)));
 }
 
-// Fields up to 16 MB live in L2 between the passes, as in the trials; larger
-// ones stream, which a trial on the same buffers does not show: variant 0.
+// Fields up to 16 MB live in L2 between the passes, as in the trials, and the
+// double-precision passes are bound by arithmetic; larger single-precision
+// fields stream, which a trial on the same buffers does not show: variant 0.
 template <class A, typename T, int L, bool NARROW, bool PROD>
 void cols_tuned(const Spectral<T>& sp, const ColJob<T>* jobs, int nj, cudaStream_t st) {
   auto run = [&](int v) {
@@ -70,7 +70,7 @@ void cols_tuned(const Spectral<T>& sp, const ColJob<T>* jobs, int nj, cudaStream
     else cols_launch<A, T, L, NARROW, PROD, 1>(sp, jobs, nj, st);
   };
   const long n = sp.grid().N;
-  if (n * (long)sizeof(T) > (16 << 20)) return run(0);
+  if (sizeof(T) == 4 && n * (long)sizeof(T) > (16 << 20)) return run(0);
   run(tuned_choice(PROD ? "cols|prod" : "cols|plain", sizeof(T), L, tune_size(n * nj), 2, st, run));
 }
 
@@ -79,37 +79,41 @@ void cols_L(const Spectral<T>& sp, const ColJob<T>* jobs, int nj, cudaStream_t s
   using A = typename Arith<T>::Main;
   const Grid& g = sp.grid();
   const long threads = (long)nj * g.Nc / L * LinePlan<L, false>::TS;
-  if (narrow_lines(threads)) return cols_tuned<A, T, L, true, PROD>(sp, jobs, nj, st);
+  if (narrow_lines(threads, sizeof(T))) return cols_tuned<A, T, L, true, PROD>(sp, jobs, nj, st);
   if constexpr (sizeof(T) == 4)
     if (threads >= 2 * 152 * 512) return cols_tuned<LinePair, T, L, false, PROD>(sp, jobs, nj, st);
   cols_tuned<A, T, L, false, PROD>(sp, jobs, nj, st);
 }
 
-// The column passes of one stage: one launch per distinct axis length.
+// The column passes of one stage: one launch per axis length, side by side
+// where there are two (each fills the other's last wave; 32 x 64 x 128 Newton
+// matvec: 3140 -> 2800 us).
 template <typename T, bool PROD>
-void run_cols(const Spectral<T>& sp, const ColJob<T>* jobs, int nj, cudaStream_t st) {
+void run_cols(Spectral<T>& sp, const ColJob<T>* jobs, int nj, cudaStream_t st) {
   const Grid& g = sp.grid();
-  bool done[kColJobs] = {false};
-  for (int a = 0; a < nj; ++a) {
-    if (done[a]) continue;
-    const int L = g.n[jobs[a].axis];
+  const bool two = nj > 1 && g.n[0] != g.n[1];
+  cudaStream_t st2 = two ? sp.fork() : st;
+  for (int axis = 0; axis < (two ? 2 : 1); ++axis) {
     ColJob<T> grp[kColJobs];
     int m = 0;
-    for (int b = a; b < nj; ++b)
-      if (!done[b] && g.n[jobs[b].axis] == L) {
-        grp[m++] = jobs[b];
-        done[b] = true;
-      }
-    switch (L) {
-      case 8: cols_L<T, 8, PROD>(sp, grp, m, st); break;
-      case 16: cols_L<T, 16, PROD>(sp, grp, m, st); break;
-      case 32: cols_L<T, 32, PROD>(sp, grp, m, st); break;
-      case 64: cols_L<T, 64, PROD>(sp, grp, m, st); break;
-      case 128: cols_L<T, 128, PROD>(sp, grp, m, st); break;
-      case 256: cols_L<T, 256, PROD>(sp, grp, m, st); break;
-      case 512: cols_L<T, 512, PROD>(sp, grp, m, st); break;
+    for (int q = 0; q < nj; ++q)
+      if (!two || jobs[q].axis == axis) grp[m++] = jobs[q];
+    if (two) tl_plain_launch = true;
+    cudaStream_t s = axis ? st2 : st;
+    switch (g.n[axis]) {
+      case 8: cols_L<T, 8, PROD>(sp, grp, m, s); break;
+      case 16: cols_L<T, 16, PROD>(sp, grp, m, s); break;
+      case 32: cols_L<T, 32, PROD>(sp, grp, m, s); break;
+      case 64: cols_L<T, 64, PROD>(sp, grp, m, s); break;
+      case 128: cols_L<T, 128, PROD>(sp, grp, m, s); break;
+      case 256: cols_L<T, 256, PROD>(sp, grp, m, s); break;
+      case 512: cols_L<T, 512, PROD>(sp, grp, m, s); break;
       default: throw StatusError{1, "unsupported axis length"};
     }
+  }
+  if (two) {
+    sp.join();
+    tl_plain_launch = true;
   }
 }
 
@@ -122,10 +126,14 @@ void rows_L(const Spectral<T>& sp, const RowArgs<T>& a, double bytes, cudaStream
     constexpr bool NARROW = decltype(narrow)::value;
     using Tile = RowTile<L, NARROW, EPI>;
     const unsigned grid = (unsigned)((a.nrows + Tile::ROWS - 1) / Tile::ROWS);
-    chain(k_rows_line<A, T, L, NARROW, EPI>, grid, Tile::NT, st, a,
+    RowArgs<T> b = a;
+    // large fields from the last row on: the column pass left its last planes in
+    // L2 (256^3 mixed matvec 158.7 -> 156.3 ms)
+    b.rev = a.nrows * (long)L * sizeof(T) >= (64 << 20);
+    chain(k_rows_line<A, T, L, NARROW, EPI>, grid, Tile::NT, st, b,
           static_cast<const typename A::W*>(sp.line_table(L, NARROW, A::TABLE)));
   };
-  if (narrow_lines(a.nrows / 2 * NF * LinePlan<L, false>::TS)) go(std::true_type{});
+  if (narrow_lines(a.nrows / 2 * NF * LinePlan<L, false>::TS, sizeof(T))) go(std::true_type{});
   else go(std::false_type{});
 }
 
