@@ -3,12 +3,8 @@
 //
 // Heun's RK2 (reading of "explicit second-order Runge-Kutta", Sec. 3.3.1):
 //   k1 = F(t_j, y_j), yh = y_j + h k1, k2 = F(t_{j+1}, yh),
-//   y_{j+1} = y_j + h/2 (k1 + k2) = acc + h/2 k2 with acc = y_j + h/2 k1.
-// The stage kernels below take the spectral derivatives of the current stage
-// input and form the right-hand sides of
-//   state        m'  = -v . grad m                      (Eq. first-order-forward)
-//   incr. state  m~' = -v . grad m~ - grad m . v~        (Eq. gauss-newton)
-// together with the Runge-Kutta combination.
+//   y_{j+1} = y_j + h/2 (k1 + k2) = y_j + ((yh - y_j) + h k2) / 2.
+// The stages themselves are in stage.cuh.
 #include <float.h>
 
 #include <type_traits>
@@ -92,26 +88,16 @@ __global__ void k_convert(const S* __restrict__ in, T* __restrict__ out, long n)
   if (x < n) out[x] = (T)in[x];
 }
 
-// k = -sum_i v_i G_i - [sum_i gm_i w_i]; Heun stage 1 or 2 update.
-template <typename T, bool SRC, bool STAGE1>
-__global__ void k_stage(const T* __restrict__ G, const T* __restrict__ vt, const T* __restrict__ gm,
-                        const T* __restrict__ wt, const T* __restrict__ y, T h, T* __restrict__ yh,
-                        T* __restrict__ acc, int d, long N) {
+// yh = -h sum_i gm_i w_i: the first predictor of the incremental state, from zero
+template <typename T>
+__global__ void k_first_predictor(const T* __restrict__ gm, const T* __restrict__ wt, T h, T* __restrict__ yh, int d,
+                                  long N) {
   chain_enter();
   long x = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= N) return;
   T k = 0;
-  if (G)
-    for (int i = 0; i < d; ++i) k -= vt[i * N + x] * G[i * N + x];
-  if (SRC)
-    for (int i = 0; i < d; ++i) k -= gm[i * N + x] * wt[i * N + x];
-  if (STAGE1) {
-    T yv = y ? y[x] : (T)0;
-    yh[x] = yv + h * k;
-    acc[x] = yv + (T)0.5 * h * k;
-  } else {
-    yh[x] = y[x] + (T)0.5 * h * k;  // y holds acc here; yh is the new state
-  }
+  for (int i = 0; i < d; ++i) k -= gm[i * N + x] * wt[i * N + x];
+  yh[x] = h * k;
 }
 
 // out_k = sum_i a_{k,i} b_i for the nodes k = blockIdx.y
@@ -384,10 +370,9 @@ template void convert<float, double>(const float*, double*, long, cudaStream_t);
 template void convert<double, double>(const double*, double*, long, cudaStream_t);
 
 template <typename T>
-void transport_stage1(const T* G, const T* vt, const T* gm, const T* wt, const T* y, T h, T* yh, T* acc, int d,
-                      long N, cudaStream_t s) {
-  ProfScope ps(KK_STAGE, s, (double)N * sizeof(T) * ((G ? 2 * d : 0) + (gm ? 2 * d : 0) + (y ? 1 : 0) + 2));
-  chain(gm ? k_stage<T, true, true> : k_stage<T, false, true>, nblk(N), 256, s, G, vt, gm, wt, y, h, yh, acc, d, N);
+void first_predictor(const T* gm, const T* wt, T h, T* yh, int d, long N, cudaStream_t s) {
+  ProfScope ps(KK_STAGE, s, (double)N * sizeof(T) * (2 * d + 1));
+  chain(k_first_predictor<T>, nblk(N), 256, s, gm, wt, h, yh, d, N);
 }
 template <typename T>
 void dot_fields(const T* a, const T* b, T* out, int d, long N, int nodes, cudaStream_t s) {
@@ -414,8 +399,7 @@ void pair_to_double(const float* hi, const float* lo, double* out, long n, cudaS
 }
 
 #define INST(T)                                                                                          \
-  template void transport_stage1<T>(const T*, const T*, const T*, const T*, const T*, T, T*, T*, int, long, \
-                                    cudaStream_t);                                                       \
+  template void first_predictor<T>(const T*, const T*, T, T*, int, long, cudaStream_t);                        \
   template void dot_fields<T>(const T*, const T*, T*, int, long, int, cudaStream_t);                             \
   template void force_acc<T>(T*, T*, const ForceNodes<T>&, int, int, long, cudaStream_t);
 INST(float)

@@ -16,12 +16,9 @@ void vel_at(const T* coef, int nc, const Coefs& b, T* out, long dN, cudaStream_t
 template <typename S, typename T>
 void convert(const S* in, T* out, long n, cudaStream_t s);
 
-// Heun stage 1 of m' = -v.G - gm.w (the gm.w source only when gm != null; G may
-// be null for a zero state; y may be null for a zero state):
-//   yh = y + h k, acc = y + h/2 k.
+// yh = -h sum_i gm_i wt_i (d fields at stride N)
 template <typename T>
-void transport_stage1(const T* G, const T* vt, const T* gm, const T* wt, const T* y, T h, T* yh, T* acc, int d,
-                      long N, cudaStream_t s);
+void first_predictor(const T* gm, const T* wt, T h, T* yh, int d, long N, cudaStream_t s);
 // out_k = sum_i a_{k,i} b_i (d fields at stride N) for `nodes` consecutive groups a_k
 template <typename T>
 void dot_fields(const T* a, const T* b, T* out, int d, long N, int nodes, cudaStream_t s);

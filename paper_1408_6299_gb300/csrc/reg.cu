@@ -103,15 +103,15 @@ template <typename T>
 struct Work {
   DBuf<T> gx, gy;          // column derivatives of a stage
   DBuf<T> gx2, gy2;        // and of the second field of a two-field stage
-  DBuf<T> yhS, accS, srcS; // state stage values and one source of the fused forward sweep
+  DBuf<T> yhS, srcS;       // state stage values and one source of the fused forward sweep
   DBuf<T> G, q, va, vb, wa, wb;  // d fields
-  DBuf<T> m, yh, acc, k, lam;    // fields
+  DBuf<T> m, yh, lam;            // fields
   DBuf<T> vcoef, wcoef;          // coefficient vectors in precision T
   DBuf<T> gm, gmh, ck;           // state gradients (all nodes or one segment), stage gradients, checkpoints
   DBuf<T> fhi, flo;              // single precision body force as a compensated pair
   DBuf<T> src;                   // source grad m_j . v~(t_j) per node (all nodes or one segment)
   DBuf<T> lamR, yhR;             // adjoint (and its predictors) of the nodes whose force is pending
-  DBuf<T> mtil, lamN, yh2, acc2, st0, st1, Gt, mR, m1;  // full Newton matvec
+  DBuf<T> mtil, lamN, yh2, st0, st1, Gt, mR, m1;  // full Newton matvec
 };
 
 // A sweep replayed as a CUDA graph. A sweep is hundreds of dependent launches
@@ -304,8 +304,8 @@ struct NodeVel {
 
 // advection stage on u: k = -a.grad u [- gm.w], Heun stage update
 template <typename T>
-void adv(reg_ctx* c, const T* u, const T* a, const T* gm, const T* wv, const T* y, T* out1, T* out2, T* Gkeep,
-         int stage, const T* src = nullptr, const T* sw = nullptr, T* Sout = nullptr) {
+void adv(reg_ctx* c, const T* u, const T* a, const T* gm, const T* wv, const T* y, T* out1, T* Gkeep, int stage,
+         const T* src = nullptr, const T* sw = nullptr, T* Sout = nullptr) {
   Work<T>& w = work<T>(c);
   const long N = c->N();
   fused::AdvEpi<T> e{};
@@ -319,8 +319,8 @@ void adv(reg_ctx* c, const T* u, const T* a, const T* gm, const T* wv, const T* 
   e.src = src;
   e.Sout = Sout;
   e.y = y;
+  e.yh = u;
   e.out1 = out1;
-  e.out2 = out2;
   e.h = (T)c->h();
   e.stage = stage;
   adv_stage<T>(spectral<T>(c), u, e, w.gx.get(N), c->d == 3 ? w.gy.get(N) : nullptr);
@@ -328,7 +328,7 @@ void adv(reg_ctx* c, const T* u, const T* a, const T* gm, const T* wv, const T* 
 
 // epilogue of an advection stage without stored-gradient source terms
 template <typename T>
-fused::AdvEpi<T> adv_epi(reg_ctx* c, const T* a, const T* y, T* out1, T* out2, int stage, const T* src = nullptr,
+fused::AdvEpi<T> adv_epi(reg_ctx* c, const T* a, const T* y, T* out1, int stage, const T* src = nullptr,
                          const T* sw = nullptr, T* Sout = nullptr) {
   const long N = c->N();
   fused::AdvEpi<T> e{};
@@ -340,7 +340,6 @@ fused::AdvEpi<T> adv_epi(reg_ctx* c, const T* a, const T* y, T* out1, T* out2, i
   e.Sout = Sout;
   e.y = y;
   e.out1 = out1;
-  e.out2 = out2;
   e.h = (T)c->h();
   e.stage = stage;
   return e;
@@ -348,8 +347,10 @@ fused::AdvEpi<T> adv_epi(reg_ctx* c, const T* a, const T* y, T* out1, T* out2, i
 
 // two 3D advection stages sharing their passes
 template <typename T>
-void adv2(reg_ctx* c, const T* uA, const fused::AdvEpi<T>& eA, const T* uB, const fused::AdvEpi<T>& eB) {
+void adv2(reg_ctx* c, const T* uA, fused::AdvEpi<T> eA, const T* uB, fused::AdvEpi<T> eB) {
   Work<T>& w = work<T>(c);
+  eA.yh = uA;
+  eB.yh = uB;
   const long N = c->N();
   T* Z[4] = {w.gx.get(N), w.gy.get(N), w.gx2.get(N), w.gy2.get(N)};
   adv2_stage<T>(spectral<T>(c), uA, eA, uB, eB, Z);
@@ -358,19 +359,19 @@ void adv2(reg_ctx* c, const T* uA, const fused::AdvEpi<T>& eA, const T* uB, cons
 // grad u into G (d fields) through the stage passes
 template <typename T>
 void grad_fused(reg_ctx* c, const T* u, T* G) {
-  adv<T>(c, u, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, G, 1);
+  adv<T>(c, u, nullptr, nullptr, nullptr, nullptr, nullptr, G, 1);
 }
 
 // fused divergence stage on lam: k = div(a lam), Heun stage update; e carries
 // the optional body-force accumulation of stage 1
 template <typename T>
-void divh(reg_ctx* c, const T* lam, const T* a, const T* y, T* out1, T* out2, int stage,
+void divh(reg_ctx* c, const T* lam, const T* a, const T* y, T* out1, int stage,
           fused::DivEpi<T> e = fused::DivEpi<T>{}) {
   Work<T>& w = work<T>(c);
   const long N = c->N();
   e.y = y;
+  e.yh = lam;
   e.out1 = out1;
-  e.out2 = out2;
   e.h = (T)c->h();
   e.stage = stage;
   div_stage<T>(spectral<T>(c), lam, a, e, w.gx.get(N), c->d == 3 ? w.gy.get(N) : nullptr);
@@ -389,14 +390,12 @@ void state_steps(reg_ctx* c, const T* vcoef, int j0, int j1, T* gm, T* gmh, int 
   const long N = c->N(), dN = c->dN();
   T* m = w.m.get(N);
   T* yh = w.yh.get(N);
-  T* acc = w.acc.get(N);
   NodeVel<T> v(c, vcoef, w.va, w.vb);
   for (int j = j0; j < j1; ++j) {
     if (ck && c->ckpt > 0 && j % c->ckpt == 0)
       REG_CUDA(cudaMemcpyAsync(ck + (long)(j / c->ckpt) * N, m, N * sizeof(T), cudaMemcpyDeviceToDevice, c->s));
-    adv<T>(c, m, v.get(j), nullptr, nullptr, m, yh, acc, gm ? gm + (long)(j - base) * dN : nullptr, 1);
-    adv<T>(c, yh, v.get(j + 1), nullptr, nullptr, acc, m, nullptr,
-           gmh ? gmh + (long)(j + 1 - base) * dN : nullptr, 2);
+    adv<T>(c, m, v.get(j), nullptr, nullptr, m, yh, gm ? gm + (long)(j - base) * dN : nullptr, 1);
+    adv<T>(c, yh, v.get(j + 1), nullptr, nullptr, m, m, gmh ? gmh + (long)(j + 1 - base) * dN : nullptr, 2);
   }
   if (ck && c->ckpt > 0 && j1 % c->ckpt == 0)
     REG_CUDA(cudaMemcpyAsync(ck + (long)(j1 / c->ckpt) * N, m, N * sizeof(T), cudaMemcpyDeviceToDevice, c->s));
@@ -423,15 +422,14 @@ void recompute_segment_src(reg_ctx* c, const T* vcoef, const T* wcoef, int j0, i
   const long N = c->N();
   T* m = w.m.get(N);
   T* yh = w.yh.get(N);
-  T* acc = w.acc.get(N);
   NodeVel<T> v(c, vcoef, w.va, w.vb), vt(c, wcoef, w.wa, w.wb);
   T* src = w.src.get((size_t)(c->ckpt + 1) * N);
   REG_CUDA(cudaMemcpyAsync(m, w.ck.p + (long)(j0 / c->ckpt) * N, N * sizeof(T), cudaMemcpyDeviceToDevice, c->s));
   for (int j = j0; j < j1; ++j) {
-    adv<T>(c, m, v.get(j), nullptr, nullptr, m, yh, acc, nullptr, 1, nullptr, vt.get(j), src + (long)(j - j0) * N);
-    adv<T>(c, yh, v.get(j + 1), nullptr, nullptr, acc, m, nullptr, nullptr, 2);
+    adv<T>(c, m, v.get(j), nullptr, nullptr, m, yh, nullptr, 1, nullptr, vt.get(j), src + (long)(j - j0) * N);
+    adv<T>(c, yh, v.get(j + 1), nullptr, nullptr, m, m, nullptr, 2);
   }
-  adv<T>(c, m, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 1, nullptr, vt.get(j1), src + (long)(j1 - j0) * N);
+  adv<T>(c, m, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 1, nullptr, vt.get(j1), src + (long)(j1 - j0) * N);
 }
 
 // Gradient slots available for node j (after ensure_segment)
@@ -529,7 +527,6 @@ void adjoint_solve(reg_ctx* c, const T* vcoef, double* f) {
   Work<T>& w = work<T>(c);
   const long N = c->N();
   const double hd = c->h();
-  T* acc = w.acc.get(N);
   T* ring = w.lamR.get((size_t)(kForceNodes + 1) * N);
   T* yhs = c->quad ? w.yhR.get((size_t)(kForceNodes + 1) * N) : w.yh.get(N);
   BodyForce<T> bf(c, f);
@@ -548,8 +545,8 @@ void adjoint_solve(reg_ctx* c, const T* vcoef, double* f) {
     for (int j = j1 - 1; j >= j0; --j) {
       T* yh = c->quad ? ring_slot(yhs, k, N) : yhs;
       T* next = ring_slot(ring, k++, N);
-      divh<T>(c, lam, v.get(j + 1), lam, yh, acc, 1);
-      divh<T>(c, yh, v.get(j), acc, next, nullptr, 2);
+      divh<T>(c, lam, v.get(j + 1), lam, yh, 1);
+      divh<T>(c, yh, v.get(j), lam, next, 2);
       if (!c->quad) {
         bf.add(lam, gm_slot<T>(c, j + 1, base), j + 1, c->trap_w(j + 1));
       } else {
@@ -577,9 +574,7 @@ void newton_adjoint(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
   const long N = c->N(), dN = c->dN();
   const size_t slots = kForceNodes + 1;
   T* yh = w.yh.get(N);
-  T* acc = w.acc.get(N);
   T* yh2 = w.yh2.get(N);
-  T* acc2 = w.acc2.get(N);
   T* sA = w.st0.get(N);
   T* sB = w.st1.get(N);
   T* ringT = w.lamR.get(slots * N);  // lam~
@@ -593,7 +588,7 @@ void newton_adjoint(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
   lincomb_t<T>((T)1, w.mR.p, (T)-1, w.m1.p, lam1, N, c->s);
   const T* lam = lam1;
   NodeVel<T> vt(c, wcoef, w.wa, w.wb);
-  divh<T>(c, lam, vt.get(c->n_t), nullptr, sB, nullptr, 0);
+  divh<T>(c, lam, vt.get(c->n_t), nullptr, sB, 0);
   int k = 0;
   const int K = c->ckpt > 0 ? c->ckpt : c->n_t;
   for (int seg = (c->n_t - 1) / K; seg >= 0; --seg) {
@@ -618,16 +613,16 @@ void newton_adjoint(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
       fused::DivEpi<T> e{};
       e.src = sB;
       const T* vB = v.get(j + 1);
-      divh<T>(c, lt, vB, lt, yh, acc, 1, e);
+      divh<T>(c, lt, vB, lt, yh, 1, e);
       // adjoint step lam_{j+1} -> lam_j
-      divh<T>(c, lam, vB, lam, yh2, acc2, 1);
+      divh<T>(c, lam, vB, lam, yh2, 1);
       const T* vA = v.get(j);
-      divh<T>(c, yh2, vA, acc2, lam2, nullptr, 2);
+      divh<T>(c, yh2, vA, lam, lam2, 2);
       // source at t_j, then incremental stage 2
-      divh<T>(c, lam2, vt.get(j), nullptr, sA, nullptr, 0);
+      divh<T>(c, lam2, vt.get(j), nullptr, sA, 0);
       fused::DivEpi<T> e2{};
       e2.src = sA;
-      divh<T>(c, yh, vA, acc, lt2, nullptr, 2, e2);
+      divh<T>(c, yh, vA, lt, lt2, 2, e2);
       std::swap(sA, sB);  // the source at t_j is the next step's source at t_{j+1}
       lt = lt2;
       lam = lam2;
@@ -651,7 +646,7 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
   const T h = (T)c->h();
   T* y = w.lam.get(N);  // the incremental state ends up as -lam~_1 in place
   T* yh = w.yh.get(N);
-  T* acc = w.acc.get(N);
+  REG_CUDA(cudaMemsetAsync(y, 0, N * sizeof(T), c->s));
   NodeVel<T> v(c, vcoef, w.va, w.vb), vt(c, wcoef, w.wa, w.wb);
   const bool use_src = !c->quad;
   const int K = c->ckpt > 0 ? c->ckpt : c->n_t;
@@ -678,7 +673,6 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
     // stage 1 of step j (source s_j, kept in one field).
     T* m = w.m.get(N);
     T* yhS = w.yhS.get(N);
-    T* accS = w.accS.get(N);
     T* sj = w.srcS.get(N);
     for (int seg = 0; seg * K < c->n_t; ++seg) {
       const int j0 = seg * K, j1 = j0 + K;
@@ -687,11 +681,11 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
       for (int j = j0; j < j1; ++j) {
         const T* vA = v.get(j);
         const T* wA = vt.get(j);
-        fused::AdvEpi<T> sA = adv_epi<T>(c, vA, m, yhS, accS, 1, nullptr, wA, sj);
+        fused::AdvEpi<T> sA = adv_epi<T>(c, vA, m, yhS, 1, nullptr, wA, sj);
         if (j == 0) {
-          adv<T>(c, m, vA, nullptr, nullptr, m, yhS, accS, nullptr, 1, nullptr, wA, sj);
+          adv<T>(c, m, vA, nullptr, nullptr, m, yhS, nullptr, 1, nullptr, wA, sj);
         } else {
-          fused::AdvEpi<T> iB = adv_epi<T>(c, vA, acc, y, nullptr, 2);
+          fused::AdvEpi<T> iB = adv_epi<T>(c, vA, y, y, 2);
           iB.src_from_a = 1;
           adv2<T>(c, m, sA, yh, iB);
           if (mtil)
@@ -699,21 +693,20 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
         }
         const T* vB = v.get(j + 1);
         if (j == 0) {
-          adv<T>(c, yhS, vB, nullptr, nullptr, accS, m, nullptr, nullptr, 2);
+          adv<T>(c, yhS, vB, nullptr, nullptr, m, m, nullptr, 2);
           lincomb_t<T>(-h, sj, (T)0, nullptr, yh, N, c->s);
-          lincomb_t<T>((T)(-0.5) * h, sj, (T)0, nullptr, acc, N, c->s);
         } else {
-          fused::AdvEpi<T> sB = adv_epi<T>(c, vB, accS, m, nullptr, 2);
-          fused::AdvEpi<T> iA = adv_epi<T>(c, vA, y, yh, acc, 1, sj);
+          fused::AdvEpi<T> sB = adv_epi<T>(c, vB, m, m, 2);
+          fused::AdvEpi<T> iA = adv_epi<T>(c, vA, y, yh, 1, sj);
           adv2<T>(c, yhS, sB, y, iA);
         }
       }
     }
     // the source at t_{n_t} from the final state, and the last incremental stage 2
     const T* vN = v.get(c->n_t);
-    fused::AdvEpi<T> sN = adv_epi<T>(c, nullptr, nullptr, nullptr, nullptr, 1, nullptr, vt.get(c->n_t),
+    fused::AdvEpi<T> sN = adv_epi<T>(c, nullptr, nullptr, nullptr, 1, nullptr, vt.get(c->n_t),
                                      sj);
-    fused::AdvEpi<T> iN = adv_epi<T>(c, vN, acc, y, nullptr, 2);
+    fused::AdvEpi<T> iN = adv_epi<T>(c, vN, y, y, 2);
     iN.src_from_a = 1;
     adv2<T>(c, m, sN, yh, iN);
     if (mtil)
@@ -735,11 +728,10 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
         const T* s2 = w.src.p + (long)(j + 1 - base) * N;
         if (j == 0) {  // zero state: k1 = -s_0
           lincomb_t<T>(-h, s1, (T)0, nullptr, yh, N, c->s);
-          lincomb_t<T>((T)(-0.5) * h, s1, (T)0, nullptr, acc, N, c->s);
         } else {
-          adv<T>(c, y, v.get(j), nullptr, nullptr, y, yh, acc, nullptr, 1, s1);
+          adv<T>(c, y, v.get(j), nullptr, nullptr, y, yh, nullptr, 1, s1);
         }
-        adv<T>(c, yh, v.get(j + 1), nullptr, nullptr, acc, y, nullptr, nullptr, 2, s2);
+        adv<T>(c, yh, v.get(j + 1), nullptr, nullptr, y, y, nullptr, 2, s2);
         if (mtil)
           REG_CUDA(cudaMemcpyAsync(mtil + (long)(j + 1) * N, y, N * sizeof(T), cudaMemcpyDeviceToDevice, c->s));
       } else {
@@ -747,11 +739,11 @@ void gn_sweeps(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
         const T* g2 = gmh_slot<T>(c, j + 1, base);
         const T* wA = vt.get(j);
         if (j == 0) {
-          transport_stage1<T>(nullptr, v.get(j), g1, wA, nullptr, h, yh, acc, c->d, N, c->s);
+          first_predictor<T>(g1, wA, h, yh, c->d, N, c->s);
         } else {
-          adv<T>(c, y, v.get(j), g1, wA, y, yh, acc, nullptr, 1);
+          adv<T>(c, y, v.get(j), g1, wA, y, yh, nullptr, 1);
         }
-        adv<T>(c, yh, v.get(j + 1), g2, vt.get(j + 1), acc, y, nullptr, nullptr, 2);
+        adv<T>(c, yh, v.get(j + 1), g2, vt.get(j + 1), y, y, nullptr, 2);
       }
     }
   }
@@ -817,16 +809,15 @@ double reg_term(reg_ctx* c, const double* v) {
 // would read or write stale memory and must be captured again
 size_t graph_signature(reg_ctx* c) {
   const void* ptrs[] = {c->f.p,        c->SV.p,       c->SF.p,       c->vlin.p,     c->gdir.p,     c->vfix.p,
-                        c->w64.gx.p,   c->w64.gy.p,    c->w64.m.p,    c->w64.yh.p,   c->w64.acc.p,
+                        c->w64.gx.p,   c->w64.gy.p,    c->w64.m.p,    c->w64.yh.p, 
                         c->w64.lam.p,  c->w64.va.p,   c->w64.vb.p,   c->w64.wa.p,   c->w64.wb.p,   c->w64.gm.p,
                         c->w64.gmh.p,  c->w64.ck.p,   c->w32.gx.p,   c->w32.gy.p,    c->w32.m.p,
-                        c->w32.yh.p,   c->w32.acc.p,  c->w32.lam.p,  c->w32.va.p,   c->w32.vb.p,   c->w32.wa.p,
+                        c->w32.yh.p,   c->w32.lam.p,  c->w32.va.p,   c->w32.vb.p,   c->w32.wa.p,
                         c->w32.wb.p,   c->w32.gm.p,   c->w32.gmh.p,  c->w32.ck.p,   c->w32.vcoef.p, c->w32.wcoef.p,
                         c->w32.fhi.p,  c->w32.flo.p,  c->w64.G.p,    c->w32.G.p,    c->w64.src.p,  c->w32.src.p,
-                        c->w64.mtil.p, c->w32.mtil.p, c->w64.lamN.p, c->w32.lamN.p, c->w64.yh2.p, c->w32.yh2.p,
-                        c->w64.acc2.p, c->w32.acc2.p, c->w64.st0.p,  c->w32.st0.p,  c->w64.st1.p,  c->w32.st1.p,
+                        c->w64.mtil.p, c->w32.mtil.p, c->w64.lamN.p, c->w32.lamN.p, c->w64.yh2.p, c->w32.yh2.p,  c->w64.st0.p,  c->w32.st0.p,  c->w64.st1.p,  c->w32.st1.p,
                         c->w64.Gt.p,   c->w32.Gt.p,   c->w64.gx2.p,  c->w32.gx2.p,  c->w64.gy2.p,  c->w32.gy2.p,
-                        c->w64.yhS.p,  c->w32.yhS.p,  c->w64.accS.p, c->w32.accS.p,
+                        c->w64.yhS.p,  c->w32.yhS.p, 
                         c->w64.srcS.p, c->w32.srcS.p, c->w64.lamR.p, c->w32.lamR.p, c->w64.yhR.p,  c->w32.yhR.p};
   size_t h = 1469598103934665603ull;
   for (const void* p : ptrs) h = (h ^ (size_t)p) * 1099511628211ull;
@@ -1107,7 +1098,6 @@ void displacement(reg_ctx* c, const double* v, double* u) {
   Work<double>& w = c->w64;
   const long N = c->N(), dN = c->dN();
   double* yh = w.yh.get(N);
-  double* acc = w.acc.get(N);
   NodeVel<double> nv(c, v, w.va, w.vb);
   double* s1 = c->disp_src.get(2 * N);
   double* s2 = s1 + N;
@@ -1119,8 +1109,8 @@ void displacement(reg_ctx* c, const double* v, double* u) {
       double* ui = u + (long)i * N;
       lincomb_t<double>(-1.0, vA + (long)i * N, 0.0, nullptr, s1, N, c->s);
       lincomb_t<double>(-1.0, vB + (long)i * N, 0.0, nullptr, s2, N, c->s);
-      adv<double>(c, ui, vA, nullptr, nullptr, ui, yh, acc, nullptr, 1, s1);
-      adv<double>(c, yh, vB, nullptr, nullptr, acc, ui, nullptr, nullptr, 2, s2);
+      adv<double>(c, ui, vA, nullptr, nullptr, ui, yh, nullptr, 1, s1);
+      adv<double>(c, yh, vB, nullptr, nullptr, ui, ui, nullptr, 2, s2);
     }
   }
 }

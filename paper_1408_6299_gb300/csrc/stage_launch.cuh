@@ -157,7 +157,7 @@ template <typename T>
 int adv_fields(const AdvEpi<T>& e, int d, const T* u) {
   int n = (e.G[0] ? d : 0) + (e.Sout ? d + 1 : 0);
   if (e.out1)
-    n += d + (e.src ? 1 : (e.gm[0] && !e.src_from_a ? 2 * d : 0)) + (e.y && e.y != u ? 1 : 0) + (e.stage == 1 ? 2 : 1);
+    n += d + (e.src ? 1 : (e.gm[0] && !e.src_from_a ? 2 * d : 0)) + (e.y && e.y != u ? 1 : 0) + 1;
   return n;
 }
 
@@ -222,7 +222,7 @@ void div_stage_impl(Spectral<T>& sp, const T* lam, const T* a, const DivEpi<T>& 
   r.gy[0] = g.d == 3 ? ky : nullptr;
   r.dv = e;
   r.nrows = g.rows;
-  const double f = 2 + g.d - 1 + (e.stage && e.y != lam ? 1 : 0) + (e.stage == 1 ? 2 : 1) + (e.src ? 1 : 0);
+  const double f = 2 + g.d - 1 + (e.stage && e.y != lam ? 1 : 0) + 1 + (e.src ? 1 : 0);
   run_rows<T, EPI_DIV>(sp, r, f * N * sizeof(T), s);
 }
 
