@@ -5,9 +5,9 @@
 // waits on the host for every inner product. reg_solve_batched therefore runs
 // the pairs concurrently: worker threads, each driving its own CUDA stream,
 // take pairs from a shared queue (largest first) and solve them with contexts
-// cached per configuration. Contexts with their own stream replay the Hessian
-// matvec as a captured CUDA graph, so a small pair's matvec costs one graph
-// launch instead of a few hundred kernel launches.
+// cached per configuration. A context replays its sweeps as CUDA graphs, so a
+// small pair's matvec costs one graph launch instead of a few hundred kernel
+// launches.
 #include <algorithm>
 #include <cstring>
 #include <string>

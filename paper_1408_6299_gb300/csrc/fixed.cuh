@@ -201,10 +201,6 @@ struct FxScale {
   // Conversions in integer arithmetic: the double-precision unit converts two
   // values per clock and SM, and the epilogues need it. Rounded to nearest.
   __device__ __forceinline__ long long in1(double x) const {
-    if (!plain) {
-      if (pre == 0.0) return 0;
-      x *= pre;
-    }
     const int hi = __double2hiint(x);
     const unsigned lo = (unsigned)__double2loint(x);
     // the 53-bit significand times 2^10, shifted right by r >= 1; r counts up for smaller values
@@ -215,12 +211,12 @@ struct FxScale {
     const long long sign = (long long)(hi >> 31);
     return (long long)(v ^ (unsigned long long)sign) - sign;
   }
+  // on the double-precision unit: one conversion and an exponent shift
   __device__ __forceinline__ double out1(long long r) const {
     const double d = __ll2double_rn(r);
-    double x = r == 0 ? 0.0 : __hiloint2double(__double2hiint(d) + down, __double2loint(d));
-    if (!plain) x *= post;
-    return x;
+    return r == 0 ? 0.0 : __hiloint2double(__double2hiint(d) + down, __double2loint(d));
   }
+  // on the integer units
   __device__ __forceinline__ double out1i(long long r) const {
     const long long sign = r >> 63;
     const unsigned long long a = (unsigned long long)((r ^ sign) - sign);
@@ -229,9 +225,7 @@ struct FxScale {
     const unsigned long long n = ((a << lz) >> 1) + 0x200;
     const unsigned hi = (unsigned)(n >> 42) + (unsigned)((1085 - lz) * (1 << 20) + down);
     const unsigned lo = __funnelshift_r((unsigned)n, (unsigned)(n >> 32), 10);
-    double x = r == 0 ? 0.0 : __hiloint2double((int)(hi | ((unsigned)(sign >> 32) & 0x80000000u)), (int)lo);
-    if (!plain) x *= post;
-    return x;
+    return r == 0 ? 0.0 : __hiloint2double((int)(hi | ((unsigned)(sign >> 32) & 0x80000000u)), (int)lo);
   }
   // A line whose sum of magnitudes l1 (see fx_l1) is far below L times its
   // largest value, as the lines of a decaying spectrum are: no partial sum
@@ -250,10 +244,30 @@ struct FxScale {
   }
   // results times 2^n as well
   __device__ __forceinline__ void times_pow2(int n) { down += n * (1 << 20); }
-  __device__ __forceinline__ FxV in(double2 x) const { return {in1(x.x), in1(x.y)}; }
-  // the conjugate of z, scaled back; out converts on the double-precision unit, outi on the integer one
-  __device__ __forceinline__ double2 out(FxV z) const { return make_double2(out1(z.x), out1(-z.y)); }
-  __device__ __forceinline__ double2 outi(FxV z) const { return make_double2(out1i(z.x), out1i(-z.y)); }
+  // v = x scaled, for the E values a thread holds of the line
+  template <int E>
+  __device__ __forceinline__ void in(const double2 (&x)[E], FxV (&v)[E]) const {
+    if (plain) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) v[e] = {in1(x[e].x), in1(x[e].y)};
+    } else {
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        v[e] = pre == 0.0 ? FxV{0, 0} : FxV{in1(x[e].x * pre), in1(x[e].y * pre)};
+    }
+  }
+  __device__ __forceinline__ double back(long long r) const { return plain ? out1(r) : out1(r) * post; }
+  // x = the conjugate of v, scaled back; INT: on the integer units
+  template <bool INT, int E>
+  __device__ __forceinline__ void out(const FxV (&v)[E], double2 (&x)[E]) const {
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+      x[e] = INT ? make_double2(out1i(v[e].x), out1i(-v[e].y)) : make_double2(out1(v[e].x), out1(-v[e].y));
+    if (!plain) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) x[e] = make_double2(x[e].x * post, x[e].y * post);
+    }
+  }
 };
 
 }  // namespace reg

@@ -40,9 +40,9 @@ struct StatusError {
 // bracketing of launches by kind (enabled per context through the C ABI).
 // ---------------------------------------------------------------------------
 enum KernelKind {
-  KK_ROWS_R2C = 0,  // real-to-complex row pass
-  KK_ROWS_C2R = 1,  // complex-to-real row pass
-  KK_COLS = 2,      // strided complex pass
+  KK_ROWS_R2C = 0,  // real-to-complex rows of whole-field transforms
+  KK_ROWS_C2R = 1,  // row pass of a stage with its epilogue, or complex-to-real rows
+  KK_COLS = 2,      // strided pass
   KK_MULT = 3,      // Fourier multipliers
   KK_STAGE = 4,     // Heun stage / transport right-hand side
   KK_FORCE = 5,     // body-force accumulation
@@ -155,12 +155,12 @@ class LineTables {
 size_t write_wide_tables(unsigned char* out, long* off);
 
 // Whether lines that take so many threads on the wide plan run the narrow one
-// (line.cuh) instead: below two warps (single precision: four) per scheduler
-// of the 152 SMs, where a pass lasts as long as one thread's serial work. Both
-// sides measured: 128^2 gradient 5600 us wide, 2170 narrow; 128^3 gradient 42.7
-// ms wide, 61.9 narrow; 128^3 mixed matvec, checkpoints every 8: 16.5 ms at the
-// lower limit for both precisions, 12.6 at this one, 14.1 at twice this one.
-inline bool narrow_lines(long wide_threads, int size) { return wide_threads < 152L * (size == 8 ? 256 : 512); }
+// (line.cuh) instead. Wide lines hold the fewest operations, narrow ones
+// shorter serial work per thread and fewer registers. Measured: 128^2 FP64
+// gradient 5600 us wide, 2170 narrow; 128^3 FP64 gradient 42.7 ms wide, 38.4
+// narrow; 128^3 mixed matvec, checkpoints every 8, 16.5 ms with this limit at
+// half, 12.6 here, 14.1 at double; 256^3 mixed matvec 180 ms wide, 246 narrow.
+inline bool narrow_lines(long wide_threads, int size) { return wide_threads < 152L * (size == 8 ? 1024 : 512); }
 
 // A grid with its stream and line tables in precision T: what the stages run on.
 template <typename T>

@@ -246,24 +246,23 @@ struct Line {
   static constexpr int E = P::E, TS = P::TS, S = P::S;
   static constexpr int R0 = P::R(0), Q0 = L / R0;
 
-  // Twiddles a thread uses in derivative(), in the order of use: forward stages
-  // s >= 1, then inverse ones. Narrow kernels load them into registers before
-  // they wait for their predecessor: a stage would otherwise begin with a miss
-  // to L2, as L1 is empty when a kernel starts.
+  // Narrow kernels load a thread's forward twiddles into registers before they
+  // wait for their predecessor, and the inverse ones ahead of the inverse
+  // stages: a stage would otherwise begin with a miss to L2, as L1 is empty when
+  // a kernel starts (128^2 mixed matvec 680 -> 613 us, 512^2 FP64 transport 4913
+  // -> 4709). Order: stages s >= 1 of one direction.
   static constexpr bool PRELOAD = NARROW;
   __host__ __device__ static constexpr int tw_index(int s, bool inv) {
     int n = 0;
-    for (int b = 0; b < 2; ++b)
-      for (int t = 1; t < S; ++t) {
-        if ((inv ? 1 : 0) == b && t == s) return n;
-        const int R = b ? P::R(S - 1 - t) : P::R(t);
-        n += E / R * (R - 1);
-      }
+    for (int t = 1; t < s; ++t) {
+      const int R = inv ? P::R(S - 1 - t) : P::R(t);
+      n += E / R * (R - 1);
+    }
     return n;
   }
-  static constexpr int NTW = PRELOAD ? tw_index(S, true) : 0;
+  static constexpr int NTW = PRELOAD ? tw_index(S, false) : 0;
   template <int s, bool INV>
-  static __device__ __forceinline__ void load_stage(W* w, int j, const W* __restrict__ tw) {
+  static __device__ __forceinline__ void load_stages(W* w, int j, const W* __restrict__ tw) {
     if constexpr (s < S) {
       constexpr int R = line_radix<P>(s, INV), NS = line_ns<P>(s, INV), TK = E / R;
       const W* t0 = tw + line_tw_offset<P>(s, INV);
@@ -272,14 +271,11 @@ struct Line {
 #pragma unroll
         for (int r = 1; r < R; ++r)
           w[tw_index(s, INV) + i * (R - 1) + r - 1] = __ldg(&t0[r * NS + ((j + i * TS) & (NS - 1))]);
-      load_stage<s + 1, INV>(w, j, tw);
+      load_stages<s + 1, INV>(w, j, tw);
     }
   }
   static __device__ __forceinline__ void preload(W* w, int j, const W* __restrict__ tw) {
-    if constexpr (PRELOAD) {
-      load_stage<1, false>(w, j, tw);
-      load_stage<1, true>(w, j, tw);
-    }
+    if constexpr (PRELOAD) load_stages<1, false>(w, j, tw);
   }
 
   // position of v[i * R0 + r]
@@ -338,13 +334,16 @@ struct Line {
     stages<0, false, false>(v, j, buf, sync, scaled ? tw : tw + line_tw_block<P>(false) + line_tw_block<P>(true), scaled);
   }
 
-  // tw: the table, or the array preload() filled (PRELOAD plans)
+  // pre: what preload() filled (PRELOAD plans)
   template <class Buf, class Sync>
-  static __device__ __forceinline__ void derivative(V* v, int j, const Buf& buf, const Sync& sync, const W* tw) {
-    stages<0, false, PRELOAD>(v, j, buf, sync, tw);
+  static __device__ __forceinline__ void derivative(V* v, int j, const Buf& buf, const Sync& sync,
+                                                    const W* __restrict__ tw, const W* pre) {
+    stages<0, false, PRELOAD>(v, j, buf, sync, PRELOAD ? pre : tw);
+    W inv[PRELOAD ? tw_index(S, true) + 1 : 1];
+    if constexpr (PRELOAD) load_stages<1, true>(inv, j, tw);
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = A::template deriv<L>(v[e], frequency(j, e));
-    stages<0, true, PRELOAD>(v, j, buf, sync, tw);
+    stages<0, true, PRELOAD>(v, j, buf, sync, PRELOAD ? inv : tw);
   }
 };
 

@@ -208,7 +208,6 @@ __global__ void __launch_bounds__(ColTile<A, L, NARROW, VAR>::NT) k_cols_line(Co
   using Ln = Line<A, L, NARROW>;
   typename A::W pre[Ln::NTW + 1];
   Ln::preload(pre, threadIdx.x / Tile::TC, tw);
-  const typename A::W* twd = Ln::PRELOAD ? pre : tw;
   chain_enter(sizeof(T) == 4);
   using V = typename A::V;
   using G = typename A::G;
@@ -247,16 +246,16 @@ __global__ void __launch_bounds__(ColTile<A, L, NARROW, VAR>::NT) k_cols_line(Co
 #pragma unroll
     for (int e = 0; e < E; ++e) mag = max(mag, fx_mag(x[e]));
     const FxScale<L, Ln::R0> sc(line_max<TC, Tile::TS>(mag, reinterpret_cast<unsigned*>(buf), c, j));
-#pragma unroll
-    for (int e = 0; e < E; ++e) v[e] = sc.in(x[e]);
-    Ln::derivative(v, j, at, sync, twd);
+    sc.in(x, v);
+    Ln::derivative(v, j, at, sync, tw, pre);
     if (!ok) return;
+    sc.template out<NARROW>(v, x);
 #pragma unroll
-    for (int e = 0; e < E; ++e) out[Ln::position(j, e) * s] = sc.out(v[e]);
+    for (int e = 0; e < E; ++e) out[Ln::position(j, e) * s] = x[e];
   } else {
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = A::in(x[e]);
-    Ln::derivative(v, j, at, sync, twd);
+    Ln::derivative(v, j, at, sync, tw, pre);
     if (!ok) return;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
@@ -285,33 +284,34 @@ struct RowArgs {
   int rev;  // blocks take the rows from the last one
 };
 
-// Rows r and r + 1 (r even) form one complex line. A block holds NSEQ lines;
-// a wide line lives in one warp, which also runs the epilogue of its rows, so
-// the warps never wait for one another. A narrow block transforms one or a few
-// lines with part of its threads and spreads their epilogue over all of them.
-template <int L, bool NARROW, int EPI>
+// Rows r and r + 1 (r even) form one complex line; a block holds NSEQ of them.
+// FEW (narrow plans): one or two lines per block, transformed by part of its
+// threads and their epilogue spread over all of them: the shortest pass where
+// lines are few. Else every thread transforms, and a line that fits a warp stays in
+// it with the epilogue of its rows, so the warps never wait for one another.
+template <int L, bool NARROW, bool FEW, int EPI>
 struct RowTile {
   using P = LinePlan<L, NARROW>;
   static constexpr int TS = P::TS;
   static constexpr int NF = EPI == EPI_ADV33 ? 2 : 1;
   static constexpr int MINSEQ = 32 / TS > NF ? 32 / TS : NF;
-  static constexpr int NSEQ = NARROW ? MINSEQ : 128 / TS;
+  static constexpr int FULLSEQ = 128 / TS > NF ? 128 / TS : NF;
+  static constexpr int NSEQ = FEW ? MINSEQ : FULLSEQ;
   static constexpr int NFFT = NSEQ * TS;  // transforming threads
   static constexpr int NT = NFFT > 128 ? NFFT : 128;
-  static constexpr bool WARP = !NARROW && 32 / TS >= NF;  // each warp alone
+  static constexpr bool WARP = !FEW && 32 / TS >= NF;  // each warp alone
   static constexpr int PADSH = P::R(0) == 16 ? 4 : (P::R(0) == 8 ? 3 : 2);
   static constexpr int RS = (L + (L >> PADSH) + 1) / 2 * 2;
   static constexpr int ROWS = NSEQ / NF * 2;  // rows of one field per block
 };
 
-template <class A, typename T, int L, bool NARROW, int EPI>
-__global__ void __launch_bounds__(RowTile<L, NARROW, EPI>::NT) k_rows_line(RowArgs<T> a,
-                                                                            const typename A::W* __restrict__ tw) {
-  using Tile = RowTile<L, NARROW, EPI>;
+template <class A, typename T, int L, bool NARROW, bool FEW, int EPI>
+__global__ void __launch_bounds__(RowTile<L, NARROW, FEW, EPI>::NT) k_rows_line(RowArgs<T> a,
+                                                                                 const typename A::W* __restrict__ tw) {
+  using Tile = RowTile<L, NARROW, FEW, EPI>;
   using Ln = Line<A, L, NARROW>;
   typename A::W pre[Ln::NTW + 1];
   if (Tile::NFFT == Tile::NT || threadIdx.x < Tile::NFFT) Ln::preload(pre, threadIdx.x % Tile::TS, tw);
-  const typename A::W* twd = Ln::PRELOAD ? pre : tw;
   chain_enter(sizeof(T) == 4);
   using V = typename A::V;
   using C = cx<T>;
@@ -350,15 +350,13 @@ __global__ void __launch_bounds__(RowTile<L, NARROW, EPI>::NT) k_rows_line(RowAr
 #pragma unroll
       for (int e = 0; e < E; ++e) mag = max(mag, fx_mag(x[e]));
       const FxScale<L, Ln::R0> sc(row_max<TS>(mag, reinterpret_cast<unsigned*>(b), j, sync));
-#pragma unroll
-      for (int e = 0; e < E; ++e) v[e] = sc.in(x[e]);
-      Ln::derivative(v, j, at, sync, twd);
-#pragma unroll
-      for (int e = 0; e < E; ++e) x[e] = sc.outi(v[e]);
+      sc.in(x, v);
+      Ln::derivative(v, j, at, sync, tw, pre);
+      sc.template out<true>(v, x);
     } else {
 #pragma unroll
       for (int e = 0; e < E; ++e) v[e] = A::in(x[e]);
-      Ln::derivative(v, j, at, sync, twd);
+      Ln::derivative(v, j, at, sync, tw, pre);
 #pragma unroll
       for (int e = 0; e < E; ++e) x[e] = A::out(v[e]);
     }

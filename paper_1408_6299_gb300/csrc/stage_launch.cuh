@@ -120,21 +120,26 @@ void run_cols(Spectral<T>& sp, const ColJob<T>* jobs, int nj, cudaStream_t st) {
 template <typename T, int L, int EPI>
 void rows_L(const Spectral<T>& sp, const RowArgs<T>& a, double bytes, cudaStream_t st) {
   using A = typename Arith<T>::Main;
-  constexpr int NF = RowTile<L, false, EPI>::NF;
+  constexpr int NF = RowTile<L, false, false, EPI>::NF;
   ProfScope ps(KK_ROWS_C2R, st, bytes, (double)a.nrows / 2 * NF * (2.0 * fft_flops<L>() + 2.0 * L));
-  auto go = [&](auto narrow) {
-    constexpr bool NARROW = decltype(narrow)::value;
-    using Tile = RowTile<L, NARROW, EPI>;
-    const unsigned grid = (unsigned)((a.nrows + Tile::ROWS - 1) / Tile::ROWS);
-    RowArgs<T> b = a;
+  auto go = [&](auto narrow, auto few) {
+    constexpr bool NARROW = decltype(narrow)::value, FEW = decltype(few)::value;
+    using Tile = RowTile<L, NARROW, FEW, EPI>;
     // large fields from the last row on: the column pass left its last planes in
     // L2 (256^3 mixed matvec 158.7 -> 156.3 ms)
+    RowArgs<T> b = a;
     b.rev = a.nrows * (long)L * sizeof(T) >= (64 << 20);
-    chain(k_rows_line<A, T, L, NARROW, EPI>, grid, Tile::NT, st, b,
+    chain(k_rows_line<A, T, L, NARROW, FEW, EPI>, (unsigned)((a.nrows + Tile::ROWS - 1) / Tile::ROWS), Tile::NT, st, b,
           static_cast<const typename A::W*>(sp.line_table(L, NARROW, A::TABLE)));
   };
-  if (narrow_lines(a.nrows / 2 * NF * LinePlan<L, false>::TS, sizeof(T))) go(std::true_type{});
-  else go(std::false_type{});
+  const long lines = a.nrows / 2 * NF;
+  // few lines: 32^2 FP64 matvec 708 -> 529 us, 128^2 mixed 817 -> 613, 64^3 mixed
+  // 1627 -> 1426. Double precision, bound by arithmetic, loses earlier: 64^3
+  // gradient (2048 lines) 3790 -> 3940 us
+  const long few = 152L * (sizeof(T) == 8 ? 8 : 24);
+  if (!narrow_lines(lines * LinePlan<L, false>::TS, sizeof(T))) go(std::false_type{}, std::false_type{});
+  else if (lines <= few) go(std::true_type{}, std::true_type{});
+  else go(std::true_type{}, std::false_type{});
 }
 
 template <typename T, int EPI>
@@ -150,6 +155,21 @@ void run_rows(const Spectral<T>& sp, const RowArgs<T>& a, double bytes, cudaStre
   }
   throw StatusError{1, "unsupported last-axis length"};
 }
+
+// Instantiated once per precision and pass (stage_cols_*.cu, stage_rows_*.cu),
+// which compile side by side: one file per precision took 105 s.
+#define REG_COLS_OF(T)                                                                         \
+  template void run_cols<T, false>(Spectral<T>&, const ColJob<T>*, int, cudaStream_t);         \
+  template void run_cols<T, true>(Spectral<T>&, const ColJob<T>*, int, cudaStream_t);
+#define REG_ROWS_OF(T, EPI) template void run_rows<T, EPI>(const Spectral<T>&, const RowArgs<T>&, double, cudaStream_t);
+#define REG_STAGES_OF(T)                                                                       \
+  extern template void run_cols<T, false>(Spectral<T>&, const ColJob<T>*, int, cudaStream_t);  \
+  extern template void run_cols<T, true>(Spectral<T>&, const ColJob<T>*, int, cudaStream_t);   \
+  extern REG_ROWS_OF(T, EPI_ADV2) extern REG_ROWS_OF(T, EPI_ADV3)                              \
+  extern REG_ROWS_OF(T, EPI_ADV33) extern REG_ROWS_OF(T, EPI_DIV)
+REG_STAGES_OF(float)
+REG_STAGES_OF(double)
+#undef REG_STAGES_OF
 
 // fields an advection epilogue reads and writes beyond u and its derivatives
 // (stage 1 reads y = u itself)

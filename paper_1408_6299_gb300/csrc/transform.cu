@@ -51,8 +51,7 @@ __global__ void __launch_bounds__(FieldRows<L, NARROW, VAR>::NT) k_field_rows_fw
   sc.by_sum(mag, l1);
   sc.times_pow2(-1);
   FxV v[E];
-#pragma unroll
-  for (int e = 0; e < E; ++e) v[e] = sc.in(x[e]);
+  sc.in(x, v);
   auto at = [&](int p) { return b + p + (p >> F::PADSH); };
   Ln::forward(v, j, at, sync, tw, sc.scaled);
   if constexpr (Ln::S > 1) sync();
@@ -71,8 +70,8 @@ __global__ void __launch_bounds__(FieldRows<L, NARROW, VAR>::NT) k_field_rows_fw
       a = {z.x + w.x, z.y - w.y};
       c = {z.y + w.y, w.x - z.x};
     }
-    o[k] = make_double2(sc.out1(a.x), sc.out1(a.y));
-    o[M + k] = make_double2(sc.out1(c.x), sc.out1(c.y));
+    o[k] = make_double2(sc.back(a.x), sc.back(a.y));
+    o[M + k] = make_double2(sc.back(c.x), sc.back(c.y));
   }
 }
 
@@ -112,17 +111,16 @@ __global__ void __launch_bounds__(FieldRows<L, NARROW, 0>::NT) k_field_rows_inv(
   sc.by_sum(mag, l1);
   sc.times_pow2(-ilog2_c(L));
   FxV v[E];
-#pragma unroll
-  for (int e = 0; e < E; ++e) v[e] = sc.in(x[e]);
+  sc.in(x, v);
   Ln::forward(v, j, [&](int p) { return b + p + (p >> F::PADSH); }, sync, tw, sc.scaled);
   if (!ok) return;
   double* o = out + row * L;
+  sc.template out<true>(v, x);
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     const int p = Ln::frequency(j, e);
-    const double2 z = sc.out(v[e]);
-    o[p] = z.x;
-    o[L + p] = z.y;
+    o[p] = x[e].x;
+    o[L + p] = x[e].y;
   }
 }
 
@@ -163,15 +161,12 @@ __global__ void __launch_bounds__(FieldCols<L, NARROW>::NT) k_field_cols(double2
   sc.by_sum(mag, l1);
   if (INV) sc.times_pow2(-ilog2_c(L));
   FxV v[E];
-#pragma unroll
-  for (int e = 0; e < E; ++e) v[e] = sc.in(x[e]);
+  sc.in(x, v);
   Ln::forward(v, j, [&](int p) { return buf + p * TC + c; }, [] { __syncthreads(); }, tw, sc.scaled);
   if (!ok) return;
+  sc.template out<false>(v, x);  // conjugated
 #pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const double2 z = sc.out(v[e]);  // conjugated
-    d[Ln::frequency(j, e) * s] = INV ? z : make_double2(z.x, -z.y);
-  }
+  for (int e = 0; e < E; ++e) d[Ln::frequency(j, e) * s] = INV ? x[e] : make_double2(x[e].x, -x[e].y);
 }
 
 template <class F>
