@@ -201,29 +201,34 @@ __device__ __forceinline__ float4 gmul(float4 a, float4 b) {
   return make_float4(a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w);
 }
 
-template <class A, typename T, int L, bool NARROW, bool PROD, int VAR>
-__global__ void __launch_bounds__(ColTile<A, L, NARROW, VAR>::NT) k_cols_line(ColJobs<T> J,
-                                                                          const typename A::W* __restrict__ tw) {
-  using Tile = ColTile<A, L, NARROW, VAR>;
-  using Ln = Line<A, L, NARROW>;
-  typename A::W pre[Ln::NTW + 1];
-  Ln::preload(pre, threadIdx.x / Tile::TC, tw);
-  chain_enter(sizeof(T) == 4);
-  using V = typename A::V;
-  using G = typename A::G;
-  constexpr int E = Ln::E, TC = Tile::TC;
-  __shared__ V buf[L * TC];
-  int q = 0, tile = blockIdx.x;
+// Job q of block tile
+template <typename T>
+__device__ __forceinline__ int col_job(const ColJobs<T>& J, int& tile) {
+  int q = 0;
 #pragma unroll
   for (int k = 1; k < kColJobs; ++k)
     if (k < J.nj && tile >= J.start[k]) q = k;
   tile -= J.start[q];
+  return q;
+}
+
+// TC neighbouring lines of job q; buf: L * TC values
+template <class A, typename T, int L, bool NARROW, bool PROD, int TC>
+__device__ __forceinline__ void cols_tile(const ColJobs<T>& J, int q, int tile, int n, typename A::V* buf,
+                                          const typename A::W* __restrict__ tw) {
+  using Ln = Line<A, L, NARROW>;
+  using V = typename A::V;
+  using G = typename A::G;
+  constexpr int E = Ln::E, TS = LinePlan<L, NARROW>::TS;
   const int c = threadIdx.x % TC, j = threadIdx.x / TC;
+  typename A::W pre[Ln::NTW + 1];
+  Ln::preload(pre, j, tw);
+  chain_enter(sizeof(T) == 4);
   const int line = tile * TC + c;
   const int ls = J.log2s[q];
   const long s = 1L << ls;
   const long off = ((long)(line >> ls) * L << ls) + (line & (int)(s - 1));
-  const bool ok = line < J.n;
+  const bool ok = line < n;
   G x[E];
   {
     const G* in = reinterpret_cast<const G*>(J.in[q]) + off;
@@ -245,7 +250,7 @@ __global__ void __launch_bounds__(ColTile<A, L, NARROW, VAR>::NT) k_cols_line(Co
     unsigned mag = 0;
 #pragma unroll
     for (int e = 0; e < E; ++e) mag = max(mag, fx_mag(x[e]));
-    const FxScale<L, Ln::R0> sc(line_max<TC, Tile::TS>(mag, reinterpret_cast<unsigned*>(buf), c, j));
+    const FxScale<L, Ln::R0> sc(line_max<TC, TS>(mag, reinterpret_cast<unsigned*>(buf), c, j));
     sc.in(x, v);
     Ln::derivative(v, j, at, sync, tw, pre);
     if (!ok) return;
@@ -262,6 +267,48 @@ __global__ void __launch_bounds__(ColTile<A, L, NARROW, VAR>::NT) k_cols_line(Co
       if (J.stream[q]) st_stream(out + Ln::position(j, e) * s, A::out(v[e]));
       else out[Ln::position(j, e) * s] = A::out(v[e]);
     }
+  }
+}
+
+template <class A, typename T, int L, bool NARROW, bool PROD, int VAR>
+__global__ void __launch_bounds__(ColTile<A, L, NARROW, VAR>::NT) k_cols_line(ColJobs<T> J,
+                                                                          const typename A::W* __restrict__ tw) {
+  constexpr int TC = ColTile<A, L, NARROW, VAR>::TC;
+  __shared__ typename A::V buf[L * TC];
+  int tile = blockIdx.x;
+  const int q = col_job(J, tile);
+  cols_tile<A, T, L, NARROW, PROD, TC>(J, q, tile, J.n, buf, tw);
+}
+
+// Jobs along axes of two lengths up to 256 (narrow plans): the length is
+// uniform in a block of 64 threads, one or several lines of it. One launch,
+// chained to its predecessor and successor, instead of one per length on forked
+// streams (one_cols_launch has the figures).
+constexpr int kTwoNT = 64;
+template <class A>
+struct TwoAxes {
+  const typename A::W* tw[2];
+  int lg[2], n[2];  // log2 of the length, lines of a field
+  int axis[kColJobs];
+};
+template <class A, typename T, bool PROD>
+__global__ void __launch_bounds__(kTwoNT) k_cols_two(const __grid_constant__ ColJobs<T> J,
+                                                    const __grid_constant__ TwoAxes<A> P) {
+  __shared__ typename A::V buf[kTwoNT * 4];
+  int tile = blockIdx.x;
+  const int q = col_job(J, tile), a = P.axis[q];
+  auto go = [&](auto len) {
+    constexpr int L = decltype(len)::value;
+    static_assert(LinePlan<L, true>::E == 4, "lines of a block fill buf");
+    cols_tile<A, T, L, true, PROD, kTwoNT / LinePlan<L, true>::TS>(J, q, tile, P.n[a], buf, P.tw[a]);
+  };
+  switch (P.lg[a]) {
+    case 3: return go(std::integral_constant<int, 8>{});
+    case 4: return go(std::integral_constant<int, 16>{});
+    case 5: return go(std::integral_constant<int, 32>{});
+    case 6: return go(std::integral_constant<int, 64>{});
+    case 7: return go(std::integral_constant<int, 128>{});
+    default: return go(std::integral_constant<int, 256>{});
   }
 }
 

@@ -85,13 +85,59 @@ void cols_L(const Spectral<T>& sp, const ColJob<T>* jobs, int nj, cudaStream_t s
   cols_tuned<A, T, L, false, PROD>(sp, jobs, nj, st);
 }
 
-// The column passes of one stage: one launch per axis length, side by side
-// where there are two (each fills the other's last wave; 32 x 64 x 128 Newton
-// matvec: 3140 -> 2800 us).
+// Whether jobs along axes of two lengths share a launch: where both run narrow
+// plans, and in double precision only while every block has an SM to itself,
+// since k_cols_two holds the registers of its longest line and does not tune its
+// tile (32 x 16 x 8 mixed matvec 287 -> 262 us, 32 x 64 x 128 mixed Newton matvec
+// 2506 -> 2437, 64 x 16 x 8 FP64 matvec 967 -> 874; beyond the limit 64 x 128 x
+// 16 FP64 transport 1056 -> 1132, 256 x 32 x 64 FP64 matvec 40.8 -> 44.5 ms).
+template <typename T>
+bool one_cols_launch(const Grid& g, int nj) {
+  for (int a = 0; a < 2; ++a) {
+    const int L = (int)g.n[a];
+    if (L > 256) return false;
+    const int wide_ts = L > 64 ? L / 16 : (L == 16 ? 1 : L / 8);
+    if (!narrow_lines((long)(nj / 2) * g.Nc / L * wide_ts, sizeof(T))) return false;
+  }
+  return sizeof(T) == 4 || nj * g.Nc / 4 <= 152L * kTwoNT;
+}
+
+// jobs along both strided axes, of two lengths, in one launch of narrow plans
+template <typename T, bool PROD>
+void cols_two(const Spectral<T>& sp, const ColJob<T>* jobs, int nj, cudaStream_t st) {
+  using A = typename Arith<T>::Main;
+  const Grid& g = sp.grid();
+  ColJobs<T> J{};
+  TwoAxes<A> P{};
+  J.nj = nj;
+  double flops = 0;
+  for (int a = 0; a < 2; ++a) {
+    P.tw[a] = static_cast<const typename A::W*>(sp.line_table((int)g.n[a], true, A::TABLE));
+    P.lg[a] = ilog2_c((int)g.n[a]);
+    P.n[a] = (int)(g.Nc / g.n[a] / A::CW);
+  }
+  for (int q = 0; q < nj; ++q) {
+    const int a = jobs[q].axis, tc = kTwoNT * 4 / (int)g.n[a];
+    J.in[q] = jobs[q].in;
+    J.mul[q] = jobs[q].mul;
+    J.out[q] = jobs[q].out;
+    J.log2s[q] = ilog2_c((int)(line_stride(g, a) / A::CW));
+    J.start[q + 1] = J.start[q] + (P.n[a] + tc - 1) / tc;
+    P.axis[q] = a;
+    flops += (double)g.Nc / g.n[a] * (10.0 * g.n[a] * P.lg[a] + 2.0 * g.n[a]);
+  }
+  ProfScope ps(KK_COLS, st, (double)nj * g.N * sizeof(T) * (PROD ? 3.0 : 2.0), flops);
+  chain(k_cols_two<A, T, PROD>, (unsigned)J.start[nj], kTwoNT, st, J, P);
+}
+
+// The column passes of one stage. Axes of two lengths: one launch
+// (one_cols_launch) or one launch per length, side by side (each fills the
+// other's last wave; 32 x 64 x 128 Newton matvec 3140 -> 2800 us).
 template <typename T, bool PROD>
 void run_cols(Spectral<T>& sp, const ColJob<T>* jobs, int nj, cudaStream_t st) {
   const Grid& g = sp.grid();
   const bool two = nj > 1 && g.n[0] != g.n[1];
+  if (two && one_cols_launch<T>(g, nj)) return cols_two<T, PROD>(sp, jobs, nj, st);
   cudaStream_t st2 = two ? sp.fork() : st;
   for (int axis = 0; axis < (two ? 2 : 1); ++axis) {
     ColJob<T> grp[kColJobs];
