@@ -16,6 +16,7 @@
 #include <algorithm>
 #include <atomic>
 #include <stdexcept>
+#include <type_traits>
 
 #include "internal.h"
 
@@ -37,32 +38,40 @@ struct GridArgs {
   long Nc;   // all stacked problems
   long Nc1;  // one problem (a power of two)
   int lg1;   // log2 Nc1
+  int lg[3];  // log2 n, of the last axis log2 M
 };
+// D: the dimension where it is a constant (indices then stay in registers), or 0
+template <int D = 0>
 __device__ inline ModeIdx decode(long q, const GridArgs& g) {
+  const int d = D ? D : g.d;
   ModeIdx m;
   int r = (int)(q & (g.Nc1 - 1));
-  m.j[g.d - 1] = r & (g.M - 1);
-  r /= g.M;
-  for (int a = g.d - 2; a >= 0; --a) {
-    m.j[a] = r & (g.n[a] - 1);
-    r /= g.n[a];
+#pragma unroll
+  for (int a = d - 1; a >= 0; --a) {
+    m.j[a] = r & ((1 << g.lg[a]) - 1);
+    r >>= g.lg[a];
   }
   return m;
 }
 // index of -k' on the slot-0 plane of the problem that holds mode q0
+template <int D = 0>
 __device__ inline long encode_neg(long q0, const ModeIdx& m, const GridArgs& g) {
   int q = 0;
-  for (int a = 0; a < g.d - 1; ++a) q = q * g.n[a] + ((g.n[a] - m.j[a]) & (g.n[a] - 1));
+#pragma unroll
+  for (int a = 0; a < (D ? D : g.d) - 1; ++a) q = q * g.n[a] + ((g.n[a] - m.j[a]) & (g.n[a] - 1));
   return (q0 & ~(g.Nc1 - 1)) + (long)q * g.M;
 }
+template <int D>
 __device__ inline int masked_k(const ModeIdx& m, const GridArgs& g, int a) {
-  if (a == g.d - 1) return m.j[a];  // slot 0 -> 0 for both DC and Nyquist halves
+  if (a == D - 1) return m.j[a];  // slot 0 -> 0 for both DC and Nyquist halves
   return kmask(m.j[a], g.n[a]);
 }
 // |k|^2 over the leading axes (full wavenumbers, Nyquist kept)
+template <int D = 0>
 __device__ inline int lead_k2(const ModeIdx& m, const GridArgs& g) {
   int kk = 0;
-  for (int a = 0; a < g.d - 1; ++a) {
+#pragma unroll
+  for (int a = 0; a < (D ? D : g.d) - 1; ++a) {
     const int k = kfull(m.j[a], g.n[a]);
     kk += k * k;
   }
@@ -83,8 +92,10 @@ __global__ void k_inv_k2(double* t, long n) {
 }
 
 // NC: n_c where it is 1, 2 or 3 (the coefficients of a component then stay in
-// registers), else 0.
-template <int NC>
+// registers), else 0. Bound by the double-precision unit, so products with one
+// and sums with zero are left out for n_c = 1, and indices come from shifts with
+// the dimension a constant (256^3: 472 -> 243 us, 177 at the copy rate).
+template <int NC, int D>
 __global__ void __launch_bounds__(256) k_spec_tail(const double2* __restrict__ V, const double2* __restrict__ F,
                                                    double2* __restrict__ out, GridArgs g, int nc_, double beta,
                                                    const double* __restrict__ Cg, int reg, int stokes,
@@ -94,25 +105,27 @@ __global__ void __launch_bounds__(256) k_spec_tail(const double2* __restrict__ V
   const long q = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= g.Nc) return;
   if (betas) beta = betas[q >> g.lg1];
-  const int d = g.d, nc = NC ? NC : nc_;
+  constexpr int d = D;
+  const int nc = NC ? NC : nc_;
   const long Nc = g.Nc;
-  const ModeIdx m = decode(q, g);
-  const int kk = lead_k2(m, g), kz = m.j[d - 1];
+  const ModeIdx m = decode<D>(q, g);
+  const int kk = lead_k2<D>(m, g), kz = m.j[d - 1];
   double alpha, delta = 0.0;
   long qn = q;
   if (kz == 0) {
     const double a0 = sym_pow(kk, reg), aN = sym_pow(kk + g.M * g.M, reg);
     alpha = 0.5 * beta * (a0 + aN);
     delta = 0.5 * beta * (a0 - aN);
-    qn = encode_neg(q, m, g);
+    qn = encode_neg<D>(q, m, g);
   } else {
     alpha = beta * sym_pow(kk + kz * kz, reg);
   }
   // masked wavenumber for K
-  int kt[3], kt2 = 0;
+  int kt[d], kt2 = 0;
   if (F && stokes)
+#pragma unroll
     for (int a = 0; a < d; ++a) {
-      kt[a] = masked_k(m, g, a);
+      kt[a] = masked_k<D>(m, g, a);
       kt2 += kt[a] * kt[a];
     }
   auto reg_term = [&](int i, int l, const double2* v, const double2* vn) {
@@ -153,7 +166,32 @@ __global__ void __launch_bounds__(256) k_spec_tail(const double2* __restrict__ V
     }
     out[(l * d + i) * Nc + q] = r;
   };
-  if constexpr (NC > 0) {
+  if constexpr (NC == 1) {
+    // the 1 x 1 Gram matrix is 1; all loads of a mode first
+    double2 v[d], f[d], vn[d];
+#pragma unroll
+    for (int i = 0; i < d; ++i) {
+      v[i] = V[i * Nc + q];
+      f[i] = F ? F[i * Nc + q] : make_double2(0, 0);
+      if (kz == 0) vn[i] = V[i * Nc + qn];
+    }
+    double2 p = make_double2(0, 0);
+    const bool leray = F && stokes && kt2 > 0;
+    if (leray) {
+#pragma unroll
+      for (int a = 0; a < d; ++a) p = make_double2(p.x + (double)kt[a] * f[a].x, p.y + (double)kt[a] * f[a].y);
+      const double w = inv_pow(kt2, 1, inv_k2);
+      p = make_double2(p.x * w, p.y * w);
+    }
+#pragma unroll
+    for (int i = 0; i < d; ++i) {
+      double2 r = make_double2(alpha * v[i].x, alpha * v[i].y);
+      if (kz == 0) r = make_double2(r.x + delta * vn[i].x, r.y - delta * vn[i].y);
+      if (F) r = make_double2(r.x + f[i].x, r.y + f[i].y);
+      if (leray) r = make_double2(r.x - (double)kt[i] * p.x, r.y - (double)kt[i] * p.y);
+      out[i * Nc + q] = r;
+    }
+  } else if constexpr (NC > 0) {
     double2 p[NC];
 #pragma unroll
     for (int l = 0; l < NC; ++l) p[l] = projection(l);
@@ -175,20 +213,23 @@ __global__ void __launch_bounds__(256) k_spec_tail(const double2* __restrict__ V
   }
 }
 
-template <int NC>
+// ib: 1 / beta, divided once on the host instead of once per mode (with the
+// changes named at k_spec_tail the 256^3 preconditioner 2085 -> 1883 us, of which
+// this kernel 242; 118 at the copy rate)
+template <int NC, int D>
 __global__ void __launch_bounds__(256) k_spec_precond(const double2* __restrict__ R, double2* __restrict__ out,
-                                                      GridArgs g, int nc_, double beta, const double* __restrict__ Ci,
+                                                      GridArgs g, int nc_, double ib, const double* __restrict__ Ci,
                                                       int reg, const double* __restrict__ betas,
                                                       const double* __restrict__ inv_k2) {
   chain_enter();
   const long q = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= g.Nc) return;
-  if (betas) beta = betas[q >> g.lg1];
-  const int d = g.d, nc = NC ? NC : nc_;
+  if (betas) ib = 1.0 / betas[q >> g.lg1];
+  constexpr int d = D;
+  const int nc = NC ? NC : nc_;
   const long Nc = g.Nc;
-  const ModeIdx m = decode(q, g);
-  const int kk = lead_k2(m, g), kz = m.j[d - 1];
-  const double ib = 1.0 / beta;
+  const ModeIdx m = decode<D>(q, g);
+  const int kk = lead_k2<D>(m, g), kz = m.j[d - 1];
   double alpha, delta = 0.0;
   long qn = q;
   if (kz == 0) {
@@ -196,9 +237,24 @@ __global__ void __launch_bounds__(256) k_spec_precond(const double2* __restrict_
     const double sN = ib * inv_pow(kk + g.M * g.M, reg, inv_k2);
     alpha = 0.5 * (s0 + sN);
     delta = 0.5 * (s0 - sN);
-    qn = encode_neg(q, m, g);
+    qn = encode_neg<D>(q, m, g);
   } else {
     alpha = ib * inv_pow(kk + kz * kz, reg, inv_k2);
+  }
+  if constexpr (NC == 1) {  // the 1 x 1 Gram matrix is 1; all loads of a mode first
+    double2 v[d], vn[d];
+#pragma unroll
+    for (int i = 0; i < d; ++i) {
+      v[i] = R[i * Nc + q];
+      if (kz == 0) vn[i] = R[i * Nc + qn];
+    }
+#pragma unroll
+    for (int i = 0; i < d; ++i) {
+      double2 r = make_double2(alpha * v[i].x, alpha * v[i].y);
+      if (kz == 0) r = make_double2(r.x + delta * vn[i].x, r.y - delta * vn[i].y);
+      out[i * Nc + q] = r;
+    }
+    return;
   }
   for (int i = 0; i < d; ++i) {
     double2 v[NC ? NC : 1], vn[NC ? NC : 1];
@@ -213,7 +269,7 @@ __global__ void __launch_bounds__(256) k_spec_precond(const double2* __restrict_
     for (int l = 0; l < nc; ++l) {
       double2 s = make_double2(0, 0), n = make_double2(0, 0);
       for (int lp = 0; lp < nc; ++lp) {
-        const double c = NC == 1 ? 1.0 : __ldg(&Ci[l * nc + lp]);  // the 1 x 1 Gram matrix is 1
+        const double c = __ldg(&Ci[l * nc + lp]);
         const double2 x = NC ? v[NC ? lp : 0] : R[(lp * d + i) * Nc + q];
         s.x += c * x.x;
         s.y += c * x.y;
@@ -260,6 +316,10 @@ GridArgs args(const Grid& g) {
   a.Nc1 = g.Nc / g.B;
   a.lg1 = 0;
   while ((1L << a.lg1) < a.Nc1) ++a.lg1;
+  for (int i = 0; i < g.d; ++i) {
+    a.lg[i] = 0;
+    while ((1 << a.lg[i]) < (i == g.d - 1 ? g.M : g.n[i])) ++a.lg[i];
+  }
   return a;
 }
 
@@ -307,21 +367,31 @@ void spec_tail(const Grid& g, cudaStream_t s, const double2* V, const double2* F
   auto run = [&](auto k) {
     chain(k, blocks_for(g.Nc), 256, s, V, F, out, args(g), nc, beta, Cg_dev, reg, stokes, betas, inv_k2);
   };
-  if (nc == 1) run(k_spec_tail<1>);
-  else if (nc == 2) run(k_spec_tail<2>);
-  else if (nc == 3) run(k_spec_tail<3>);
-  else run(k_spec_tail<0>);
+  auto dim = [&](auto d) {
+    constexpr int D = decltype(d)::value;
+    if (nc == 1) run(k_spec_tail<1, D>);
+    else if (nc == 2) run(k_spec_tail<2, D>);
+    else if (nc == 3) run(k_spec_tail<3, D>);
+    else run(k_spec_tail<0, D>);
+  };
+  if (g.d == 2) dim(std::integral_constant<int, 2>{});
+  else dim(std::integral_constant<int, 3>{});
 }
 
 void spec_precond(const Grid& g, cudaStream_t s, const double2* R, double2* out, int nc, double beta,
                   const double* Ci_dev, int reg, const double* betas, const double* inv_k2) {
   auto run = [&](auto k) {
-    chain(k, blocks_for(g.Nc), 256, s, R, out, args(g), nc, beta, Ci_dev, reg, betas, inv_k2);
+    chain(k, blocks_for(g.Nc), 256, s, R, out, args(g), nc, 1.0 / beta, Ci_dev, reg, betas, inv_k2);
   };
-  if (nc == 1) run(k_spec_precond<1>);
-  else if (nc == 2) run(k_spec_precond<2>);
-  else if (nc == 3) run(k_spec_precond<3>);
-  else run(k_spec_precond<0>);
+  auto dim = [&](auto d) {
+    constexpr int D = decltype(d)::value;
+    if (nc == 1) run(k_spec_precond<1, D>);
+    else if (nc == 2) run(k_spec_precond<2, D>);
+    else if (nc == 3) run(k_spec_precond<3, D>);
+    else run(k_spec_precond<0, D>);
+  };
+  if (g.d == 2) dim(std::integral_constant<int, 2>{});
+  else dim(std::integral_constant<int, 3>{});
 }
 
 void spec_gauss(const Grid& g, cudaStream_t s, double2* U, double2* out, double sigma) {
