@@ -40,12 +40,19 @@ template <typename T>
 struct NodeWeights {
   T hi[16], lo[16];
 };
-// NC: n_c where it is 2, 3 or 4 (the loads of a point are then issued
-// together: 64^3 with three coefficients 16 -> 4 us), else 0. VEC: 16-byte
-// accesses, else single values (callers' arrays may be offset views).
+// The velocity at up to kVelGroup nodes, dN values each. NC: n_c where it is 2,
+// 3 or 4 (the loads of a point are then issued together and serve every node:
+// 64^3 with three coefficients 16 -> 4 us for one node), else 0. VEC: 16-byte
+// accesses, else single values.
+template <typename T>
+struct VelNodes {
+  NodeWeights<T> b[kVelGroup];
+  int count;
+};
 template <typename T, int NC, bool VEC>
-__global__ void __launch_bounds__(128) k_vel_at(const T* __restrict__ coef, int nc_, NodeWeights<T> b,
-                                                T* __restrict__ out, long dN) {
+__global__ void __launch_bounds__(128) k_vel_at(const T* __restrict__ coef, int nc_,
+                                                const __grid_constant__ VelNodes<T> nodes, T* __restrict__ out,
+                                                long dN) {
   chain_enter();
   using Q = std::conditional_t<VEC, Quad<T>, One<T>>;
   const int nc = NC ? NC : nc_;
@@ -57,28 +64,33 @@ __global__ void __launch_bounds__(128) k_vel_at(const T* __restrict__ coef, int 
 #pragma unroll
     for (int l = 0; l < NC; ++l) v[l] = c[l * n];
   }
-  Q s{}, err{};
 #pragma unroll
-  for (int l = 0; l < nc; ++l) {
-    if (!NC) v[0] = c[l * n];
-    const Q u = v[NC ? l : 0];
+  for (int k = 0; k < kVelGroup; ++k) {
+    if (k == nodes.count) return;
+    const NodeWeights<T>& b = nodes.b[k];
+    Q s{}, err{};
 #pragma unroll
-    for (int w = 0; w < Q::W; ++w) {
-      if constexpr (sizeof(T) == 8) {
-        s.v[w] += b.hi[l] * u.v[w];
-      } else {
-        const float p = __fmul_rn(b.hi[l], u.v[w]);
-        const float e = fmaf(b.hi[l], u.v[w], -p) + b.lo[l] * u.v[w];
-        const float t = __fadd_rn(s.v[w], p), z = __fsub_rn(t, s.v[w]);
-        err.v[w] += e + __fadd_rn(__fsub_rn(s.v[w], __fsub_rn(t, z)), __fsub_rn(p, z));
-        s.v[w] = t;
+    for (int l = 0; l < nc; ++l) {
+      if (!NC) v[0] = c[l * n];
+      const Q u = v[NC ? l : 0];
+#pragma unroll
+      for (int w = 0; w < Q::W; ++w) {
+        if constexpr (sizeof(T) == 8) {
+          s.v[w] += b.hi[l] * u.v[w];
+        } else {
+          const float p = __fmul_rn(b.hi[l], u.v[w]);
+          const float e = fmaf(b.hi[l], u.v[w], -p) + b.lo[l] * u.v[w];
+          const float t = __fadd_rn(s.v[w], p), z = __fsub_rn(t, s.v[w]);
+          err.v[w] += e + __fadd_rn(__fsub_rn(s.v[w], __fsub_rn(t, z)), __fsub_rn(p, z));
+          s.v[w] = t;
+        }
       }
     }
-  }
-  if (sizeof(T) == 4)
+    if (sizeof(T) == 4)
 #pragma unroll
-    for (int w = 0; w < Q::W; ++w) s.v[w] += err.v[w];
-  reinterpret_cast<Q*>(out)[x] = s;
+      for (int w = 0; w < Q::W; ++w) s.v[w] += err.v[w];
+    reinterpret_cast<Q*>(out)[k * n + x] = s;
+  }
 }
 
 template <typename S, typename T>
@@ -100,13 +112,16 @@ __global__ void k_first_predictor(const T* __restrict__ gm, const T* __restrict_
   yh[x] = h * k;
 }
 
-// out_k = sum_i a_{k,i} b_i for the nodes k = blockIdx.y
+// out_k = sum_i a_{k,i} b_{k,i} for the nodes k = blockIdx.y; bs: distance of the
+// nodes of b (0: one b for all)
 template <typename T>
-__global__ void k_dot_fields(const T* __restrict__ a, const T* __restrict__ b, T* __restrict__ out, int d, long N) {
+__global__ void k_dot_fields(const T* __restrict__ a, const T* __restrict__ b, long bs, T* __restrict__ out, int d,
+                             long N) {
   chain_enter();
   long x = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= N) return;
   a += blockIdx.y * d * N;
+  b += blockIdx.y * bs;
   T s = 0;
   for (int i = 0; i < d; ++i) s += a[i * N + x] * b[i * N + x];
   out[blockIdx.y * N + x] = s;
@@ -346,20 +361,23 @@ __global__ void k_reduce_final(const double* __restrict__ part, double* __restri
 }  // namespace
 
 template <typename T>
-void vel_at(const T* coef, int nc, const Coefs& b, T* out, long dN, cudaStream_t s) {
-  NodeWeights<T> w;
-  for (int l = 0; l < 16; ++l) {
-    w.hi[l] = l < nc ? (T)b.c[l] : (T)0;
-    w.lo[l] = l < nc ? (T)(b.c[l] - (double)w.hi[l]) : (T)0;
-  }
+void vel_at(const T* coef, int nc, const Coefs* b, int count, T* out, long dN, cudaStream_t s) {
+  VelNodes<T> w;
+  w.count = count;
+  for (int k = 0; k < kVelGroup; ++k)
+    for (int l = 0; l < 16; ++l) {
+      const double c = k < count && l < nc ? b[k].c[l] : 0.0;
+      w.b[k].hi[l] = (T)c;
+      w.b[k].lo[l] = (T)(c - (double)w.b[k].hi[l]);
+    }
   const bool vec = ((reinterpret_cast<uintptr_t>(coef) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
   auto kern = !vec ? k_vel_at<T, 0, false>
                    : (nc == 2 ? k_vel_at<T, 2, true>
                               : (nc == 3 ? k_vel_at<T, 3, true> : (nc == 4 ? k_vel_at<T, 4, true> : k_vel_at<T, 0, true>)));
   chain(kern, nblk(vec ? dN / Quad<T>::W : dN, 128), 128, s, coef, nc, w, out, dN);
 }
-template void vel_at<float>(const float*, int, const Coefs&, float*, long, cudaStream_t);
-template void vel_at<double>(const double*, int, const Coefs&, double*, long, cudaStream_t);
+template void vel_at<float>(const float*, int, const Coefs*, int, float*, long, cudaStream_t);
+template void vel_at<double>(const double*, int, const Coefs*, int, double*, long, cudaStream_t);
 
 template <typename S, typename T>
 void convert(const S* in, T* out, long n, cudaStream_t s) {
@@ -375,11 +393,11 @@ void first_predictor(const T* gm, const T* wt, T h, T* yh, int d, long N, cudaSt
   chain(k_first_predictor<T>, nblk(N), 256, s, gm, wt, h, yh, d, N);
 }
 template <typename T>
-void dot_fields(const T* a, const T* b, T* out, int d, long N, int nodes, cudaStream_t s) {
+void dot_fields(const T* a, const T* b, long bs, T* out, int d, long N, int nodes, cudaStream_t s) {
   ProfScope ps(KK_STAGE, s, (double)nodes * N * sizeof(T) * (2 * d + 1));
   for (int k = 0; k < nodes; k += 65535)  // grid.y is limited to 65535
-    chain(k_dot_fields<T>, dim3(nblk(N), (unsigned)(nodes - k < 65535 ? nodes - k : 65535)), 256, s, a + (long)k * d * N, b,
-          out + (long)k * N, d, N);
+    chain(k_dot_fields<T>, dim3(nblk(N), (unsigned)(nodes - k < 65535 ? nodes - k : 65535)), 256, s, a + (long)k * d * N,
+          b + k * bs, bs, out + (long)k * N, d, N);
 }
 
 template <typename T>
@@ -400,7 +418,7 @@ void pair_to_double(const float* hi, const float* lo, double* out, long n, cudaS
 
 #define INST(T)                                                                                          \
   template void first_predictor<T>(const T*, const T*, T, T*, int, long, cudaStream_t);                        \
-  template void dot_fields<T>(const T*, const T*, T*, int, long, int, cudaStream_t);                             \
+  template void dot_fields<T>(const T*, const T*, long, T*, int, long, int, cudaStream_t);                       \
   template void force_acc<T>(T*, T*, const ForceNodes<T>&, int, int, long, cudaStream_t);
 INST(float)
 INST(double)

@@ -10,18 +10,24 @@ struct Coefs {
   double c[16];
 };
 
-// out[x] = sum_l b_l coef[l*dN + x], x < dN, rounded once to T
+constexpr int kVelGroup = 4;
+// out[k*dN + x] = sum_l b[k]_l coef[l*dN + x], x < dN, k < count <= kVelGroup,
+// rounded once to T
 template <typename T>
-void vel_at(const T* coef, int nc, const Coefs& b, T* out, long dN, cudaStream_t s);
+void vel_at(const T* coef, int nc, const Coefs* b, int count, T* out, long dN, cudaStream_t s);
+inline void vel_at(const double* coef, int nc, const Coefs& b, double* out, long dN, cudaStream_t s) {
+  vel_at<double>(coef, nc, &b, 1, out, dN, s);
+}
 template <typename S, typename T>
 void convert(const S* in, T* out, long n, cudaStream_t s);
 
 // yh = -h sum_i gm_i wt_i (d fields at stride N)
 template <typename T>
 void first_predictor(const T* gm, const T* wt, T h, T* yh, int d, long N, cudaStream_t s);
-// out_k = sum_i a_{k,i} b_i (d fields at stride N) for `nodes` consecutive groups a_k
+// out_k = sum_i a_{k,i} b_{k,i} (d fields at stride N) for `nodes` consecutive
+// groups a_k; bs: distance of the b_k (0: one for all)
 template <typename T>
-void dot_fields(const T* a, const T* b, T* out, int d, long N, int nodes, cudaStream_t s);
+void dot_fields(const T* a, const T* b, long bs, T* out, int d, long N, int nodes, cudaStream_t s);
 // Body force of up to kForceNodes time nodes (see ForceNodes):
 //   f[l][i] += cA_l (yA gA_i + yC gC_i) + cB_l yB gB_i   for every node in order,
 // a plain sum into fhi (flo null) or a compensated (fhi, flo) pair of precision T

@@ -49,6 +49,11 @@ def velocity(n, size):
     return torch.stack([smooth(n, 2, 40 + i) for i in range(len(n))])[None].mul_(size).contiguous()
 
 
+def torch_cat(*t):
+    import torch
+    return torch.cat(t).contiguous()
+
+
 def derivative(u, axis):
     import torch
     n = u.shape[axis]
@@ -155,6 +160,30 @@ def test_force_groups(n_t, ckpt):
         for _ in range(3):  # launched, captured and replayed
             R.hessvec(cuda(vt), Hv)
             assert rel(host(Hv), P.hessvec(v, mT, vt)) < tol
+
+
+@pytest.mark.parametrize("n,n_t", [((64, 32), 7), ((32, 32, 32), 6), ((256, 256, 128), 3)],
+                         ids=["64x32", "32c", "256x256x128"])
+def test_time_dependent_velocity(n, n_t):
+    # nodes formed in groups of four (the last one partial), and one by one in the largest fields
+    d = len(n)
+    size = 0.2 * n_t / (d * max(n) / 2)
+    v = torch_cat(velocity(n, size), velocity(n, 0.5 * size).flip(1))
+    u = white(n, 5)
+    R = lib.Registration(n, n_t, 2, 1e-2, lib.REG_H1, False, lib.REG_FP64, 0)
+    m1 = empty(n)
+    R.transport(v, u, m1)
+    h = 1.0 / n_t
+
+    def rhs(y, j):
+        a = v[0] + (2.0 * j / n_t - 1.0) * v[1]
+        return -sum(a[i] * derivative(y, i) for i in range(d))
+
+    for j in range(n_t):
+        k1 = rhs(u, j)
+        u = u + 0.5 * h * (k1 + rhs(u + h * k1, j + 1))
+    assert float((m1 - u).norm() / u.norm()) < FP64_TOL
+    R.close()
 
 
 @pytest.mark.parametrize("ckpt", [0, 3])
