@@ -35,6 +35,14 @@ struct StatusError {
     REG_CUDA(cudaGetLastError()); \
   } while (0)
 
+// Host data to device memory, complete on return. cudaMemcpy from pageable memory
+// may return with the transfer still under way on the NULL stream, and a
+// non-blocking stream has no order behind that stream.
+inline void upload(void* dst, const void* src, size_t bytes) {
+  REG_CUDA(cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice));
+  REG_CUDA(cudaStreamSynchronize(nullptr));
+}
+
 // ---------------------------------------------------------------------------
 // Kernel accounting: a process-wide launch counter, and optional CUDA-event
 // bracketing of launches by kind (enabled per context through the C ABI).

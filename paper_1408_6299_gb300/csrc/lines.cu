@@ -106,7 +106,7 @@ LineTables<T>::LineTables(const Grid& g) {
       }
   h.resize(h.size() + 16);
   REG_CUDA(cudaMalloc(&dev_, h.size()));
-  REG_CUDA(cudaMemcpy(dev_, h.data(), h.size(), cudaMemcpyHostToDevice));
+  upload(dev_, h.data(), h.size());
 }
 template <typename T>
 LineTables<T>::~LineTables() {

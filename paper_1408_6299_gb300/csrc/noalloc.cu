@@ -74,6 +74,7 @@ int setup_device(int dev) {
   if (n > kTableBytes) return (int)cudaErrorInvalidValue;
   write_wide_tables(g_table_image, S.tw_off);
   e = cudaMemcpy(p, g_table_image, n, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // the transfer may still be under way (see upload)
   if (e != cudaSuccess) return (int)e;
   S.base = (unsigned char*)p;
   S.ready = true;

@@ -2159,8 +2159,8 @@ reg_ctx* create_ctx(int d, const int64_t* n, int n_t, int n_c, double beta, int 
   for (int a = 0; a < n_c; ++a)
     for (int b = 0; b < n_c; ++b) c->Cg[a * n_c + b] = cheb_gram_entry(a, b);
   if (!invert_small(n_c, c->Cg, c->Ci)) throw StatusError{REG_EINVAL, "singular Gram matrix"};
-  REG_CUDA(cudaMemcpy(c->Cg_dev.get(n_c * n_c), c->Cg.data(), n_c * n_c * sizeof(double), cudaMemcpyHostToDevice));
-  REG_CUDA(cudaMemcpy(c->Ci_dev.get(n_c * n_c), c->Ci.data(), n_c * n_c * sizeof(double), cudaMemcpyHostToDevice));
+  upload(c->Cg_dev.get(n_c * n_c), c->Cg.data(), n_c * n_c * sizeof(double));
+  upload(c->Ci_dev.get(n_c * n_c), c->Ci.data(), n_c * n_c * sizeof(double));
   c->sp64.reset(new Spectral<double>(g, c->s));
   c->ft.reset(new FieldTransforms(
       g, c->s, [c](int L, bool narrow) { return c->sp64->line_table(L, narrow, 1); }, true));
