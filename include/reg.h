@@ -29,9 +29,10 @@
  * All work is ordered on the context's stream (a context created on the NULL
  * stream works on a stream of its own that first waits for what the NULL
  * stream holds); calls return after that work has finished (results are valid
- * on return). From their second call on, the sweeps of a context are captured
- * and replayed as CUDA graphs. A context is not thread-safe:
- * use one context per host thread.
+ * on return). From their second call on, the sweeps of a context are captured,
+ * on a private stream, and replayed as CUDA graphs on the context's stream,
+ * which other contexts and threads may use as well. A context is not
+ * thread-safe: use one context per host thread.
  *
  * Errors: every call returns a reg_status; reg_last_error() describes the most
  * recent failure of that context. No call aborts, traps or exits the process.
@@ -85,8 +86,9 @@ typedef enum {
  * coefficients, regularisation weight beta > 0, regulariser type, Stokes flag
  * gamma, precision of the matvec sweeps, state checkpoint interval
  * ckpt_every (0 = store the whole state trajectory; K > 0 = keep every K-th
- * state and recompute the others), and a cudaStream_t (NULL = the legacy
- * default stream). Requires n_t % ckpt_every == 0 when ckpt_every > 0.
+ * state and recompute the others), and a cudaStream_t (NULL or
+ * cudaStreamLegacy: a stream of the context's own, ordered behind the legacy
+ * default stream at every call). Requires n_t % ckpt_every == 0 when ckpt_every > 0.
  * Errors: REG_EINVAL, REG_ENOMEM, REG_ECUDA. On error *out is NULL. */
 REG_API reg_status reg_create(reg_ctx** out, int d, const int64_t* n, int n_t, int n_c, double beta, int reg_type,
                       int stokes, int precision, int ckpt_every, void* cuda_stream);

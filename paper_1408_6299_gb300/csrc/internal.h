@@ -200,6 +200,7 @@ class Spectral {
   }
   const Grid& grid() const { return g_; }
   cudaStream_t stream() const { return s_; }
+  void set_stream(cudaStream_t s) { s_ = s; }
   const void* line_table(int L, bool narrow, int kind) const { return lines_.get(L, narrow, kind); }
 
  private:

@@ -178,9 +178,11 @@ struct reg_ctx {
   Replay rp_state, rp_store, rp_adj, rp_hess;
   DBuf<double> vfix, gdir;
   // a context created on the NULL stream works on a stream of its own, ordered
-  // behind the NULL stream at every call (captures are not allowed there)
+  // behind the NULL stream at every call (graphs are not launched there)
   cudaStream_t own = nullptr;
   cudaEvent_t own_ev = nullptr;
+  // where sweeps are captured: nobody else enqueues on it
+  cudaStream_t cap = nullptr;
   // device-driven lockstep loops (stacked problems): per-problem scalars, the
   // control block, and the graphs of the PCG and line-search loops
   DBuf<double> lk;
@@ -194,6 +196,7 @@ struct reg_ctx {
     if (lk_ls) cudaGraphExecDestroy(lk_ls);
     if (own_ev) cudaEventDestroy(own_ev);
     if (own) cudaStreamDestroy(own);
+    if (cap) cudaStreamDestroy(cap);
   }
 
   long N() const { return g.N; }
@@ -837,13 +840,31 @@ size_t graph_signature(reg_ctx* c) {
   return h;
 }
 
+// The context's launches go to its private stream while this object lives. A
+// capture there takes in nothing that other threads or contexts enqueue on the
+// caller's stream, and their synchronisations do not break it.
+struct OnCaptureStream {
+  reg_ctx* c;
+  cudaStream_t s;
+  explicit OnCaptureStream(reg_ctx* c_) : c(c_), s(c_->s) {
+    if (!c->cap) REG_CUDA(cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking));
+    set(c->cap);
+  }
+  ~OnCaptureStream() { set(s); }
+  void set(cudaStream_t to) {
+    c->s = to;
+    c->sp64->set_stream(to);
+    if (c->sp32) c->sp32->set_stream(to);
+  }
+};
+
 // Runs body, a sequence of launches on the context's stream whose arguments
 // depend on the signature alone, as a graph where it repeats (see Replay).
 template <typename Body>
 void replay(reg_ctx* c, Replay& g, Body body) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (c->s) REG_CUDA(cudaStreamIsCapturing(c->s, &cs));
-  if (!c->s || c->prof.mask || cs != cudaStreamCaptureStatusNone) return body();  // timed by kernel, or inside a capture
+  REG_CUDA(cudaStreamIsCapturing(c->s, &cs));
+  if (c->prof.mask || cs != cudaStreamCaptureStatusNone) return body();  // timed by kernel, or inside a capture
   const size_t sig = graph_signature(c);
   if (!g.exec || g.sig != sig) {
     g.drop();
@@ -854,15 +875,18 @@ void replay(reg_ctx* c, Replay& g, Body body) {
     }
     const long l0 = launch_count();
     cudaGraph_t graph = nullptr;
-    REG_CUDA(cudaStreamBeginCapture(c->s, cudaStreamCaptureModeThreadLocal));
-    try {
-      body();
-    } catch (...) {
-      cudaStreamEndCapture(c->s, &graph);
-      if (graph) cudaGraphDestroy(graph);
-      throw;
+    {
+      OnCaptureStream on(c);
+      REG_CUDA(cudaStreamBeginCapture(c->s, cudaStreamCaptureModeThreadLocal));
+      try {
+        body();
+      } catch (...) {
+        cudaStreamEndCapture(c->s, &graph);
+        if (graph) cudaGraphDestroy(graph);
+        throw;
+      }
+      REG_CUDA(cudaStreamEndCapture(c->s, &graph));
     }
-    REG_CUDA(cudaStreamEndCapture(c->s, &graph));
     const cudaError_t e = cudaGraphInstantiate(&g.exec, graph, 0);
     cudaGraphDestroy(graph);
     REG_CUDA(e);
@@ -2147,7 +2171,7 @@ reg_ctx* create_ctx(int d, const int64_t* n, int n_t, int n_c, double beta, int 
   c->prec = precision;
   c->ckpt = ckpt_every;
   c->s = (cudaStream_t)cuda_stream;
-  if (!c->s) {
+  if (!c->s || c->s == cudaStreamLegacy) {  // two names of the NULL stream
     REG_CUDA(cudaEventCreateWithFlags(&c->own_ev, cudaEventDisableTiming));
     REG_CUDA(cudaStreamCreateWithFlags(&c->own, cudaStreamNonBlocking));
     c->s = c->own;

@@ -42,3 +42,95 @@ def test_fresh_context_reads_complete_tables():
         ref = ref or out
         assert all(torch.equal(a, b) for a, b in zip(out, ref)), k
         R.close()
+
+
+LEGACY, PER_THREAD = 1, 2  # cudaStreamLegacy, cudaStreamPerThread
+
+
+@pytest.mark.parametrize("handle", [LEGACY, PER_THREAD], ids=["legacy", "per-thread"])
+def test_special_stream_handles(handle):
+    # launched, captured and replayed; the inputs are written on the NULL stream just before
+    import torch
+    n = (32, 32)
+    v, u = coefs(n, 1, 0.1), field(n, 7)
+    R = lib.Registration(n, 6, 1, 1e-2, lib.REG_H1, False, lib.REG_FP64, 0, stream=handle)
+    one, g1, H1 = empty(n), empty(R.coef_shape()), empty(R.coef_shape())
+    R.set_images(u, field(n, 8))
+    R.transport(v, u, one)
+    R.gradient(v, g1)
+    R.hessvec(v, H1)
+    for k in range(1, 5):
+        x, m1, g, H = u.clone(), empty(n), empty(R.coef_shape()), empty(R.coef_shape())
+        x.mul_(2.0 ** k)  # exact, and transport is linear in the image
+        if handle == PER_THREAD:
+            torch.cuda.synchronize()
+        R.transport(v, x, m1)
+        R.gradient(v, g)
+        R.hessvec(v, H)
+        assert torch.equal(m1, one * 2.0 ** k) and torch.equal(g, g1) and torch.equal(H, H1), k
+    R.close()
+
+
+def test_stream_shared_with_other_threads():
+    # Two contexts and a counter, each in its own thread, on one stream. The contexts are made to capture again
+    # and again; what the others enqueue meanwhile has to run once, and their synchronisations to succeed.
+    import threading
+
+    import torch
+    n = (32, 32)
+    s = torch.cuda.Stream()
+    v, u = coefs(n, 1, 0.1), field(n, 7)
+    torch.cuda.synchronize()
+    refs, outs, errors, stop = {}, {0: [], 1: []}, [], threading.Event()
+    for n_t in (4, 6):
+        R = lib.Registration(n, n_t, 1, 1e-2, lib.REG_H1, False, lib.REG_FP64, 0)
+        refs[n_t] = empty(n)
+        R.transport(v, u, refs[n_t])
+        R.close()
+    counter = torch.zeros(1024, dtype=torch.float64, device="cuda")
+    bufs = {w: [torch.empty_like(u) for _ in range(120)] for w in outs}
+    torch.cuda.synchronize()
+
+    def guard(f):
+        def go():
+            try:
+                f()
+            except BaseException as e:
+                errors.append(repr(e))
+        return threading.Thread(target=go)
+
+    def context(w):
+        def go():
+            R = lib.Registration(n, 4, 1, 1e-2, lib.REG_H1, False, lib.REG_FP64, 0, stream=s.cuda_stream)
+            for i, m1 in enumerate(bufs[w]):
+                if i % 4 == 0:  # each setting twice launched, captured and replayed
+                    R.set_time_steps(6 if R.n_t == 4 else 4)
+                R.transport(v, u, m1)
+                outs[w].append(R.n_t)
+            R.close()
+        return go
+
+    added = [0]
+
+    def count():
+        with torch.cuda.stream(s):
+            while not stop.is_set():
+                counter.add_(1.0)
+                added[0] += 1
+                if added[0] % 64 == 0:
+                    s.synchronize()
+
+    workers, other = [guard(context(w)) for w in outs], guard(count)
+    other.start()
+    for t in workers:
+        t.start()
+    for t in workers:
+        t.join()
+    stop.set()
+    other.join()
+    torch.cuda.synchronize()
+    assert not errors, errors
+    assert added[0] and bool((counter == float(added[0])).all())
+    for w in outs:
+        for m1, n_t in zip(bufs[w], outs[w]):
+            assert torch.equal(m1, refs[n_t]), (w, n_t)
