@@ -2628,7 +2628,8 @@ reg_status reg_solve_lockstep(const reg_problem* problems, int count, int precis
       for (;;) {
         // a stack of the problems in `slot` (positions in ids), loaded from the callers' arrays
         const int B = (int)slot.size();
-        c = create_ctx(p0.d, p0.n, p0.n_t, p0.n_c, p0.beta, p0.reg_type, p0.stokes, precision, 0, st, B);
+        // beta: used where one problem is left (B = 1), else betas
+        c = create_ctx(p0.d, p0.n, p0.n_t, p0.n_c, problems[ids[slot[0]]].beta, p0.reg_type, p0.stokes, precision, 0, st, B);
         const long N1 = c->g.N1, N = c->N();
         const int K = c->n_c * c->d;
         c->betas.resize(B);

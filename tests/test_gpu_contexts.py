@@ -134,3 +134,26 @@ def test_stream_shared_with_other_threads():
     for w in outs:
         for m1, n_t in zip(bufs[w], outs[w]):
             assert torch.equal(m1, refs[n_t]), (w, n_t)
+
+
+def test_last_problem_of_a_stack_keeps_its_beta():
+    # seven of eight stacked problems start at their minimum, so the eighth goes on in a stack of its own
+    import torch
+    n = (32, 32)
+    u, mR = field(n, 7), empty(n)
+    M = lib.Registration(n, 8, 1, 1e-2, lib.REG_H1, False, lib.REG_FP64, 0)
+    M.transport(coefs(n, 1, 0.2), u, mR)
+    M.close()
+    probs = [dict(n=n, n_t=8, beta=1e-1 if i else 1e-3, mT=u, mR=u, v=torch.zeros((1, 2) + n, dtype=torch.float64,
+                                                                                 device="cuda")) for i in range(8)]
+    probs[5].update(mR=mR, beta=1e-2)
+    reps = lib.solve_lockstep(probs, lib.REG_FP64, grad_rtol=1e-3)
+    R = lib.Registration(n, 8, 1, 1e-2, lib.REG_H1, False, lib.REG_FP64, 0)
+    R.set_images(u, mR)
+    v = torch.zeros((1, 2) + n, dtype=torch.float64, device="cuda")
+    rep = R.solve(v, grad_rtol=1e-3)
+    for k in ("outer", "pcg_iters", "ls_trials", "status"):
+        assert reps[5][k] == rep[k], (k, reps[5][k], rep[k])
+    assert float((probs[5]["v"] - v).norm() / v.norm()) < 1e-9
+    assert abs(reps[5]["J"] - rep["J"]) <= 1e-11 * rep["J"]
+    R.close()
