@@ -151,6 +151,7 @@ struct reg_ctx {
   std::unique_ptr<Spectral<double>> sp64;
   std::unique_ptr<FieldTransforms> ft;
   DBuf<double> ik2;    // reciprocals of the squared wavenumbers (spec_tail, spec_precond)
+  bool ik2_filled = false;
   std::unique_ptr<Spectral<float>> sp32;
   Work<double> w64;
   Work<float> w32;
@@ -774,10 +775,16 @@ namespace {
 // Fourier-diagonal tail (FP64): out = beta (C (x) A) V + K^gamma F
 // (App. A Eq. control-equation-expansion; Eq. eliminated-control). F may be null.
 // ---------------------------------------------------------------------------
+// Null (the kernels then divide) inside a capture before the first use: the
+// filling would only be recorded.
 const double* inv_k2(reg_ctx* c) {
-  if (!c->ik2.p) {
+  if (!c->ik2_filled) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    REG_CUDA(cudaStreamIsCapturing(c->s, &cs));
+    if (cs != cudaStreamCaptureStatusNone) return nullptr;
     const long n = inv_k2_count(c->g);
     fill_inv_k2(c->ik2.get(n), n, c->s);
+    c->ik2_filled = true;
   }
   return c->ik2.p;
 }

@@ -157,3 +157,31 @@ def test_last_problem_of_a_stack_keeps_its_beta():
     assert float((probs[5]["v"] - v).norm() / v.norm()) < 1e-9
     assert abs(reps[5]["J"] - rep["J"]) <= 1e-11 * rep["J"]
     R.close()
+
+
+def test_call_refused_under_capture_leaves_nothing_half_done():
+    # a call synchronises, so a capture of the caller's refuses it; what it set up meanwhile was only recorded
+    import ctypes
+
+    import torch
+    drv = ctypes.CDLL("libcuda.so.1")
+    n = (32, 64)
+    r = coefs(n, 1, 1.0)
+    ref, z = empty((1, 2) + n), empty((1, 2) + n)
+    R = lib.Registration(n, 4, 1, 1e-2, lib.REG_H1, False, lib.REG_FP64, 0)
+    R.precond(r, ref)
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    S = lib.Registration(n, 4, 1, 1e-2, lib.REG_H1, False, lib.REG_FP64, 0, stream=s.cuda_stream)
+    graph = ctypes.c_void_p()
+    assert drv.cuStreamBeginCapture_v2(ctypes.c_void_p(s.cuda_stream), 2) == 0  # relaxed
+    try:
+        with pytest.raises(lib.RegError):
+            S.precond(r, z)
+    finally:
+        assert drv.cuStreamEndCapture(ctypes.c_void_p(s.cuda_stream), ctypes.byref(graph)) != 0
+    torch.cuda.synchronize()
+    S.precond(r, z)
+    assert torch.equal(z, ref)
+    S.close()
+    R.close()
