@@ -60,6 +60,7 @@ enum KernelKind {
 void count_launch();
 void add_launches(long n);  // kernels launched by a graph replay
 long launch_count();
+long thread_launch_count();  // those of count_launch() on this thread
 
 // Launch of a kernel that begins with chain_enter(): it may be set up while its
 // predecessor on the stream still runs, and waits there for its results. The

@@ -880,7 +880,7 @@ void replay(reg_ctx* c, Replay& g, Body body) {
       g.seen = graph_signature(c);
       return;
     }
-    const long l0 = launch_count();
+    const long l0 = thread_launch_count();
     cudaGraph_t graph = nullptr;
     {
       OnCaptureStream on(c);
@@ -897,7 +897,7 @@ void replay(reg_ctx* c, Replay& g, Body body) {
     const cudaError_t e = cudaGraphInstantiate(&g.exec, graph, 0);
     cudaGraphDestroy(graph);
     REG_CUDA(e);
-    g.kernels = launch_count() - l0;
+    g.kernels = thread_launch_count() - l0;
     add_launches(-g.kernels);
     g.sig = sig;
   }
@@ -2152,6 +2152,7 @@ reg_status fail(reg_ctx* c, int st, const std::string& msg) {
     return fail(c_, e.status, e.what);                                                                \
   }                                                                                                   \
   catch (const CudaError& e) {                                                                        \
+    (void)cudaGetLastError(); /* reported here, not by the next call too */                            \
     return fail(c_, e.code == cudaErrorMemoryAllocation ? REG_ENOMEM : REG_ECUDA, e.what);            \
   }                                                                                                   \
   catch (const std::bad_alloc&) {                                                                     \

@@ -458,7 +458,12 @@ void spec_upsample(const Grid& c, const Grid& f, cudaStream_t s, const double2* 
 namespace reg {
 
 static std::atomic<long> g_launches{0};
-void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
+static thread_local long tl_launches = 0;
+void count_launch() {
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+  ++tl_launches;
+}
+long thread_launch_count() { return tl_launches; }
 void add_launches(long n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 long launch_count() { return g_launches.load(std::memory_order_relaxed); }
 

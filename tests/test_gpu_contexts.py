@@ -137,26 +137,26 @@ def test_stream_shared_with_other_threads():
 
 
 def test_last_problem_of_a_stack_keeps_its_beta():
-    # seven of eight stacked problems start at their minimum, so the eighth goes on in a stack of its own
+    # seven of eight stacked problems start at their minimum, so the eighth goes on in a stack of its own: the
+    # iterates of that problem solved as a stack of one, bit for bit
     import torch
     n = (32, 32)
     u, mR = field(n, 7), empty(n)
     M = lib.Registration(n, 8, 1, 1e-2, lib.REG_H1, False, lib.REG_FP64, 0)
     M.transport(coefs(n, 1, 0.2), u, mR)
     M.close()
-    probs = [dict(n=n, n_t=8, beta=1e-1 if i else 1e-3, mT=u, mR=u, v=torch.zeros((1, 2) + n, dtype=torch.float64,
-                                                                                 device="cuda")) for i in range(8)]
-    probs[5].update(mR=mR, beta=1e-2)
-    reps = lib.solve_lockstep(probs, lib.REG_FP64, grad_rtol=1e-3)
-    R = lib.Registration(n, 8, 1, 1e-2, lib.REG_H1, False, lib.REG_FP64, 0)
-    R.set_images(u, mR)
-    v = torch.zeros((1, 2) + n, dtype=torch.float64, device="cuda")
-    rep = R.solve(v, grad_rtol=1e-3)
-    for k in ("outer", "pcg_iters", "ls_trials", "status"):
-        assert reps[5][k] == rep[k], (k, reps[5][k], rep[k])
-    assert float((probs[5]["v"] - v).norm() / v.norm()) < 1e-9
-    assert abs(reps[5]["J"] - rep["J"]) <= 1e-11 * rep["J"]
-    R.close()
+
+    def problem(ref, beta):
+        return dict(n=n, n_t=8, beta=beta, mT=u, mR=ref, v=torch.zeros((1, 2) + n, dtype=torch.float64, device="cuda"))
+
+    probs = [problem(u, 1e-1 if i else 1e-3) for i in range(8)]
+    probs[5] = problem(mR, 1e-2)
+    one = problem(mR, 1e-2)
+    rep = lib.solve_lockstep(probs, lib.REG_FP64, grad_rtol=1e-3)[5]
+    alone = lib.solve_lockstep([one], lib.REG_FP64, grad_rtol=1e-3)[0]
+    for k in ("outer", "pcg_iters", "ls_trials", "status", "J"):
+        assert rep[k] == alone[k], (k, rep[k], alone[k])
+    assert torch.equal(probs[5]["v"], one["v"])
 
 
 def test_call_refused_under_capture_leaves_nothing_half_done():
@@ -185,3 +185,26 @@ def test_call_refused_under_capture_leaves_nothing_half_done():
     assert torch.equal(z, ref)
     S.close()
     R.close()
+
+
+def test_launches_counted_alike_by_one_and_by_many_workers():
+    # eight problems of one shape and eight weights: one context each, whoever solves it
+    import torch
+    n = (32, 32)
+    u, mR = field(n, 7), empty(n)
+    M = lib.Registration(n, 8, 1, 1e-2, lib.REG_H1, False, lib.REG_FP64, 0)
+    M.transport(coefs(n, 1, 0.2), u, mR)
+    M.close()
+
+    def launches(workers):
+        probs = [dict(n=n, n_t=8, beta=1e-2 * (1 + i), mT=u, mR=mR, v=torch.zeros((1, 2) + n, dtype=torch.float64,
+                                                                                 device="cuda")) for i in range(8)]
+        before = lib.launch_count()
+        lib.solve_batched(probs, lib.REG_FP64, workers=workers, grad_rtol=1e-3)
+        return lib.launch_count() - before
+
+    launches(1)  # settles the autotuner
+    one = launches(1)
+    assert one > 0
+    for _ in range(3):
+        assert launches(8) == one
