@@ -524,27 +524,53 @@ struct BodyForce {
   }
 };
 
-// slot k of a ring of kForceNodes + 1 fields
+// Time nodes whose force terms a backward sweep collects before it adds them:
+// kForceNodes, or fewer where the rings that keep their operands, fields * K + more
+// fields for K nodes, would take more than `bytes`. The terms are added in the same
+// order in any case, so the sums do not depend on it.
 template <typename T>
-T* ring_slot(T* ring, int k, long stride) {
-  return ring + (long)(k % (kForceNodes + 1)) * stride;
+int force_group(const reg_ctx* c, int fields, int more, long bytes) {
+  int K = kForceNodes;
+  while (K > 1 && ((long)fields * K + more) * c->N() * (long)sizeof(T) > bytes) --K;
+  return K;
+}
+// The full Newton matvec keeps lam~, lam and the d fields of grad m~, the discrete
+// adjoint lam and its predictors: 1.2 GB, which bounds them to 3 nodes and 1 at 256^3
+// (single, double precision) and 4 (discrete adjoint, double). The trapezoid rule
+// keeps lam alone: 4.8 GB, 8 nodes up to 512^3 in single precision, 3 in double.
+constexpr long kRingBytes = 9L << 27, kLamRingBytes = 9L << 29;
+template <typename T>
+int adjoint_group(const reg_ctx* c) {
+  return c->quad ? force_group<T>(c, 2, 1, kRingBytes) : force_group<T>(c, 1, 1, kLamRingBytes);
+}
+template <typename T>
+int newton_group(const reg_ctx* c) {
+  return force_group<T>(c, 2 + c->d, 2, kRingBytes);
+}
+
+// entry k of a ring of `slots` entries: slots for K pending nodes, or K + 1 where the
+// next one is written before they are added
+template <typename T>
+T* ring_slot(T* ring, int k, int slots, long stride) {
+  return ring + (long)(k % slots) * stride;
 }
 
 // Adjoint solve (Eq. first-order-adjoint) backward from lam (in w.lam at n_t),
 // accumulating the body force f_l = int b_l lam grad m dt into f (double): the
 // trapezoid term of every node, or the two stage terms per step of the
 // discrete adjoint. lam (and the predictors of the discrete adjoint) are kept
-// for the nodes whose force is still to be added; lam_0 ends in slot n_t - 1.
+// for the nodes whose force is still to be added; lam_0 ends in entry n_t - 1.
 template <typename T>
 void adjoint_solve(reg_ctx* c, const T* vcoef, double* f) {
   Work<T>& w = work<T>(c);
   const long N = c->N();
   const double hd = c->h();
-  T* ring = w.lamR.get((size_t)(kForceNodes + 1) * N);
-  T* yhs = c->quad ? w.yhR.get((size_t)(kForceNodes + 1) * N) : w.yh.get(N);
+  const int group = adjoint_group<T>(c);
+  T* ring = w.lamR.get((size_t)(group + 1) * N);
+  T* yhs = c->quad ? w.yhR.get((size_t)group * N) : w.yh.get(N);
   BodyForce<T> bf(c, f);
   const T* lam = w.lam.p;
-  int k = 0;  // ring slots used
+  int k = 0;  // ring entries used
   const int K = c->ckpt > 0 ? c->ckpt : c->n_t;
   for (int seg = (c->n_t - 1) / K; seg >= 0; --seg) {
     int j0 = seg * K, j1 = j0 + K;
@@ -556,8 +582,8 @@ void adjoint_solve(reg_ctx* c, const T* vcoef, double* f) {
     }
     NodeVel<T> v(c, vcoef, w.va, w.vb);
     for (int j = j1 - 1; j >= j0; --j) {
-      T* yh = c->quad ? ring_slot(yhs, k, N) : yhs;
-      T* next = ring_slot(ring, k++, N);
+      T* yh = c->quad ? ring_slot(yhs, k, group, N) : yhs;
+      T* next = ring_slot(ring, k++, group + 1, N);
       divh<T>(c, lam, v.get(j + 1), lam, yh, 1);
       divh<T>(c, yh, v.get(j), lam, next, 2);
       if (!c->quad) {
@@ -567,7 +593,7 @@ void adjoint_solve(reg_ctx* c, const T* vcoef, double* f) {
         bf.also(yh, gm_slot<T>(c, j, base), j, 0.5 * hd);
       }
       lam = next;
-      if (bf.F.count == kForceNodes) bf.flush();
+      if (bf.F.count == group) bf.flush();
     }
     if (j0 == 0 && !c->quad) bf.add(lam, gm_slot<T>(c, 0, base), 0, c->trap_w(0));
   }
@@ -585,19 +611,19 @@ template <typename T>
 void newton_adjoint(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
   Work<T>& w = work<T>(c);
   const long N = c->N(), dN = c->dN();
-  const size_t slots = kForceNodes + 1;
+  const int group = newton_group<T>(c), slots = group + 1;
   T* yh = w.yh.get(N);
   T* yh2 = w.yh2.get(N);
   T* sA = w.st0.get(N);
   T* sB = w.st1.get(N);
-  T* ringT = w.lamR.get(slots * N);  // lam~
-  T* ringL = w.lamN.get(slots * N);  // lam
-  T* Gt = w.Gt.get(slots * dN);
+  T* ringT = w.lamR.get((size_t)slots * N);  // lam~
+  T* ringL = w.lamN.get((size_t)slots * N);  // lam
+  T* Gt = w.Gt.get((size_t)group * dN);
   const T* mtil = w.mtil.p;
   BodyForce<T> bf(c, f);
   const T* lt = w.lam.p;
   // lam_1 = m_R - m_1 and the source at t_1
-  T* lam1 = ring_slot(ringL, kForceNodes, N);
+  T* lam1 = ring_slot(ringL, group, slots, N);
   lincomb_t<T>((T)1, w.mR.p, (T)-1, w.m1.p, lam1, N, c->s);
   const T* lam = lam1;
   NodeVel<T> vt(c, wcoef, w.wa, w.wb);
@@ -614,9 +640,9 @@ void newton_adjoint(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
     }
     NodeVel<T> v(c, vcoef, w.va, w.vb);
     for (int j = j1 - 1; j >= j0; --j) {
-      T* gt = ring_slot(Gt, k, dN);
-      T* lt2 = ring_slot(ringT, k, N);
-      T* lam2 = ring_slot(ringL, k, N);
+      T* gt = ring_slot(Gt, k, group, dN);
+      T* lt2 = ring_slot(ringT, k, slots, N);
+      T* lam2 = ring_slot(ringL, k, slots, N);
       ++k;
       // force of node j+1
       grad_fused<T>(c, mtil + (long)(j + 1) * N, gt);
@@ -639,7 +665,7 @@ void newton_adjoint(reg_ctx* c, const T* vcoef, const T* wcoef, double* f) {
       std::swap(sA, sB);  // the source at t_j is the next step's source at t_{j+1}
       lt = lt2;
       lam = lam2;
-      if (bf.F.count == kForceNodes) bf.flush();
+      if (bf.F.count == group) bf.flush();
     }
     if (j0 == 0)  // node 0: m~_0 = 0, so only the Gauss-Newton term
       bf.add(lt, gm_slot<T>(c, 0, base), 0, c->trap_w(0));
@@ -2365,7 +2391,7 @@ reg_status reg_transport_adjoint(reg_ctx* ctx, const double* v, const double* m0
   lincomb_t<double>(-1.0, Gd, 0.0, nullptr, w.lam.get(N), N, c_->s);  // lam_1 = -G
   double* f = c_->f.get(c_->ncdN());
   replay(c_, c_->rp_adj, [&] { adjoint_solve<double>(c_, vc, f); });
-  const double* lam0 = ring_slot(w.lamR.p, c_->n_t - 1, N);  // where the last step left lam_0
+  const double* lam0 = ring_slot(w.lamR.p, c_->n_t - 1, adjoint_group<double>(c_) + 1, N);  // where the last step left lam_0
   if (grad_v) {
     Output o(c_, grad_v, c_->ncdN(), c_->stage_out);
     REG_CUDA(cudaMemcpyAsync(o.dev, f, c_->ncdN() * sizeof(double), cudaMemcpyDeviceToDevice, c_->s));

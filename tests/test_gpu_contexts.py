@@ -208,3 +208,82 @@ def test_launches_counted_alike_by_one_and_by_many_workers():
     assert one > 0
     for _ in range(3):
         assert launches(8) == one
+
+
+@pytest.mark.parametrize("n_t,ckpt", [(20, 0), (20, 4), (20, 10), (9, 9)])
+def test_newton_over_more_nodes_than_a_force_group(n_t, ckpt):
+    # the rings of the backward sweep wrap; tolerances of the Newton parity tests
+    from oracle import oracle as O
+    from paper_1408_6299_gb300 import synth
+    from gpu_util import cuda, host, pair, rel
+    c = synth.stokes_3d(16, n_t=n_t, n_c=3)
+    P = O.Problem(c["n"], n_t, c["n_c"], c["beta"], c["reg"], c["stokes"])
+    mR = P.state(c["v_true"], c["mT"])[-1]
+    v = 0.5 * c["v_true"]
+    ref = P.hessvec_newton(v, c["mT"], mR, c["vt"])
+    for precision, tol in ((lib.REG_FP64, 1e-10), (lib.REG_MIXED, 1e-5)):
+        R, _ = pair(c, precision=precision, ckpt=ckpt)
+        R.set_hessian(lib.REG_HESS_NEWTON)
+        R.set_images(cuda(c["mT"]), cuda(mR))
+        R.linearize(cuda(v))
+        Hv = empty(R.coef_shape())
+        for _ in range(3):  # launched, captured and replayed
+            R.hessvec(cuda(c["vt"]), Hv)
+            assert rel(host(Hv), ref) < tol
+        R.close()
+
+
+# grids whose rings hold fewer than eight nodes: full Newton 3 and 1, discrete adjoint 4, trapezoid 3
+@pytest.mark.parametrize("what,n,n_t,ckpt", [
+    ("newton", (256, 256, 128), 7, 0), ("newton", (256, 256, 256), 5, 0), ("newton", (256, 256, 128), 8, 4),
+    ("adjoint", (256, 256, 256), 9, 0), ("gradient", (512, 512, 512), 5, 0)])
+def test_rings_bounded_by_memory(what, n, n_t, ckpt):
+    # fields that do not vary along the first axis: the same on 8 points there, where the rings hold eight nodes
+    import torch
+    small = (8,) + n[1:]
+    d, size = 3, 0.4 * n_t / (3 * max(n) / 2)
+    out = []
+    for m in (small, n):
+        def make(seed, count=None):
+            f = torch.stack([field(small[1:], seed + i) for i in range(count or 1)])
+            f = f[:, None].expand((count or 1,) + m).contiguous()
+            return f[None] if count else f[0]
+        R = lib.Registration(m, n_t, 1, 1e-2, lib.REG_H1, False, lib.REG_FP64, ckpt,
+                             quadrature=lib.REG_QUAD_DISCRETE if what == "adjoint" else lib.REG_QUAD_TRAPEZOID,
+                             hessian=lib.REG_HESS_NEWTON if what == "newton" else lib.REG_HESS_GN)
+        u, v, res = make(7), make(20, d) * size, empty((1, d) + m)
+        if what == "adjoint":
+            gm = empty(m)
+            R.transport_adjoint(v, u, make(8), res, gm)
+            out.append([res[0, :, :8].clone(), gm[:8].clone()])
+        else:
+            R.set_images(u, make(8))
+            if what == "gradient":
+                R.gradient(v, res)
+            else:
+                R.linearize(v)
+                R.hessvec(make(30, d), res)
+            out.append([res[0, :, :8].clone()])
+        R.close()
+        del R, u, v, res
+        torch.cuda.empty_cache()
+    for a, b in zip(*out):
+        assert float((a - b).norm() / b.norm()) < 1e-10
+
+
+def test_newton_matvec_memory():
+    # 59 fields of a store-all context with two steps; the matvec held 58 before its body force was summed in
+    # groups, and five more fields than that are allowed here
+    import torch
+    n = (256, 256, 128)
+    u, v = field(n, 7), coefs(n, 1, 0.001)
+    Hv = torch.empty_like(v)
+    R = lib.Registration(n, 2, 1, 1e-2, lib.REG_H1, False, lib.REG_FP64, 0, hessian=lib.REG_HESS_NEWTON)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    R.set_images(u, u)
+    R.linearize(v)
+    R.hessvec(v, Hv)
+    assert (free - torch.cuda.mem_get_info()[0]) / (8.0 * u.numel()) < 63
+    R.close()
