@@ -71,7 +71,10 @@ void cols_tuned(const Spectral<T>& sp, const ColJob<T>* jobs, int nj, cudaStream
   };
   const long n = sp.grid().N;
   if (sizeof(T) == 4 && n * (long)sizeof(T) > (16 << 20)) return run(0);
-  run(tuned_choice(PROD ? "cols|prod" : "cols|plain", sizeof(T), L, tune_size(n * nj), 2, st, run));
+  const char* kind = NARROW ? (PROD ? "cols|prod|narrow" : "cols|plain|narrow")
+                            : A::CW == 2 ? (PROD ? "cols|prod|pair" : "cols|plain|pair")
+                                         : (PROD ? "cols|prod|wide" : "cols|plain|wide");
+  run(tuned_choice(kind, sizeof(T), L, tune_size(n * nj), 2, st, run));
 }
 
 template <typename T, int L, bool PROD>

@@ -232,7 +232,7 @@ void FieldTransforms::fwd(const double* u, double2* U, int nf) const {
         else
           chain(k_field_rows_fwd<L, NW, 1>, (unsigned)((lines + F1::NSEQ - 1) / F1::NSEQ), F1::NT, s_, u, U, rows, tw);
       };
-      run(tuned_ ? tuned_choice("rows_r2c", sizeof(double), L, tune_size(rows), 2, s_, run) : 0);
+      run(tuned_ ? tuned_choice(NW ? "rows_r2c|narrow" : "rows_r2c|wide", sizeof(double), L, tune_size(rows), 2, s_, run) : 0);
     });
   });
   for (int a = g_.d - 2; a >= 0; --a) cols(U, a, nf, false);

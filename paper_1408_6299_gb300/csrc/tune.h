@@ -14,7 +14,8 @@
 
 namespace reg {
 
-// Variant 0..nv-1 for pass `kind` on elements of `size` bytes, lines of length
+// Variant 0..nv-1 for pass `kind` (which names the line plan: sizes are rounded, so
+// two plans may meet in one size) on elements of `size` bytes, lines of length
 // L and `work` lines: the choice of this process for the shape, or the
 // persistent one (tune.cu), else, outside a stream capture, each variant runs
 // three times on the call's own buffers after one untimed run, timed with

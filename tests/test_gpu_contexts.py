@@ -287,3 +287,37 @@ def test_newton_matvec_memory():
     R.hessvec(v, Hv)
     assert (free - torch.cuda.mem_get_info()[0]) / (8.0 * u.numel()) < 63
     R.close()
+
+
+def stack(n, count, n_t=2):
+    """count problems of one shape, the first two the same in every stack."""
+    import torch
+    out = []
+    for i in range(count):
+        u = field(n, 7 + i)
+        out.append(dict(n=n, n_t=n_t, beta=1e-2, mT=u, mR=torch.roll(u, 1, 0).contiguous(),
+                        v=torch.zeros((1, 2) + n, dtype=torch.float64, device="cuda")))
+    return out
+
+
+TUNED_STACKS = r"""
+import sys
+sys.path[:0] = [%r, %r]
+from test_gpu_contexts import stack
+from paper_1408_6299_gb300 import lib
+for count in (37, 39):  # on either side of the line between the plans, one rounded size
+    lib.solve_lockstep(stack((256, 256), count), lib.REG_MIXED, max_outer=1)
+"""
+
+
+def test_tuner_keeps_the_plans_apart(tmp_path):
+    import json
+    import os
+    import subprocess
+    import sys
+    here = os.path.dirname(os.path.abspath(__file__))
+    cache = tmp_path / "tune_cache.json"
+    subprocess.run([sys.executable, "-c", TUNED_STACKS % (os.path.dirname(here), here)], check=True, timeout=600,
+                   env=dict(os.environ, REG_TUNE_CACHE=str(cache)))
+    keys = [k for k in json.loads(cache.read_text()) if "cols|plain" in k and k.endswith("|f32|L256|n4194304")]
+    assert len(keys) == 2, keys
