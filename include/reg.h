@@ -360,7 +360,8 @@ REG_API reg_status reg_solve_batched(const reg_problem* problems, int count, int
  * Alg. 1 (PCG or Picard, CFL halving, line search, stopping rule: opts) runs
  * for all problems of a stack at once with per-problem Krylov and line-search
  * scalars, so each problem takes the iterates it would take alone (up to the
- * order of its inner-product sums); a problem that stops keeps its iterate
+ * order of its inner-product sums and, with REG_MIXED, the rounding of its
+ * single-precision sweeps); a problem that stops keeps its iterate
  * while the others continue. Stacks run concurrently, one stream each.
  * Checkpointing is off (every state gradient is stored). Arrays may be host
  * or device memory; reports (may be NULL): one per problem, in the order of

@@ -170,6 +170,11 @@ size_t write_wide_tables(unsigned char* out, long* off);
 // narrow; 128^3 mixed matvec, checkpoints every 8, 16.5 ms with this limit at
 // half, 12.6 here, 14.1 at double; 256^3 mixed matvec 180 ms wide, 246 narrow.
 inline bool narrow_lines(long wide_threads, int size) { return wide_threads < 152L * (size == 8 ? 1024 : 512); }
+// The lines that count for it. Plans round differently. In double precision the
+// plan follows the size of one problem, so that a problem has the same bits in any
+// stack and after its stack is rebuilt; in single precision that of the whole stack,
+// which a narrow plan would slow down by up to 1.4 (256^3 above).
+inline long plan_lines(const Grid& g, long lines, int size) { return size == 8 ? lines / g.B : lines; }
 
 // A grid with its stream and line tables in precision T: what the stages run on.
 template <typename T>

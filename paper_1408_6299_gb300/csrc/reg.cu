@@ -1550,9 +1550,12 @@ int continuation(reg_ctx* c, double* v, const reg_solve_opts& so, const reg_cont
 // Stacked problems (g.B > 1): per-problem objective and gradient, and the
 // outer loop of Alg. 1 run for all problems in lockstep. Every kernel of a
 // matvec, gradient or objective evaluation covers all problems at once; the
-// Krylov and line-search scalars are per problem, so each problem follows
-// exactly the iteration it would follow alone. A problem that has stopped
-// keeps its iterate: its update coefficients are zero.
+// Krylov and line-search scalars are per problem, so each problem follows the
+// iteration it would follow alone: in double precision the same bits in any
+// stack (and those of a single solve up to the order of its inner products), in
+// the mixed mode up to the rounding of its sweeps, whose plans follow the size of
+// the stack. A problem that has stopped keeps its iterate: its update coefficients
+// are zero.
 // ---------------------------------------------------------------------------
 struct Seg {
   reg_ctx* c;

@@ -81,7 +81,7 @@ template <typename T, int L, bool PROD>
 void cols_L(const Spectral<T>& sp, const ColJob<T>* jobs, int nj, cudaStream_t st) {
   using A = typename Arith<T>::Main;
   const Grid& g = sp.grid();
-  const long threads = (long)nj * g.Nc / L * LinePlan<L, false>::TS;
+  const long threads = plan_lines(g, (long)nj * g.Nc / L, sizeof(T)) * LinePlan<L, false>::TS;
   if (narrow_lines(threads, sizeof(T))) return cols_tuned<A, T, L, true, PROD>(sp, jobs, nj, st);
   if constexpr (sizeof(T) == 4)
     if (threads >= 2 * 152 * 512) return cols_tuned<LinePair, T, L, false, PROD>(sp, jobs, nj, st);
@@ -100,7 +100,7 @@ bool one_cols_launch(const Grid& g, int nj) {
     const int L = (int)g.n[a];
     if (L > 256) return false;
     const int wide_ts = L > 64 ? L / 16 : (L == 16 ? 1 : L / 8);
-    if (!narrow_lines((long)(nj / 2) * g.Nc / L * wide_ts, sizeof(T))) return false;
+    if (!narrow_lines(plan_lines(g, (long)(nj / 2) * g.Nc / L, sizeof(T)) * wide_ts, sizeof(T))) return false;
   }
   return sizeof(T) == 4 || nj * g.Nc / 4 <= 152L * kTwoNT;
 }
@@ -186,7 +186,7 @@ void rows_L(const Spectral<T>& sp, const RowArgs<T>& a, double bytes, cudaStream
   // 1627 -> 1426. Double precision, bound by arithmetic, loses earlier: 64^3
   // gradient (2048 lines) 3790 -> 3940 us
   const long few = 152L * (sizeof(T) == 8 ? 8 : 24);
-  if (!narrow_lines(lines * LinePlan<L, false>::TS, sizeof(T))) go(std::false_type{}, std::false_type{});
+  if (!narrow_lines(plan_lines(sp.grid(), lines, sizeof(T)) * LinePlan<L, false>::TS, sizeof(T))) go(std::false_type{}, std::false_type{});
   else if (lines <= few) go(std::true_type{}, std::true_type{});
   else go(std::true_type{}, std::false_type{});
 }

@@ -321,3 +321,15 @@ def test_tuner_keeps_the_plans_apart(tmp_path):
                    env=dict(os.environ, REG_TUNE_CACHE=str(cache)))
     keys = [k for k in json.loads(cache.read_text()) if "cols|plain" in k and k.endswith("|f32|L256|n4194304")]
     assert len(keys) == 2, keys
+
+
+def test_double_precision_bits_do_not_depend_on_the_stack():
+    # the larger stack alone would run wide plans
+    import torch
+    n, vs = (256, 256), []
+    for count in (2, 80):
+        probs = stack(n, count)
+        lib.solve_lockstep(probs, lib.REG_FP64, max_outer=1)
+        vs.append([p["v"] for p in probs[:2]])
+    for a, b in zip(*vs):
+        assert bool(a.any()) and torch.equal(a, b)
