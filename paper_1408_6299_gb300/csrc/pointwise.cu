@@ -10,6 +10,7 @@
 #include <type_traits>
 
 #include "pointwise.h"
+#include "velsum.cuh"
 
 namespace reg {
 
@@ -32,13 +33,22 @@ struct One {
   T v[1];
 };
 
-// Weights of a velocity combination. In single precision every weight is a
-// pair of floats: products and sums keep their rounding errors and the sum is
-// rounded once, accurate to the last bit without the double-precision unit
-// (two operations per clock and SM).
+// Weights of a velocity combination, and the sum over the coefficients
 template <typename T>
 struct NodeWeights {
-  T hi[16], lo[16];
+  double w[16];
+  struct Sum {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double c, double u) { s += c * u; }
+    __device__ __forceinline__ double rounded() const { return s; }
+  };
+  void set(int l, double c) { w[l] = c; }
+};
+template <>
+struct NodeWeights<float> {
+  FloatWeight w[16];
+  using Sum = FloatSum;
+  void set(int l, double c) { w[l] = split_weight(c); }
 };
 // The velocity at up to kVelGroup nodes, dN values each. NC: n_c where it is 2,
 // 3 or 4 (the loads of a point are then issued together and serve every node:
@@ -68,27 +78,17 @@ __global__ void __launch_bounds__(128) k_vel_at(const T* __restrict__ coef, int 
   for (int k = 0; k < kVelGroup; ++k) {
     if (k == nodes.count) return;
     const NodeWeights<T>& b = nodes.b[k];
-    Q s{}, err{};
+    typename NodeWeights<T>::Sum sum[Q::W];
 #pragma unroll
     for (int l = 0; l < nc; ++l) {
       if (!NC) v[0] = c[l * n];
       const Q u = v[NC ? l : 0];
 #pragma unroll
-      for (int w = 0; w < Q::W; ++w) {
-        if constexpr (sizeof(T) == 8) {
-          s.v[w] += b.hi[l] * u.v[w];
-        } else {
-          const float p = __fmul_rn(b.hi[l], u.v[w]);
-          const float e = fmaf(b.hi[l], u.v[w], -p) + b.lo[l] * u.v[w];
-          const float t = __fadd_rn(s.v[w], p), z = __fsub_rn(t, s.v[w]);
-          err.v[w] += e + __fadd_rn(__fsub_rn(s.v[w], __fsub_rn(t, z)), __fsub_rn(p, z));
-          s.v[w] = t;
-        }
-      }
+      for (int w = 0; w < Q::W; ++w) sum[w].add(b.w[l], u.v[w]);
     }
-    if (sizeof(T) == 4)
+    Q s;
 #pragma unroll
-      for (int w = 0; w < Q::W; ++w) s.v[w] += err.v[w];
+    for (int w = 0; w < Q::W; ++w) s.v[w] = sum[w].rounded();
     reinterpret_cast<Q*>(out)[k * n + x] = s;
   }
 }
@@ -367,8 +367,7 @@ void vel_at(const T* coef, int nc, const Coefs* b, int count, T* out, long dN, c
   for (int k = 0; k < kVelGroup; ++k)
     for (int l = 0; l < 16; ++l) {
       const double c = k < count && l < nc ? b[k].c[l] : 0.0;
-      w.b[k].hi[l] = (T)c;
-      w.b[k].lo[l] = (T)(c - (double)w.b[k].hi[l]);
+      w.b[k].set(l, c);
     }
   const bool vec = ((reinterpret_cast<uintptr_t>(coef) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
   auto kern = !vec ? k_vel_at<T, 0, false>
