@@ -33,21 +33,42 @@ struct One {
   T v[1];
 };
 
-// Weights of a velocity combination, and the sum over the coefficients
+// Weights of a velocity combination, and the sum over the coefficients (velsum.cuh
+// for single precision, four values as two pairs)
 template <typename T>
 struct NodeWeights {
   double w[16];
+  template <int W>
   struct Sum {
-    double s = 0.0;
-    __device__ __forceinline__ void add(double c, double u) { s += c * u; }
-    __device__ __forceinline__ double rounded() const { return s; }
+    double s[W];
+    __device__ __forceinline__ void add(int l, double c, const double* u) {
+#pragma unroll
+      for (int k = 0; k < W; ++k) s[k] = l ? s[k] + c * u[k] : c * u[k];
+    }
+    __device__ __forceinline__ void rounded(double* r) const {
+#pragma unroll
+      for (int k = 0; k < W; ++k) r[k] = s[k];
+    }
   };
   void set(int l, double c) { w[l] = c; }
 };
 template <>
 struct NodeWeights<float> {
   FloatWeight w[16];
-  using Sum = FloatSum;
+  template <int W>
+  struct Sum {
+    static constexpr int P = W > 1 ? 2 : 1;
+    using V = std::conditional_t<P == 2, float2, float>;
+    FloatSum<V> s[W / P];
+    __device__ __forceinline__ void add(int l, const FloatWeight& c, const float* u) {
+#pragma unroll
+      for (int k = 0; k < W / P; ++k) s[k].add(l, c, reinterpret_cast<const V*>(u)[k]);
+    }
+    __device__ __forceinline__ void rounded(float* r) const {
+#pragma unroll
+      for (int k = 0; k < W / P; ++k) s[k].rounded(r + k * P);
+    }
+  };
   void set(int l, double c) { w[l] = split_weight(c); }
 };
 // The velocity at up to kVelGroup nodes, dN values each. NC: n_c where it is 2,
@@ -78,17 +99,14 @@ __global__ void __launch_bounds__(128) k_vel_at(const T* __restrict__ coef, int 
   for (int k = 0; k < kVelGroup; ++k) {
     if (k == nodes.count) return;
     const NodeWeights<T>& b = nodes.b[k];
-    typename NodeWeights<T>::Sum sum[Q::W];
+    typename NodeWeights<T>::template Sum<Q::W> sum;
 #pragma unroll
     for (int l = 0; l < nc; ++l) {
       if (!NC) v[0] = c[l * n];
-      const Q u = v[NC ? l : 0];
-#pragma unroll
-      for (int w = 0; w < Q::W; ++w) sum[w].add(b.w[l], u.v[w]);
+      sum.add(l, b.w[l], v[NC ? l : 0].v);
     }
     Q s;
-#pragma unroll
-    for (int w = 0; w < Q::W; ++w) s.v[w] = sum[w].rounded();
+    sum.rounded(s.v);
     reinterpret_cast<Q*>(out)[k * n + x] = s;
   }
 }

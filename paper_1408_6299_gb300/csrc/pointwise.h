@@ -12,7 +12,7 @@ struct Coefs {
 
 constexpr int kVelGroup = 4;
 // out[k*dN + x] = sum_l b[k]_l coef[l*dN + x], x < dN, k < count <= kVelGroup,
-// rounded once to T
+// rounded once to T; b[k]_0 = 1 (T_0)
 template <typename T>
 void vel_at(const T* coef, int nc, const Coefs* b, int count, T* out, long dN, cudaStream_t s);
 inline void vel_at(const double* coef, int nc, const Coefs& b, double* out, long dN, cudaStream_t s) {
