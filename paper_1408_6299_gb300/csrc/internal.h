@@ -260,17 +260,19 @@ void div_stage(Spectral<T>& sp, const T* lam, const T* a, const fused::DivEpi<T>
 // Fourier-diagonal operators on whole coefficient vectors (FP64), with the
 // DC/Nyquist pairing of the packed last-axis slot 0.
 // ---------------------------------------------------------------------------
-// inv_k2 (device): 1/m for m = 1 .. sum_a (n_a/2)^2 at [m], the reciprocals of
-// every squared wavenumber; null: computed per mode.
+// Tables of every squared wavenumber m = 1 .. sum_a (n_a/2)^2, at [m] (device):
+// 1 / (beta m^reg), rounded as one division.
 long inv_k2_count(const Grid& g);
-void fill_inv_k2(double* inv_k2, long count, cudaStream_t s);
+void fill_inv_k2(double* t, long count, double beta, int reg, cudaStream_t s);
 // out_l = beta sum_l' Cg[l][l'] a(k) V_l' + (stokes ? K F_l : F_l); F may be null.
 // betas (device, may be null): one beta per stacked problem, replacing beta.
+// inv_k2: the table of 1 / m; null: divided per mode
 void spec_tail(const Grid& g, cudaStream_t s, const double2* V, const double2* F, double2* out, int nc,
                double beta, const double* Cg_dev, int reg, int stokes, const double* betas, const double* inv_k2);
 // out_l = sum_l' Ci[l][l'] s(k) R_l' with s = 1/(beta a(k)), s = 1 at k = 0.
+// inv: the table of 1 / (beta m^reg); null: divided per mode
 void spec_precond(const Grid& g, cudaStream_t s, const double2* R, double2* out, int nc, double beta,
-                  const double* Ci_dev, int reg, const double* betas, const double* inv_k2);
+                  const double* Ci_dev, int reg, const double* betas, const double* inv);
 // Gaussian filter exp(-sigma^2 |k|^2 / 2) of one packed FP64 field (out may not alias U)
 void spec_gauss(const Grid& g, cudaStream_t s, double2* U, double2* out, double sigma);
 // trigonometric interpolation of nfields packed FP64 spectra of grid c onto the

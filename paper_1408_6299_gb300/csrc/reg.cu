@@ -150,8 +150,8 @@ struct reg_ctx {
 
   std::unique_ptr<Spectral<double>> sp64;
   std::unique_ptr<FieldTransforms> ft;
-  DBuf<double> ik2;    // reciprocals of the squared wavenumbers (spec_tail, spec_precond)
-  bool ik2_filled = false;
+  DBuf<double> ik2, ipk;     // tables of 1 / |k|^2 (spec_tail) and 1 / (beta a(k)) (spec_precond)
+  double ik2_beta = 0, ipk_beta = 0;  // the beta they are filled for (0: not filled)
   std::unique_ptr<Spectral<float>> sp32;
   Work<double> w64;
   Work<float> w32;
@@ -803,16 +803,16 @@ namespace {
 // ---------------------------------------------------------------------------
 // Null (the kernels then divide) inside a capture before the first use: the
 // filling would only be recorded.
-const double* inv_k2(reg_ctx* c) {
-  if (!c->ik2_filled) {
+const double* inv_table(reg_ctx* c, DBuf<double>& t, double& filled, double beta, int reg) {
+  if (filled != beta) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     REG_CUDA(cudaStreamIsCapturing(c->s, &cs));
     if (cs != cudaStreamCaptureStatusNone) return nullptr;
     const long n = inv_k2_count(c->g);
-    fill_inv_k2(c->ik2.get(n), n, c->s);
-    c->ik2_filled = true;
+    fill_inv_k2(t.get(n), n, beta, reg, c->s);
+    filled = beta;
   }
-  return c->ik2.p;
+  return t.p;
 }
 
 // Without the Leray projection the body force passes the tail unchanged, so it
@@ -826,7 +826,7 @@ void tail(reg_ctx* c, const double* V, const double* F, double* out) {
   c->ft->fwd(V, SV, ncd);
   if (fspec) c->ft->fwd(F, SF, ncd);
   spec_tail(c->g, c->s, SV, fspec ? SF : nullptr, SF, c->n_c, c->beta, c->Cg_dev.p, c->rtype, c->stokes,
-            c->g.B > 1 ? c->betas_dev.p : nullptr, inv_k2(c));
+            c->g.B > 1 ? c->betas_dev.p : nullptr, fspec ? inv_table(c, c->ik2, c->ik2_beta, 1.0, 1) : nullptr);
   c->ft->inv(SF, out, ncd);
   if (F && !fspec) lincomb_t<double>(1.0, out, 1.0, F, out, (long)ncd * N, c->s);
 }
@@ -837,8 +837,9 @@ void precond(reg_ctx* c, const double* r, double* z) {
   double2* SV = c->SV.get((size_t)ncd * Nc);
   double2* SF = c->SF.get((size_t)ncd * Nc);
   c->ft->fwd(r, SV, ncd);
-  spec_precond(c->g, c->s, SV, SF, c->n_c, c->beta, c->Ci_dev.p, c->rtype, c->g.B > 1 ? c->betas_dev.p : nullptr,
-               inv_k2(c));
+  const bool one = c->g.B == 1;  // a stack has a beta per problem: divided per mode
+  spec_precond(c->g, c->s, SV, SF, c->n_c, c->beta, c->Ci_dev.p, c->rtype, one ? nullptr : c->betas_dev.p,
+               one ? inv_table(c, c->ipk, c->ipk_beta, c->beta, c->rtype) : nullptr);
   c->ft->inv(SF, z, ncd);
 }
 

@@ -77,18 +77,20 @@ __device__ inline int lead_k2(const ModeIdx& m, const GridArgs& g) {
   }
   return kk;
 }
-// |k|^2 or |k|^4 (exact: |k|^2 <= 3 256^2) and its reciprocal
+// |k|^2 or |k|^4 (exact: |k|^2 <= 3 256^2)
 __device__ inline double sym_pow(int kk, int reg) { return (double)(reg == 1 ? (long long)kk : (long long)kk * kk); }
-__device__ inline double inv_pow(int kk, int reg, const double* __restrict__ inv_k2) {
-  const double r = inv_k2 ? __ldg(&inv_k2[kk]) : 1.0 / (double)kk;
-  return reg == 1 ? r : r * r;
+// p / kk from the rounded reciprocal w = 1 / kk: the remainder corrects the product
+__device__ inline double quotient(double p, double w, double kk) {
+  const double q = p * w;
+  return fma(w, fma(-q, kk, p), q);
 }
 
 constexpr int kMaxNc = 16;
 
-__global__ void k_inv_k2(double* t, long n) {
+// t[m] = 1 / (beta m^reg)
+__global__ void k_inv_k2(double* t, long n, double beta, int reg) {
   const long m = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (m < n) t[m] = m ? 1.0 / (double)m : 0.0;
+  if (m < n) t[m] = m ? 1.0 / (beta * sym_pow((int)m, reg)) : 0.0;
 }
 
 // NC: n_c where it is 1, 2 or 3 (the coefficients of a component then stay in
@@ -147,6 +149,8 @@ __global__ void __launch_bounds__(256) k_spec_tail(const double2* __restrict__ V
     return r;
   };
   // k . f_l / |k|^2; out may be F, so it is formed before any component of f_l is overwritten
+  const double wk = kt2 > 0 && F && stokes ? (inv_k2 ? __ldg(&inv_k2[kt2]) : 1.0 / (double)kt2) : 0.0;
+  auto over_k2 = [&](double2 p) { return make_double2(quotient(p.x, wk, (double)kt2), quotient(p.y, wk, (double)kt2)); };
   auto projection = [&](int l) {
     double2 p = make_double2(0, 0);
     if (!(F && stokes && kt2 > 0)) return p;
@@ -155,8 +159,7 @@ __global__ void __launch_bounds__(256) k_spec_tail(const double2* __restrict__ V
       p.x += (double)kt[a] * fa.x;
       p.y += (double)kt[a] * fa.y;
     }
-    const double w = inv_pow(kt2, 1, inv_k2);
-    return make_double2(p.x * w, p.y * w);
+    return over_k2(p);
   };
   auto store = [&](int i, int l, double2 r, double2 p) {
     if (F) {
@@ -180,8 +183,7 @@ __global__ void __launch_bounds__(256) k_spec_tail(const double2* __restrict__ V
     if (leray) {
 #pragma unroll
       for (int a = 0; a < d; ++a) p = make_double2(p.x + (double)kt[a] * f[a].x, p.y + (double)kt[a] * f[a].y);
-      const double w = inv_pow(kt2, 1, inv_k2);
-      p = make_double2(p.x * w, p.y * w);
+      p = over_k2(p);
     }
 #pragma unroll
     for (int i = 0; i < d; ++i) {
@@ -213,18 +215,18 @@ __global__ void __launch_bounds__(256) k_spec_tail(const double2* __restrict__ V
   }
 }
 
-// ib: 1 / beta, divided once on the host instead of once per mode (with the
-// changes named at k_spec_tail the 256^3 preconditioner 2085 -> 1883 us, of which
-// this kernel 242; 118 at the copy rate)
+// inv: 1 / (beta |k|^2) or 1 / (beta |k|^4) by |k|^2; null: divided per mode (with
+// the changes named at k_spec_tail the 256^3 preconditioner 2085 -> 1883 us, of
+// which this kernel 242; 118 at the copy rate)
 template <int NC, int D>
 __global__ void __launch_bounds__(256) k_spec_precond(const double2* __restrict__ R, double2* __restrict__ out,
-                                                      GridArgs g, int nc_, double ib, const double* __restrict__ Ci,
+                                                      GridArgs g, int nc_, double beta, const double* __restrict__ Ci,
                                                       int reg, const double* __restrict__ betas,
-                                                      const double* __restrict__ inv_k2) {
+                                                      const double* __restrict__ inv) {
   chain_enter();
   const long q = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= g.Nc) return;
-  if (betas) ib = 1.0 / betas[q >> g.lg1];
+  if (betas) beta = betas[q >> g.lg1];
   constexpr int d = D;
   const int nc = NC ? NC : nc_;
   const long Nc = g.Nc;
@@ -232,14 +234,15 @@ __global__ void __launch_bounds__(256) k_spec_precond(const double2* __restrict_
   const int kk = lead_k2<D>(m, g), kz = m.j[d - 1];
   double alpha, delta = 0.0;
   long qn = q;
+  auto scale = [&](int k2) { return inv ? __ldg(&inv[k2]) : 1.0 / (beta * sym_pow(k2, reg)); };
   if (kz == 0) {
-    const double s0 = kk == 0 ? 1.0 : ib * inv_pow(kk, reg, inv_k2);  // k = 0: the inverse is replaced by one
-    const double sN = ib * inv_pow(kk + g.M * g.M, reg, inv_k2);
+    const double s0 = kk == 0 ? 1.0 : scale(kk);  // k = 0: the inverse is replaced by one
+    const double sN = scale(kk + g.M * g.M);
     alpha = 0.5 * (s0 + sN);
     delta = 0.5 * (s0 - sN);
     qn = encode_neg<D>(q, m, g);
   } else {
-    alpha = ib * inv_pow(kk + kz * kz, reg, inv_k2);
+    alpha = scale(kk + kz * kz);
   }
   if constexpr (NC == 1) {  // the 1 x 1 Gram matrix is 1; all loads of a mode first
     double2 v[d], vn[d];
@@ -254,34 +257,34 @@ __global__ void __launch_bounds__(256) k_spec_precond(const double2* __restrict_
       if (kz == 0) r = make_double2(r.x + delta * vn[i].x, r.y - delta * vn[i].y);
       out[i * Nc + q] = r;
     }
-    return;
-  }
-  for (int i = 0; i < d; ++i) {
-    double2 v[NC ? NC : 1], vn[NC ? NC : 1];
-    if (NC) {
+  } else {
+    for (int i = 0; i < d; ++i) {
+      double2 v[NC ? NC : 1], vn[NC ? NC : 1];
+      if (NC) {
 #pragma unroll
-      for (int lp = 0; lp < NC; ++lp) {
-        v[lp] = R[(lp * d + i) * Nc + q];
-        if (kz == 0) vn[lp] = R[(lp * d + i) * Nc + qn];
-      }
-    }
-#pragma unroll
-    for (int l = 0; l < nc; ++l) {
-      double2 s = make_double2(0, 0), n = make_double2(0, 0);
-      for (int lp = 0; lp < nc; ++lp) {
-        const double c = __ldg(&Ci[l * nc + lp]);
-        const double2 x = NC ? v[NC ? lp : 0] : R[(lp * d + i) * Nc + q];
-        s.x += c * x.x;
-        s.y += c * x.y;
-        if (kz == 0) {
-          const double2 y = NC ? vn[NC ? lp : 0] : R[(lp * d + i) * Nc + qn];
-          n.x += c * y.x;
-          n.y += c * y.y;
+        for (int lp = 0; lp < NC; ++lp) {
+          v[lp] = R[(lp * d + i) * Nc + q];
+          if (kz == 0) vn[lp] = R[(lp * d + i) * Nc + qn];
         }
       }
-      double2 r = make_double2(alpha * s.x, alpha * s.y);
-      if (kz == 0) r = make_double2(r.x + delta * n.x, r.y - delta * n.y);
-      out[(l * d + i) * Nc + q] = r;
+#pragma unroll
+      for (int l = 0; l < nc; ++l) {
+        double2 s = make_double2(0, 0), n = make_double2(0, 0);
+        for (int lp = 0; lp < nc; ++lp) {
+          const double c = __ldg(&Ci[l * nc + lp]);
+          const double2 x = NC ? v[NC ? lp : 0] : R[(lp * d + i) * Nc + q];
+          s.x += c * x.x;
+          s.y += c * x.y;
+          if (kz == 0) {
+            const double2 y = NC ? vn[NC ? lp : 0] : R[(lp * d + i) * Nc + qn];
+            n.x += c * y.x;
+            n.y += c * y.y;
+          }
+        }
+        double2 r = make_double2(alpha * s.x, alpha * s.y);
+        if (kz == 0) r = make_double2(r.x + delta * n.x, r.y - delta * n.y);
+        out[(l * d + i) * Nc + q] = r;
+      }
     }
   }
 }
@@ -356,8 +359,8 @@ long inv_k2_count(const Grid& g) {
   return n;
 }
 
-void fill_inv_k2(double* inv_k2, long count, cudaStream_t s) {
-  k_inv_k2<<<blocks_for(count), 256, 0, s>>>(inv_k2, count);
+void fill_inv_k2(double* t, long count, double beta, int reg, cudaStream_t s) {
+  k_inv_k2<<<blocks_for(count), 256, 0, s>>>(t, count, beta, reg);
   REG_LAUNCH();
 }
 
@@ -379,9 +382,9 @@ void spec_tail(const Grid& g, cudaStream_t s, const double2* V, const double2* F
 }
 
 void spec_precond(const Grid& g, cudaStream_t s, const double2* R, double2* out, int nc, double beta,
-                  const double* Ci_dev, int reg, const double* betas, const double* inv_k2) {
+                  const double* Ci_dev, int reg, const double* betas, const double* inv) {
   auto run = [&](auto k) {
-    chain(k, blocks_for(g.Nc), 256, s, R, out, args(g), nc, 1.0 / beta, Ci_dev, reg, betas, inv_k2);
+    chain(k, blocks_for(g.Nc), 256, s, R, out, args(g), nc, beta, Ci_dev, reg, betas, inv);
   };
   auto dim = [&](auto d) {
     constexpr int D = decltype(d)::value;
