@@ -16,6 +16,10 @@
 // sum of the derivative matrix: 406 at L = 256, 924 at L = 512). G = 61, and 60
 // at L = 512, keeps every sum below 2^63.
 //
+// The two real lines of a complex line may have a scale each, since the operator is
+// real: rows do (k_rows_line), so that a row keeps its own accuracy beside one of
+// another size (with one scale 4e-9 of itself beside a row 10^8 times larger). Neighbouring columns share one: every column meets every row.
+//
 // Accuracy. The rounding of the inputs to 2^(e - S0) and of the products to one
 // unit is below that of double-precision butterflies: on smooth, blob and
 // white-noise lines the error against extended precision is 0.1 to 0.45 of the
@@ -150,9 +154,12 @@ __host__ __device__ constexpr int fx_headroom() {
   return L == 512 ? 60 : 61;
 }
 
-// the largest magnitude of a pair, as the high word of a double (ordered as an
-// unsigned number), its lowest bit set by low words: subnormal values without a
-// high word are not zero
+// a magnitude as the high word of a double (ordered as an unsigned number), its
+// lowest bit set by low words: subnormal values without a high word are not zero
+__device__ __forceinline__ unsigned fx_mag(double x) {
+  return ((unsigned)__double2hiint(x) & 0x7fffffffu) | min((unsigned)__double2loint(x), 1u);
+}
+// the larger one of a pair
 __device__ __forceinline__ unsigned fx_mag(double2 x) {
   return max((unsigned)__double2hiint(x.x) & 0x7fffffffu, (unsigned)__double2hiint(x.y) & 0x7fffffffu) |
          min((unsigned)(__double2loint(x.x) | __double2loint(x.y)), 1u);
@@ -174,29 +181,23 @@ __device__ __forceinline__ float fx_l1(double2 x) {
 template <int L, int R0>
 struct FxScale {
   static constexpr int S0 = fx_headroom<L>() - ilog2_c(R0), S = fx_headroom<L>() - ilog2_c(L);
+  enum Kind { PLAIN, TINY, HUGE_, NONFINITE, ZERO };
   int right, down;  // in1: shift of a value with exponent field 0; exponent shift of the results (high word)
+  Kind kind;
   bool plain;
   bool scaled = true;  // the forward stages scale (see Line::forward)
-  double pre, post;
   __device__ __forceinline__ explicit FxScale(unsigned mag) {
-    pre = post = 1.0;
     int e = (int)(mag >> 20);
-    plain = mag == 0 || (e >= 64 && e <= 1990);
-    if (mag == 0) e = 1023;
-    if (!plain) {
-      const double m = __hiloint2double((int)mag, -1);
-      if (e == 2047) {
-        pre = 0.0;
-        post = __hiloint2double(0x7ff80000, 0);
-        e = 1023;
-      } else {
-        pre = e < 64 ? 0x1p300 : 0x1p-300;
-        post = e < 64 ? 0x1p-300 : 0x1p300;
-        e = __double2hiint(m * pre) >> 20;
-      }
-    }
+    kind = mag == 0 ? ZERO : (e < 64 ? TINY : (e <= 1990 ? PLAIN : (e < 2047 ? HUGE_ : NONFINITE)));
+    plain = kind == PLAIN || kind == ZERO;
+    if (kind == ZERO || kind == NONFINITE) e = 1023;
+    else if (kind != PLAIN) e = __double2hiint(__hiloint2double((int)mag, -1) * pre()) >> 20;
     right = 63 - S0 + e;
     down = (e - 1022 - S) * (1 << 20);
+  }
+  __device__ __forceinline__ double pre() const { return kind == TINY ? 0x1p300 : (kind == HUGE_ ? 0x1p-300 : 1.0); }
+  __device__ __forceinline__ double post() const {
+    return kind == TINY ? 0x1p-300 : (kind == HUGE_ ? 0x1p300 : (kind == NONFINITE ? __hiloint2double(0x7ff80000, 0) : 1.0));
   }
   // Conversions in integer arithmetic: the double-precision unit converts two
   // values per clock and SM, and the epilogues need it. Rounded to nearest.
@@ -244,28 +245,49 @@ struct FxScale {
   }
   // results times 2^n as well
   __device__ __forceinline__ void times_pow2(int n) { down += n * (1 << 20); }
-  // v = x scaled, for the E values a thread holds of the line
+  // v = x scaled, for the E values a thread holds of the line; im: the scale of the
+  // imaginary parts, a real line of its own
   template <int E>
   __device__ __forceinline__ void in(const double2 (&x)[E], FxV (&v)[E]) const {
-    if (plain) {
+    in(*this, x, v);
+  }
+  template <int E>
+  __device__ __forceinline__ void in(const FxScale& im, const double2 (&x)[E], FxV (&v)[E]) const {
+    if (plain && im.plain) {
 #pragma unroll
-      for (int e = 0; e < E; ++e) v[e] = {in1(x[e].x), in1(x[e].y)};
+      for (int e = 0; e < E; ++e) v[e] = {in1(x[e].x), im.in1(x[e].y)};
     } else {
 #pragma unroll
       for (int e = 0; e < E; ++e)
-        v[e] = pre == 0.0 ? FxV{0, 0} : FxV{in1(x[e].x * pre), in1(x[e].y * pre)};
+        v[e] = {kind == NONFINITE ? 0 : in1(x[e].x * pre()), im.kind == NONFINITE ? 0 : im.in1(x[e].y * im.pre())};
     }
   }
-  __device__ __forceinline__ double back(long long r) const { return plain ? out1(r) : out1(r) * post; }
+  __device__ __forceinline__ double back(long long r) const { return plain ? out1(r) : out1(r) * post(); }
   // x = the conjugate of v, scaled back; INT: on the integer units
   template <bool INT, int E>
   __device__ __forceinline__ void out(const FxV (&v)[E], double2 (&x)[E]) const {
+    out<INT>(*this, v, x);
+  }
+  template <bool INT, int E>
+  __device__ __forceinline__ void out(const FxScale& im, const FxV (&v)[E], double2 (&x)[E]) const {
 #pragma unroll
     for (int e = 0; e < E; ++e)
-      x[e] = INT ? make_double2(out1i(v[e].x), out1i(-v[e].y)) : make_double2(out1(v[e].x), out1(-v[e].y));
-    if (!plain) {
+      x[e] = INT ? make_double2(out1i(v[e].x), im.out1i(-v[e].y)) : make_double2(out1(v[e].x), im.out1(-v[e].y));
+    if (!(plain && im.plain)) {
 #pragma unroll
-      for (int e = 0; e < E; ++e) x[e] = make_double2(x[e].x * post, x[e].y * post);
+      for (int e = 0; e < E; ++e) x[e] = make_double2(x[e].x * post(), x[e].y * im.post());
+    }
+  }
+  // a zero line beside another takes its roundings: none of them is its own
+  template <int E>
+  __device__ __forceinline__ void keep_zero(const FxScale& im, double2 (&x)[E]) const {
+    if (kind == ZERO) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) x[e].x = 0.0;
+    }
+    if (im.kind == ZERO) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) x[e].y = 0.0;
     }
   }
 };

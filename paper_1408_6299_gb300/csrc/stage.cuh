@@ -331,6 +331,16 @@ struct RowArgs {
   int rev;  // blocks take the rows from the last one
 };
 
+// In single precision the two rows of a complex line are brought to one size by
+// powers of two, and back: their errors mix, and a row keeps its own accuracy beside
+// a larger one (its derivative is its own, where those along strided axes mix all
+// rows; without, a row came out 1e-2 of itself wrong beside one 10^6 times its
+// size). row_binade: the power of two of a row's largest magnitude, as the bits of a
+// float, from the bits of that magnitude; 0 for a zero row, which so stays zero.
+__device__ __forceinline__ unsigned row_binade(unsigned mag) {
+  return min(max(mag & 0x7f800000u, min(mag, 1u) << 23), 253u << 23);
+}
+
 // Rows r and r + 1 (r even) form one complex line; a block holds NSEQ of them.
 // FEW (narrow plans): one or two lines per block, transformed by part of its
 // threads and their epilogue spread over all of them: the shortest pass where
@@ -350,11 +360,15 @@ struct RowTile {
   static constexpr int PADSH = P::R(0) == 16 ? 4 : (P::R(0) == 8 ? 3 : 2);
   static constexpr int RS = (L + (L >> PADSH) + 1) / 2 * 2;
   static constexpr int ROWS = NSEQ / NF * 2;  // rows of one field per block
+  // blocks per SM asked of the compiler (0: its choice). The wide two-field pass in
+  // single precision, bound by memory, is held to 56 registers: 256^3 mixed matvec
+  // 157.4 ms with 58, 154 so
+  static constexpr int min_blocks(int size) { return size == 4 && !NARROW && L <= 256 && EPI == EPI_ADV33 ? 9 : 0; }
 };
 
 template <class A, typename T, int L, bool NARROW, bool FEW, int EPI>
-__global__ void __launch_bounds__(RowTile<L, NARROW, FEW, EPI>::NT) k_rows_line(RowArgs<T> a,
-                                                                                 const typename A::W* __restrict__ tw) {
+__global__ void __launch_bounds__(RowTile<L, NARROW, FEW, EPI>::NT, RowTile<L, NARROW, FEW, EPI>::min_blocks(sizeof(T)))
+    k_rows_line(RowArgs<T> a, const typename A::W* __restrict__ tw) {
   using Tile = RowTile<L, NARROW, FEW, EPI>;
   using Ln = Line<A, L, NARROW>;
   typename A::W pre[Ln::NTW + 1];
@@ -393,19 +407,36 @@ __global__ void __launch_bounds__(RowTile<L, NARROW, FEW, EPI>::NT) k_rows_line(
     const RowSync<TS, Tile::NFFT> sync;
     auto at = [&](int p) { return b + p + (p >> Tile::PADSH); };
     if constexpr (A::SCALED) {
-      unsigned mag = 0;
+      unsigned mx = 0, my = 0;
 #pragma unroll
-      for (int e = 0; e < E; ++e) mag = max(mag, fx_mag(x[e]));
-      const FxScale<L, Ln::R0> sc(row_max<TS>(mag, reinterpret_cast<unsigned*>(b), j, sync));
-      sc.in(x, v);
+      for (int e = 0; e < E; ++e) {
+        mx = max(mx, fx_mag(x[e].x));
+        my = max(my, fx_mag(x[e].y));
+      }
+      row_max<TS>(mx, my, reinterpret_cast<unsigned*>(b), j, sync);
+      const FxScale<L, Ln::R0> sx(mx), sy(my);
+      sx.in(sy, x, v);
       Ln::derivative(v, j, at, sync, tw, pre);
-      sc.template out<true>(v, x);
+      sx.template out<true>(sy, v, x);
+      sx.keep_zero(sy, x);
     } else {
+      float mx = 0.f, my = 0.f;
 #pragma unroll
-      for (int e = 0; e < E; ++e) v[e] = A::in(x[e]);
+      for (int e = 0; e < E; ++e) {
+        mx = fmaxf(mx, fabsf(x[e].x));
+        my = fmaxf(my, fabsf(x[e].y));
+      }
+      unsigned bx = __float_as_uint(mx), by = __float_as_uint(my);
+      row_max<TS>(bx, by, reinterpret_cast<unsigned*>(b), j, sync);
+      bx = row_binade(bx);
+      by = row_binade(by);
+      const float2 to_one = make_float2(__uint_as_float(0x7f000000u - bx), __uint_as_float(0x7f000000u - by));
+      const float2 back = make_float2(__uint_as_float(bx), -__uint_as_float(by));  // of the conjugate
+#pragma unroll
+      for (int e = 0; e < E; ++e) v[e] = A::in(__fmul2_rn(x[e], to_one));
       Ln::derivative(v, j, at, sync, tw, pre);
 #pragma unroll
-      for (int e = 0; e < E; ++e) x[e] = A::out(v[e]);
+      for (int e = 0; e < E; ++e) x[e] = __fmul2_rn(v[e], back);
     }
     // the two real rows of the derivative, in place of the exchanged values
     if constexpr (Ln::S > 1) sync();

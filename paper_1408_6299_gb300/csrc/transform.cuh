@@ -34,19 +34,30 @@ __device__ __forceinline__ unsigned line_max(unsigned mag, unsigned* red, int c,
   }
 }
 
-// the same for the TS neighbouring threads j < TS of a row line; red: scratch of the line
+// the largest of two mags over the TS neighbouring threads j < TS of a row line; red: scratch of the line
 template <int TS, class Sync>
-__device__ __forceinline__ unsigned row_max(unsigned mag, unsigned* red, int j, const Sync& sync) {
+__device__ __forceinline__ void row_max(unsigned& mx, unsigned& my, unsigned* red, int j, const Sync& sync) {
+  if constexpr (TS < 32) {
 #pragma unroll
-  for (int o = 1; o < (TS < 32 ? TS : 32); o *= 2) mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, o));
+    for (int o = 1; o < TS; o *= 2) {
+      mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      my = max(my, __shfl_xor_sync(0xffffffffu, my, o));
+    }
+  } else {
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    my = __reduce_max_sync(0xffffffffu, my);
+  }
   if constexpr (TS > 32) {  // the line's warps exchange their maxima
-    red[j / 32] = mag;
+    red[j / 32] = mx;
+    red[TS / 32 + j / 32] = my;
     sync();
 #pragma unroll
-    for (int w = 0; w < TS / 32; ++w) mag = max(mag, red[w]);
+    for (int w = 0; w < TS / 32; ++w) {
+      mx = max(mx, red[w]);
+      my = max(my, red[TS / 32 + w]);
+    }
     sync();
   }
-  return mag;
 }
 
 // the same with the sum of l1
