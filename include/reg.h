@@ -64,7 +64,7 @@ typedef enum {
   REG_ECFL = 6,          /* CFL bound could not be met by step halving */
   REG_ELINESEARCH = 7,   /* Armijo line search exhausted its trials */
   REG_EMAXIT = 8,        /* outer iteration cap reached before the tolerance */
-  REG_ETIMEOUT = 9       /* a bounded device wait ran out */
+  REG_ETIMEOUT = 9       /* reserved: no call waits on the device with a bound */
 } reg_status;
 
 typedef enum { REG_H1 = 1, REG_H2 = 2 } reg_type;
@@ -372,8 +372,10 @@ REG_API reg_status reg_solve_batched(const reg_problem* problems, int count, int
  * CUDA graph whose conditional WHILE node iterates a check kernel (per-problem
  * forcing-term, curvature and Armijo decisions, the same operations as the
  * host loop) and an IF node with one iteration, so the host waits once per
- * loop instead of once per reduction (report device_loops = 1; the
- * environment variable REG_LOCKSTEP_GRAPHS=0 keeps the host-driven loops). */
+ * loop instead of once per reduction (report device_loops = 1). The
+ * environment variable REG_LOCKSTEP_GRAPHS=0 keeps the host-driven loops, which
+ * take the same iterates and were 7 to 17% faster on 256 pairs of 64^2 to 256^2.
+ * Read at every solve. */
 REG_API reg_status reg_solve_lockstep(const reg_problem* problems, int count, int precision,
                                       const reg_solve_opts* opts, reg_solve_report* reports, int max_stack);
 
@@ -453,16 +455,18 @@ REG_API reg_status reg_profile_flops(reg_ctx* ctx, double* flops);
  * per FMA): independent FMA chains in every thread of one wave of resident
  * blocks, the best of three launches timed with CUDA events after a warm-up.
  * Allocates and frees a small buffer; changes no device setting. The bench
- * reports the transforms' rate in the FP64 sweeps against it. Errors: REG_ECUDA (message in reg_last_error(NULL)). */
+ * reports the transforms' rate in the FP64 sweeps against it. Errors: REG_ECUDA
+ * (message in reg_last_error(NULL)). */
 REG_API reg_status reg_fp64_peak(double* gflops);
 
 /* Number of kernel launches issued by the library in this process so far. */
 REG_API long reg_launch_count(void);
 
-/* Failure-path check of the bounded waits (no counterpart in the paper): one
- * block polls an mbarrier that nothing completes, gives up after a bounded
- * number of polls, and counts the timeout. *counted: the timeouts read back and cleared (1 expected).
- * Faults, traps and hangs nothing; uses the current device. */
+/* Check of a bounded device wait (no counterpart in the paper): one block polls
+ * an mbarrier that nothing completes, gives up after a bounded number of polls,
+ * and counts the timeout. It stands for itself: no other kernel of the library
+ * waits. *counted: the timeouts read back and cleared (1 expected). Faults, traps
+ * and hangs nothing; uses the current device. */
 REG_API reg_status reg_selftest_copy_timeout(int* counted);
 
 #ifdef __cplusplus

@@ -12,16 +12,20 @@
 
 namespace reg {
 
+constexpr int kSMs = 152;
+
 // First statement of a kernel launched by chain() (internal.h): waits until the
 // previous kernel of the stream has finished and its writes are visible, then
 // lets the next one be set up. No effect under an ordinary launch. Blocks of
 // the next kernel that are placed early are spread unevenly, which costs more
 // than the launch gap where a kernel fills the GPU and its double-precision
 // unit (128^3 FP64 gradient: 47.6 -> 56.3 ms), so only single-precision stages
-// (early) and grids of at most one block per SM let it in before they end.
+// (early) and grids of at most one block per SM in x let it in before they end
+// (y: the time nodes of k_dot_fields, the one kernel with two dimensions, which runs
+// once or n_t / 4 times a sweep).
 __device__ __forceinline__ void chain_enter(bool early = false) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (early || gridDim.x <= 152) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (early || gridDim.x <= kSMs) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 template <typename T> struct Cx;

@@ -169,7 +169,7 @@ size_t write_wide_tables(unsigned char* out, long* off);
 // gradient 5600 us wide, 2170 narrow; 128^3 FP64 gradient 42.7 ms wide, 38.4
 // narrow; 128^3 mixed matvec, checkpoints every 8, 16.5 ms with this limit at
 // half, 12.6 here, 14.1 at double; 256^3 mixed matvec 180 ms wide, 246 narrow.
-inline bool narrow_lines(long wide_threads, int size) { return wide_threads < 152L * (size == 8 ? 1024 : 512); }
+inline bool narrow_lines(long wide_threads, int size) { return wide_threads < (long)kSMs * (size == 8 ? 1024 : 512); }
 // The lines that count for it. Plans round differently. In double precision the
 // plan follows the size of one problem, so that a problem has the same bits in any
 // stack and after its stack is rebuilt; in single precision that of the whole stack,

@@ -24,7 +24,7 @@ namespace reg {
 // Plans. Wide: radices 16 and 8, the fewest operations and exchanges per
 // point, for fields that fill the GPU. Narrow: radix 4, four values per
 // thread, four times the threads and a quarter of the serial work of one
-// thread, for fields whose wide form would leave most of the 152 SMs idle.
+// thread, for fields whose wide form would leave most of the SMs idle.
 // ---------------------------------------------------------------------------
 template <int L, bool NARROW>
 struct LinePlan;
@@ -54,6 +54,19 @@ REG_LINE_PLAN(256, true, 4, 4, 4, 4, 4, 1, 4)
 REG_LINE_PLAN(512, true, 5, 4, 4, 4, 4, 2, 4)
 #undef REG_LINE_PLAN
 
+// threads of a wide line
+inline int wide_threads(int L) {
+  switch (L) {
+    case 8: return LinePlan<8, false>::TS;
+    case 16: return LinePlan<16, false>::TS;
+    case 32: return LinePlan<32, false>::TS;
+    case 64: return LinePlan<64, false>::TS;
+    case 128: return LinePlan<128, false>::TS;
+    case 256: return LinePlan<256, false>::TS;
+    default: return LinePlan<512, false>::TS;
+  }
+}
+
 // radix of forward stage s, of inverse stage s, and the product of the
 // radices before stage s
 template <class P>
@@ -80,6 +93,16 @@ __host__ __device__ constexpr int line_tw_offset(int s, bool inv) {
   int off = inv ? line_tw_block<P>(false) : 0;
   for (int t = 1; t < s; ++t) off += line_ns<P>(t, inv) * line_radix<P>(t, inv);
   return off;
+}
+
+// Bytes of the fixed-point tables of the wide plans of every length: 3 blocks of
+// 16-byte entries (50,688 bytes).
+template <int L = 512>
+__host__ __device__ constexpr size_t wide_table_bytes() {
+  using P = LinePlan<L, false>;
+  const size_t n = (size_t)(2 * line_tw_block<P>(false) + line_tw_block<P>(true)) * 16;
+  if constexpr (L > 8) return n + wide_table_bytes<L / 2>();
+  else return n;
 }
 
 // Real additions and multiplications of one forward transform along the wide
@@ -249,8 +272,8 @@ struct Line {
   // Narrow kernels load a thread's forward twiddles into registers before they
   // wait for their predecessor, and the inverse ones ahead of the inverse
   // stages: a stage would otherwise begin with a miss to L2, as L1 is empty when
-  // a kernel starts (128^2 mixed matvec 680 -> 613 us, 512^2 FP64 transport 4913
-  // -> 4709). Order: stages s >= 1 of one direction.
+  // a kernel starts (128^2 mixed matvec 613 us, without it 680; 512^2 FP64 transport
+  // 4709 and 4913). Order: stages s >= 1 of one direction.
   static constexpr bool PRELOAD = NARROW;
   __host__ __device__ static constexpr int tw_index(int s, bool inv) {
     int n = 0;

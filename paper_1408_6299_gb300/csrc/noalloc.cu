@@ -23,6 +23,7 @@
 
 #include "../../include/reg.h"
 #include "internal.h"
+#include "line.cuh"
 
 using namespace reg;
 
@@ -30,7 +31,7 @@ namespace {
 
 // Fixed scratch: 64 MiB per GPU that loads the library, held until exit.
 constexpr size_t kScratchBytes = 64ull << 20;
-constexpr size_t kTableBytes = 64ull << 10;   // twiddle tables (about 25 KiB used)
+constexpr size_t kTableBytes = 64ull << 10;   // twiddle tables (write_wide_tables)
 constexpr size_t kGramBytes = 16 * 16 * 8;    // inverse Gram matrix, n_c <= 16
 static __device__ __align__(256) unsigned char g_precond_scratch[kScratchBytes];
 
@@ -70,8 +71,8 @@ int setup_device(int dev) {
   void* p = nullptr;
   cudaError_t e = cudaGetSymbolAddress(&p, g_precond_scratch);
   if (e != cudaSuccess) return (int)e;
+  static_assert(wide_table_bytes() <= kTableBytes, "the tables have to fit");
   const size_t n = write_wide_tables(nullptr, S.tw_off);
-  if (n > kTableBytes) return (int)cudaErrorInvalidValue;
   write_wide_tables(g_table_image, S.tw_off);
   e = cudaMemcpy(p, g_table_image, n, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // the transfer may still be under way (see upload)

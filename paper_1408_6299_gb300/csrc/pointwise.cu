@@ -425,7 +425,7 @@ void force_acc(T* fhi, T* flo, const ForceNodes<T>& F, int nc, int d, long N, cu
   ProfScope ps(KK_FORCE, s, (double)N * sizeof(T) * fields);
   const long n = N / Quad<T>::W;
   // double precision is bound by its unit: more threads up to larger grids
-  if (n * d <= 152L * (sizeof(T) == 8 ? 16384 : 2048)) chain(k_force<T, true>, nblk(n, 128) * d, 128, s, fhi, flo, F, nc, d, N);
+  if (n * d <= (long)kSMs * (sizeof(T) == 8 ? 16384 : 2048)) chain(k_force<T, true>, nblk(n, 128) * d, 128, s, fhi, flo, F, nc, d, N);
   else chain(k_force<T, false>, nblk(n, 128), 128, s, fhi, flo, F, nc, d, N);
 }
 

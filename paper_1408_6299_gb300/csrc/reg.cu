@@ -104,7 +104,8 @@ struct Work {
   DBuf<T> gx, gy;          // column derivatives of a stage
   DBuf<T> gx2, gy2;        // and of the second field of a two-field stage
   DBuf<T> yhS, srcS;       // state stage values and one source of the fused forward sweep
-  DBuf<T> G, q, va, vb, wa, wb;  // d fields
+  DBuf<T> G;               // d fields
+  DBuf<T> va, vb, wa, wb;  // velocities at time nodes (NodeVel)
   DBuf<T> m, yh, lam;            // fields
   DBuf<T> vcoef, wcoef;          // coefficient vectors in precision T
   DBuf<T> gm, gmh, ck;           // state gradients (all nodes or one segment), stage gradients, checkpoints
@@ -287,8 +288,8 @@ Spectral<float>& spectral<float>(reg_ctx* c) {
 // fields. For n_c > 1 the nodes are formed in groups of four, in two buffers by
 // turns: one launch and one read of the coefficients per group, and steps share
 // their nodes (64^3, n_c = 3: mixed matvec 1331 -> 1258 us, FP64 gradient 3739 ->
-// 3610). Fields of more than 128 MB take one node per launch, to bound the memory. A pointer stays valid while
-// only its node and the neighbouring ones are asked for.
+// 3610). Fields of more than 128 MB take one node per launch, to bound the memory. A
+// pointer stays valid while only its node and the neighbouring ones are asked for.
 template <typename T>
 struct NodeVel {
   reg_ctx* c;
@@ -375,8 +376,7 @@ void grad_fused(reg_ctx* c, const T* u, T* G) {
   adv<T>(c, u, nullptr, nullptr, nullptr, nullptr, nullptr, G, 1);
 }
 
-// fused divergence stage on lam: k = div(a lam), Heun stage update; e carries
-// the optional body-force accumulation of stage 1
+// divergence stage on lam: k = div(a lam), Heun stage update; e: an added source
 template <typename T>
 void divh(reg_ctx* c, const T* lam, const T* a, const T* y, T* out1, int stage,
           fused::DivEpi<T> e = fused::DivEpi<T>{}) {

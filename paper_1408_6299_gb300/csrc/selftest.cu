@@ -1,5 +1,6 @@
-// selftest.cu -- failure path of a bounded device wait: a wait that runs out is
-// counted and reported to the host, and the device stays usable.
+// selftest.cu -- a bounded device wait that runs out is counted and reported to the
+// host, and the device stays usable. The probe stands for itself: no kernel of the
+// solver waits on a copy or on another block.
 #include "../../include/reg.h"
 #include "internal.h"
 

@@ -451,7 +451,7 @@ __global__ void k_spec_upsample(const double2* __restrict__ P, double2* __restri
 
 void spec_upsample(const Grid& c, const Grid& f, cudaStream_t s, const double2* P, double2* Q, int nfields) {
   const long total = (long)nfields * f.Nc;
-  const int blocks = (int)std::min<long>((total + 255) / 256, 152L * 16);
+  const int blocks = (int)std::min<long>((total + 255) / 256, (long)kSMs * 16);
   k_spec_upsample<<<blocks, 256, 0, s>>>(P, Q, args(c), args(f), nfields, (double)f.N / (double)c.N);
   REG_LAUNCH();
 }

@@ -64,10 +64,11 @@ __device__ __forceinline__ void st_stream(C* p, C v) {
 }
 
 // y_{j+1} = y_j + h/2 (k_1 + k_2) from the predictor yh = y_j + h k_1, which
-// carries k_1: the first stage stores no second field. yh - y_j is exact, and
-// h k_2 and the result are rounded once each (256^3 mixed matvec 166 -> 156 ms
-// against storing y_j + h/2 k_1 as well; error of 32 steps against extended
-// precision 3.1e-16, 4.1e-16 that way).
+// carries k_1: the first stage stores no second field. yh - y_j is exact while the
+// increment is below y_j, else rounded to half a unit of the increment; h k_2 and
+// the result are rounded once each (256^3 mixed matvec 166 -> 156 ms against storing
+// y_j + h/2 k_1 as well; error of 32 steps against extended precision 3.1e-16,
+// 4.1e-16 that way).
 template <typename T>
 __device__ __forceinline__ T heun_end(T y, T yh, T k, T h) {
   return y + (T)0.5 * ((yh - y) + h * k);
@@ -181,8 +182,8 @@ struct ColJobs {
 // Threads of a block: TS along a line times TC neighbouring lines. VAR: 0, or 1
 // for the other block size the autotuner may choose; both give the same bits.
 // Wide: 128-byte row segments where the block allows it. Narrow: one warp or
-// one line (the most blocks; against four lines 512^2 FP64 transport 6370 ->
-// 4700 us, 128^2 mixed matvec 670 -> 613), or four lines and at least 128 threads.
+// one line (the most blocks; 512^2 FP64 transport 4700 us, with four lines at least
+// 6370, 128^2 mixed matvec 613 and 671), or four lines and at least 128 threads.
 template <class A, int L, bool NARROW, int VAR>
 struct ColTile {
   static constexpr int TS = LinePlan<L, NARROW>::TS;

@@ -84,25 +84,24 @@ void cols_L(const Spectral<T>& sp, const ColJob<T>* jobs, int nj, cudaStream_t s
   const long threads = plan_lines(g, (long)nj * g.Nc / L, sizeof(T)) * LinePlan<L, false>::TS;
   if (narrow_lines(threads, sizeof(T))) return cols_tuned<A, T, L, true, PROD>(sp, jobs, nj, st);
   if constexpr (sizeof(T) == 4)
-    if (threads >= 2 * 152 * 512) return cols_tuned<LinePair, T, L, false, PROD>(sp, jobs, nj, st);
+    if (threads >= 2 * kSMs * 512) return cols_tuned<LinePair, T, L, false, PROD>(sp, jobs, nj, st);
   cols_tuned<A, T, L, false, PROD>(sp, jobs, nj, st);
 }
 
 // Whether jobs along axes of two lengths share a launch: where both run narrow
 // plans, and in double precision only while every block has an SM to itself,
 // since k_cols_two holds the registers of its longest line and does not tune its
-// tile (32 x 16 x 8 mixed matvec 287 -> 262 us, 32 x 64 x 128 mixed Newton matvec
-// 2506 -> 2437, 64 x 16 x 8 FP64 matvec 967 -> 874; beyond the limit 64 x 128 x
+// tile (32 x 16 x 8 mixed matvec 287 -> 254 us, 32 x 64 x 128 mixed Newton matvec
+// 2506 -> 2422, 64 x 16 x 8 FP64 matvec 967 -> 871; beyond the limit 64 x 128 x
 // 16 FP64 transport 1056 -> 1132, 256 x 32 x 64 FP64 matvec 40.8 -> 44.5 ms).
 template <typename T>
 bool one_cols_launch(const Grid& g, int nj) {
   for (int a = 0; a < 2; ++a) {
     const int L = (int)g.n[a];
     if (L > 256) return false;
-    const int wide_ts = L > 64 ? L / 16 : (L == 16 ? 1 : L / 8);
-    if (!narrow_lines(plan_lines(g, (long)(nj / 2) * g.Nc / L, sizeof(T)) * wide_ts, sizeof(T))) return false;
+    if (!narrow_lines(plan_lines(g, (long)(nj / 2) * g.Nc / L, sizeof(T)) * wide_threads(L), sizeof(T))) return false;
   }
-  return sizeof(T) == 4 || nj * g.Nc / 4 <= 152L * kTwoNT;
+  return sizeof(T) == 4 || nj * g.Nc / 4 <= (long)kSMs * kTwoNT;
 }
 
 // jobs along both strided axes, of two lengths, in one launch of narrow plans
@@ -182,10 +181,10 @@ void rows_L(const Spectral<T>& sp, const RowArgs<T>& a, double bytes, cudaStream
           static_cast<const typename A::W*>(sp.line_table(L, NARROW, A::TABLE)));
   };
   const long lines = a.nrows / 2 * NF;
-  // few lines: 32^2 FP64 matvec 708 -> 529 us, 128^2 mixed 817 -> 613, 64^3 mixed
-  // 1627 -> 1426. Double precision, bound by arithmetic, loses earlier: 64^3
-  // gradient (2048 lines) 3790 -> 3940 us
-  const long few = 152L * (sizeof(T) == 8 ? 8 : 24);
+  // few lines, against full blocks at any size, all else equal: 32^2 FP64 matvec 529
+  // us (708 full), 128^2 mixed 613 (817), 64^3 mixed 1426 (1627). Double precision,
+  // bound by arithmetic, loses earlier: 64^3 gradient (2048 lines) 3940 us (3790)
+  const long few = (long)kSMs * (sizeof(T) == 8 ? 8 : 24);
   if (!narrow_lines(plan_lines(sp.grid(), lines, sizeof(T)) * LinePlan<L, false>::TS, sizeof(T))) go(std::false_type{}, std::false_type{});
   else if (lines <= few) go(std::true_type{}, std::true_type{});
   else go(std::true_type{}, std::false_type{});

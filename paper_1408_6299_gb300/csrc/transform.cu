@@ -194,8 +194,7 @@ FieldTransforms::FieldTransforms(const Grid& g, cudaStream_t s, TableFn tables, 
     : g_(g), s_(s), tables_(std::move(tables)), tuned_(tuned) {}
 
 bool FieldTransforms::narrow(int L, long lines) const {
-  return tuned_ && narrow_lines(plan_lines(g_, lines, sizeof(double)) *
-                                    (L == 512 ? 32 : (L > 64 ? L / 16 : (L == 16 ? 1 : L / 8))), sizeof(double));
+  return tuned_ && narrow_lines(plan_lines(g_, lines, sizeof(double)) * wide_threads(L), sizeof(double));
 }
 
 void FieldTransforms::cols(double2* U, int axis, int nf, bool inverse) const {

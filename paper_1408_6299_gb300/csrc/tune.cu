@@ -1,6 +1,6 @@
-// tune.cu -- the persistent store of the autotuner's choices (the column-pass
-// variant and the row-block size of the real-to-complex pass per shape,
-// precision and stack size; see fused_launch.cuh). Choices are kept per
+// tune.cu -- the persistent store of the autotuner's choices (tune.h: the tile of
+// a column pass and the lines per block of the whole-field real-to-complex rows, per
+// plan, precision, length and size). Choices are kept per
 // process and in a JSON file, one object of "key": choice pairs, so later
 // processes reuse them without timing trials. The file is
 // $REG_TUNE_CACHE when that is set (an empty value disables the file), else
