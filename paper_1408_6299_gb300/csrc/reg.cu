@@ -535,10 +535,12 @@ int force_group(const reg_ctx* c, int fields, int more, long bytes) {
   return K;
 }
 // The full Newton matvec keeps lam~, lam and the d fields of grad m~, the discrete
-// adjoint lam and its predictors: 1.2 GB, which bounds them to 3 nodes and 1 at 256^3
-// (single, double precision) and 4 (discrete adjoint, double). The trapezoid rule
-// keeps lam alone: 4.8 GB, 8 nodes up to 512^3 in single precision, 3 in double.
-constexpr long kRingBytes = 9L << 27, kLamRingBytes = 9L << 29;
+// adjoint lam and its predictors: 2.8 GB, all eight nodes of a full Newton matvec at
+// 256^3 in single precision (3 nodes: 4.13 -> 3.97 matvecs/s), 3 in double, where it
+// takes no more than the stages of half spectra before it did, and 1 beyond. The
+// trapezoid rule keeps lam alone: 4.8 GB, 8 nodes up to 512^3 in single precision, 3
+// in double.
+constexpr long kRingBytes = 21L << 27, kLamRingBytes = 9L << 29;
 template <typename T>
 int adjoint_group(const reg_ctx* c) {
   return c->quad ? force_group<T>(c, 2, 1, kRingBytes) : force_group<T>(c, 1, 1, kLamRingBytes);

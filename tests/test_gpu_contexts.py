@@ -235,8 +235,8 @@ def test_newton_over_more_nodes_than_a_force_group(n_t, ckpt):
 
 # grids whose rings hold fewer than eight nodes: full Newton 3 and 1, discrete adjoint 4, trapezoid 3
 @pytest.mark.parametrize("what,n,n_t,ckpt", [
-    ("newton", (256, 256, 128), 7, 0), ("newton", (256, 256, 256), 5, 0), ("newton", (256, 256, 128), 8, 4),
-    ("adjoint", (256, 256, 256), 9, 0), ("gradient", (512, 512, 512), 5, 0)])
+    ("newton", (256, 256, 256), 7, 0), ("newton", (512, 256, 256), 5, 0), ("newton", (256, 256, 256), 8, 4),
+    ("adjoint", (512, 256, 256), 9, 0), ("gradient", (512, 512, 512), 5, 0)])
 def test_rings_bounded_by_memory(what, n, n_t, ckpt):
     # fields that do not vary along the first axis: the same on 8 points there, where the rings hold eight nodes
     import torch
@@ -272,10 +272,10 @@ def test_rings_bounded_by_memory(what, n, n_t, ckpt):
 
 
 def test_newton_matvec_memory():
-    # 59 fields of a store-all context with two steps; the matvec held 58 before its body force was summed in
-    # groups, and five more fields than that are allowed here
+    # 59 fields of a store-all context with two steps where the rings are bounded; the matvec held 58 before its
+    # body force was summed in groups, and five more fields than that are allowed here
     import torch
-    n = (256, 256, 128)
+    n = (256, 256, 256)
     u, v = field(n, 7), coefs(n, 1, 0.001)
     Hv = torch.empty_like(v)
     R = lib.Registration(n, 2, 1, 1e-2, lib.REG_H1, False, lib.REG_FP64, 0, hessian=lib.REG_HESS_NEWTON)
