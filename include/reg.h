@@ -373,9 +373,9 @@ REG_API reg_status reg_solve_batched(const reg_problem* problems, int count, int
  * forcing-term, curvature and Armijo decisions, the same operations as the
  * host loop) and an IF node with one iteration, so the host waits once per
  * loop instead of once per reduction (report device_loops = 1). The
- * environment variable REG_LOCKSTEP_GRAPHS=0 keeps the host-driven loops, which
- * take the same iterates and were 7 to 17% faster on 256 pairs of 64^2 to 256^2.
- * Read at every solve. */
+ * environment variable REG_LOCKSTEP_GRAPHS=0, read at every solve, keeps the
+ * host-driven loops, which take the same iterates: on 256 pairs of 64^2 to 256^2
+ * from 3% slower to 17% faster, run by run. */
 REG_API reg_status reg_solve_lockstep(const reg_problem* problems, int count, int precision,
                                       const reg_solve_opts* opts, reg_solve_report* reports, int max_stack);
 
