@@ -21,8 +21,8 @@ constexpr int kSMs = 152;
 // than the launch gap where a kernel fills the GPU and its double-precision
 // unit (128^3 FP64 gradient: 47.6 -> 56.3 ms), so only single-precision stages
 // (early) and grids of at most one block per SM in x let it in before they end
-// (y: the time nodes of k_dot_fields, the one kernel with two dimensions, which runs
-// once or n_t / 4 times a sweep).
+// (y: the time nodes of k_dot_fields, the one kernel with two dimensions; 128^2 mixed
+// matvec 610 us whether they count or not).
 __device__ __forceinline__ void chain_enter(bool early = false) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (early || gridDim.x <= kSMs) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -333,3 +333,30 @@ def test_double_precision_bits_do_not_depend_on_the_stack():
         vs.append([p["v"] for p in probs[:2]])
     for a, b in zip(*vs):
         assert bool(a.any()) and torch.equal(a, b)
+
+
+TUNED_TRANSPORT = r"""
+import sys
+sys.path[:0] = [%r, %r]
+from test_gpu_contexts import coefs, empty, field
+from paper_1408_6299_gb300 import lib
+n = (512, 512)
+R = lib.Registration(n, 4, 1, 1e-2, lib.REG_H1, False, lib.REG_FP64, 0)
+R.transport(coefs(n, 1, 0.01), field(n, 7), empty(n))
+"""
+
+
+def test_tuner_takes_the_shorter_tile_each_time(tmp_path):
+    # columns of 512 points in double precision: one line per block, with four of them a transport takes 1.3 times
+    # as long
+    import json
+    import os
+    import subprocess
+    import sys
+    here = os.path.dirname(os.path.abspath(__file__))
+    for k in range(3):
+        cache = tmp_path / f"tune_cache_{k}.json"
+        subprocess.run([sys.executable, "-c", TUNED_TRANSPORT % (os.path.dirname(here), here)], check=True, timeout=600,
+                       env=dict(os.environ, REG_TUNE_CACHE=str(cache)))
+        picks = [v for key, v in json.loads(cache.read_text()).items() if "cols|plain" in key and "|f64|L512|" in key]
+        assert picks == [0], picks
