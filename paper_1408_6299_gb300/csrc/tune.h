@@ -45,22 +45,28 @@ int tuned_choice(const char* kind, int size, int L, long work, int nv, cudaStrea
     cudaEvent_t e0, e1;
     REG_CUDA(cudaEventCreate(&e0));
     REG_CUDA(cudaEventCreate(&e1));
+    auto timed = [&](int v, int launches) {
+      REG_CUDA(cudaEventRecord(e0, st));
+      for (int k = 0; k < launches; ++k) run(v);
+      REG_CUDA(cudaEventRecord(e1, st));
+      REG_CUDA(cudaEventSynchronize(e1));
+      float ms = 0;
+      REG_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+      return ms;
+    };
     // In turn, so that a disturbance does not meet one variant alone, and the shortest of
-    // them; four launches at a time, which overlap as in a sweep. Three single launches
-    // each, summed, took the slower one now and then: 512^2 FP64 transport 6200 us
-    // instead of 4660, 64^3 Stokes mixed matvec 1400 instead of 1305.
-    constexpr int kReps = 6, kChain = 4, kMaxVariants = 4;
+    // six; several launches at a time, which overlap as in a sweep, more of short ones.
+    // Three single launches each, summed, took the slower one now and then: 512^2 FP64
+    // transport 6200 us instead of 4660, 64^3 Stokes mixed matvec 1400 instead of 1305;
+    // with four of the 2 us passes at 32^2 (matvec 489 or 505 us) it was still chance.
+    constexpr int kReps = 6, kMaxVariants = 4;
     float best[kMaxVariants] = {1e30f, 1e30f, 1e30f, 1e30f};
     nv = nv < kMaxVariants ? nv : kMaxVariants;
     for (int v = 0; v < nv; ++v) run(v);
+    const int launches = timed(0, 1) < 0.03f ? 16 : 4;
     for (int r = 0; r < kReps; ++r)
       for (int v = 0; v < nv; ++v) {
-        REG_CUDA(cudaEventRecord(e0, st));
-        for (int k = 0; k < kChain; ++k) run(v);
-        REG_CUDA(cudaEventRecord(e1, st));
-        REG_CUDA(cudaEventSynchronize(e1));
-        float ms = 0;
-        REG_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+        const float ms = timed(v, launches);
         best[v] = ms < best[v] ? ms : best[v];
       }
     pick = 0;
