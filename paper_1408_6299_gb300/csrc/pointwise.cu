@@ -41,6 +41,7 @@ struct NodeWeights {
   template <int W>
   struct Sum {
     double s[W];
+    template <bool SHORT>
     __device__ __forceinline__ void add(int l, double c, const double* u) {
 #pragma unroll
       for (int k = 0; k < W; ++k) s[k] = l ? s[k] + c * u[k] : c * u[k];
@@ -50,7 +51,10 @@ struct NodeWeights {
       for (int k = 0; k < W; ++k) r[k] = s[k];
     }
   };
-  void set(int l, double c) { w[l] = c; }
+  bool set(int l, double c) {
+    w[l] = c;
+    return true;
+  }
 };
 template <>
 struct NodeWeights<float> {
@@ -60,27 +64,33 @@ struct NodeWeights<float> {
     static constexpr int P = W > 1 ? 2 : 1;
     using V = std::conditional_t<P == 2, float2, float>;
     FloatSum<V> s[W / P];
+    template <bool SHORT>
     __device__ __forceinline__ void add(int l, const FloatWeight& c, const float* u) {
 #pragma unroll
-      for (int k = 0; k < W / P; ++k) s[k].add(l, c, reinterpret_cast<const V*>(u)[k]);
+      for (int k = 0; k < W / P; ++k) s[k].template add<SHORT>(l, c, reinterpret_cast<const V*>(u)[k]);
     }
     __device__ __forceinline__ void rounded(float* r) const {
 #pragma unroll
       for (int k = 0; k < W / P; ++k) s[k].rounded(r + k * P);
     }
   };
-  void set(int l, double c) { w[l] = split_weight(c); }
+  // whether the weight is one float
+  bool set(int l, double c) {
+    w[l] = split_weight(c);
+    return w[l].mid == 0.f;
+  }
 };
 // The velocity at up to kVelGroup nodes, dN values each. NC: n_c where it is 2,
 // 3 or 4 (the loads of a point are then issued together and serve every node:
 // 64^3 with three coefficients 16 -> 4 us for one node), else 0. VEC: 16-byte
-// accesses, else single values.
+// accesses, else single values. SHORT: every weight is one float, as for powers of
+// two of time steps (double precision: one form).
 template <typename T>
 struct VelNodes {
   NodeWeights<T> b[kVelGroup];
   int count;
 };
-template <typename T, int NC, bool VEC>
+template <typename T, int NC, bool VEC, bool SHORT>
 __global__ void __launch_bounds__(128) k_vel_at(const T* __restrict__ coef, int nc_,
                                                 const __grid_constant__ VelNodes<T> nodes, T* __restrict__ out,
                                                 long dN) {
@@ -103,7 +113,7 @@ __global__ void __launch_bounds__(128) k_vel_at(const T* __restrict__ coef, int 
 #pragma unroll
     for (int l = 0; l < nc; ++l) {
       if (!NC) v[0] = c[l * n];
-      sum.add(l, b.w[l], v[NC ? l : 0].v);
+      sum.template add<SHORT>(l, b.w[l], v[NC ? l : 0].v);
     }
     Q s;
     sum.rounded(s.v);
@@ -382,16 +392,21 @@ template <typename T>
 void vel_at(const T* coef, int nc, const Coefs* b, int count, T* out, long dN, cudaStream_t s) {
   VelNodes<T> w;
   w.count = count;
+  bool one = true;
   for (int k = 0; k < kVelGroup; ++k)
-    for (int l = 0; l < 16; ++l) {
-      const double c = k < count && l < nc ? b[k].c[l] : 0.0;
-      w.b[k].set(l, c);
-    }
+    for (int l = 0; l < 16; ++l) one = w.b[k].set(l, k < count && l < nc ? b[k].c[l] : 0.0) && one;
   const bool vec = ((reinterpret_cast<uintptr_t>(coef) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
-  auto kern = !vec ? k_vel_at<T, 0, false>
-                   : (nc == 2 ? k_vel_at<T, 2, true>
-                              : (nc == 3 ? k_vel_at<T, 3, true> : (nc == 4 ? k_vel_at<T, 4, true> : k_vel_at<T, 0, true>)));
-  chain(kern, nblk(vec ? dN / Quad<T>::W : dN, 128), 128, s, coef, nc, w, out, dN);
+  auto run = [&](auto shrt) {
+    constexpr bool S = decltype(shrt)::value;
+    auto kern = !vec ? k_vel_at<T, 0, false, S>
+                     : (nc == 2 ? k_vel_at<T, 2, true, S>
+                                : (nc == 3 ? k_vel_at<T, 3, true, S>
+                                           : (nc == 4 ? k_vel_at<T, 4, true, S> : k_vel_at<T, 0, true, S>)));
+    chain(kern, nblk(vec ? dN / Quad<T>::W : dN, 128), 128, s, coef, nc, w, out, dN);
+  };
+  if constexpr (sizeof(T) == 4)
+    if (!one) return run(std::false_type{});
+  run(std::true_type{});
 }
 template void vel_at<float>(const float*, int, const Coefs*, int, float*, long, cudaStream_t);
 template void vel_at<double>(const double*, int, const Coefs*, int, double*, long, cudaStream_t);

@@ -104,7 +104,8 @@ struct FloatSum {
     two_sum(e, x, e, f);
     t = add_rn(t, f);
   }
-  // term l of the sum, in order
+  // term l of the sum, in order; SHORT: no weight has a second word
+  template <bool SHORT>
   REG_HD void add(int l, const FloatWeight& w, V u) {
     if (l == 0) {
       s = u;
@@ -121,7 +122,7 @@ struct FloatSum {
       put(fma_rn(h, u, n));
       put(d);
     }
-    if (w.mid != 0.f) {  // the weights of a power of two of time steps have none
+    if (!SHORT) {
       const V q = mul_rn(splat(w.mid, u), u);
       put(q);
       t = fma_rn(splat(w.lo, u), u, sub_rn(t, fma_rn(splat(-w.mid, u), u, q)));
